@@ -7,14 +7,15 @@
 //                  its tiles' gradient in registers and writes one partial vector
 //   k_mlp_adam     sums the partials in a fixed order, Adam update of the FP32 master
 //                  copy, refreshes the BF16 image used by the next forward pass
-//   k_mlp_forward  inference, one thread per sample
-//   k_mlp_invert   bisection on kappa for a target sigma, one thread per query
-// The weights are read as BF16 and every product is accumulated in FP32 (fmaf, in the
-// order of the sums' indices), so the training forward pass and k_mlp_forward give the
-// same bits for the same sample.
+//   k_mlp_forward  inference, one warp per sample or pair of samples
+//   k_mlp_invert   bisection on kappa for a target sigma, one warp per query or pair
+// The weights are read as BF16 and every product is accumulated in FP32 (fmaf; the hidden
+// layers in the order of the sums' indices, the output layer of inference over a fixed
+// butterfly of the lanes).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -335,30 +336,92 @@ __global__ void k_mlp_refresh_bf16(const float *__restrict__ master, __nv_bfloat
     if (p < NP) wbf[p] = __float2bfloat16_rn(master[p]);
 }
 
-// One sample through the network (weights in shared memory), standardised output.
-__device__ void forward_one(const SmemW &w, const float (&xs)[3], float (&o)[3]) {
-    float a[H];
+// ---------------------------------------------------------------------------------
+// Inference. A warp carries Q samples at a time; lane l owns hidden units 2l and 2l + 1 of
+// both layers and keeps their W2 rows in registers as unit pairs, so the 64 x 64 layer is 64
+// packed multiply-adds per lane and sample, each lane's sum in the order of k. The layer's
+// inputs go round the warp through shared memory, every activation stored twice (a, a) so
+// that one 16-byte broadcast load feeds two packed multiply-adds. The output sums are a
+// fixed butterfly over the lanes.
+// What bounds it: the serial chain of one evaluation (two erf-based activations and a
+// 64-long sum), times 42 evaluations for the inversion. One thread per sample (weights re-read
+// from shared memory) took 2346 us for 4097 inversions and as long for 24, 33 CTAs busy; a
+// warp per sample shortens the chain by 30 and fills the chip: lb_mlp_forward and
+// lb_mlp_invert_kappa of 4097 samples, copies included, 181 us against 2449 us.
+// ---------------------------------------------------------------------------------
+constexpr int kInferThreads = 128, kInferWarps = kInferThreads / 32;
+constexpr int kInferCtas = 2;      // resident CTAs per SM (the weights take 128 registers a thread)
+
+struct LaneWeights {
+    float2 w2[H];                  // (W2[2l][k], W2[2l+1][k])
+    float2 w1[IN], b1, b2;
+};
+
+__device__ __forceinline__ float2 bf16_pair(const __nv_bfloat16 *__restrict__ w, int i, int j) {
+    return make_float2(__bfloat162float(w[i]), __bfloat162float(w[j]));
+}
+
+__device__ __forceinline__ void load_lane_weights(LaneWeights &L, const __nv_bfloat16 *__restrict__ w) {
+    const int j = 2 * (threadIdx.x & 31);
+    const uint4 *r0 = reinterpret_cast<const uint4 *>(w + OW2 + j * H);   // 16-byte aligned rows
+    const uint4 *r1 = reinterpret_cast<const uint4 *>(w + OW2 + (j + 1) * H);
 #pragma unroll
-    for (int j = 0; j < H; ++j) {
-        float z = w.b1[j];
+    for (int c = 0; c < H / 8; ++c) {
+        const uint4 u = r0[c], v = r1[c];
+        const unsigned a[4] = {u.x, u.y, u.z, u.w}, b[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-        for (int i = 0; i < IN; ++i) z = fmaf(w.w1[j * IN + i], xs[i], z);
-        a[j] = gelu(z);
+        for (int e = 0; e < 4; ++e) {
+            L.w2[8 * c + 2 * e] = make_float2(__uint_as_float(a[e] << 16), __uint_as_float(b[e] << 16));
+            L.w2[8 * c + 2 * e + 1] = make_float2(__uint_as_float(a[e] & 0xffff0000u),
+                                                  __uint_as_float(b[e] & 0xffff0000u));
+        }
     }
-    // the outputs accumulate over j in order, like the output layer of k_mlp_grad
-    float acc0 = w.b3[0], acc1 = w.b3[1], acc2 = w.b3[2];
-    for (int j = 0; j < H; ++j) {
-        float z = w.b2[j];
 #pragma unroll
-        for (int k = 0; k < H; ++k) z = fmaf(w.w2[j * kW2Pitch + k], a[k], z);
-        const float g = gelu(z);
-        acc0 = fmaf(w.w3[0 * H + j], g, acc0);
-        acc1 = fmaf(w.w3[1 * H + j], g, acc1);
-        acc2 = fmaf(w.w3[2 * H + j], g, acc2);
+    for (int i = 0; i < IN; ++i) L.w1[i] = bf16_pair(w, OW1 + j * IN + i, OW1 + (j + 1) * IN + i);
+    L.b1 = bf16_pair(w, OB1 + j, OB1 + j + 1);
+    L.b2 = bf16_pair(w, OB2 + j, OB2 + j + 1);
+}
+static_assert((OW2 * 2) % 16 == 0 && (H * 2) % 16 == 0, "W2 rows are read in 16-byte words");
+
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
+// second-layer activations of the lane's two units for Q standardised samples
+template <int Q>
+__device__ __forceinline__ void hidden_units(const LaneWeights &L, const float (&xs)[Q][IN],
+                                             float4 (*act)[H / 2], float2 (&g)[Q]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        float2 z = L.b1;
+#pragma unroll
+        for (int i = 0; i < IN; ++i) z = fma2(L.w1[i], make_float2(xs[q][i], xs[q][i]), z);
+        const float a0 = gelu(z.x), a1 = gelu(z.y);
+        act[q][lane] = make_float4(a0, a0, a1, a1);
     }
-    o[0] = acc0;
-    o[1] = acc1;
-    o[2] = acc2;
+    __syncwarp();
+    float2 z[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) z[q] = L.b2;
+#pragma unroll
+    for (int k = 0; k < H / 2; ++k) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const float4 a = act[q][k];
+            z[q] = fma2(L.w2[2 * k], make_float2(a.x, a.y), z[q]);
+            z[q] = fma2(L.w2[2 * k + 1], make_float2(a.z, a.w), z[q]);
+        }
+    }
+    __syncwarp();                  // the activations are read: the next call may overwrite them
+#pragma unroll
+    for (int q = 0; q < Q; ++q) g[q] = make_float2(gelu(z[q].x), gelu(z[q].y));
+}
+
+// output c of one sample from the lanes' second-layer activations (the same in every lane)
+__device__ __forceinline__ float output_unit(float2 w3, float b3, float2 g) {
+    float p = fmaf(w3.y, g.y, w3.x * g.x);
+#pragma unroll
+    for (int m = 16; m > 0; m >>= 1) p += __shfl_xor_sync(0xffffffffu, p, m);
+    return p + b3;
 }
 
 __device__ __forceinline__ void standardise(const MlpNorm &nm, const float (&x)[3], float (&xs)[3]) {
@@ -370,57 +433,113 @@ __device__ __forceinline__ float sigma_of(const MlpNorm &nm, float o0) {
     return expf(fmaf(o0, nm.out_scale[0], nm.out_mean[0]));
 }
 
-__global__ void __launch_bounds__(128)
+template <int Q>
+__global__ void __launch_bounds__(kInferThreads, kInferCtas)
 k_mlp_forward(const __nv_bfloat16 *__restrict__ wbf, const MlpNorm *__restrict__ norm,
               const float *__restrict__ x, float *__restrict__ y, int n) {
-    __shared__ SmemW w;
-    __shared__ MlpNorm nm;
-    load_weights(w, wbf);
-    if (threadIdx.x == 0) nm = *norm;
-    __syncthreads();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float xv[3] = {x[3 * i], x[3 * i + 1], x[3 * i + 2]}, xs[3], o[3];
-    standardise(nm, xv, xs);
-    forward_one(w, xs, o);
-    y[3 * i + 0] = sigma_of(nm, o[0]);
-    y[3 * i + 1] = fmaf(o[1], nm.out_scale[1], nm.out_mean[1]);
-    y[3 * i + 2] = expf(fmaf(o[2], nm.out_scale[2], nm.out_mean[2]));
+    __shared__ float4 act[kInferWarps][Q][H / 2];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    LaneWeights L;
+    load_lane_weights(L, wbf);
+    float2 w3[OUT];
+    float b3[OUT];
+#pragma unroll
+    for (int c = 0; c < OUT; ++c) {
+        w3[c] = bf16_pair(wbf, OW3 + c * H + 2 * lane, OW3 + c * H + 2 * lane + 1);
+        b3[c] = __bfloat162float(wbf[OB3 + c]);
+    }
+    const MlpNorm nm = *norm;
+    for (int i = (blockIdx.x * kInferWarps + warp) * Q; i < n; i += gridDim.x * kInferWarps * Q) {
+        float xs[Q][IN];
+        float2 g[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int s = min(i + q, n - 1);   // a ragged last group repeats its last sample
+            const float xv[3] = {x[3 * s], x[3 * s + 1], x[3 * s + 2]};
+            standardise(nm, xv, xs[q]);
+        }
+        hidden_units<Q>(L, xs, act[warp], g);
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            float o[OUT];
+#pragma unroll
+            for (int c = 0; c < OUT; ++c) o[c] = output_unit(w3[c], b3[c], g[q]);
+            if (lane == 0 && i + q < n) {
+                y[3 * (i + q) + 0] = sigma_of(nm, o[0]);
+                y[3 * (i + q) + 1] = fmaf(o[1], nm.out_scale[1], nm.out_mean[1]);
+                y[3 * (i + q) + 2] = expf(fmaf(o[2], nm.out_scale[2], nm.out_mean[2]));
+            }
+        }
+    }
 }
 
-__global__ void __launch_bounds__(128)
+template <int Q>
+__global__ void __launch_bounds__(kInferThreads, kInferCtas)
 k_mlp_invert(const __nv_bfloat16 *__restrict__ wbf, const MlpNorm *__restrict__ norm,
-             const float *__restrict__ q, int n, float lo0, float hi0, float *__restrict__ kappa) {
-    __shared__ SmemW w;
-    __shared__ MlpNorm nm;
-    load_weights(w, wbf);
-    if (threadIdx.x == 0) nm = *norm;
-    __syncthreads();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float tt = q[3 * i], tau = q[3 * i + 1], target = q[3 * i + 2];
-    auto sigma = [&](float k) {
-        float xv[3] = {tt, k, tau}, xs[3], o[3];
-        standardise(nm, xv, xs);
-        forward_one(w, xs, o);
-        return sigma_of(nm, o[0]);
-    };
-    // one call site of the network (the bracket check is iterations -2 and -1)
-    float lo = lo0, hi = hi0;
-    bool ok = true;
-    for (int it = -2; it < kBisect && ok; ++it) {
-        const float k = it == -2 ? lo : (it == -1 ? hi : 0.5f * (lo + hi));
-        const float s = sigma(k);
-        if (it == -2) ok = s >= target;
-        else if (it == -1) ok = s <= target;
-        else if (s > target) lo = k;
-        else hi = k;
+             const float *__restrict__ qs, int n, float lo0, float hi0, float *__restrict__ kappa) {
+    __shared__ float4 act[kInferWarps][Q][H / 2];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    LaneWeights L;
+    load_lane_weights(L, wbf);
+    const float2 w3 = bf16_pair(wbf, OW3 + 2 * lane, OW3 + 2 * lane + 1);
+    const float b3 = __bfloat162float(wbf[OB3]);
+    const MlpNorm nm = *norm;
+    for (int i = (blockIdx.x * kInferWarps + warp) * Q; i < n; i += gridDim.x * kInferWarps * Q) {
+        float xs[Q][IN], lo[Q], hi[Q], target[Q];
+        bool ok[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int s = min(i + q, n - 1);   // a ragged last group repeats its last query
+            const float xv[3] = {qs[3 * s], 0.f, qs[3 * s + 1]};
+            standardise(nm, xv, xs[q]);        // T/T_c and tau_v stay through the bisection
+            target[q] = qs[3 * s + 2];
+            lo[q] = lo0;
+            hi[q] = hi0;
+            ok[q] = true;
+        }
+        // one call site of the network (the bracket check is iterations -2 and -1)
+#pragma unroll 1
+        for (int it = -2; it < kBisect; ++it) {
+            float k[Q];
+            float2 g[Q];
+            bool any = false;
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                k[q] = it == -2 ? lo[q] : (it == -1 ? hi[q] : 0.5f * (lo[q] + hi[q]));
+                xs[q][1] = (input_feature(k[q], 1) - nm.in_mean[1]) / nm.in_scale[1];
+            }
+            hidden_units<Q>(L, xs, act[warp], g);
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const float s = sigma_of(nm, output_unit(w3, b3, g[q]));
+                if (it == -2) ok[q] = s >= target[q];
+                else if (it == -1) ok[q] = ok[q] && s <= target[q];
+                else if (s > target[q]) lo[q] = k[q];
+                else hi[q] = k[q];
+                any |= ok[q];
+            }
+            if (!any) break;                   // the same in every lane
+        }
+#pragma unroll
+        for (int q = 0; q < Q; ++q)
+            if (lane == 0 && i + q < n)
+                kappa[i + q] = ok[q] ? 0.5f * (lo[q] + hi[q]) : __int_as_float(0x7fc00000);
     }
-    if (!ok) {
-        kappa[i] = __int_as_float(0x7fc00000);
-        return;
-    }
-    kappa[i] = 0.5f * (lo + hi);
+}
+
+// Samples per warp and grid for n samples: one per warp while every sample finds a resident
+// warp (the chain of one sample is then all there is), else two (their chains overlap and
+// share the weights' registers); the grid is at most the resident CTAs, which walk on.
+struct InferLaunch {
+    int q, grid;
+};
+
+InferLaunch infer_launch(int sms, int n) {
+    InferLaunch l;
+    l.q = n <= sms * kInferCtas * kInferWarps ? 1 : 2;
+    const int per_cta = kInferWarps * l.q;
+    l.grid = std::min((n + per_cta - 1) / per_cta, sms * kInferCtas);
+    return l;
 }
 
 }  // namespace
@@ -428,6 +547,7 @@ k_mlp_invert(const __nv_bfloat16 *__restrict__ wbf, const MlpNorm *__restrict__ 
 struct lb_mlp {
     cudaStream_t stream = nullptr;
     int max_samples = 0, n = 0, grad_ctas = 0;
+    int sms = 1;
     float *master = nullptr, *m1 = nullptr, *m2 = nullptr, *xn = nullptr, *tn = nullptr;
     float *part = nullptr, *lpart = nullptr, *grad = nullptr;
     __nv_bfloat16 *wbf = nullptr;
@@ -524,7 +644,10 @@ lb_status lb_mlp_create(lb_mlp **out, int max_samples, void *stream) {
     m->stream = static_cast<cudaStream_t>(stream);
     m->max_samples = max_samples;
     const size_t ns = (size_t)max_samples;
-    bool ok = cudaMalloc(&m->master, NP * sizeof(float)) == cudaSuccess &&
+    int dev = 0;
+    bool ok = cudaGetDevice(&dev) == cudaSuccess &&
+              cudaDeviceGetAttribute(&m->sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+              cudaMalloc(&m->master, NP * sizeof(float)) == cudaSuccess &&
               cudaMalloc(&m->m1, NP * sizeof(float)) == cudaSuccess &&
               cudaMalloc(&m->m2, NP * sizeof(float)) == cudaSuccess &&
               cudaMalloc(&m->grad, NP * sizeof(float)) == cudaSuccess &&
@@ -688,8 +811,9 @@ lb_status lb_mlp_forward(lb_mlp *m, const float *x, float *y, int n) {
     if (s != LB_OK) return s;
     LB_MCUDA(m, cudaStreamSynchronize(m->stream));
     LB_MCUDA(m, cudaMemcpy(m->io, x, (size_t)n * 3 * sizeof(float), cudaMemcpyHostToDevice));
-    k_mlp_forward<<<(n + 127) / 128, 128, 0, m->stream>>>(m->wbf, m->norm, m->io,
-                                                          m->io + (size_t)n * 3, n);
+    const InferLaunch l = infer_launch(m->sms, n);
+    (l.q == 1 ? k_mlp_forward<1> : k_mlp_forward<2>)<<<l.grid, kInferThreads, 0, m->stream>>>(
+        m->wbf, m->norm, m->io, m->io + (size_t)n * 3, n);
     LB_MCUDA(m, cudaGetLastError());
     LB_MCUDA(m, cudaStreamSynchronize(m->stream));
     LB_MCUDA(m, cudaMemcpy(y, m->io + (size_t)n * 3, (size_t)n * 3 * sizeof(float),
@@ -710,8 +834,9 @@ lb_status lb_mlp_invert_kappa(lb_mlp *m, const float *q, int n, float kappa_lo,
     if (s != LB_OK) return s;
     LB_MCUDA(m, cudaStreamSynchronize(m->stream));
     LB_MCUDA(m, cudaMemcpy(m->io, q, (size_t)n * 3 * sizeof(float), cudaMemcpyHostToDevice));
-    k_mlp_invert<<<(n + 127) / 128, 128, 0, m->stream>>>(m->wbf, m->norm, m->io, n, kappa_lo,
-                                                         kappa_hi, m->io + (size_t)n * 3);
+    const InferLaunch l = infer_launch(m->sms, n);
+    (l.q == 1 ? k_mlp_invert<1> : k_mlp_invert<2>)<<<l.grid, kInferThreads, 0, m->stream>>>(
+        m->wbf, m->norm, m->io, n, kappa_lo, kappa_hi, m->io + (size_t)n * 3);
     LB_MCUDA(m, cudaGetLastError());
     LB_MCUDA(m, cudaStreamSynchronize(m->stream));
     LB_MCUDA(m, cudaMemcpy(kappa, m->io + (size_t)n * 3, (size_t)n * sizeof(float),
