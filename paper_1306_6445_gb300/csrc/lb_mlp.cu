@@ -3,7 +3,7 @@
 //   k_mlp_prepare  one CTA: FP64 means / scales of the input features
 //                  (ln(1 - T/T_c), ln(1 - kappa), tau_v) and of the transformed targets,
 //                  standardised copies (float)
-//   k_mlp_grad     forward + backward over tiles of kTile samples; each CTA accumulates
+//   k_mlp_grad     forward + backward over tiles of 4 or 16 samples; each CTA accumulates
 //                  its tiles' gradient in registers and writes one partial vector
 //   k_mlp_adam     sums the partials in a fixed order, Adam update of the FP32 master
 //                  copy, refreshes the BF16 image used by the next forward pass
@@ -33,10 +33,10 @@ constexpr int OW1 = 0, OB1 = OW1 + H * IN, OW2 = OB1 + H, OB2 = OW2 + H * H, OW3
               OB3 = OW3 + OUT * H;
 static_assert(OB3 + OUT == NP, "parameter layout");
 
-constexpr int kTile = 16;          // samples per tile of k_mlp_grad
+constexpr int kSmallTile = 4, kLargeTile = 16;   // samples per tile of k_mlp_grad
 constexpr int kThreads = 256;      // k_mlp_grad block
 constexpr int kMaxGradCtas = 304;  // 2 x 152 SMs: bounds the partial-gradient buffer
-constexpr int kW2Pitch = H + 1;    // padded rows of W2 in shared memory (no bank conflicts)
+constexpr int kW2Pitch = H + 4;    // padded rows of W2 in shared memory (16-byte rows, no bank conflicts)
 constexpr int kGraphSteps = 50;
 constexpr int kMaxSamples = 1 << 20;
 constexpr int kMaxForward = 1 << 22;
@@ -52,6 +52,7 @@ struct MlpState {
     float lr, beta1, beta2, eps;
     float loss;        // loss of the last forward pass of k_mlp_grad (set by k_mlp_adam)
     int pad;
+    double pow1, pow2; // beta1^step, beta2^step of this step (advanced with step)
 };
 
 __device__ __forceinline__ float gelu(float z) {
@@ -66,19 +67,43 @@ __device__ __forceinline__ float gelu_grad(float z) {
 
 // Weights as float in shared memory; W2 rows padded to kW2Pitch.
 struct SmemW {
-    float w1[H * IN], b1[H], w2[H * kW2Pitch], b2[H], w3[OUT * H], b3[4];
+    __align__(16) float w2[H * kW2Pitch];
+    float w1[H * IN], b1[H], b2[H], w3[OUT * H], b3[4];
 };
 
-__device__ void load_weights(SmemW &w, const __nv_bfloat16 *__restrict__ wbf) {
-    for (int p = threadIdx.x; p < NP; p += blockDim.x) {
+__device__ __forceinline__ void load_weights(SmemW &w, const __nv_bfloat16 *__restrict__ wbf) {
+    static_assert(OW2 * 2 % 16 == 0 && H % 8 == 0, "W2 is read in 16-byte words of one row");
+    const uint4 *w2 = reinterpret_cast<const uint4 *>(wbf + OW2);
+#pragma unroll
+    for (int p = threadIdx.x; p < H * H / 8; p += kThreads) {
+        const uint4 u = w2[p];
+        const unsigned v[4] = {u.x, u.y, u.z, u.w};
+        float4 *d = reinterpret_cast<float4 *>(&w.w2[(p / (H / 8)) * kW2Pitch + (p % (H / 8)) * 8]);
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+            d[e] = make_float4(__uint_as_float(v[2 * e] << 16), __uint_as_float(v[2 * e] & 0xffff0000u),
+                               __uint_as_float(v[2 * e + 1] << 16),
+                               __uint_as_float(v[2 * e + 1] & 0xffff0000u));
+    }
+    for (int p = threadIdx.x; p < OW2; p += kThreads) {
         const float v = __bfloat162float(wbf[p]);
         if (p < OB1) w.w1[p] = v;
-        else if (p < OW2) w.b1[p - OB1] = v;
-        else if (p < OB2) { const int q = p - OW2; w.w2[(q / H) * kW2Pitch + q % H] = v; }
-        else if (p < OW3) w.b2[p - OB2] = v;
+        else w.b1[p - OB1] = v;
+    }
+    for (int p = OB2 + threadIdx.x; p < NP; p += kThreads) {
+        const float v = __bfloat162float(wbf[p]);
+        if (p < OW3) w.b2[p - OB2] = v;
         else if (p < OB3) w.w3[p - OW3] = v;
         else w.b3[p - OB3] = v;
     }
+}
+
+// output c of one sample from the lanes' second-layer activations (the same in every lane)
+__device__ __forceinline__ float output_unit(float2 w3, float b3, float2 g) {
+    float p = fmaf(w3.y, g.y, w3.x * g.x);
+#pragma unroll
+    for (int m = 16; m > 0; m >>= 1) p += __shfl_xor_sync(0xffffffffu, p, m);
+    return p + b3;
 }
 
 // Input features (ln(1 - T/T_c), ln(1 - kappa), tau_v) in float, as inference computes them.
@@ -162,23 +187,46 @@ k_mlp_prepare(float *__restrict__ x, float *__restrict__ y, int n, MlpNorm *__re
 }
 
 // ---------------------------------------------------------------------------------
-// Forward + backward. Block of 256 threads, tiles of 16 samples; the CTA walks tiles
+// Forward + backward. Block of 256 threads, tiles of TILE samples; the CTA walks tiles
 // blockIdx.x, blockIdx.x + gridDim.x, ... and keeps the gradient entries it owns in
 // registers:
-//   gW2: 16 per thread (k = t & 63, j = (t >> 6) + 4q)     gb2: threads 0..63
+//   gW2: 16 per thread (k = t & 63, j = 16 (t >> 6) + q)   gb2: threads 0..63
 //   gW3 / gb3: threads 0..191 / 192..194                   gW1 / gb1: 0..191 / 192..255
 // Activations of a tile live in shared memory; dz overwrites z in place.
+// What bounds it: the chain load weights -> layer -> layer -> back, once per tile, not the
+// arithmetic (14 MFLOP at 512 samples). So the tile is 4 samples (one per thread in the
+// hidden layers) while that gives at most kMaxGradCtas tiles, and 16 beyond, where a CTA's
+// weight load and partial vector are shared by more samples. Rows of W2 are padded to 68
+// floats: 16-byte row reads (forward) and column reads (backward) are both free of bank
+// conflicts. 50 Adam steps at 512 samples (both kernels, the call included): 439 us, against
+// 1469 us with 16-sample tiles (32 CTAs), a serial partial sum and no launch overlap.
 // ---------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads)
+__device__ __forceinline__ void grid_dependency_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void grid_dependents_launch() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <int TILE>
+__global__ void __launch_bounds__(kThreads, 2)
 k_mlp_grad(const __nv_bfloat16 *__restrict__ wbf, const float *__restrict__ xn,
            const float *__restrict__ tn, MlpState *__restrict__ st, int bump_step,
            float *__restrict__ part, float *__restrict__ lpart) {
+    constexpr int NQ = TILE / 4;          // samples per thread in the hidden layers
     __shared__ SmemW w;
-    __shared__ float sx[kTile * IN], dout[kTile * OUT];
-    __shared__ float z1[kTile * H], a1[kTile * H], z2[kTile * H], a2[kTile * H];
-    const int t = threadIdx.x;
+    __shared__ float sx[TILE * IN], dout[TILE * OUT], res[TILE * OUT];
+    __shared__ __align__(16) float z1[TILE * H], a1[TILE * H], z2[TILE * H], a2[TILE * H];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    // the weights are the previous kernel's: wait for it (programmatic dependent launch)
+    grid_dependency_wait();
+    grid_dependents_launch();
     const int n = st->n;
-    if (bump_step && blockIdx.x == 0 && t == 0) st->step += 1;
+    if (bump_step && blockIdx.x == 0 && t == 0) {
+        st->step += 1;
+        st->pow1 *= (double)st->beta1;
+        st->pow2 *= (double)st->beta2;
+    }
     load_weights(w, wbf);
     const float dscale = 2.0f / (3.0f * (float)n);
 
@@ -187,17 +235,14 @@ k_mlp_grad(const __nv_bfloat16 *__restrict__ wbf, const float *__restrict__ xn,
     for (int q = 0; q < 16; ++q) gw2[q] = 0.f;
     float gb2 = 0.f, g3 = 0.f, g1 = 0.f, lsum = 0.f;
 
-    const int jj = t & 63, sg = t >> 6;   // unit and sample group of the 4-per-thread loops
-    for (int base = blockIdx.x * kTile; base < n; base += gridDim.x * kTile) {
+    const int jj = t & 63, sg = t >> 6;   // unit and sample group (uniform in a warp)
+    for (int base = blockIdx.x * TILE; base < n; base += gridDim.x * TILE) {
         __syncthreads();   // weights loaded / previous tile consumed
-        if (t < kTile * IN) {
-            const int s = t / IN;
-            sx[t] = base + s < n ? xn[(size_t)base * IN + t] : 0.f;
-        }
+        if (t < TILE * IN) sx[t] = base + t / IN < n ? xn[(size_t)base * IN + t] : 0.f;
         __syncthreads();
         // layer 1
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < NQ; ++q) {
             const int s = sg + 4 * q;
             float z = w.b1[jj];
 #pragma unroll
@@ -208,44 +253,59 @@ k_mlp_grad(const __nv_bfloat16 *__restrict__ wbf, const float *__restrict__ xn,
         __syncthreads();
         // layer 2
         {
-            float acc[4];
+            float acc[NQ];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) acc[q] = w.b2[jj];
-#pragma unroll 8
-            for (int k = 0; k < H; ++k) {
-                const float wv = w.w2[jj * kW2Pitch + k];
+            for (int q = 0; q < NQ; ++q) acc[q] = w.b2[jj];
+#pragma unroll 4
+            for (int k = 0; k < H; k += 4) {
+                const float4 wv = *reinterpret_cast<const float4 *>(&w.w2[jj * kW2Pitch + k]);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) acc[q] = fmaf(wv, a1[(sg + 4 * q) * H + k], acc[q]);
+                for (int q = 0; q < NQ; ++q) {
+                    const float4 av = *reinterpret_cast<const float4 *>(&a1[(sg + 4 * q) * H + k]);
+                    acc[q] = fmaf(wv.x, av.x, acc[q]);
+                    acc[q] = fmaf(wv.y, av.y, acc[q]);
+                    acc[q] = fmaf(wv.z, av.z, acc[q]);
+                    acc[q] = fmaf(wv.w, av.w, acc[q]);
+                }
             }
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
+            for (int q = 0; q < NQ; ++q) {
                 z2[(sg + 4 * q) * H + jj] = acc[q];
                 a2[(sg + 4 * q) * H + jj] = gelu(acc[q]);
             }
         }
         __syncthreads();
-        // output layer and loss residual
-        if (t < kTile * OUT) {
-            const int s = t / OUT, c = t % OUT;
-            float o = w.b3[c];
-            for (int k = 0; k < H; ++k) o = fmaf(w.w3[c * H + k], a2[s * H + k], o);
-            const float r = base + s < n ? o - tn[(size_t)base * OUT + t] : 0.f;
-            dout[t] = r * dscale;
-            sx[t] = r;   // the tile's inputs are re-read below only by gW1: kept in xn
+        // output layer (summed as in inference) and loss residual: one warp per output
+        for (int p = warp; p < TILE * OUT; p += kThreads / 32) {
+            const int s = p / OUT, c = p % OUT;
+            const float2 g = *reinterpret_cast<const float2 *>(&a2[s * H + 2 * lane]);
+            const float o = output_unit(make_float2(w.w3[c * H + 2 * lane], w.w3[c * H + 2 * lane + 1]),
+                                        w.b3[c], g);
+            if (lane == 0) {
+                const float r = base + s < n ? o - tn[(size_t)base * OUT + p] : 0.f;
+                dout[p] = r * dscale;
+                res[p] = r;
+            }
         }
         __syncthreads();
-        if (t == 0)
-            for (int k = 0; k < kTile * OUT; ++k) lsum = fmaf(sx[k], sx[k], lsum);
+        if (warp == kThreads / 32 - 1) {
+            float l = lane < TILE * OUT ? res[lane] * res[lane] : 0.f;
+            if (TILE * OUT > 32 && lane + 32 < TILE * OUT) l = fmaf(res[lane + 32], res[lane + 32], l);
+#pragma unroll
+            for (int m = 16; m > 0; m >>= 1) l += __shfl_xor_sync(0xffffffffu, l, m);
+            lsum += l;
+        }
         // gW3, gb3; dz2 = (dout W3) * gelu'(z2) in place
         if (t < OUT * H) {
             const int c = t >> 6, k = t & 63;
-            for (int s = 0; s < kTile; ++s) g3 = fmaf(dout[s * OUT + c], a2[s * H + k], g3);
+#pragma unroll
+            for (int s = 0; s < TILE; ++s) g3 = fmaf(dout[s * OUT + c], a2[s * H + k], g3);
         } else if (t < OUT * H + OUT) {
             const int c = t - OUT * H;
-            for (int s = 0; s < kTile; ++s) g3 += dout[s * OUT + c];
+            for (int s = 0; s < TILE; ++s) g3 += dout[s * OUT + c];
         }
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < NQ; ++q) {
             const int s = sg + 4 * q;
             float d = 0.f;
 #pragma unroll
@@ -254,65 +314,102 @@ k_mlp_grad(const __nv_bfloat16 *__restrict__ wbf, const float *__restrict__ xn,
         }
         __syncthreads();
         // gW2, gb2; dz1 = (dz2 W2) * gelu'(z1) in place
-        for (int s = 0; s < kTile; ++s) {
+#pragma unroll 4
+        for (int s = 0; s < TILE; ++s) {
             const float av = a1[s * H + jj];
 #pragma unroll
-            for (int q = 0; q < 16; ++q) gw2[q] = fmaf(z2[s * H + sg + 4 * q], av, gw2[q]);
+            for (int q = 0; q < 16; q += 4) {
+                const float4 d = *reinterpret_cast<const float4 *>(&z2[s * H + 16 * sg + q]);
+                gw2[q] = fmaf(d.x, av, gw2[q]);
+                gw2[q + 1] = fmaf(d.y, av, gw2[q + 1]);
+                gw2[q + 2] = fmaf(d.z, av, gw2[q + 2]);
+                gw2[q + 3] = fmaf(d.w, av, gw2[q + 3]);
+            }
         }
         if (t < H)
-            for (int s = 0; s < kTile; ++s) gb2 += z2[s * H + t];
+            for (int s = 0; s < TILE; ++s) gb2 += z2[s * H + t];
         {
-            float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 8
-            for (int j = 0; j < H; ++j) {
-                const float wv = w.w2[j * kW2Pitch + jj];
+            float acc[NQ];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) acc[q] = fmaf(z2[(sg + 4 * q) * H + j], wv, acc[q]);
+            for (int q = 0; q < NQ; ++q) acc[q] = 0.f;
+#pragma unroll 4
+            for (int j = 0; j < H; j += 4) {
+                float wv[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) wv[e] = w.w2[(j + e) * kW2Pitch + jj];
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) {
+                    const float4 d = *reinterpret_cast<const float4 *>(&z2[(sg + 4 * q) * H + j]);
+                    acc[q] = fmaf(d.x, wv[0], acc[q]);
+                    acc[q] = fmaf(d.y, wv[1], acc[q]);
+                    acc[q] = fmaf(d.z, wv[2], acc[q]);
+                    acc[q] = fmaf(d.w, wv[3], acc[q]);
+                }
             }
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
+            for (int q = 0; q < NQ; ++q) {
                 const int s = sg + 4 * q;
                 z1[s * H + jj] = acc[q] * gelu_grad(z1[s * H + jj]);
             }
         }
         __syncthreads();
-        // gW1, gb1 (inputs re-read from global memory: sx now holds residuals)
+        // gW1, gb1
         if (t < H * IN) {
             const int j = t / IN, i = t % IN;
-            for (int s = 0; s < kTile; ++s) {
-                const float xv = base + s < n ? xn[(size_t)(base + s) * IN + i] : 0.f;
-                g1 = fmaf(z1[s * H + j], xv, g1);
-            }
+#pragma unroll
+            for (int s = 0; s < TILE; ++s) g1 = fmaf(z1[s * H + j], sx[s * IN + i], g1);
         } else {
             const int j = t - H * IN;
-            for (int s = 0; s < kTile; ++s) g1 += z1[s * H + j];
+#pragma unroll
+            for (int s = 0; s < TILE; ++s) g1 += z1[s * H + j];
         }
     }
     float *out = part + (size_t)blockIdx.x * NP;
 #pragma unroll
-    for (int q = 0; q < 16; ++q) out[OW2 + (sg + 4 * q) * H + jj] = gw2[q];
+    for (int q = 0; q < 16; ++q) out[OW2 + (16 * sg + q) * H + jj] = gw2[q];
     if (t < H) out[OB2 + t] = gb2;
     if (t < OUT * H) out[OW3 + t] = g3;
     else if (t < OUT * H + OUT) out[OB3 + t - OUT * H] = g3;
     if (t < H * IN) out[OW1 + t] = g1;
     else out[OB1 + t - H * IN] = g1;
-    if (t == 0) lpart[blockIdx.x] = lsum;
+    if (t == kThreads - 1) lpart[blockIdx.x] = lsum;
 }
 
-// Sum of the partial gradients in CTA order, then Adam on the FP32 master copy.
-__global__ void __launch_bounds__(256)
+// Sum of the partial gradients in a fixed order, then Adam on the FP32 master copy. A CTA
+// owns 32 parameters: warp w sums partials w, w + 8, ... (128-byte reads, several in
+// flight), then the eight sums are added in warp order; the bias corrections come from the
+// running powers of beta1 and beta2 that k_mlp_grad advances in FP64. One thread per
+// parameter with a serial sum of 32 partials and two FP64 pow took 17.6 us at 512 samples.
+constexpr int kAdamThreads = 256, kAdamParams = 32;
+
+__global__ void __launch_bounds__(kAdamThreads)
 k_mlp_adam(const float *__restrict__ part, const float *__restrict__ lpart, int nparts,
            MlpState *__restrict__ st, float *__restrict__ master, float *__restrict__ m1,
            float *__restrict__ m2, __nv_bfloat16 *__restrict__ wbf, float *__restrict__ grad_out) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        double l = 0.0;
-        for (int c = 0; c < nparts; ++c) l += (double)lpart[c];
-        st->loss = (float)(l / (3.0 * st->n));
-    }
-    if (p >= NP) return;
+    constexpr int NW = kAdamThreads / 32;
+    __shared__ float sums[NW][kAdamParams];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int p = blockIdx.x * kAdamParams + lane;
+    grid_dependency_wait();
+    grid_dependents_launch();
     float g = 0.f;
-    for (int c = 0; c < nparts; ++c) g += part[(size_t)c * NP + p];
+    if (p < NP) {
+#pragma unroll 8
+        for (int c = warp; c < nparts; c += NW) g += part[(size_t)c * NP + p];
+    }
+    sums[warp][lane] = g;
+    __syncthreads();
+    if (blockIdx.x == 0 && warp == 1) {   // the loss: lanes take every 32nd partial, then a butterfly
+        double l = 0.0;
+        for (int c = lane; c < nparts; c += 32) l += (double)lpart[c];
+#pragma unroll
+        for (int m = 16; m > 0; m >>= 1) l += __shfl_xor_sync(0xffffffffu, l, m);
+        if (lane == 0) st->loss = (float)(l / (3.0 * st->n));
+    }
+    if (warp != 0 || p >= NP) return;
+    g = 0.f;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) g += sums[w][lane];
     if (grad_out) {   // gradient only (no update)
         grad_out[p] = g;
         return;
@@ -322,9 +419,8 @@ k_mlp_adam(const float *__restrict__ part, const float *__restrict__ lpart, int 
     const float v = fmaf(b2, m2[p], (1.f - b2) * g * g);
     m1[p] = m;
     m2[p] = v;
-    const double tstep = (double)st->step;
-    const float c1 = (float)(1.0 - pow((double)b1, tstep));
-    const float c2 = (float)(1.0 - pow((double)b2, tstep));
+    const float c1 = (float)(1.0 - st->pow1);
+    const float c2 = (float)(1.0 - st->pow2);
     const float upd = st->lr * (m / c1) / (sqrtf(v / c2) + st->eps);
     const float th = master[p] - upd;
     master[p] = th;
@@ -414,14 +510,6 @@ __device__ __forceinline__ void hidden_units(const LaneWeights &L, const float (
     __syncwarp();                  // the activations are read: the next call may overwrite them
 #pragma unroll
     for (int q = 0; q < Q; ++q) g[q] = make_float2(gelu(z[q].x), gelu(z[q].y));
-}
-
-// output c of one sample from the lanes' second-layer activations (the same in every lane)
-__device__ __forceinline__ float output_unit(float2 w3, float b3, float2 g) {
-    float p = fmaf(w3.y, g.y, w3.x * g.x);
-#pragma unroll
-    for (int m = 16; m > 0; m >>= 1) p += __shfl_xor_sync(0xffffffffu, p, m);
-    return p + b3;
 }
 
 __device__ __forceinline__ void standardise(const MlpNorm &nm, const float (&x)[3], float (&xs)[3]) {
@@ -547,6 +635,7 @@ InferLaunch infer_launch(int sms, int n) {
 struct lb_mlp {
     cudaStream_t stream = nullptr;
     int max_samples = 0, n = 0, grad_ctas = 0;
+    int tile = 0;
     int sms = 1;
     float *master = nullptr, *m1 = nullptr, *m2 = nullptr, *xn = nullptr, *tn = nullptr;
     float *part = nullptr, *lpart = nullptr, *grad = nullptr;
@@ -579,16 +668,36 @@ bool finite3(const float *v) {
     return std::isfinite(v[0]) && std::isfinite(v[1]) && std::isfinite(v[2]);
 }
 
+// launch with programmatic dependent launch: the kernel's set-up overlaps the previous
+// kernel's end, it waits (griddepcontrol.wait) before its first access to global memory
+template <typename K, typename... A>
+cudaError_t launch_dependent(K kern, int grid, int block, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+// samples per tile for n samples (see k_mlp_grad)
+int tile_for(int n) { return n <= kSmallTile * kMaxGradCtas ? kSmallTile : kLargeTile; }
+
 cudaError_t launch_grad(lb_mlp *m, int bump, cudaStream_t s) {
-    k_mlp_grad<<<m->grad_ctas, kThreads, 0, s>>>(m->wbf, m->xn, m->tn, m->st, bump, m->part,
-                                                 m->lpart);
-    return cudaGetLastError();
+    return launch_dependent(tile_for(m->n) == kSmallTile ? k_mlp_grad<kSmallTile> : k_mlp_grad<kLargeTile>,
+                            m->grad_ctas, kThreads, s, (const __nv_bfloat16 *)m->wbf,
+                            (const float *)m->xn, (const float *)m->tn, m->st, bump, m->part,
+                            m->lpart);
 }
 
 cudaError_t launch_adam(lb_mlp *m, float *grad_out, cudaStream_t s) {
-    k_mlp_adam<<<(NP + 255) / 256, 256, 0, s>>>(m->part, m->lpart, m->grad_ctas, m->st,
-                                                m->master, m->m1, m->m2, m->wbf, grad_out);
-    return cudaGetLastError();
+    return launch_dependent(k_mlp_adam, (NP + kAdamParams - 1) / kAdamParams, kAdamThreads, s,
+                            (const float *)m->part, (const float *)m->lpart, m->grad_ctas, m->st,
+                            m->master, m->m1, m->m2, m->wbf, grad_out);
 }
 
 lb_status ensure_graph(lb_mlp *m) {
@@ -727,9 +836,11 @@ lb_status lb_mlp_set_data(lb_mlp *m, const float *x, const float *y, int n) {
     LB_MCUDA(m, cudaMemcpyAsync(&m->st->n, &n, sizeof(int), cudaMemcpyHostToDevice, m->stream));
     LB_MCUDA(m, cudaStreamSynchronize(m->stream));
     m->n = n;
-    const int tiles = (n + kTile - 1) / kTile;
+    const int tile = tile_for(n), tiles = (n + tile - 1) / tile;
     const int ctas = tiles < kMaxGradCtas ? tiles : kMaxGradCtas;
-    if (ctas != m->grad_ctas) drop_graph(m);
+    // the captured graph carries the grid and the tile kernel
+    if (ctas != m->grad_ctas || tile != m->tile) drop_graph(m);
+    m->tile = tile;
     m->grad_ctas = ctas;
     m->have_norm = true;
     return LB_OK;
@@ -778,8 +889,11 @@ lb_status lb_mlp_train(lb_mlp *m, int steps, float lr, float beta1, float beta2,
           beta2 < 1.f && eps > 0.f && std::isfinite(eps)))
         return mfail(m, LB_EINVAL, "bad Adam hyper-parameters");
     const float hp[4] = {lr, beta1, beta2, eps};
+    const double pw[2] = {std::pow((double)beta1, (double)m->steps),
+                          std::pow((double)beta2, (double)m->steps)};
     LB_MCUDA(m, cudaMemcpyAsync(&m->st->lr, hp, sizeof hp, cudaMemcpyHostToDevice, m->stream));
-    // the host array must stay valid until the copy ran
+    LB_MCUDA(m, cudaMemcpyAsync(&m->st->pow1, pw, sizeof pw, cudaMemcpyHostToDevice, m->stream));
+    // the host arrays must stay valid until the copies ran
     LB_MCUDA(m, cudaStreamSynchronize(m->stream));
     int left = steps;
     while (left >= kGraphSteps) {
