@@ -28,21 +28,26 @@ using Arith = typename ArithOf<T>::type;
 
 template <typename T>
 struct DevConsts {
-    T a, b4, RT;
+    T b4;                                  // Carnahan-Starling, 2/G folded in: see eos_psi
+    T rtc, ac, c3;
     T psi0, rho0;
     T th_v, th_m, th_l, rho1, rho2, p_rho1, p_rho2;
     T two_over_G;
-    T G, kG2, sig_coef;
-    T s_e, s_z, s_q, s_v;
-    // Eq. 17 coefficients per relaxed moment k: (1 - s_k), s_k, (1 - s_k/2) and the source
-    // weights 3 s_k / 2 (e, zeta) and -s_v (p_xx, p_xy), rounded once from FP64
-    T e_keep, e_half, e_src, z_keep, z_half, z_src, q_keep, q_half, v_keep, v_half, v_src;
-    // storage shift w_a rho_s: LB_BF16 stores f_a - w_a rho_s (zero for FP32 / FP64)
+    T G, mG12, qk3;                        // G, -G/12, kappa G / 6
+    // Eq. 17 coefficients of the moments as M^-1 uses them (collide): e/36, zeta/36, q/12,
+    // p/4. *_m multiplies the moment itself (1 - s); the others, in the order of the terms of
+    // collide, the equilibrium, the forcing (1 - s/2) and the source. Rounded once from FP64.
+    T e_m, e_w, e_r, e_fs, e_ss, e_tr;
+    T z_m, z_w, z_r, z_fs, z_ss, z_tr;
+    T q_m, q_j, q_f;
+    T v_m, v_u, v_f2, v_f4, v_q4, v_q16;
+    // storage shift w_a rho_s: LB_BF16 stores f_a - w_a rho_s (zero for FP32 / FP64); e_c and
+    // z_c are what it adds to e/36 and zeta/36 (collide)
     T wshift[9];
-    T rho_s;
+    T rho_s, e_c, z_c;
     // nu(rho) (open-boundary kernels only): sites with rho < rho_sw relax p_xx, p_xy at
-    // s_vV; the Eq. 17 coefficients for that rate
-    T rho_sw, s_vV, v_keep_V, v_half_V, v_src_V;
+    // s_vV; the v_* coefficients for that rate
+    T rho_sw, v_m_V, v_u_V, v_f2_V, v_f4_V, v_q4_V, v_q16_V;
     int stall_row;
     // LB_BF16 stochastic rounding: the step of the launch (the counter)
     unsigned sr_step;
@@ -61,25 +66,36 @@ struct BatchLattice {
 template <typename T>
 inline DevConsts<T> to_dev(const Consts &c) {
     DevConsts<T> d;
-    d.a = T(c.a); d.b4 = T(c.b4); d.RT = T(c.RT);
+    d.b4 = T(c.b4);
+    d.rtc = T(c.RT * c.two_over_G);
+    d.ac = T(c.a * c.two_over_G);
+    d.c3 = T(c.two_over_G / 3.0);
     d.psi0 = T(c.psi0); d.rho0 = T(c.rho0);
     d.th_v = T(c.th_v); d.th_m = T(c.th_m); d.th_l = T(c.th_l);
     d.rho1 = T(c.rho1); d.rho2 = T(c.rho2); d.p_rho1 = T(c.p_rho1); d.p_rho2 = T(c.p_rho2);
     d.two_over_G = T(c.two_over_G);
-    d.G = T(c.G); d.kG2 = T(c.kG2); d.sig_coef = T(c.sig_coef);
-    d.s_e = T(c.s_e); d.s_z = T(c.s_z); d.s_q = T(c.s_q); d.s_v = T(c.s_v);
-    d.e_keep = T(1.0 - c.s_e); d.e_half = T(1.0 - 0.5 * c.s_e); d.e_src = T(1.5 * c.s_e);
-    d.z_keep = T(1.0 - c.s_z); d.z_half = T(1.0 - 0.5 * c.s_z); d.z_src = T(1.5 * c.s_z);
-    d.q_keep = T(1.0 - c.s_q); d.q_half = T(1.0 - 0.5 * c.s_q);
-    d.v_keep = T(1.0 - c.s_v); d.v_half = T(1.0 - 0.5 * c.s_v); d.v_src = T(-c.s_v);
+    d.G = T(c.G); d.mG12 = T(-c.G / 12.0); d.qk3 = T(c.kG2 / 3.0);
+    const double e_keep = 1.0 - c.s_e, e_half = 1.0 - 0.5 * c.s_e;
+    d.e_m = T(e_keep / 36.0); d.e_w = T(c.s_e / 12.0); d.e_r = T(-c.s_e / 18.0);
+    d.e_fs = T(e_half / 6.0); d.e_ss = T(e_half * c.sig_coef / 5184.0); d.e_tr = T(c.s_e / 24.0);
+    const double z_keep = 1.0 - c.s_z, z_half = 1.0 - 0.5 * c.s_z;
+    d.z_m = T(z_keep / 36.0); d.z_w = T(-c.s_z / 12.0); d.z_r = T(c.s_z / 36.0);
+    d.z_fs = T(-z_half / 6.0); d.z_ss = T(-z_half * c.sig_coef / 5184.0); d.z_tr = T(-c.s_z / 24.0);
+    d.q_m = T((1.0 - c.s_q) / 12.0); d.q_j = T(-c.s_q / 12.0);
+    d.q_f = T(-(1.0 - 0.5 * c.s_q) / 12.0);
+    auto rate_v = [](double s, T &m, T &u, T &f2, T &f4, T &q4, T &q16) {
+        const double h = 1.0 - 0.5 * s;
+        m = T((1.0 - s) / 4.0); u = T(s / 4.0); f2 = T(h / 2.0); f4 = T(h / 4.0);
+        q4 = T(-s / 4.0); q16 = T(-s / 16.0);
+    };
+    rate_v(c.s_v, d.v_m, d.v_u, d.v_f2, d.v_f4, d.v_q4, d.v_q16);
+    rate_v(c.s_v_vapour, d.v_m_V, d.v_u_V, d.v_f2_V, d.v_f4_V, d.v_q4_V, d.v_q16_V);
     for (int a = 0; a < 9; ++a)
         d.wshift[a] = T((a == 0 ? 4.0 / 9.0 : (a <= 4 ? 1.0 / 9.0 : 1.0 / 36.0)) * c.shift_rho);
     d.rho_s = T(c.shift_rho);
+    d.e_c = T(c.shift_rho * (1.0 - e_keep) / 18.0);
+    d.z_c = T(c.shift_rho * (z_keep - 1.0) / 36.0);
     d.rho_sw = T(c.rho_sw);
-    d.s_vV = T(c.s_v_vapour);
-    d.v_keep_V = T(1.0 - c.s_v_vapour);
-    d.v_half_V = T(1.0 - 0.5 * c.s_v_vapour);
-    d.v_src_V = T(-c.s_v_vapour);
     d.stall_row = c.stall_row;
     d.sr_step = c.step_key;
     return d;
@@ -187,20 +203,22 @@ __device__ __forceinline__ T eos_psi(T rho, const DevConsts<T> &P, bool &bad) {
         bad |= !(rho > T(0));
         return rmul(P.psi0, lb_exp(-lb_div(P.rho0, rho)));
     } else {
-        T p;
+        T arg;   // 2 (p_EOS - rho/3) / G
         if constexpr (EOS == LB_EOS_CS) {
-            // rho RT (1 + eta + eta^2 - eta^3) / (1 - eta)^3 - a rho^2
+            // p = rho RT (1 + eta + eta^2 - eta^3) / (1 - eta)^3 - a rho^2; with 2/G folded
+            // into the constants, arg = rho RT' poly / den - rho (a' rho + 2/(3G))
             const T eta = rmul(P.b4, rho);
             const T om = rsub(T(1), eta);
-            const T poly = rfma(eta, rfma(eta, rsub(T(1), eta), T(1)), T(1));
-            const T num = rmul(rmul(rho, P.RT), poly);
-            p = rsub(lb_div(num, rmul(rmul(om, om), om)), rmul(P.a, rmul(rho, rho)));
+            const T poly = rfma(eta, rfma(eta, om, T(1)), T(1));
+            const T num = rmul(rmul(rho, P.rtc), poly);
+            const T low = rmul(rho, rfma(P.ac, rho, P.c3));
+            arg = rfma(num, lb_rcp(rmul(rmul(om, om), om)), -low);
         } else {
-            p = (rho <= P.rho1) ? rmul(rho, P.th_v)
-              : (rho < P.rho2) ? rfma(rsub(rho, P.rho1), P.th_m, P.p_rho1)
-                               : rfma(rsub(rho, P.rho2), P.th_l, P.p_rho2);
+            const T p = (rho <= P.rho1) ? rmul(rho, P.th_v)
+                      : (rho < P.rho2) ? rfma(rsub(rho, P.rho1), P.th_m, P.p_rho1)
+                                       : rfma(rsub(rho, P.rho2), P.th_l, P.p_rho2);
+            arg = rmul(rsub(p, rmul(rho, T(1.0 / 3.0))), P.two_over_G);
         }
-        const T arg = rmul(rsub(p, rmul(rho, T(1.0 / 3.0))), P.two_over_G);
         bad |= !(arg > T(0)) || !(rho > T(0));
         return lb_sqrt_pos(arg);
     }
@@ -260,6 +278,39 @@ __device__ __forceinline__ V2<double> vfma(V2<double> a, V2<double> b, V2<double
 }
 __device__ __forceinline__ V2<double> operator-(V2<double> a) { return {-a.x, -a.y}; }
 
+// one site (the lane of the scalar kernels), the same operations
+template <typename T>
+struct V1 {
+    T v;
+    __device__ __forceinline__ V1() {}
+    __device__ __forceinline__ V1(T a) : v(a) {}
+    __device__ __forceinline__ static V1 all(T a) { return V1(a); }
+};
+template <typename T>
+__device__ __forceinline__ V1<T> operator+(V1<T> a, V1<T> b) { return radd(a.v, b.v); }
+template <typename T>
+__device__ __forceinline__ V1<T> operator*(V1<T> a, V1<T> b) { return rmul(a.v, b.v); }
+template <typename T>
+__device__ __forceinline__ V1<T> operator-(V1<T> a, V1<T> b) { return rsub(a.v, b.v); }
+template <typename T>
+__device__ __forceinline__ V1<T> operator-(V1<T> a) { return V1<T>(-a.v); }
+template <typename T>
+__device__ __forceinline__ V1<T> vfma(V1<T> a, V1<T> b, V1<T> c) { return rfma(a.v, b.v, c.v); }
+
+template <typename T>
+__device__ __forceinline__ V2<T> vrcp(V2<T> a) { return V2<T>(lb_rcp(a.lo()), lb_rcp(a.hi())); }
+template <typename T>
+__device__ __forceinline__ V1<T> vrcp(V1<T> a) { return V1<T>(lb_rcp(a.v)); }
+// per lane: a >= limit ? x : y
+template <typename T>
+__device__ __forceinline__ V2<T> pick_ge(V2<T> a, T limit, T x, T y) {
+    return V2<T>(a.lo() >= limit ? x : y, a.hi() >= limit ? x : y);
+}
+template <typename T>
+__device__ __forceinline__ V1<T> pick_ge(V1<T> a, T limit, T x, T y) {
+    return V1<T>(a.v >= limit ? x : y);
+}
+
 // psi of two densities; lane by lane the same operations, in the same order and with
 // the same rounding, as eos_psi (so a site's psi does not depend on which lane or which
 // kernel computes it). `hi_valid` = false: the second lane is padding and is not checked.
@@ -271,12 +322,10 @@ __device__ __forceinline__ V2<T> eos_psi2(V2<T> rho, const DevConsts<T> &P, bool
         const V one = V::all(T(1));
         const V eta = V::all(P.b4) * rho;
         const V om = one - eta;
-        const V poly = vfma(eta, vfma(eta, one - eta, one), one);
-        const V num = (rho * V::all(P.RT)) * poly;
-        const V den = (om * om) * om;
-        const V q(lb_div(num.lo(), den.lo()), lb_div(num.hi(), den.hi()));
-        const V p = q - V::all(P.a) * (rho * rho);
-        const V arg = (p - rho * V::all(T(1.0 / 3.0))) * V::all(P.two_over_G);
+        const V poly = vfma(eta, vfma(eta, om, one), one);
+        const V num = (rho * V::all(P.rtc)) * poly;
+        const V low = rho * vfma(V::all(P.ac), rho, V::all(P.c3));
+        const V arg = vfma(num, vrcp((om * om) * om), -low);
         bad |= !(arg.lo() > T(0)) || !(rho.lo() > T(0));
         if (hi_valid) bad |= !(arg.hi() > T(0)) || !(rho.hi() > T(0));
         return V(lb_sqrt_pos(arg.lo()), lb_sqrt_pos(arg.hi()));
@@ -289,46 +338,50 @@ __device__ __forceinline__ V2<T> eos_psi2(V2<T> rho, const DevConsts<T> &P, bool
     }
 }
 
-// One collision for two sites: f[9] (populations after streaming, pre-collision) and the
-// potential at the sites and their neighbours pn[a] = psi(x + e_a) (pn[0] = psi(x)) give
-// f*[9] in place.
+// One collision for the sites of a vector V (V2: two sites, V1: one): f[9] (populations
+// after streaming, pre-collision) and the potential at the sites and their neighbours
+// pn[a] = psi(x + e_a) (pn[0] = psi(x)) give f*[9] in place.
 //
 // Arithmetic (identical in exact arithmetic to Eqs. 3, 5-8, 17-19 and f* = M^-1 m*):
-//   Sx, Sy = sum_a w_a psi(x+e_a) e_a,       F = -G psi(x) (Sx, Sy)                 (Eq. 7)
-//   Q = kappa G/2 psi(x) sum_a w_a (psi_a - psi) e_a e_a                           (Eq. 19)
-//   v = (j + F/2) / rho                                                             (Eq. 6)
-//   |F|^2 / psi^2 in Eq. 8 is evaluated as G^2 (Sx^2 + Sy^2) (no division by psi)
+//   12 S = 12 sum_a w_a psi(x+e_a) e_a,      F = -G psi(x) S                        (Eq. 7)
+//   Q = kappa G/2 psi(x) sum_a w_a (psi_a - psi) e_a e_a enters only as Q_xx + Q_yy,
+//   Q_xx - Q_yy and 4 Q_xy                                                         (Eq. 19)
+//   rho v = j + F/2                                                                 (Eq. 6)
+//   |F|^2 / psi^2 in Eq. 8 is evaluated as G^2 |S|^2 (no division by psi)
 //   m*_rho = rho and m*_j = j + F for every s_j (relaxing j towards rho v = j + F/2 and
 //   adding (1 - s_j/2) F cancels s_j exactly), so s_rho and s_j drop out;
-//   m*_k = (1 - s_k) m_k + s_k m_eq_k + (1 - s_k/2) S_k + C_k for the other moments.
+//   m*_k = (1 - s_k) m_k + s_k m_eq_k + (1 - s_k/2) S_k + C_k for the other moments, formed
+//   directly as e/36, zeta/36, q/12 and p/4, the multiples that M^-1 adds up, with the
+//   products with rho v taken before the division by rho is multiplied back.
+//   That is 124 operations and one reciprocal per site (FP64, whose pipe is the bound of
+//   the FP64 step; the form with unscaled moments took 150: 1000 x 700 FP64 steps in 280
+//   against 333 us, BF16 2048^2 steps in 63 against 65 us, FP32 2048^2 1 % faster).
 //   VSW: nu(rho) of Sec. V.C, the rate of p_xx, p_xy (and the weight of their source
 //   terms) taken per site as s_v where rho >= rho_sw, else s_vV.
 //   SH (LB_BF16): f holds the stored shifted populations f_a - w_a rho_s. The shift only
-//   moves the moments rho, e and zeta (M w = (1, -2, 1, 0, ..., 0)), so those are corrected
-//   by rho_s, and the same is taken off m* before M^-1 gives the shifted f* that is stored;
-//   f*_0 from mass conservation reads the same in shifted terms.
-template <typename T, bool VSW = false, bool SH = false>
-__device__ __forceinline__ void collide_pair(V2<T> (&f)[9], const V2<T> (&pn)[9],
-                                             const DevConsts<T> &P) {
-    using V = V2<T>;
-    const V third = V::all(T(1.0 / 3.0)), twelfth = V::all(T(1.0 / 12.0));
-    const V two = V::all(T(2)), four = V::all(T(4)), half = V::all(T(0.5));
+//   moves the moments rho, e and zeta (M w = (1, -2, 1, 0, ..., 0)): rho is corrected by
+//   rho_s, and what the shift adds to e and zeta before, and takes off after, the collision
+//   is one constant each (e_c, z_c); M^-1 then gives the shifted f* that is stored.
+template <typename T, bool VSW = false, bool SH = false, typename V>
+__device__ __forceinline__ void collide(V (&f)[9], const V (&pn)[9], const DevConsts<T> &P) {
+    const V four = V::all(T(4)), half = V::all(T(0.5)), mtwo = V::all(T(-2)), mfour = V::all(T(-4));
     const V pc = pn[0];
 
-    // Eq. 7 neighbour sums and Eq. 19 differences
+    // Eq. 7 neighbour sums (times 12) and the three combinations of Eq. 19
     const V dg_pp = pn[5] - pn[7];
     const V dg_mp = pn[6] - pn[8];
-    const V Sx = vfma(third, pn[1] - pn[3], twelfth * (dg_pp - dg_mp));
-    const V Sy = vfma(third, pn[2] - pn[4], twelfth * (dg_pp + dg_mp));
-    const V mGpc = V::all(-P.G) * pc;
-    const V Fx = mGpc * Sx;
-    const V Fy = mGpc * Sy;
-    const V dsum = vfma(V::all(T(-4)), pc, (pn[5] + pn[6]) + (pn[7] + pn[8]));
-    const V qpre = V::all(P.kG2) * pc;
-    const V tdsum = twelfth * dsum;
-    const V Qxx = qpre * vfma(third, vfma(V::all(T(-2)), pc, pn[1] + pn[3]), tdsum);
-    const V Qyy = qpre * vfma(third, vfma(V::all(T(-2)), pc, pn[2] + pn[4]), tdsum);
-    const V Qxy = qpre * (twelfth * ((pn[5] + pn[7]) - (pn[6] + pn[8])));
+    const V Sx = vfma(four, pn[1] - pn[3], dg_pp - dg_mp);
+    const V Sy = vfma(four, pn[2] - pn[4], dg_pp + dg_mp);
+    const V gp = V::all(P.mG12) * pc;
+    const V Fx = gp * Sx;
+    const V Fy = gp * Sy;
+    const V pa = pn[1] + pn[3], pb = pn[2] + pn[4];
+    const V p57 = pn[5] + pn[7], p68 = pn[6] + pn[8];
+    const V qp = V::all(P.qk3) * pc;
+    const V dsum = vfma(mfour, pc, p57 + p68);
+    const V tr = qp * vfma(half, dsum, vfma(mfour, pc, pa + pb));   // Q_xx + Q_yy
+    const V dq = qp * (pa - pb);                                     // Q_xx - Q_yy
+    const V qxy4 = qp * (p57 - p68);                                 // 4 Q_xy
 
     // moments m = M f
     const V ax = f[1] + f[3], ay = f[2] + f[4];
@@ -337,93 +390,81 @@ __device__ __forceinline__ void collide_pair(V2<T> (&f)[9], const V2<T> (&pn)[9]
     const V d57 = f[5] - f[7], d68 = f[6] - f[8];
     const V axis = ax + ay, diag = s57 + s68;
     const V rsum = f[0] + (axis + diag);       // sum of f (of the shifted f when SH)
-    V rs;                                      // rho_s in both lanes (SH)
-    if constexpr (SH) rs = V::all(P.rho_s);
     V rho = rsum;
-    if constexpr (SH) rho = rsum + rs;
-    const V jx = d13 + (d57 - d68);
-    const V jy = d24 + (d57 + d68);
-    V m1 = vfma(two, diag, vfma(V::all(T(-4)), f[0], -axis));
-    V m2 = vfma(four, f[0], vfma(V::all(T(-2)), axis, diag));
-    if constexpr (SH) {
-        m1 = vfma(V::all(T(-2)), rs, m1);
-        m2 = m2 + rs;
-    }
-    const V m4 = vfma(V::all(T(-2)), d13, d57 - d68);
-    const V m6 = vfma(V::all(T(-2)), d24, d57 + d68);
+    if constexpr (SH) rho = rsum + V::all(P.rho_s);
+    const V dm = d57 - d68, dp = d57 + d68;
+    const V jx = d13 + dm;
+    const V jy = d24 + dp;
+    const V m1 = vfma(-mtwo, diag, vfma(mfour, f[0], -axis));
+    const V m2 = vfma(four, f[0], vfma(mtwo, axis, diag));
+    const V m4 = vfma(mtwo, d13, dm);
+    const V m6 = vfma(mtwo, d24, dp);
     const V m7 = ax - ay;
     const V m8 = s57 - s68;
 
-    // Eq. 6 velocity and Eq. 3 equilibria
-    const V rinv(lb_rcp(rho.lo()), lb_rcp(rho.hi()));
-    const V vx = vfma(half, Fx, jx) * rinv;
-    const V vy = vfma(half, Fy, jy) * rinv;
-    const V vxx = vx * vx, vyy = vy * vy;
-    const V v2 = vxx + vyy;
-    const V meq1 = rho * vfma(V::all(T(3)), v2, V::all(T(-2)));
-    const V meq2 = rho * vfma(V::all(T(-3)), v2, V::all(T(1)));
-    const V rvx = rho * vx, rvy = rho * vy;
-    const V meq7 = rho * (vxx - vyy);
-    const V meq8 = rvx * vy;
-
-    // Eq. 5 forcing with S_1 of Eq. 8
-    const V S1 = vfma(V::all(T(6)), vfma(vx, Fx, vy * Fy), V::all(P.sig_coef) * vfma(Sx, Sx, Sy * Sy));
-    const V S7 = two * (vx * Fx - vy * Fy);
+    // Eq. 6 velocity; products for Eqs. 3, 5 and 8
+    const V rinv = vrcp(rho);
+    const V rvx = vfma(half, Fx, jx), rvy = vfma(half, Fy, jy);
+    const V vx = rvx * rinv, vy = rvy * rinv;
+    const V ryy = rvy * vy;
+    const V w = vfma(rvx, vx, ryy), u = vfma(rvx, vx, -ryy);     // rho (v_x^2 +- v_y^2)
+    const V xy = rvx * vy;
+    const V fyy = vy * Fy;
+    const V fs = vfma(vx, Fx, fyy), fd = vfma(vx, Fx, -fyy);     // v_x F_x +- v_y F_y
     const V S8 = vfma(vx, Fy, vy * Fx);
+    const V ss = vfma(Sx, Sx, Sy * Sy);
 
-    // Eq. 18 source
-    const V tr = Qxx + Qyy;
-
-    // Eq. 17, written as (1 - s) m + s m_eq + (1 - s/2) S + C
-    const V ms0 = rho;
-    V ms1 = vfma(V::all(P.e_keep), m1, vfma(V::all(P.s_e), meq1,
-                  vfma(V::all(P.e_half), S1, V::all(P.e_src) * tr)));
-    V ms2 = vfma(V::all(P.z_keep), m2, vfma(V::all(P.s_z), meq2,
-                  -vfma(V::all(P.z_half), S1, V::all(P.z_src) * tr)));
-    const V ms3 = jx + Fx;
-    const V ms4 = vfma(V::all(P.q_keep), m4, -vfma(V::all(P.s_q), rvx, V::all(P.q_half) * Fx));
-    const V ms5 = jy + Fy;
-    const V ms6 = vfma(V::all(P.q_keep), m6, -vfma(V::all(P.s_q), rvy, V::all(P.q_half) * Fy));
-    V vkeep = V::all(P.v_keep), vs = V::all(P.s_v), vhalf = V::all(P.v_half);
-    V vsrc = V::all(P.v_src);
-    if constexpr (VSW) {
-        const bool lo = rho.lo() >= P.rho_sw, hi = rho.hi() >= P.rho_sw;
-        vkeep = V(lo ? P.v_keep : P.v_keep_V, hi ? P.v_keep : P.v_keep_V);
-        vs = V(lo ? P.s_v : P.s_vV, hi ? P.s_v : P.s_vV);
-        vhalf = V(lo ? P.v_half : P.v_half_V, hi ? P.v_half : P.v_half_V);
-        vsrc = V(lo ? P.v_src : P.v_src_V, hi ? P.v_src : P.v_src_V);
+    // Eq. 17, scaled as M^-1 uses the moments
+    V et = V::all(P.e_tr) * tr, zt = V::all(P.z_tr) * tr;
+    if constexpr (SH) {
+        et = vfma(V::all(P.e_tr), tr, V::all(P.e_c));
+        zt = vfma(V::all(P.z_tr), tr, V::all(P.z_c));
     }
-    const V ms7 = vfma(vkeep, m7, vfma(vs, meq7, vfma(vhalf, S7, vsrc * (Qxx - Qyy))));
-    const V ms8 = vfma(vkeep, m8, vfma(vs, meq8, vfma(vhalf, S8, vsrc * Qxy)));
+    const V e36 = vfma(V::all(P.e_m), m1, vfma(V::all(P.e_r), rho, vfma(V::all(P.e_w), w,
+                       vfma(V::all(P.e_fs), fs, vfma(V::all(P.e_ss), ss, et)))));
+    const V z36 = vfma(V::all(P.z_m), m2, vfma(V::all(P.z_r), rho, vfma(V::all(P.z_w), w,
+                       vfma(V::all(P.z_fs), fs, vfma(V::all(P.z_ss), ss, zt)))));
+    const V qx = vfma(V::all(P.q_m), m4, vfma(V::all(P.q_j), rvx, V::all(P.q_f) * Fx));
+    const V qy = vfma(V::all(P.q_m), m6, vfma(V::all(P.q_j), rvy, V::all(P.q_f) * Fy));
+    V vm = V::all(P.v_m), vu = V::all(P.v_u), vf2 = V::all(P.v_f2), vf4 = V::all(P.v_f4);
+    V vq4 = V::all(P.v_q4), vq16 = V::all(P.v_q16);
+    if constexpr (VSW) {
+        vm = pick_ge(rho, P.rho_sw, P.v_m, P.v_m_V);
+        vu = pick_ge(rho, P.rho_sw, P.v_u, P.v_u_V);
+        vf2 = pick_ge(rho, P.rho_sw, P.v_f2, P.v_f2_V);
+        vf4 = pick_ge(rho, P.rho_sw, P.v_f4, P.v_f4_V);
+        vq4 = pick_ge(rho, P.rho_sw, P.v_q4, P.v_q4_V);
+        vq16 = pick_ge(rho, P.rho_sw, P.v_q16, P.v_q16_V);
+    }
+    const V pxx = vfma(vm, m7, vfma(vu, u, vfma(vf2, fd, vq4 * dq)));
+    const V pxy = vfma(vm, m8, vfma(vu, xy, vfma(vf4, S8, vq16 * qxy4)));
 
     // f* = M^-1 m*, M^-1 = M^T diag(1/9, 1/36, 1/36, 1/6, 1/12, 1/6, 1/12, 1/4, 1/4)
-    if constexpr (SH) {   // back to the moments of the shifted f*
-        ms1 = vfma(two, rs, ms1);
-        ms2 = ms2 - rs;
-    }
-    const V c9 = V::all(T(1.0 / 9.0)), c18 = V::all(T(1.0 / 18.0)), c36 = V::all(T(1.0 / 36.0));
-    const V c6 = V::all(T(1.0 / 6.0)), c12 = V::all(T(1.0 / 12.0)), c4 = V::all(T(0.25));
-    const V a0 = c9 * (SH ? rsum : ms0);
-    const V base_axis = a0 - vfma(c36, ms1, c18 * ms2);
-    const V base_diag = vfma(c18, ms1, vfma(c36, ms2, a0));
-    const V jx6 = c6 * ms3, qx6 = c6 * ms4, jy6 = c6 * ms5, qy6 = c6 * ms6;
-    const V pxx4 = c4 * ms7, pxy4 = c4 * ms8;
-    const V ax1 = jx6 - qx6, ay1 = jy6 - qy6;
-    f[1] = base_axis + (ax1 + pxx4);
-    f[3] = base_axis + (pxx4 - ax1);
-    f[2] = base_axis + (ay1 - pxx4);
-    f[4] = base_axis - (ay1 + pxx4);
-    const V xp = vfma(c12, ms4, jx6), yp = vfma(c12, ms6, jy6);
+    const V c6 = V::all(T(1.0 / 6.0));
+    const V a0 = V::all(T(1.0 / 9.0)) * rsum;
+    const V base_axis = vfma(mtwo, z36, a0 - e36);
+    const V base_diag = vfma(-mtwo, e36, a0 + z36);
+    const V jx6 = c6 * (jx + Fx), jy6 = c6 * (jy + Fy);
+    const V ax1 = vfma(mtwo, qx, jx6), ay1 = vfma(mtwo, qy, jy6);
+    f[1] = base_axis + (ax1 + pxx);
+    f[3] = base_axis + (pxx - ax1);
+    f[2] = base_axis + (ay1 - pxx);
+    f[4] = base_axis - (ay1 + pxx);
+    const V xp = jx6 + qx, yp = jy6 + qy;
     const V xy_p = xp + yp, xy_m = xp - yp;
-    f[5] = base_diag + (xy_p + pxy4);
-    f[6] = base_diag - (xy_m + pxy4);
-    f[7] = base_diag - (xy_p - pxy4);
-    f[8] = base_diag + (xy_m - pxy4);
+    f[5] = base_diag + (xy_p + pxy);
+    f[6] = base_diag - (xy_m + pxy);
+    f[7] = base_diag - (xy_p - pxy);
+    f[8] = base_diag + (xy_m - pxy);
     // f*_0 from mass conservation, rho - sum_{a>0} f*_a, instead of (m*_0 - m*_1 + m*_2)/9:
-    // with the rounded constants 1/9, 1/18, 1/36 the column sums of M^-1 are not exactly
-    // (1, 0, ..., 0), which in FP32 adds mass at about 7e-9 per step; this way the only
-    // error is one unbiased rounding.
-    f[0] = rsum - (((f[1] + f[3]) + (f[2] + f[4])) + ((f[5] + f[7]) + (f[6] + f[8])));
+    // with the rounded constants the column sums of M^-1 are not exactly (1, 0, ..., 0), which
+    // in FP32 adds mass at about 7e-9 per step; this way the only error is one unbiased
+    // rounding. In FP64 the eight f*_a sum to 4 (base_axis + base_diag) up to their own
+    // unbiased roundings, two operations instead of eight.
+    if constexpr (std::is_same<T, double>::value)
+        f[0] = vfma(mfour, base_axis + base_diag, rsum);
+    else
+        f[0] = rsum - (((f[1] + f[3]) + (f[2] + f[4])) + ((f[5] + f[7]) + (f[6] + f[8])));
 }
 
 }  // namespace lbm

@@ -239,7 +239,7 @@ __device__ __forceinline__ V2<T> lds_pair(const T *p) {
 
 // The step kernels work on the stored values themselves: for LB_BF16 the shifted
 // f_a - w_a rho_s (exactly, as FP32), which the collision corrects in moment space
-// (collide_pair with SH), so neither the loads nor the stores apply the shift.
+// (collide with SH), so neither the loads nor the stores apply the shift.
 template <typename T>
 __device__ __forceinline__ Arith<T> stored_val(T v) {
     if constexpr (std::is_same<T, __nv_bfloat16>::value) return __bfloat162float(v);
@@ -545,7 +545,7 @@ __device__ __forceinline__ int march(const CUtensorMap *tmap, T *__restrict__ go
             pn[6] = V2<A>(qL, q0.lo());
             pn[7] = V2<A>(mL, m0.lo());
             pn[8] = V2<A>(m0.hi(), mR);
-            collide_pair<A, BC == 2, std::is_same<T, __nv_bfloat16>::value>(fc, pn, P);
+            collide<A, BC == 2, std::is_same<T, __nv_bfloat16>::value>(fc, pn, P);
 
             const int x = x0 + c0;
             const unsigned idx = (unsigned)yr * (unsigned)pitch + (unsigned)(x + GH<T>);
@@ -824,7 +824,7 @@ __device__ __forceinline__ int march_stage(const CUtensorMap *tmap, T *__restric
             pn[6] = V2<A>(qL, q0.lo());
             pn[7] = V2<A>(mL, m0.lo());
             pn[8] = V2<A>(m0.hi(), mR);
-            collide_pair<A, BC == 2, std::is_same<T, __nv_bfloat16>::value>(fc, pn, P);
+            collide<A, BC == 2, std::is_same<T, __nv_bfloat16>::value>(fc, pn, P);
 
             const int x = x0 + c0;
             const unsigned idx = (unsigned)y * (unsigned)pitch + (unsigned)(x + GH<T>);
