@@ -29,22 +29,22 @@ using Arith = typename ArithOf<T>::type;
 template <typename T>
 struct DevConsts {
     T b4;                                  // Carnahan-Starling, 2/G folded in: see eos_psi
-    T rtc, ac, c3;
+    T rtc, a2, c3;
     T psi0, rho0;
     T th_v, th_m, th_l, rho1, rho2, p_rho1, p_rho2;
     T two_over_G;
     T G, mG12, qk3;                        // G, -G/12, kappa G / 6
-    // Eq. 17 coefficients of the moments as M^-1 uses them (collide): e/36, zeta/36, q/12,
-    // p/4. *_m multiplies the moment itself (1 - s); the others, in the order of the terms of
-    // collide, the equilibrium, the forcing (1 - s/2) and the source. Rounded once from FP64.
-    T e_m, e_w, e_r, e_fs, e_ss, e_tr;
-    T z_m, z_w, z_r, z_fs, z_ss, z_tr;
+    // Eq. 17 coefficients of the moments as M^-1 uses them (collide): (e + 2 rho)/36,
+    // (zeta - rho)/36, q/12, p/4. *_m multiplies the moment itself (1 - s); the others, in the
+    // order of the terms of collide, the equilibrium, the forcing (1 - s/2) and the source.
+    // Rounded once from FP64.
+    T e_m, e_w, e_fs, e_ss, e_tr;
+    T z_m, z_w, z_fs, z_ss, z_tr;
     T q_m, q_j, q_f;
     T v_m, v_u, v_f2, v_f4, v_q4, v_q16;
-    // storage shift w_a rho_s: LB_BF16 stores f_a - w_a rho_s (zero for FP32 / FP64); e_c and
-    // z_c are what it adds to e/36 and zeta/36 (collide)
+    // storage shift w_a rho_s: LB_BF16 stores f_a - w_a rho_s (zero for FP32 / FP64)
     T wshift[9];
-    T rho_s, e_c, z_c;
+    T rho_s;
     // nu(rho) (open-boundary kernels only): sites with rho < rho_sw relax p_xx, p_xy at
     // s_vV; the v_* coefficients for that rate
     T rho_sw, v_m_V, v_u_V, v_f2_V, v_f4_V, v_q4_V, v_q16_V;
@@ -68,7 +68,7 @@ inline DevConsts<T> to_dev(const Consts &c) {
     DevConsts<T> d;
     d.b4 = T(c.b4);
     d.rtc = T(c.RT * c.two_over_G);
-    d.ac = T(c.a * c.two_over_G);
+    d.a2 = T(c.a * c.two_over_G);
     d.c3 = T(c.two_over_G / 3.0);
     d.psi0 = T(c.psi0); d.rho0 = T(c.rho0);
     d.th_v = T(c.th_v); d.th_m = T(c.th_m); d.th_l = T(c.th_l);
@@ -76,10 +76,10 @@ inline DevConsts<T> to_dev(const Consts &c) {
     d.two_over_G = T(c.two_over_G);
     d.G = T(c.G); d.mG12 = T(-c.G / 12.0); d.qk3 = T(c.kG2 / 3.0);
     const double e_keep = 1.0 - c.s_e, e_half = 1.0 - 0.5 * c.s_e;
-    d.e_m = T(e_keep / 36.0); d.e_w = T(c.s_e / 12.0); d.e_r = T(-c.s_e / 18.0);
+    d.e_m = T(e_keep / 36.0); d.e_w = T(c.s_e / 12.0);
     d.e_fs = T(e_half / 6.0); d.e_ss = T(e_half * c.sig_coef / 5184.0); d.e_tr = T(c.s_e / 24.0);
     const double z_keep = 1.0 - c.s_z, z_half = 1.0 - 0.5 * c.s_z;
-    d.z_m = T(z_keep / 36.0); d.z_w = T(-c.s_z / 12.0); d.z_r = T(c.s_z / 36.0);
+    d.z_m = T(z_keep / 12.0); d.z_w = T(-c.s_z / 12.0);   // times (zeta - rho)/3 = f_0 - sum f_1..4
     d.z_fs = T(-z_half / 6.0); d.z_ss = T(-z_half * c.sig_coef / 5184.0); d.z_tr = T(-c.s_z / 24.0);
     d.q_m = T((1.0 - c.s_q) / 12.0); d.q_j = T(-c.s_q / 12.0);
     d.q_f = T(-(1.0 - 0.5 * c.s_q) / 12.0);
@@ -93,8 +93,6 @@ inline DevConsts<T> to_dev(const Consts &c) {
     for (int a = 0; a < 9; ++a)
         d.wshift[a] = T((a == 0 ? 4.0 / 9.0 : (a <= 4 ? 1.0 / 9.0 : 1.0 / 36.0)) * c.shift_rho);
     d.rho_s = T(c.shift_rho);
-    d.e_c = T(c.shift_rho * (1.0 - e_keep) / 18.0);
-    d.z_c = T(c.shift_rho * (z_keep - 1.0) / 36.0);
     d.rho_sw = T(c.rho_sw);
     d.stall_row = c.stall_row;
     d.sr_step = c.step_key;
@@ -206,13 +204,16 @@ __device__ __forceinline__ T eos_psi(T rho, const DevConsts<T> &P, bool &bad) {
         T arg;   // 2 (p_EOS - rho/3) / G
         if constexpr (EOS == LB_EOS_CS) {
             // p = rho RT (1 + eta + eta^2 - eta^3) / (1 - eta)^3 - a rho^2; with 2/G folded
-            // into the constants, arg = rho RT' poly / den - rho (a' rho + 2/(3G))
+            // into the constants, arg = rho RT' poly / den - a' rho^2 - 2 rho/(3G)
             const T eta = rmul(P.b4, rho);
             const T om = rsub(T(1), eta);
             const T poly = rfma(eta, rfma(eta, om, T(1)), T(1));
             const T num = rmul(rmul(rho, P.rtc), poly);
-            const T low = rmul(rho, rfma(P.ac, rho, P.c3));
-            arg = rfma(num, lb_rcp(rmul(rmul(om, om), om)), -low);
+            const T q = rmul(num, lb_rcp(rmul(rmul(om, om), om)));
+            if constexpr (std::is_same<T, float>::value)   // the three terms rounded apart: see eos_psi2
+                arg = rsub(rsub(q, rmul(P.a2, rmul(rho, rho))), rmul(rho, P.c3));
+            else
+                arg = rfma(rho, -rfma(P.a2, rho, P.c3), q);
         } else {
             const T p = (rho <= P.rho1) ? rmul(rho, P.th_v)
                       : (rho < P.rho2) ? rfma(rsub(rho, P.rho1), P.th_m, P.p_rho1)
@@ -324,8 +325,16 @@ __device__ __forceinline__ V2<T> eos_psi2(V2<T> rho, const DevConsts<T> &P, bool
         const V om = one - eta;
         const V poly = vfma(eta, vfma(eta, om, one), one);
         const V num = (rho * V::all(P.rtc)) * poly;
-        const V low = rho * vfma(V::all(P.ac), rho, V::all(P.c3));
-        const V arg = vfma(num, vrcp((om * om) * om), -low);
+        const V q = num * vrcp((om * om) * om);
+        // In FP32 the three terms are rounded one by one: arg is a small difference of terms of
+        // the order of rho, and the fused form (two operations fewer) rounds 2 a rho + 2/3, twice
+        // their size; the pressure it left in a liquid at 0.8 T_c doubled the error of a droplet
+        // after 200 steps against FP64 (1.3e-6 against 6e-7).
+        V arg;
+        if constexpr (std::is_same<T, float>::value)
+            arg = (q - V::all(P.a2) * (rho * rho)) - rho * V::all(P.c3);
+        else
+            arg = vfma(rho, -vfma(V::all(P.a2), rho, V::all(P.c3)), q);
         bad |= !(arg.lo() > T(0)) || !(rho.lo() > T(0));
         if (hi_valid) bad |= !(arg.hi() > T(0)) || !(rho.hi() > T(0));
         return V(lb_sqrt_pos(arg.lo()), lb_sqrt_pos(arg.hi()));
@@ -351,17 +360,17 @@ __device__ __forceinline__ V2<T> eos_psi2(V2<T> rho, const DevConsts<T> &P, bool
 //   m*_rho = rho and m*_j = j + F for every s_j (relaxing j towards rho v = j + F/2 and
 //   adding (1 - s_j/2) F cancels s_j exactly), so s_rho and s_j drop out;
 //   m*_k = (1 - s_k) m_k + s_k m_eq_k + (1 - s_k/2) S_k + C_k for the other moments, formed
-//   directly as e/36, zeta/36, q/12 and p/4, the multiples that M^-1 adds up, with the
-//   products with rho v taken before the division by rho is multiplied back.
-//   That is 124 operations and one reciprocal per site (FP64, whose pipe is the bound of
+//   directly as (e + 2 rho)/36, (zeta - rho)/36, q/12 and p/4: the multiples that M^-1 adds
+//   up, and e and zeta as departures from rest, which are small, so that their roundings are
+//   too. The products with rho v are taken before the division by rho is multiplied back.
+//   That is 120 operations and one reciprocal per site (FP64, whose pipe is the bound of
 //   the FP64 step; the form with unscaled moments took 150: 1000 x 700 FP64 steps in 280
 //   against 333 us, BF16 2048^2 steps in 63 against 65 us, FP32 2048^2 1 % faster).
 //   VSW: nu(rho) of Sec. V.C, the rate of p_xx, p_xy (and the weight of their source
 //   terms) taken per site as s_v where rho >= rho_sw, else s_vV.
-//   SH (LB_BF16): f holds the stored shifted populations f_a - w_a rho_s. The shift only
-//   moves the moments rho, e and zeta (M w = (1, -2, 1, 0, ..., 0)): rho is corrected by
-//   rho_s, and what the shift adds to e and zeta before, and takes off after, the collision
-//   is one constant each (e_c, z_c); M^-1 then gives the shifted f* that is stored.
+//   SH (LB_BF16): f holds the stored shifted populations f_a - w_a rho_s. Of the quantities
+//   above the shift only moves rho (to which rho_s is added) and the rest state w_a rho, in
+//   which the shifted sum then gives the shifted f* that is stored.
 template <typename T, bool VSW = false, bool SH = false, typename V>
 __device__ __forceinline__ void collide(V (&f)[9], const V (&pn)[9], const DevConsts<T> &P) {
     const V four = V::all(T(4)), half = V::all(T(0.5)), mtwo = V::all(T(-2)), mfour = V::all(T(-4));
@@ -389,14 +398,15 @@ __device__ __forceinline__ void collide(V (&f)[9], const V (&pn)[9], const DevCo
     const V s57 = f[5] + f[7], s68 = f[6] + f[8];
     const V d57 = f[5] - f[7], d68 = f[6] - f[8];
     const V axis = ax + ay, diag = s57 + s68;
-    const V rsum = f[0] + (axis + diag);       // sum of f (of the shifted f when SH)
+    const V moving = axis + diag;
+    const V rsum = f[0] + moving;              // sum of f (of the shifted f when SH)
     V rho = rsum;
     if constexpr (SH) rho = rsum + V::all(P.rho_s);
     const V dm = d57 - d68, dp = d57 + d68;
     const V jx = d13 + dm;
     const V jy = d24 + dp;
-    const V m1 = vfma(-mtwo, diag, vfma(mfour, f[0], -axis));
-    const V m2 = vfma(four, f[0], vfma(mtwo, axis, diag));
+    const V m1 = vfma(four, diag, vfma(mtwo, f[0], axis));      // e + 2 rho
+    const V m2 = f[0] - axis;                                    // (zeta - rho)/3
     const V m4 = vfma(mtwo, d13, dm);
     const V m6 = vfma(mtwo, d24, dp);
     const V m7 = ax - ay;
@@ -415,15 +425,10 @@ __device__ __forceinline__ void collide(V (&f)[9], const V (&pn)[9], const DevCo
     const V ss = vfma(Sx, Sx, Sy * Sy);
 
     // Eq. 17, scaled as M^-1 uses the moments
-    V et = V::all(P.e_tr) * tr, zt = V::all(P.z_tr) * tr;
-    if constexpr (SH) {
-        et = vfma(V::all(P.e_tr), tr, V::all(P.e_c));
-        zt = vfma(V::all(P.z_tr), tr, V::all(P.z_c));
-    }
-    const V e36 = vfma(V::all(P.e_m), m1, vfma(V::all(P.e_r), rho, vfma(V::all(P.e_w), w,
-                       vfma(V::all(P.e_fs), fs, vfma(V::all(P.e_ss), ss, et)))));
-    const V z36 = vfma(V::all(P.z_m), m2, vfma(V::all(P.z_r), rho, vfma(V::all(P.z_w), w,
-                       vfma(V::all(P.z_fs), fs, vfma(V::all(P.z_ss), ss, zt)))));
+    const V de = vfma(V::all(P.e_m), m1, vfma(V::all(P.e_w), w, vfma(V::all(P.e_fs), fs,
+                      vfma(V::all(P.e_ss), ss, V::all(P.e_tr) * tr))));
+    const V dz = vfma(V::all(P.z_m), m2, vfma(V::all(P.z_w), w, vfma(V::all(P.z_fs), fs,
+                      vfma(V::all(P.z_ss), ss, V::all(P.z_tr) * tr))));
     const V qx = vfma(V::all(P.q_m), m4, vfma(V::all(P.q_j), rvx, V::all(P.q_f) * Fx));
     const V qy = vfma(V::all(P.q_m), m6, vfma(V::all(P.q_j), rvy, V::all(P.q_f) * Fy));
     V vm = V::all(P.v_m), vu = V::all(P.v_u), vf2 = V::all(P.v_f2), vf4 = V::all(P.v_f4);
@@ -441,30 +446,34 @@ __device__ __forceinline__ void collide(V (&f)[9], const V (&pn)[9], const DevCo
 
     // f* = M^-1 m*, M^-1 = M^T diag(1/9, 1/36, 1/36, 1/6, 1/12, 1/6, 1/12, 1/4, 1/4)
     const V c6 = V::all(T(1.0 / 6.0));
-    const V a0 = V::all(T(1.0 / 9.0)) * rsum;
-    const V base_axis = vfma(mtwo, z36, a0 - e36);
-    const V base_diag = vfma(-mtwo, e36, a0 + z36);
-    const V jx6 = c6 * (jx + Fx), jy6 = c6 * (jy + Fy);
-    const V ax1 = vfma(mtwo, qx, jx6), ay1 = vfma(mtwo, qy, jy6);
+    const V base_axis = vfma(V::all(T(1.0 / 9.0)), rsum, -vfma(V::all(T(2)), dz, de));
+    const V base_diag = vfma(V::all(T(1.0 / 36.0)), rsum, vfma(V::all(T(2)), de, dz));
+    // j* = j + F as 4 (j*/6 + q/12) along the diagonals and the rest along the axes, so that a
+    // rounded 1/6 (which in FP32 adds 3e-8 of the momentum at every step) does not enter it (a
+    // 600 x 225 splash after 160 steps, error against FP64: 2.6e-7 against 1.5e-6)
+    const V jxn = jx + Fx, jyn = jy + Fy;
+    const V xp = vfma(c6, jxn, qx), yp = vfma(c6, jyn, qy);
+    const V ax1 = vfma(mtwo, xp, half * jxn), ay1 = vfma(mtwo, yp, half * jyn);
     f[1] = base_axis + (ax1 + pxx);
     f[3] = base_axis + (pxx - ax1);
     f[2] = base_axis + (ay1 - pxx);
     f[4] = base_axis - (ay1 + pxx);
-    const V xp = jx6 + qx, yp = jy6 + qy;
     const V xy_p = xp + yp, xy_m = xp - yp;
     f[5] = base_diag + (xy_p + pxy);
     f[6] = base_diag - (xy_m + pxy);
     f[7] = base_diag - (xy_p - pxy);
     f[8] = base_diag + (xy_m - pxy);
-    // f*_0 from mass conservation, rho - sum_{a>0} f*_a, instead of (m*_0 - m*_1 + m*_2)/9:
-    // with the rounded constants the column sums of M^-1 are not exactly (1, 0, ..., 0), which
-    // in FP32 adds mass at about 7e-9 per step; this way the only error is one unbiased
-    // rounding. In FP64 the eight f*_a sum to 4 (base_axis + base_diag) up to their own
-    // unbiased roundings, two operations instead of eight.
+    // f*_0 from mass conservation instead of (m*_0 - m*_1 + m*_2)/9: with the rounded
+    // constants the column sums of M^-1 are not exactly (1, 0, ..., 0), which in FP32 adds mass
+    // at about 7e-9 per step. In FP32 it is f_0 plus what the moving populations lost, the two
+    // sums over them formed alike: in a uniform fluid their roundings cancel, where rho - sum
+    // f*_a adds the same one at every step (a 501 x 383 droplet after 200 steps, error against
+    // FP64: 7e-7 against 1.1e-6). In FP64 the eight f*_a sum to 4 (base_axis + base_diag) up
+    // to their own unbiased roundings, two operations instead of nine.
     if constexpr (std::is_same<T, double>::value)
         f[0] = vfma(mfour, base_axis + base_diag, rsum);
     else
-        f[0] = rsum - (((f[1] + f[3]) + (f[2] + f[4])) + ((f[5] + f[7]) + (f[6] + f[8])));
+        f[0] = f[0] + (moving - (((f[1] + f[3]) + (f[2] + f[4])) + ((f[5] + f[7]) + (f[6] + f[8]))));
 }
 
 }  // namespace lbm
