@@ -124,11 +124,17 @@ lb_status lb_init_ex(lb_ctx **out, int nx, int ny, const lb_eos *eos, double G, 
                      double sigma_force, const lb_rates *rates, int prec, int bc, void *stream,
                      void *f_a, void *f_b);
 
-/* Number of compiled variants of the step kernel: strip width x shared-memory ring depth
- * x ring kind. Variants 0-3 stage whole stored rows of the strip (all nine populations,
- * three rows in use at a time); variants 4-6 stage, per psi row, exactly the three plane
- * groups that row is pulled from (one stage in use at a time, so more CTAs fit on an SM).
- * Every variant gives identical results. Contexts and batches start with variant 4. */
+/* Number of variants of the step kernel. Variants 0-6 march over rows with a shared-memory
+ * ring (strip width x ring depth x ring kind): 0-3 stage whole stored rows of the strip (all
+ * nine populations, three rows in use at a time); 4-6 stage, per psi row, exactly the three
+ * plane groups that row is pulled from (one stage in use at a time, so more CTAs fit on an
+ * SM). Variant 7 has no ring: one CTA per tile of 64 x 4 sites (LB_FP32, LB_BF16), or a psi
+ * and a collision launch with one site per thread (LB_FP64, with psi scratch of 1/18 of the
+ * two population buffers, allocated by the library); its launch shape is fixed. Lattices of
+ * more than 65535 rows, and LB_FP64 lattices whose scratch cannot be allocated, take variant 4
+ * in its place. Every variant gives identical results. Contexts start with variant 7, or with
+ * variant 4 where an LB_FP32 or LB_BF16 state is too large for the L2 cache (a buffer above
+ * 72 MiB); batches have variants 0-6 and start with variant 4. */
 int lb_launch_variants(void);
 
 /* Density-dependent viscosity of Sec. V.C (LB_BC_OPEN contexts): sites with rho < rho_1
@@ -157,12 +163,13 @@ enum { LB_ROUND_NEAREST = 0, LB_ROUND_STOCHASTIC = 1 };
 lb_status lb_set_storage_rounding(lb_ctx *ctx, int mode);
 
 /* Choose the step kernel's variant (0 .. lb_launch_variants()-1) and the number of rows
- * each CTA marches over (rows = 0: about three waves of resident CTAs, at least 8 rows).
- * Synchronises the stream. Errors: LB_EINVAL for an unknown variant or rows < 0. */
+ * each CTA marches over (rows = 0: about three waves of resident CTAs, at least 8 rows;
+ * variant 7 takes no rows). Synchronises the stream. Errors: LB_EINVAL for an unknown variant or rows < 0. */
 lb_status lb_set_launch(lb_ctx *ctx, int variant, int rows);
 
 /* Autotuner: time every compiled variant with rows per CTA from {default, 6, 8, 9, 10,
- * 11, 12, 13, 14, 15, 16, 20, 24} (at most ny) on this lattice and keep the fastest. Each
+ * 11, 12, 13, 14, 15, 16, 20, 24} (at most ny; variant 7 once) on this lattice and keep the
+ * fastest. Each
  * candidate runs one untimed launch and then three timed runs of `trial_steps` >= 1
  * launches (its time is the fastest run). The trial launches take real steps on a scratch
  * copy of the state (a temporary device buffer of lb_buffer_bytes, freed before return),
@@ -179,7 +186,7 @@ lb_status lb_get_launch(const lb_ctx *ctx, int *variant, int *tx, int *rows, int
 
 /* Test hook for the failure path of the bounded device-side waits: from the next lb_step
  * on, the step kernel never requests lattice row `row` (as staged in its shared-memory
- * ring), so the CTAs that need it give up after about one second and the next
+ * ring; a context with variant 7 changes to variant 4), so the CTAs that need it give up after about one second and the next
  * synchronising call returns LB_ETIMEOUT. Nothing faults and no copy is left in flight.
  * INT_MIN (the default) switches it off. Not part of the method; for tests only. */
 lb_status lb_debug_stall_row(lb_ctx *ctx, int row);
@@ -190,7 +197,7 @@ lb_status lb_debug_stall_row(lb_ctx *ctx, int row);
  * and positive at some site (rho <= 0, or (p_EOS - rho/3)/G <= 0), LB_ECUDA. */
 lb_status lb_set_rho_u(lb_ctx *ctx, const double *rho, const double *ux, const double *uy);
 
-/* Advance n >= 0 time steps (Eqs. 4-8, 17-19), one kernel launch per step. Queued on the
+/* Advance n >= 0 time steps (Eqs. 4-8, 17-19), lb_kernels_per_step launches each. Queued on the
  * stream; returns without waiting. A psi-domain violation found on the device is reported
  * by the next call that synchronises (lb_sync, lb_get_*, lb_reduce) as LB_EDOMAIN; a
  * device-side wait that gave up (about one second) as LB_ETIMEOUT. */

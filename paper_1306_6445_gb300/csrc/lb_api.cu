@@ -33,6 +33,7 @@ struct lb_ctx {
     double *d_out8 = nullptr;      // 8 doubles
     int *d_first = nullptr;        // interface height: nx ints
     double *d_host_in = nullptr; // 3*nx*ny staging for lb_set_rho_u
+    void *d_psi = nullptr;       // FP64 direct kernels: psi of the step, ny * pitch elements
     lbm::StepLaunch launch{};
     long long steps = 0;
     lb_status sticky = LB_OK;
@@ -207,13 +208,27 @@ lb_status make_maps(lb_ctx *c) {
     return LB_OK;
 }
 
+// whether the direct kernels can run this lattice: its rows fit a grid, and the psi scratch of
+// the FP64 ones (1/18 of the two population buffers) could be allocated
+bool direct_usable(lb_ctx *c) {
+    if (!lbm::direct_fits(c->geom)) return false;
+    if (c->prec != LB_FP64 || c->d_psi) return true;
+    if (cudaMalloc(&c->d_psi, (size_t)c->geom.plane * c->elem) == cudaSuccess) return true;
+    (void)cudaGetLastError();
+    c->d_psi = nullptr;
+    return false;
+}
+
 lb_status apply_launch(lb_ctx *c, int variant, int rows) {
     if (variant < 0 || variant >= lbm::step_variant_count())
         return fail(c, LB_EINVAL, "unknown launch variant");
     if (rows < 0) return fail(c, LB_EINVAL, "rows must be >= 0");
+    if (variant == lbm::direct_variant() && !direct_usable(c)) {
+        variant = lbm::default_ring_variant();   // same results
+    }
     c->launch = lbm::make_step_launch(c->prec, c->consts.eos_kind, c->geom, c->num_sms, variant, rows);
     LB_CUDA(c, lbm::configure_step(c->prec, c->consts, c->geom, c->launch));
-    return make_maps(c);
+    return variant == lbm::direct_variant() ? LB_OK : make_maps(c);
 }
 
 lb_status check_usable(lb_ctx *c) {
@@ -302,7 +317,7 @@ lb_status create(lb_ctx **out, int nx, int ny, const lb_eos *eos, double G, doub
         lb_free(c);
         return LB_ECUDA;
     }
-    if ((s = apply_launch(c, lbm::default_step_variant(), 0)) != LB_OK) {
+    if ((s = apply_launch(c, lbm::default_variant(prec, c->geom), 0)) != LB_OK) {
         std::fprintf(stderr, "lb_init: %s\n", c->msg.c_str());
         lb_free(c);
         return s;
@@ -410,25 +425,31 @@ lb_status lb_autotune(lb_ctx *c, int trial_steps, int *variant, int *rows) {
     cudaError_t e = cudaSuccess;
     for (int v = 0; v < lbm::step_variant_count() && e == cudaSuccess; ++v) {
         int tried_rows[16], n_tried = 0;
+        const bool direct = v == lbm::direct_variant();
+        if (direct && !direct_usable(c)) continue;
         for (int r : cand) {
+            if (direct && r != 0) break;      // one launch shape
             if ((s = apply_launch(c, v, r)) != LB_OK) break;
             const int rr = c->launch.rows;
             bool seen = false;
             for (int i = 0; i < n_tried; ++i) seen |= tried_rows[i] == rr;
             if (seen) continue;
             tried_rows[n_tried++] = rr;
-            if (scratch && (s = encode_map(c, scratch, &scratch_map)) != LB_OK) break;
+            if (scratch && !direct && (s = encode_map(c, scratch, &scratch_map)) != LB_OK) break;
             // trial k reads the scratch copy (k even) or the spare buffer (k odd) and
             // writes the other, in visiting order k & 1
             int k = 0;
             auto once = [&]() {
                 const bool from_scratch = (k & 1) == 0;
-                const CUtensorMap *src = !scratch       ? &c->tmap[c->cur]
-                                         : from_scratch ? &scratch_map
-                                                        : &c->tmap[c->cur ^ 1];
-                void *dst = (!scratch || from_scratch) ? c->f[c->cur ^ 1] : scratch;
+                lbm::StepBuffers b;
+                b.tensor_map_in = !scratch       ? &c->tmap[c->cur]
+                                  : from_scratch ? &scratch_map
+                                                 : &c->tmap[c->cur ^ 1];
+                b.gin = !scratch ? c->f[c->cur] : from_scratch ? scratch : c->f[c->cur ^ 1];
+                b.gout = (!scratch || from_scratch) ? c->f[c->cur ^ 1] : scratch;
+                b.psi = c->d_psi;
                 const cudaError_t r = lbm::launch_step(c->prec, c->consts, c->geom, c->launch,
-                                                       k & 1, src, dst, c->d_err, c->stream);
+                                                       k & 1, b, c->d_err, c->stream);
                 ++k;
                 return r;
             };
@@ -511,6 +532,9 @@ lb_status lb_debug_stall_row(lb_ctx *c, int row) {
     lb_status s = check_usable(c);
     if (s != LB_OK) return s;
     c->consts.stall_row = row;
+    // the direct kernels stage no rows: a stalled row needs a ring
+    if (row != INT_MIN && c->launch.variant == lbm::direct_variant())
+        return apply_launch(c, lbm::default_ring_variant(), 0);
     return LB_OK;
 }
 
@@ -548,8 +572,9 @@ lb_status lb_step(lb_ctx *c, int n) {
         // alternate the visiting order: each step first reads the rows the previous one
         // wrote last (still in L2 when the state is not much larger than L2)
         c->consts.step_key = (unsigned)c->steps;   // the stochastic-rounding counter
+        const lbm::StepBuffers b{c->f[c->cur], &c->tmap[c->cur], c->f[c->cur ^ 1], c->d_psi};
         LB_CUDA(c, lbm::launch_step(c->prec, c->consts, c->geom, c->launch, (int)(c->steps & 1),
-                                    &c->tmap[c->cur], c->f[c->cur ^ 1], c->d_err, c->stream));
+                                    b, c->d_err, c->stream));
         c->cur ^= 1;
         ++c->steps;
     }
@@ -668,7 +693,10 @@ lb_status lb_interface_height(lb_ctx *c, double rho_mid, double *heights) {
 
 long long lb_steps_done(const lb_ctx *c) { return c ? c->steps : 0; }
 
-int lb_kernels_per_step(const lb_ctx *c) { return c ? 1 : 0; }
+int lb_kernels_per_step(const lb_ctx *c) {
+    if (!c) return 0;
+    return c->prec == LB_FP64 && c->launch.variant == lbm::direct_variant() ? 2 : 1;
+}
 
 const char *lb_last_error(const lb_ctx *c) { return c ? c->msg.c_str() : kNoCtx; }
 
@@ -688,6 +716,7 @@ void lb_free(lb_ctx *c) {
     cudaFree(c->d_out8);
     cudaFree(c->d_first);
     cudaFree(c->d_host_in);
+    cudaFree(c->d_psi);
     delete c;
 }
 

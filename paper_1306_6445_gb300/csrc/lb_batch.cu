@@ -134,7 +134,7 @@ void drop_graphs(lb_batch *b) {
 }
 
 lb_status apply_batch_launch(lb_batch *b, int variant, int rows) {
-    if (variant < 0 || variant >= lbm::step_variant_count())
+    if (variant < 0 || variant >= lbm::ring_variant_count())
         return bfail(b, LB_EINVAL, "unknown launch variant");
     if (rows <= 0) rows = 16;
     const int tx = lbm::step_variant_tx(variant);
@@ -366,7 +366,7 @@ lb_status lb_batch_create(lb_batch **out, int n, const lb_lattice_desc *descs, i
     b->active.assign(n, 1);
     b->lat_steps.assign(n, 0);
     s = prec == LB_FP32 ? upload_lattices<float>(b) : upload_lattices<double>(b);
-    if (s == LB_OK) s = apply_batch_launch(b, lbm::default_step_variant(), 16);
+    if (s == LB_OK) s = apply_batch_launch(b, lbm::default_ring_variant(), 16);
     if (s != LB_OK) {
         std::fprintf(stderr, "lb_batch_create: %s\n", b->msg.c_str());
         lb_batch_free(b);
@@ -426,7 +426,7 @@ lb_status lb_batch_autotune(lb_batch *b, int trial_steps, int *variant, int *row
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (e == cudaSuccess) e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
-    for (int v = 0; v < lbm::step_variant_count() && e == cudaSuccess; ++v) {
+    for (int v = 0; v < lbm::ring_variant_count() && e == cudaSuccess; ++v) {
         for (int r : cand_rows) {
             if (apply_batch_launch(b, v, r) != LB_OK) continue;
             if (launch_steps(b, 1) != LB_OK) continue;                 // warm-up

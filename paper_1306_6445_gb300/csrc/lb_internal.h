@@ -88,9 +88,14 @@ struct StepLaunch {
 
 // ---- kernels (lb_kernels.cu) -------------------------------------------------------
 int step_variant_count();
+int ring_variant_count();               // variants 0 .. ring_variant_count() - 1 use a TMA ring
+int direct_variant();                   // the variant of the direct kernels (lb_tile.cuh)
+bool direct_fits(const Geom &g);        // the direct kernels' grid holds the lattice
+int default_variant(int prec, const Geom &g);   // what a context starts with
+constexpr int DIRECT_COLS = 64, DIRECT_ROWS = 4;   // tile of the direct FP32 and BF16 kernels
 int step_variant_tx(int variant);
 int step_variant_planes(int variant);   // population planes per TMA box (9 or 3)
-int default_step_variant();
+int default_ring_variant();
 StepLaunch make_step_launch(int prec, int eos_kind, const Geom &g, int num_sms, int variant,
                             int rows_override);
 cudaError_t configure_step(int prec, const Consts &c, const Geom &g, const StepLaunch &l);
@@ -122,9 +127,25 @@ LB_DECLARE_BATCH_UNIT(f64, 0)
 LB_DECLARE_BATCH_UNIT(f64, 1)
 #undef LB_DECLARE_BATCH_UNIT
 
+// direct step units (lb_tile_f32.cu, lb_tile_bf16.cu, lb_split_f64.cu); psi: ny * pitch elements
+cudaError_t tile_f32(const Consts &c, const Geom &g, int order, const void *gin,
+                     void *gout, int *err, cudaStream_t st);
+cudaError_t tile_bf16(const Consts &c, const Geom &g, int order, const void *gin,
+                      void *gout, int *err, cudaStream_t st);
+cudaError_t split_f64(const Consts &c, const Geom &g, const void *gin, void *psi, void *gout,
+                      int *err, cudaStream_t st);
+
+// What a step reads and writes: the input buffer (the ring variants reach it through its
+// tensor map), the output buffer, and psi scratch (FP64 direct kernels only).
+struct StepBuffers {
+    const void *gin;
+    const void *tensor_map_in;
+    void *gout;
+    void *psi;
+};
 // order 0 / 1: visit the row blocks (and the rows inside them) forward / in reverse
 cudaError_t launch_step(int prec, const Consts &c, const Geom &g, const StepLaunch &l, int order,
-                        const void *tensor_map_in, void *gout, int *err, cudaStream_t stream);
+                        const StepBuffers &b, int *err, cudaStream_t stream);
 // packed: f in the host layout [a][y][x] (no pitch, no ghosts) instead of the padded one
 cudaError_t launch_unstream(int prec, const Geom &g, const void *f, void *gbuf, bool packed,
                             cudaStream_t stream);

@@ -383,25 +383,47 @@ k_reduce_final(const double *__restrict__ partials, int nblocks, double *__restr
 
 // the variants of LB_STEP_VARIANTS (lb_step.cuh): strip width and planes per TMA box (9:
 // whole stored rows, 3: one plane group of the stage ring)
-int step_variant_count() { return 7; }
+int step_variant_count() { return 8; }
+int ring_variant_count() { return 7; }
+int direct_variant() { return 7; }
 
 int step_variant_tx(int variant) {
-    static const int tx[] = {128, 128, 240, 64, 128, 128, 240};
-    return (variant >= 0 && variant < 7) ? tx[variant] : 0;
+    static const int tx[] = {128, 128, 240, 64, 128, 128, 240, 64};
+    return (variant >= 0 && variant < 8) ? tx[variant] : 0;
 }
 
 int step_variant_kind(int variant) { return variant >= 4 ? 1 : 0; }
 
+bool direct_fits(const Geom &g) { return g.ny <= 65535; }   // one grid row per lattice row (FP64)
+
+// The direct kernels, except where the state of an FP32 or BF16 lattice does not stay in L2:
+// there the step is bound by memory, which the ring's TMA loads keep busier. FP32 periodic
+// droplets on GB300, direct against autotuned ring: 64^2 2.3 / 9.4 us, 512^2 4.6 / 8.5,
+// 1024^2 12.1 / 15.1, 1448^2 26.5 / 26.4 (75.5 MB a buffer), 2048^2 51.6 / 48.7. FP64 is
+// bound by its pipe at every size: 128^2 9.1 / 118 us, 1000 x 700 225 / 341.
+int default_variant(int prec, const Geom &g) {
+    if (!direct_fits(g)) return default_ring_variant();
+    const long long bytes = 9 * g.plane * (prec == LB_FP32 ? 4 : 2);
+    return prec == LB_FP64 || bytes <= (72ll << 20) ? direct_variant() : default_ring_variant();
+}
+
 int step_variant_planes(int variant) { return step_variant_kind(variant) ? 3 : 9; }
 
-// the launch a new context or batch starts with: the stage ring, 128-column strips, S = 3
-int default_step_variant() { return 4; }
+// the ring launch that batches, and contexts the direct kernels do not fit, start with: the
+// stage ring, 128-column strips, S = 3
+int default_ring_variant() { return 4; }
 
 StepLaunch make_step_launch(int prec, int eos_kind, const Geom &g, int num_sms, int variant,
                             int rows_override) {
     StepLaunch l;
     l.variant = variant;
     l.tx = step_variant_tx(variant);
+    if (variant == direct_variant()) {
+        // its grid is fixed by the lattice: rows_override does not apply
+        l.rows = prec == LB_FP64 ? 1 : std::min(DIRECT_ROWS, g.ny);
+        l.ctas_per_sm = prec == LB_FP64 ? 2048 / DIRECT_COLS : 65536 / (32 * DIRECT_ROWS * 80);
+        return l;
+    }
     const bool st = step_variant_kind(variant) == 1;
     const int per_sm =
         prec == LB_FP32 ? (st ? occupancy_f32_k1 : occupancy_f32_k0)(variant, eos_kind, g.walls)
@@ -436,13 +458,18 @@ static cudaError_t launch_step_unit(int prec, const Consts &c, const Geom &g, co
 }
 
 cudaError_t configure_step(int prec, const Consts &c, const Geom &g, const StepLaunch &l) {
+    if (l.variant == direct_variant()) return cudaSuccess;
     static const CUtensorMap dummy{};
     return launch_step_unit(prec, c, g, l, 0, &dummy, nullptr, nullptr, nullptr, true);
 }
 
 cudaError_t launch_step(int prec, const Consts &c, const Geom &g, const StepLaunch &l, int order,
-                        const void *tensor_map_in, void *gout, int *err, cudaStream_t st) {
-    return launch_step_unit(prec, c, g, l, order, tensor_map_in, gout, err, st, false);
+                        const StepBuffers &b, int *err, cudaStream_t st) {
+    if (l.variant == direct_variant()) {
+        if (prec == LB_FP64) return split_f64(c, g, b.gin, b.psi, b.gout, err, st);
+        return (prec == LB_FP32 ? tile_f32 : tile_bf16)(c, g, order, b.gin, b.gout, err, st);
+    }
+    return launch_step_unit(prec, c, g, l, order, b.tensor_map_in, b.gout, err, st, false);
 }
 
 cudaError_t launch_unstream(int prec, const Geom &g, const void *f, void *gbuf, bool packed,

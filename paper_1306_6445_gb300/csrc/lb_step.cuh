@@ -373,6 +373,32 @@ __device__ __forceinline__ unsigned store_bits(unsigned key, int a, const DevCon
         return 0u;
 }
 
+// the ghost columns that the site pair (x, x + 1) of the row starting at element rowi has an
+// image in: periodic images of columns 0, 1 (right of nx-1) and nx-2, nx-1 (left of 0), or,
+// with open sides, copies of the edge columns (zero gradient)
+template <typename T, int BC, bool SR>
+__device__ __forceinline__ void store_ghosts(T *__restrict__ gout, const V2<Arith<T>> (&f)[9], int x,
+                                             unsigned rowi, int nx, unsigned plane, bool both,
+                                             unsigned key, const DevConsts<Arith<T>> &P) {
+    if (BC == 2 ? !(x == 0 || x + 1 >= nx - 1) : !(x < 2 || x + 1 >= nx - 2)) return;
+#pragma unroll
+    for (int a = 0; a < 9; ++a) {
+        const unsigned r = store_bits<T, SR>(key, a, P);
+        const T v0 = stored_enc<T, SR>(f[a].lo(), r), v1 = stored_enc<T, SR>(f[a].hi(), r >> 16);
+        T *rb = gout + (rowi + plane_of(a) * plane);
+        if (BC == 2) {
+            if (x == 0) rb[GH<T> - 1] = rb[GH<T> - 2] = v0;
+            if (x == nx - 1) rb[nx + GH<T>] = rb[nx + GH<T> + 1] = v0;
+            if (both && x + 1 == nx - 1) rb[nx + GH<T>] = rb[nx + GH<T> + 1] = v1;
+        } else {
+            if (x < 2) rb[nx + GH<T> + x] = v0;
+            if (both && x + 1 < 2) rb[nx + GH<T> + x + 1] = v1;
+            if (x >= nx - 2) rb[x - nx + GH<T>] = v0;
+            if (both && x + 1 >= nx - 2) rb[x + 1 - nx + GH<T>] = v1;
+        }
+    }
+}
+
 __device__ __forceinline__ void grid_dependency_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
@@ -554,34 +580,7 @@ __device__ __forceinline__ int march(const CUtensorMap *tmap, T *__restrict__ go
             for (int a = 0; a < 9; ++a)
                 store_pop_pair<T, SR>(gout + (idx + plane_of(a) * plane), fc[a], both, a, P,
                                   store_bits<T, SR>(key, a, P));
-            if (BC == 2) {
-                // open sides: the ghost columns repeat the edge columns (zero gradient)
-                if (x == 0 || x + 1 >= nx - 1) {
-                    const unsigned rowi = (unsigned)yr * (unsigned)pitch;
-#pragma unroll
-                    for (int a = 0; a < 9; ++a) {
-                        const unsigned r = store_bits<T, SR>(key, a, P);
-                        const T v0 = stored_enc<T, SR>(fc[a].lo(), r), v1 = stored_enc<T, SR>(fc[a].hi(), r >> 16);
-                        T *rb = gout + (rowi + plane_of(a) * plane);
-                        if (x == 0) rb[GH<T> - 1] = rb[GH<T> - 2] = v0;
-                        if (x == nx - 1) rb[nx + GH<T>] = rb[nx + GH<T> + 1] = v0;
-                        if (both && x + 1 == nx - 1) rb[nx + GH<T>] = rb[nx + GH<T> + 1] = v1;
-                    }
-                }
-            } else if (x < 2 || x + 1 >= nx - 2) {
-                // ghost images of columns 0, 1 (right of nx-1) and nx-2, nx-1 (left of 0)
-                const unsigned rowi = (unsigned)yr * (unsigned)pitch;
-#pragma unroll
-                for (int a = 0; a < 9; ++a) {
-                    const unsigned r = store_bits<T, SR>(key, a, P);
-                    const T v0 = stored_enc<T, SR>(fc[a].lo(), r), v1 = stored_enc<T, SR>(fc[a].hi(), r >> 16);
-                    T *rb = gout + (rowi + plane_of(a) * plane);
-                    if (x < 2) rb[nx + GH<T> + x] = v0;
-                    if (both && x + 1 < 2) rb[nx + GH<T> + x + 1] = v1;
-                    if (x >= nx - 2) rb[x - nx + GH<T>] = v0;
-                    if (both && x + 1 >= nx - 2) rb[x + 1 - nx + GH<T>] = v1;
-                }
-            }
+            store_ghosts<T, BC, SR>(gout, fc, x, (unsigned)yr * (unsigned)pitch, nx, plane, both, key, P);
         }
         return true;
     };
@@ -840,32 +839,7 @@ __device__ __forceinline__ int march_stage(const CUtensorMap *tmap, T *__restric
                     store_pop_pair<T, SR>(gout + (idx + plane_of(a) * plane), fc[a], both, a, P,
                                       store_bits<T, SR>(key, a, P));
             }
-            if (BC == 2) {
-                if (x == 0 || x + 1 >= nx - 1) {
-                    const unsigned rowi = (unsigned)y * (unsigned)pitch;
-#pragma unroll
-                    for (int a = 0; a < 9; ++a) {
-                        const unsigned r = store_bits<T, SR>(key, a, P);
-                        const T v0 = stored_enc<T, SR>(fc[a].lo(), r), v1 = stored_enc<T, SR>(fc[a].hi(), r >> 16);
-                        T *rb = gout + (rowi + plane_of(a) * plane);
-                        if (x == 0) rb[GH<T> - 1] = rb[GH<T> - 2] = v0;
-                        if (x == nx - 1) rb[nx + GH<T>] = rb[nx + GH<T> + 1] = v0;
-                        if (both && x + 1 == nx - 1) rb[nx + GH<T>] = rb[nx + GH<T> + 1] = v1;
-                    }
-                }
-            } else if (x < 2 || x + 1 >= nx - 2) {
-                const unsigned rowi = (unsigned)y * (unsigned)pitch;
-#pragma unroll
-                for (int a = 0; a < 9; ++a) {
-                    const unsigned r = store_bits<T, SR>(key, a, P);
-                    const T v0 = stored_enc<T, SR>(fc[a].lo(), r), v1 = stored_enc<T, SR>(fc[a].hi(), r >> 16);
-                    T *rb = gout + (rowi + plane_of(a) * plane);
-                    if (x < 2) rb[nx + GH<T> + x] = v0;
-                    if (both && x + 1 < 2) rb[nx + GH<T> + x + 1] = v1;
-                    if (x >= nx - 2) rb[x - nx + GH<T>] = v0;
-                    if (both && x + 1 >= nx - 2) rb[x + 1 - nx + GH<T>] = v1;
-                }
-            }
+            store_ghosts<T, BC, SR>(gout, fc, x, (unsigned)y * (unsigned)pitch, nx, plane, both, key, P);
         }
         return true;
     };
