@@ -39,6 +39,10 @@ struct BatchCommon {
     size_t stage_sites = 0;
     double *d_radius = nullptr;
     double *d_meas = nullptr;
+    lbm::MeasureChunk *d_chunks = nullptr;   // CTAs of a measurement (all lattices)
+    int *d_first = nullptr;                  // first chunk of lattice i, n + 1 entries
+    double *d_partials = nullptr;            // 8 doubles per chunk
+    int n_chunks = 0;
     int variant = 0, rows = 16, grid = 0, ctas_per_sm = 1, num_sms = 0;
     int phase = 0;                       // which buffer holds the active lattices' state
     std::vector<unsigned char> active;   // lattices stepped by lb_batch_step
@@ -124,6 +128,32 @@ bool make_items(const lb_batch *b, int tx, int rows, std::vector<lbm::BatchItem>
         }
     }
     return true;
+}
+
+// The chunks of a measurement: whole rows, about 8192 sites each (32 per thread), at most 256
+// per lattice (one pass of k_batch_measure_sum's lanes over eight).
+lb_status make_chunks(lb_batch *b) {
+    std::vector<lbm::MeasureChunk> chunks;
+    std::vector<int> first(b->n + 1);
+    for (int i = 0; i < b->n; ++i) {
+        first[i] = (int)chunks.size();
+        const int nx = b->geom[i].nx, ny = b->geom[i].ny;
+        const int rows = std::max(std::max(1, 8192 / nx), (ny + 255) / 256);
+        for (int y = 0; y < ny; y += rows) chunks.push_back({i, y, std::min(rows, ny - y)});
+    }
+    first[b->n] = b->n_chunks = (int)chunks.size();
+    if (cudaMalloc(&b->d_chunks, chunks.size() * sizeof(chunks[0])) != cudaSuccess ||
+        cudaMalloc(&b->d_first, first.size() * sizeof(int)) != cudaSuccess ||
+        cudaMalloc(&b->d_partials, chunks.size() * 8 * sizeof(double)) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return LB_ENOMEM;
+    }
+    if (cudaMemcpy(b->d_chunks, chunks.data(), chunks.size() * sizeof(chunks[0]),
+                   cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(b->d_first, first.data(), first.size() * sizeof(int),
+                   cudaMemcpyHostToDevice) != cudaSuccess)
+        return LB_ECUDA;
+    return LB_OK;
 }
 
 void drop_graphs(lb_batch *b) {
@@ -365,6 +395,10 @@ lb_status lb_batch_create(lb_batch **out, int n, const lb_lattice_desc *descs, i
     }
     b->active.assign(n, 1);
     b->lat_steps.assign(n, 0);
+    if ((s = make_chunks(b)) != LB_OK) {
+        lb_batch_free(b);
+        return s;
+    }
     s = prec == LB_FP32 ? upload_lattices<float>(b) : upload_lattices<double>(b);
     if (s == LB_OK) s = apply_batch_launch(b, lbm::default_ring_variant(), 16);
     if (s != LB_OK) {
@@ -548,8 +582,9 @@ lb_status lb_batch_measure(lb_batch *b, const double *radius, double *out) {
     if (b->sticky != LB_OK) return b->sticky;
     LB_BCUDA(b, cudaMemcpyAsync(b->d_radius, radius, b->n * sizeof(double), cudaMemcpyHostToDevice,
                                 b->stream));
-    LB_BCUDA(b, lbm::launch_batch_measure(b->prec, b->eos_kind, b->d_lats, b->n, b->phase,
-                                          b->d_radius, b->d_meas, b->stream));
+    LB_BCUDA(b, lbm::launch_batch_measure(b->prec, b->eos_kind, b->d_lats, b->n, b->d_chunks,
+                                          b->d_first, b->n_chunks, b->phase, b->d_radius,
+                                          b->d_partials, b->d_meas, b->stream));
     std::vector<double> raw(8 * (size_t)b->n);
     LB_BCUDA(b, cudaMemcpyAsync(raw.data(), b->d_meas, raw.size() * sizeof(double),
                                 cudaMemcpyDeviceToHost, b->stream));
@@ -598,6 +633,9 @@ void lb_batch_free(lb_batch *b) {
     cudaFree(b->d_stage);
     cudaFree(b->d_radius);
     cudaFree(b->d_meas);
+    cudaFree(b->d_chunks);
+    cudaFree(b->d_first);
+    cudaFree(b->d_partials);
     delete b;
 }
 

@@ -1,66 +1,127 @@
 // Batched-lattice kernels: the persistent step over work items with the whole-row ring
 // (FP32, FP64; the stage ring is in lb_batch_stage.cu) and the per-lattice Laplace
 // measurement.
+#include <climits>
+
 #include "lb_step.cuh"
 
 namespace lbm {
 
 namespace {
 
-// Per-lattice Laplace sums for the batched sweep: one CTA per lattice, fixed per-thread
-// order and fixed tree (deterministic). Inside: r < R/2; outside: r > R + 0.3 min(nx,ny)/2,
-// around the lattice centre ((nx-1)/2, (ny-1)/2); p = rho/3 + (G/2) psi^2.
+// Squared distances from the lattice centre ((nx-1)/2, (ny-1)/2) are quarters of integers
+// D = (2x - nx + 1)^2 + (2y - ny + 1)^2, so r < r_in is D < below(r_in) and r > r_out is
+// D >= above(r_out) exactly as with r = sqrt(D / 4), without a root per site.
+__device__ long long below(double r) {      // smallest D with sqrt(D / 4) >= r
+    if (!(r > 0)) return 0;
+    if (r > 1e9) return LLONG_MAX;
+    long long d = (long long)(4.0 * r * r);
+    while (d > 0 && sqrt(0.25 * (double)(d - 1)) >= r) --d;
+    while (sqrt(0.25 * (double)d) < r) ++d;
+    return d;
+}
+__device__ long long above(double r) {      // smallest D with sqrt(D / 4) > r
+    if (r < 0) return 0;
+    if (!(r <= 1e9)) return LLONG_MAX;
+    long long d = (long long)(4.0 * r * r);
+    while (d > 0 && sqrt(0.25 * (double)(d - 1)) > r) --d;
+    while (!(sqrt(0.25 * (double)d) > r)) ++d;
+    return d;
+}
+
+// Laplace sums of a chunk of rows of one lattice (fixed per-thread order and fixed tree, so
+// deterministic). Inside: r < R/2; outside: r > R + 0.3 min(nx,ny)/2; p = rho/3 + (G/2) psi^2,
+// summed as sums of rho and psi^2.
+// What bounds it: memory (36 bytes a site in FP32) next to the FP64 pipe (2 operations per
+// clock and SM): 4 FP64 operations a site are left (two conversions, two sums). One CTA per
+// lattice with a root and a division per site took 8.97 ms for 512 lattices of 64^2 to 512^2
+// (51.6 M sites); in chunks of 8192 sites 64 steps and a measurement take 49.9 against 57.8 ms.
 template <typename T, int EOS>
 __global__ void __launch_bounds__(RED_THREADS)
-k_batch_measure(const BatchLattice<T> *__restrict__ lats, int phase,
-                const double *__restrict__ radius, double *__restrict__ out) {
-    __shared__ double s[8][RED_THREADS];
-    const BatchLattice<T> &L = lats[blockIdx.x];
+k_batch_measure(const BatchLattice<T> *__restrict__ lats, const MeasureChunk *__restrict__ chunks,
+                int phase, const double *__restrict__ radius, double *__restrict__ partials) {
+    __shared__ double s[8][RED_THREADS / 32];
+    __shared__ long long limit[2];
+    const MeasureChunk ch = chunks[blockIdx.x];
+    const BatchLattice<T> &L = lats[ch.lat];
     const DevConsts<T> P = L.P;
-    const int nx = L.nx, ny = L.ny;
-    const T *g = L.g[L.frozen ? 0 : phase];
-    const double R = radius[blockIdx.x];
-    const double cx = 0.5 * (nx - 1), cy = 0.5 * (ny - 1);
-    const double r_in = 0.5 * R, r_out = R + 0.3 * 0.5 * min(nx, ny);
-    double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    const long long n = (long long)nx * ny;
-    for (long long i = threadIdx.x; i < n; i += RED_THREADS) {
-        const int y = (int)(i / nx), x = (int)(i % nx);
+    const int nx = L.nx, ny = L.ny, pitch = L.pitch;
+    const T *__restrict__ g = L.g[L.frozen ? 0 : phase];
+    if (threadIdx.x < 2) {
+        const double R = radius[ch.lat];
+        limit[threadIdx.x] = threadIdx.x == 0 ? below(0.5 * R) : above(R + 0.3 * 0.5 * min(nx, ny));
+    }
+    __syncthreads();
+    const long long d_in = limit[0], d_out = limit[1];
+    double m_in = 0, m_out = 0, m_rest = 0, q_in = 0, q_out = 0;
+    int n_in = 0, n_out = 0, n_bad = 0;
+    const unsigned n = (unsigned)ch.rows * (unsigned)nx;
+    for (unsigned i = threadIdx.x; i < n; i += RED_THREADS) {
+        const unsigned row = i / (unsigned)nx;
+        const int x = (int)(i - row * (unsigned)nx), y = ch.row0 + (int)row;
         T v[9];
 #pragma unroll
-        for (int a = 0; a < 9; ++a)
-            v[a] = pull_global<T, false>(g, a, x, y, nx, ny, L.pitch, (long long)L.plane);
+        for (int a = 0; a < 9; ++a) v[a] = pull_padded<T>(g, a, x, y, ny, pitch, L.plane);
         const T rho = sum9(v);
         bool bad = false;
         const T psi = eos_psi<T, EOS>(rho, P, bad);
-        const double dr = double(rho);
-        const double p = dr / 3.0 + 0.5 * double(P.G) * double(psi) * double(psi);
-        acc[0] += dr;
-        const double r = sqrt((x - cx) * (x - cx) + (y - cy) * (y - cy));
-        if (r < r_in) { acc[1] += dr; acc[2] += 1; acc[5] += p; }
-        if (r > r_out) { acc[3] += dr; acc[4] += 1; acc[6] += p; }
-        if (bad || !(dr == dr) || !(p == p)) acc[7] += 1;
-    }
-#pragma unroll
-    for (int q = 0; q < 8; ++q) s[q][threadIdx.x] = acc[q];
-    __syncthreads();
-    for (int wdt = RED_THREADS / 2; wdt > 0; wdt >>= 1) {
-        if (threadIdx.x < wdt) {
-#pragma unroll
-            for (int q = 0; q < 8; ++q) s[q][threadIdx.x] += s[q][threadIdx.x + wdt];
+        const double dr = double(rho), ds = double(psi);
+        const int a = 2 * x - (nx - 1), b = 2 * y - (ny - 1);
+        const long long d = (long long)a * a + (long long)b * b;
+        if (d < d_in) {
+            m_in += dr;
+            q_in = fma(ds, ds, q_in);
+            ++n_in;
+        } else if (d >= d_out) {
+            m_out += dr;
+            q_out = fma(ds, ds, q_out);
+            ++n_out;
+        } else {
+            m_rest += dr;
         }
-        __syncthreads();
+        if (bad || !(rho == rho) || !(psi == psi)) ++n_bad;
     }
-    if (threadIdx.x < 8) out[blockIdx.x * 8 + threadIdx.x] = s[threadIdx.x][0];
+    const double hg = 0.5 * double(P.G);
+    double acc[8] = {m_in + m_out + m_rest, m_in, (double)n_in, m_out, (double)n_out,
+                     m_in / 3.0 + hg * q_in, m_out / 3.0 + hg * q_out, (double)n_bad};
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+#pragma unroll
+        for (int w = 16; w > 0; w >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], w);
+        if ((threadIdx.x & 31) == 0) s[k][threadIdx.x >> 5] = acc[k];
+    }
+    __syncthreads();
+    if (threadIdx.x < 8) {
+        double t = 0;
+#pragma unroll
+        for (int w = 0; w < RED_THREADS / 32; ++w) t += s[threadIdx.x][w];
+        partials[(size_t)blockIdx.x * 8 + threadIdx.x] = t;
+    }
+}
+
+// Sum of the chunks of each lattice in a fixed order: warp k of CTA i adds quantity k.
+__global__ void __launch_bounds__(RED_THREADS)
+k_batch_measure_sum(const double *__restrict__ partials, const int *__restrict__ first,
+                    double *__restrict__ out) {
+    static_assert(RED_THREADS == 8 * 32, "one warp per quantity");
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int c0 = first[blockIdx.x], c1 = first[blockIdx.x + 1];
+    double t = 0;
+    for (int c = c0 + lane; c < c1; c += 32) t += partials[(size_t)c * 8 + k];
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1) t += __shfl_xor_sync(0xffffffffu, t, w);
+    if (lane == 0) out[blockIdx.x * 8 + k] = t;
 }
 
 }  // namespace
 
-cudaError_t launch_batch_measure(int prec, int eos_kind, const void *lats, int n_lat, int phase,
-                                 const double *radius, double *out, cudaStream_t st) {
+cudaError_t launch_batch_measure(int prec, int eos_kind, const void *lats, int n_lat,
+                                 const MeasureChunk *chunks, const int *first, int n_chunks,
+                                 int phase, const double *radius, double *partials, double *out,
+                                 cudaStream_t st) {
 #define LB_BM(T, EOSK)                                                                         \
-    k_batch_measure<T, EOSK><<<n_lat, RED_THREADS, 0, st>>>(                                   \
-        static_cast<const BatchLattice<T> *>(lats), phase, radius, out)
+    k_batch_measure<T, EOSK><<<n_chunks, RED_THREADS, 0, st>>>(                                \
+        static_cast<const BatchLattice<T> *>(lats), chunks, phase, radius, partials)
     if (prec == LB_FP32) {
         if (eos_kind == LB_EOS_CS) LB_BM(float, LB_EOS_CS);
         else if (eos_kind == LB_EOS_EXP) LB_BM(float, LB_EOS_EXP);
@@ -71,6 +132,9 @@ cudaError_t launch_batch_measure(int prec, int eos_kind, const void *lats, int n
         else LB_BM(double, LB_EOS_PIECEWISE);
     }
 #undef LB_BM
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    k_batch_measure_sum<<<n_lat, RED_THREADS, 0, st>>>(partials, first, out);
     return cudaGetLastError();
 }
 

@@ -79,6 +79,11 @@ struct BatchItem {
     int yb, n, dir;     // first row, row count, march direction (+1 / -1)
 };
 
+// One CTA's share of a batched measurement: rows row0 .. row0 + rows - 1 of a lattice.
+struct MeasureChunk {
+    int lat, row0, rows;
+};
+
 struct StepLaunch {
     int variant;        // compiled (strip width, ring depth) choice, see step_variant_tx
     int tx;             // lattice columns per CTA (two per thread)
@@ -202,9 +207,12 @@ cudaError_t launch_batch_step(int prec, int eos_kind, int variant, int grid, con
                               const void *lats, const BatchItem *items, int n_items, int phase,
                               int *errs, cudaStream_t stream);
 // per lattice: out[8*i ..] = mass, sum rho (r < R/2), count, sum rho (outside), count,
-// sum p (inside), sum p (outside), non-finite count; FP64, fixed order
-cudaError_t launch_batch_measure(int prec, int eos_kind, const void *lats, int n_lat, int phase,
-                                 const double *radius, double *out, cudaStream_t stream);
+// sum p (inside), sum p (outside), non-finite count; FP64, fixed order. Lattice i is measured
+// by chunks first[i] .. first[i+1] - 1; partials: 8 * n_chunks doubles
+cudaError_t launch_batch_measure(int prec, int eos_kind, const void *lats, int n_lat,
+                                 const MeasureChunk *chunks, const int *first, int n_chunks,
+                                 int phase, const double *radius, double *partials, double *out,
+                                 cudaStream_t stream);
 
 // ---- read-only view of a context for entry points outside lb_api.cu (lb_noalloc.cu) ---
 struct CtxView {

@@ -176,6 +176,16 @@ __device__ __forceinline__ T pull_global(const T *__restrict__ g, int a, int x, 
     return g[plane_of(a) * plane + (long long)sy * pitch + sx + GH<T>];
 }
 
+// f_a(x, y) of a periodic lattice pulled from g through its ghost columns (no wrap in x)
+template <typename T>
+__device__ __forceinline__ T pull_padded(const T *__restrict__ g, int a, int x, int y, int ny,
+                                         int pitch, unsigned plane) {
+    int sy = y - EYv(a);
+    sy = sy < 0 ? sy + ny : (sy >= ny ? sy - ny : sy);
+    const T *pl = g + (size_t)plane_of(a) * plane;
+    return pl[(unsigned)sy * (unsigned)pitch + (unsigned)(x - EXv(a) + GH<T>)];
+}
+
 // the value of f_a(x, y) (decoded from the storage type)
 template <typename T, int BC>
 __device__ __forceinline__ Arith<T> pull_val(const T *__restrict__ g, int a, int x, int y,
