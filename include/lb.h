@@ -128,13 +128,15 @@ lb_status lb_init_ex(lb_ctx **out, int nx, int ny, const lb_eos *eos, double G, 
  * ring (strip width x ring depth x ring kind): 0-3 stage whole stored rows of the strip (all
  * nine populations, three rows in use at a time); 4-6 stage, per psi row, exactly the three
  * plane groups that row is pulled from (one stage in use at a time, so more CTAs fit on an
- * SM). Variant 7 has no ring: one CTA per tile of 64 x 4 sites (LB_FP32, LB_BF16), or a psi
- * and a collision launch with one site per thread (LB_FP64, with psi scratch of 1/18 of the
- * two population buffers, allocated by the library); its launch shape is fixed. Lattices of
- * more than 65535 rows, and LB_FP64 lattices whose scratch cannot be allocated, take variant 4
- * in its place. Every variant gives identical results. Contexts start with variant 7, or with
- * variant 4 where an LB_FP32 or LB_BF16 state is too large for the L2 cache (a buffer above
- * 72 MiB); batches have variants 0-6 and start with variant 4. */
+ * SM). Variants 7 and 8 have no ring and a fixed launch shape: one CTA per tile of 64 x 4
+ * sites, which reads memory (7) or brings its tile into shared memory first (8). LB_FP64 has
+ * a psi and a collision launch with one site per thread for both (psi scratch of 1/18 of the
+ * two population buffers, allocated by the library). Lattices of more than 65535 rows, and
+ * LB_FP64 lattices whose scratch cannot be allocated, take variant 4 in their place. Every
+ * variant gives identical results. Contexts start with the variant that suits their type and
+ * size: 7 for LB_FP64 and for LB_FP32 up to 40 MiB a buffer, 8 for LB_BF16, for LB_BC_OPEN
+ * and up to 72 MiB, 4 beyond. LB_FP32 batches have variants 0-6 and 8 (7 is taken as 8) and
+ * start with 8, LB_FP64 batches 0-6 (7 and 8 are taken as 4) and start with 4. */
 int lb_launch_variants(void);
 
 /* Density-dependent viscosity of Sec. V.C (LB_BC_OPEN contexts): sites with rho < rho_1
@@ -164,11 +166,11 @@ lb_status lb_set_storage_rounding(lb_ctx *ctx, int mode);
 
 /* Choose the step kernel's variant (0 .. lb_launch_variants()-1) and the number of rows
  * each CTA marches over (rows = 0: about three waves of resident CTAs, at least 8 rows;
- * variant 7 takes no rows). Synchronises the stream. Errors: LB_EINVAL for an unknown variant or rows < 0. */
+ * variants 7 and 8 take no rows). Synchronises the stream. Errors: LB_EINVAL for an unknown variant or rows < 0. */
 lb_status lb_set_launch(lb_ctx *ctx, int variant, int rows);
 
 /* Autotuner: time every compiled variant with rows per CTA from {default, 6, 8, 9, 10,
- * 11, 12, 13, 14, 15, 16, 20, 24} (at most ny; variant 7 once) on this lattice and keep the
+ * 11, 12, 13, 14, 15, 16, 20, 24} (at most ny; variants 7 and 8 once) on this lattice and keep the
  * fastest. Each
  * candidate runs one untimed launch and then three timed runs of `trial_steps` >= 1
  * launches (its time is the fastest run). The trial launches take real steps on a scratch
@@ -186,7 +188,7 @@ lb_status lb_get_launch(const lb_ctx *ctx, int *variant, int *tx, int *rows, int
 
 /* Test hook for the failure path of the bounded device-side waits: from the next lb_step
  * on, the step kernel never requests lattice row `row` (as staged in its shared-memory
- * ring; a context with variant 7 changes to variant 4), so the CTAs that need it give up after about one second and the next
+ * ring; a context with variant 7 or 8 changes to variant 4), so the CTAs that need it give up after about one second and the next
  * synchronising call returns LB_ETIMEOUT. Nothing faults and no copy is left in flight.
  * INT_MIN (the default) switches it off. Not part of the method; for tests only. */
 lb_status lb_debug_stall_row(lb_ctx *ctx, int row);
@@ -285,9 +287,12 @@ void lb_free(lb_ctx *ctx);
 /* ---------------------------------------------------------------------------------
  * Batched lattices: many independent periodic lattices of uneven size and parameters
  * (for example a sweep of droplets over temperature, kappa and viscosity) advanced
- * together. Each time step is ONE launch of a persistent kernel whose CTAs walk a fixed
- * list of work items (lattice, strip, row block); runs of 64 steps are captured once in a
- * CUDA graph and replayed. The update of each lattice is the one of lb_step (Eqs. 4-8,
+ * together. With the ring variants each time step is ONE launch of a persistent kernel whose
+ * CTAs walk a fixed list of work items (lattice, strip, row block), and runs of 64 steps are
+ * captured once in a CUDA graph and replayed. With variant 8 (LB_FP32) the lattices form groups
+ * that stay in the L2 cache: a group takes all the steps of a call before the next one, three
+ * groups side by side on the batch's stream and two streams of its own that it forks and joins
+ * (work queued on the stream before and after a call is ordered as ever). The update of each lattice is the one of lb_step (Eqs. 4-8,
  * 17-19), bit for bit. All lattices share the precision and the EOS kind.
  * --------------------------------------------------------------------------------- */
 typedef struct {
@@ -342,8 +347,9 @@ lb_status lb_batch_get_populations(lb_batch *b, int i, void *dst, size_t bytes);
  * Synchronises. */
 lb_status lb_batch_measure(lb_batch *b, const double *radius, double *out);
 
-/* Time a few steps of every compiled variant and rows-per-item choice in {8, 12, 16, 24,
- * 32} on this batch and keep the fastest. The trial launches take real steps of the
+/* Time a few steps of every variant, the ring ones with rows per item in {8, 12, 16, 24,
+ * 32}, on this batch and keep the fastest (variant 8 over 16 steps, the others over trial_steps
+ * >= 2). The trial launches take real steps of the
  * current states (set them first: the cost of a step depends on the state), after the
  * populations, per-lattice error flags, phase and step count have been saved to a
  * temporary device buffer the size of the batch's pool; they are restored afterwards, so

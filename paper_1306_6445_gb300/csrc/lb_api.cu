@@ -176,15 +176,19 @@ EncodeTiledFn encode_fn() {
 // 3-D map over one population buffer: (padded column, row, population); one box is a
 // lattice row of the strip plus its apron, (tx + ghost + 4) x 1 x planes: all nine
 // populations for the whole-row ring, one for the stage ring (the left apron is as wide as
-// the ghost offset, so a box starts at the strip's own first element).
+// the ghost offset, so a box starts at the strip's own first element), or the rows of a tile
+// for the direct kernels.
 lb_status encode_map(lb_ctx *c, void *buffer, CUtensorMap *map) {
     EncodeTiledFn enc = encode_fn();
     if (!enc) return fail(c, LB_ECUDA, "cuTensorMapEncodeTiled unavailable");
     const Geom &g = c->geom;
     const cuuint64_t dims[3] = {(cuuint64_t)g.pitch, (cuuint64_t)g.ny, 9};
     const cuuint64_t strides[2] = {(cuuint64_t)g.pitch * c->elem, (cuuint64_t)g.plane * c->elem};
-    const cuuint32_t box[3] = {(cuuint32_t)(c->launch.tx + lbm::ghost_of_prec(c->prec) + 4), 1,
-                               (cuuint32_t)lbm::step_variant_planes(c->launch.variant)};
+    const bool direct = c->launch.variant >= lbm::direct_variant();
+    const cuuint32_t box[3] = {
+        (cuuint32_t)(direct ? lbm::TILE_BOX_W : c->launch.tx + lbm::ghost_of_prec(c->prec) + 4),
+        (cuuint32_t)(direct ? lbm::TILE_BOX_ROWS : 1),
+        (cuuint32_t)lbm::step_variant_planes(c->launch.variant)};
     const cuuint32_t estr[3] = {1, 1, 1};
     const CUtensorMapDataType dt = c->prec == LB_FP32   ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
                                  : c->prec == LB_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
@@ -223,12 +227,13 @@ lb_status apply_launch(lb_ctx *c, int variant, int rows) {
     if (variant < 0 || variant >= lbm::step_variant_count())
         return fail(c, LB_EINVAL, "unknown launch variant");
     if (rows < 0) return fail(c, LB_EINVAL, "rows must be >= 0");
-    if (variant == lbm::direct_variant() && !direct_usable(c)) {
-        variant = lbm::default_ring_variant();   // same results
+    if (variant >= lbm::direct_variant()) {
+        if (c->prec == LB_FP64) variant = lbm::direct_variant();     // no staged FP64 kernel
+        if (!direct_usable(c)) variant = lbm::default_ring_variant();
     }
     c->launch = lbm::make_step_launch(c->prec, c->consts.eos_kind, c->geom, c->num_sms, variant, rows);
     LB_CUDA(c, lbm::configure_step(c->prec, c->consts, c->geom, c->launch));
-    return variant == lbm::direct_variant() ? LB_OK : make_maps(c);
+    return variant >= lbm::direct_variant() && c->prec == LB_FP64 ? LB_OK : make_maps(c);
 }
 
 lb_status check_usable(lb_ctx *c) {
@@ -425,8 +430,9 @@ lb_status lb_autotune(lb_ctx *c, int trial_steps, int *variant, int *rows) {
     cudaError_t e = cudaSuccess;
     for (int v = 0; v < lbm::step_variant_count() && e == cudaSuccess; ++v) {
         int tried_rows[16], n_tried = 0;
-        const bool direct = v == lbm::direct_variant();
+        const bool direct = v >= lbm::direct_variant();
         if (direct && !direct_usable(c)) continue;
+        if (v == lbm::staged_variant() && c->prec == LB_FP64) continue;
         for (int r : cand) {
             if (direct && r != 0) break;      // one launch shape
             if ((s = apply_launch(c, v, r)) != LB_OK) break;
@@ -435,7 +441,7 @@ lb_status lb_autotune(lb_ctx *c, int trial_steps, int *variant, int *rows) {
             for (int i = 0; i < n_tried; ++i) seen |= tried_rows[i] == rr;
             if (seen) continue;
             tried_rows[n_tried++] = rr;
-            if (scratch && !direct && (s = encode_map(c, scratch, &scratch_map)) != LB_OK) break;
+            if (scratch && !(direct && c->prec == LB_FP64) && (s = encode_map(c, scratch, &scratch_map)) != LB_OK) break;
             // trial k reads the scratch copy (k even) or the spare buffer (k odd) and
             // writes the other, in visiting order k & 1
             int k = 0;
@@ -533,7 +539,7 @@ lb_status lb_debug_stall_row(lb_ctx *c, int row) {
     if (s != LB_OK) return s;
     c->consts.stall_row = row;
     // the direct kernels stage no rows: a stalled row needs a ring
-    if (row != INT_MIN && c->launch.variant == lbm::direct_variant())
+    if (row != INT_MIN && c->launch.variant >= lbm::direct_variant())
         return apply_launch(c, lbm::default_ring_variant(), 0);
     return LB_OK;
 }

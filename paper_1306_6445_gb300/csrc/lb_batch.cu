@@ -19,6 +19,14 @@
 namespace {
 
 constexpr int kGraphSteps = 64;   // steps per captured graph (even: the phase returns)
+// Most sites of a group of the direct launch (or one lattice): both buffers of the kChains groups
+// that run side by side (57 MB in FP32) stay in L2 over their steps. 64 steps of 512 lattices of
+// 64^2 to 512^2, sites / groups side by side: 2^18 / 3 39.4 ms, 2^18 / 2 45.8, 2^18 / 4 41.4, 0.7 2^18
+// / 3 40.4, 1.4 2^18 / 3 41.0, 2^19 / 2 40.4, 2^20 / 1 51.7; of 512 lattices of 128^2: 6.7, 6.8, 8.6,
+// 6.6, 8.5, 7.8, 9.2. All lattices in one launch of the ring kernel: 50.2 ms.
+constexpr long long kGroupSites = 1 << 18;
+constexpr long long kShortSites = 1 << 17;   // a smaller batch is one group (and one graph)
+constexpr int kChains = 3;        // groups that run side by side, see queue_groups
 
 struct BatchCommon {
     int n = 0;
@@ -34,6 +42,15 @@ struct BatchCommon {
     void *d_lats = nullptr;              // BatchLattice<T> table
     lbm::BatchItem *d_items = nullptr;
     int n_items = 0;
+    // Lattices that take their steps together (lb_batch_step): the direct launch (variant 7) has
+    // groups that stay in L2, the ring variants one group of all items.
+    struct Group {
+        lbm::BatchGroup lattices{};      // direct launch: the lattices, how many, most tiles of one
+        int n = 0, max_tiles = 0;
+    };
+    std::vector<Group> groups;
+    cudaStream_t side[kChains - 1] = {};             // see queue_groups
+    cudaEvent_t fork = nullptr, join[kChains - 1] = {};
     int *d_errs = nullptr;
     double *d_stage = nullptr;           // rho, ux, uy staging for one lattice
     size_t stage_sites = 0;
@@ -156,6 +173,41 @@ lb_status make_chunks(lb_batch *b) {
     return LB_OK;
 }
 
+// The groups of the direct launch: active lattices by size (so that the lattices of a group have
+// about as many tiles), each group of at most kGroupSites sites (or one lattice) and of at most
+// GROUP_LATTICES lattices. Returns the number of tiles.
+int make_groups(lb_batch *b) {
+    b->groups.clear();
+    std::vector<int> order;
+    for (int i = 0; i < b->n; ++i)
+        if (b->active[i]) order.push_back(i);
+    auto sites = [&](int i) { return (long long)b->geom[i].nx * b->geom[i].ny; };
+    std::stable_sort(order.begin(), order.end(), [&](int i, int j) { return sites(i) > sites(j); });
+    // a batch of fewer sites is split evenly over the groups that run side by side, unless a group
+    // would be too short to be worth a launch of its own
+    long long all = 0, in_group = 0, most = kGroupSites;
+    for (int i : order) all += sites(i);
+    if (all <= kShortSites) most = all;
+    else if (all < kChains * kGroupSites) most = (all + kChains - 1) / kChains;
+    int total = 0;
+    for (int i : order) {
+        const lbm::Geom &g = b->geom[i];
+        if (b->groups.empty() || in_group + sites(i) > most ||
+            b->groups.back().n == lbm::GROUP_LATTICES) {
+            b->groups.emplace_back();
+            in_group = 0;
+        }
+        auto &gr = b->groups.back();
+        const int tx = (g.nx + lbm::DIRECT_COLS - 1) / lbm::DIRECT_COLS;
+        const int tiles = tx * ((g.ny + lbm::DIRECT_ROWS - 1) / lbm::DIRECT_ROWS);
+        gr.lattices.l[gr.n++] = {{buf(b, i, 0), buf(b, i, 1)}, g.nx, g.ny, g.pitch, (unsigned)g.plane, tx, i};
+        gr.max_tiles = std::max(gr.max_tiles, tiles);
+        in_group += sites(i);
+        total += tiles;
+    }
+    return total;
+}
+
 void drop_graphs(lb_batch *b) {
     for (auto &g : b->graph) {
         if (g) cudaGraphExecDestroy(g);
@@ -163,10 +215,49 @@ void drop_graphs(lb_batch *b) {
     }
 }
 
+// the tensor maps of every lattice's two buffers, for boxes of cols x rows x planes
+lb_status make_maps(lb_batch *b, int cols, int rows, int planes) {
+    EncodeTiledFn enc = batch_encode_fn();
+    if (!enc) return bfail(b, LB_ECUDA, "cuTensorMapEncodeTiled unavailable");
+    std::vector<CUtensorMap> maps(2 * (size_t)b->n);
+    const CUtensorMapDataType dt =
+        b->prec == LB_FP32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64;
+    for (int i = 0; i < b->n; ++i) {
+        const lbm::Geom &g = b->geom[i];
+        const cuuint64_t dims[3] = {(cuuint64_t)g.pitch, (cuuint64_t)g.ny, 9};
+        const cuuint64_t strides[2] = {(cuuint64_t)g.pitch * b->elem, (cuuint64_t)g.plane * b->elem};
+        const cuuint32_t box[3] = {(cuuint32_t)cols, (cuuint32_t)rows, (cuuint32_t)planes};
+        const cuuint32_t estr[3] = {1, 1, 1};
+        for (int w = 0; w < 2; ++w) {
+            CUresult r = enc(&maps[2 * i + w], dt, 3, buf(b, i, w), dims, strides, box, estr,
+                             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+            if (r != CUDA_SUCCESS) return bfail(b, LB_ECUDA, "cuTensorMapEncodeTiled failed");
+        }
+    }
+    LB_BCUDA(b, cudaMemcpy(b->d_maps, maps.data(), maps.size() * sizeof(CUtensorMap),
+                           cudaMemcpyHostToDevice));
+    return LB_OK;
+}
+
 lb_status apply_batch_launch(lb_batch *b, int variant, int rows) {
-    if (variant < 0 || variant >= lbm::ring_variant_count())
+    if (variant < 0 || variant >= lbm::step_variant_count())
         return bfail(b, LB_EINVAL, "unknown launch variant");
     if (rows <= 0) rows = 16;
+    // of the direct kernels batches have the staged tiles, compiled for LB_FP32
+    if (variant >= lbm::direct_variant())
+        variant = b->prec == LB_FP32 ? lbm::staged_variant() : lbm::default_ring_variant();
+    if (variant == lbm::staged_variant()) {
+        b->n_items = make_groups(b);
+        const lb_status st = make_maps(b, lbm::TILE_BOX_W, lbm::TILE_BOX_ROWS, 3);
+        if (st != LB_OK) return st;
+        b->variant = variant;
+        b->rows = lbm::DIRECT_ROWS;
+        b->ctas_per_sm = 1;
+        b->grid = b->groups.empty() ? 0 : b->groups[0].n * b->groups[0].max_tiles;
+        drop_graphs(b);
+        return LB_OK;
+    }
     const int tx = lbm::step_variant_tx(variant);
     int occ = 0;
     LB_BCUDA(b, lbm::configure_batch(b->prec, b->eos_kind, variant, &occ));
@@ -182,28 +273,10 @@ lb_status apply_batch_launch(lb_batch *b, int variant, int rows) {
     b->rows = rows;
     b->ctas_per_sm = std::max(occ, 1);
     b->grid = std::min(b->n_items, b->num_sms * b->ctas_per_sm);
-    // tensor maps: the box width follows the strip width of the variant
-    EncodeTiledFn enc = batch_encode_fn();
-    if (!enc) return bfail(b, LB_ECUDA, "cuTensorMapEncodeTiled unavailable");
-    std::vector<CUtensorMap> maps(2 * (size_t)b->n);
-    const CUtensorMapDataType dt =
-        b->prec == LB_FP32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64;
-    for (int i = 0; i < b->n; ++i) {
-        const lbm::Geom &g = b->geom[i];
-        const cuuint64_t dims[3] = {(cuuint64_t)g.pitch, (cuuint64_t)g.ny, 9};
-        const cuuint64_t strides[2] = {(cuuint64_t)g.pitch * b->elem, (cuuint64_t)g.plane * b->elem};
-        const cuuint32_t box[3] = {(cuuint32_t)(tx + lbm::ghost_of_prec(b->prec) + 4), 1,
-                                   (cuuint32_t)lbm::step_variant_planes(variant)};
-        const cuuint32_t estr[3] = {1, 1, 1};
-        for (int w = 0; w < 2; ++w) {
-            CUresult r = enc(&maps[2 * i + w], dt, 3, buf(b, i, w), dims, strides, box, estr,
-                             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-            if (r != CUDA_SUCCESS) return bfail(b, LB_ECUDA, "cuTensorMapEncodeTiled failed");
-        }
-    }
-    LB_BCUDA(b, cudaMemcpy(b->d_maps, maps.data(), maps.size() * sizeof(CUtensorMap),
-                           cudaMemcpyHostToDevice));
+    b->groups.assign(b->n_items > 0 ? 1 : 0, {});
+    const lb_status st = make_maps(b, tx + lbm::ghost_of_prec(b->prec) + 4, 1,
+                                   lbm::step_variant_planes(variant));
+    if (st != LB_OK) return st;
     drop_graphs(b);
     return LB_OK;
 }
@@ -236,15 +309,60 @@ void count_steps(lb_batch *b, int n) {
         if (b->active[i]) b->lat_steps[i] += n;
 }
 
-lb_status launch_steps(lb_batch *b, int n) {
-    for (int i = 0; i < n; ++i) {
-        if (b->n_items > 0)
-            LB_BCUDA(b, lbm::launch_batch_step(b->prec, b->eos_kind, b->variant, b->grid,
-                                               b->d_maps, b->d_lats, b->d_items, b->n_items,
-                                               b->phase, b->d_errs, b->stream));
-        b->phase ^= 1;
-        count_steps(b, 1);
+cudaError_t launch_group(const lb_batch *b, const BatchCommon::Group &g, int phase, cudaStream_t st) {
+    if (b->variant == lbm::staged_variant())
+        return lbm::batch_tile_f32(b->eos_kind, g.lattices, g.n, g.max_tiles, b->d_maps, b->d_lats,
+                                   phase, b->d_errs, st);
+    return lbm::launch_batch_step(b->prec, b->eos_kind, b->variant, b->grid, b->d_maps, b->d_lats,
+                                  b->d_items, b->n_items, phase, b->d_errs, st);
+}
+
+// n steps of a batch of one group from phase `phase`, queued on st
+cudaError_t queue_steps(const lb_batch *b, int n, int phase, cudaStream_t st) {
+    cudaError_t e = cudaSuccess;
+    for (const auto &g : b->groups)
+        for (int i = 0; i < n && e == cudaSuccess; ++i) e = launch_group(b, g, phase ^ (i & 1), st);
+    return e;
+}
+
+// The side streams of several groups, made on first use.
+cudaError_t ensure_side(lb_batch *b) {
+    cudaError_t e = cudaSuccess;
+    if (!b->fork) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
+    for (int c = 0; c < kChains - 1 && e == cudaSuccess; ++c) {
+        if (!b->side[c]) e = cudaStreamCreateWithFlags(&b->side[c], cudaStreamNonBlocking);
+        if (e == cudaSuccess && !b->join[c])
+            e = cudaEventCreateWithFlags(&b->join[c], cudaEventDisableTiming);
     }
+    return e;
+}
+
+// n steps of a batch of several groups: a group takes all its steps before the next one (lattices
+// are independent), so that its state stays in L2, and kChains groups run side by side: one
+// computes while another starts a launch or drains one.
+cudaError_t queue_groups(lb_batch *b, int n) {
+    cudaError_t e = ensure_side(b);
+    if (e == cudaSuccess) e = cudaEventRecord(b->fork, b->stream);
+    for (int c = 0; c < kChains - 1 && e == cudaSuccess; ++c)
+        e = cudaStreamWaitEvent(b->side[c], b->fork, 0);
+    for (size_t k = 0; k < b->groups.size() && e == cudaSuccess; k += kChains)
+        for (int i = 0; i < n && e == cudaSuccess; ++i)
+            for (size_t c = 0; c < kChains && k + c < b->groups.size() && e == cudaSuccess; ++c)
+                e = launch_group(b, b->groups[k + c], b->phase ^ (i & 1),
+                                 c == 0 ? b->stream : b->side[c - 1]);
+    for (int c = 0; c < kChains - 1; ++c) {       // also after an error: nothing is left unjoined
+        cudaError_t j = cudaEventRecord(b->join[c], b->side[c]);
+        if (j == cudaSuccess) j = cudaStreamWaitEvent(b->stream, b->join[c], 0);
+        if (e == cudaSuccess) e = j;
+    }
+    return e;
+}
+
+lb_status launch_steps(lb_batch *b, int n) {
+    LB_BCUDA(b, b->groups.size() > 1 ? queue_groups(b, n)
+                                     : queue_steps(b, n, b->phase, b->stream));
+    b->phase ^= n & 1;
+    count_steps(b, n);
     return LB_OK;
 }
 
@@ -255,10 +373,7 @@ lb_status ensure_graph(lb_batch *b, int phase) {
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        for (int i = 0; i < kGraphSteps && e == cudaSuccess; ++i)
-            e = lbm::launch_batch_step(b->prec, b->eos_kind, b->variant, b->grid, b->d_maps,
-                                       b->d_lats, b->d_items, b->n_items, phase ^ (i & 1),
-                                       b->d_errs, cap);
+        e = queue_steps(b, kGraphSteps, phase, cap);
         cudaError_t e2 = cudaStreamEndCapture(cap, &g);
         if (e == cudaSuccess) e = e2;
     }
@@ -400,7 +515,7 @@ lb_status lb_batch_create(lb_batch **out, int n, const lb_lattice_desc *descs, i
         return s;
     }
     s = prec == LB_FP32 ? upload_lattices<float>(b) : upload_lattices<double>(b);
-    if (s == LB_OK) s = apply_batch_launch(b, lbm::default_ring_variant(), 16);
+    if (s == LB_OK) s = apply_batch_launch(b, lbm::staged_variant(), 16);
     if (s != LB_OK) {
         std::fprintf(stderr, "lb_batch_create: %s\n", b->msg.c_str());
         lb_batch_free(b);
@@ -460,20 +575,26 @@ lb_status lb_batch_autotune(lb_batch *b, int trial_steps, int *variant, int *row
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (e == cudaSuccess) e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
-    for (int v = 0; v < lbm::ring_variant_count() && e == cudaSuccess; ++v) {
+    for (int v = 0; v < lbm::step_variant_count() && e == cudaSuccess; ++v) {
         for (int r : cand_rows) {
+            if (v == lbm::direct_variant()) break;   // batches take the staged tiles
+            if (v == lbm::staged_variant() && (b->prec != LB_FP32 || r != cand_rows[0])) break;
             if (apply_batch_launch(b, v, r) != LB_OK) continue;
+            // the groups of the staged tiles keep their state in L2 over the steps of a call: they
+            // are timed over a call of some length
+            const int steps = v == lbm::staged_variant() ? std::max(trial_steps, 16) : trial_steps;
             if (launch_steps(b, 1) != LB_OK) continue;                 // warm-up
             cudaEventRecord(e0, b->stream);
-            if (launch_steps(b, trial_steps) != LB_OK) continue;
+            if (launch_steps(b, steps) != LB_OK) continue;
             cudaEventRecord(e1, b->stream);
             e = cudaEventSynchronize(e1);
             float ms = 0;
             if (e == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
+            ms /= (float)steps;
             if (ms > 0 && ms < best) {
                 best = ms;
                 bv = v;
-                br = r;
+                br = b->rows;
             }
         }
     }
@@ -525,7 +646,9 @@ lb_status lb_batch_step(lb_batch *b, int n) {
     const lbm::NvtxRange nvtx_range("lb_batch_step");
     if (!b || n < 0) return LB_EINVAL;
     if (b->sticky != LB_OK) return b->sticky;
-    while (n >= kGraphSteps) {
+    // several groups are launched one by one: a graph of all their steps would cost more to build
+    // (2 us a node) than the launches, which run ahead of the GPU
+    while (n >= kGraphSteps && b->groups.size() <= 1) {
         if (b->n_items > 0) {
             lb_status s = ensure_graph(b, b->phase);
             if (s != LB_OK) return s;
@@ -625,6 +748,11 @@ void lb_batch_free(lb_batch *b) {
     if (b->stream) cudaStreamSynchronize(b->stream);
     else cudaDeviceSynchronize();
     drop_graphs(b);
+    for (int c = 0; c < kChains - 1; ++c) {
+        if (b->side[c]) cudaStreamDestroy(b->side[c]);
+        if (b->join[c]) cudaEventDestroy(b->join[c]);
+    }
+    if (b->fork) cudaEventDestroy(b->fork);
     cudaFree(b->pool);
     cudaFree(b->d_maps);
     cudaFree(b->d_lats);

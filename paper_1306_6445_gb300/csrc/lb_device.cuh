@@ -26,28 +26,34 @@ struct ArithOf<__nv_bfloat16> { using type = float; };
 template <typename T>
 using Arith = typename ArithOf<T>::type;
 
-template <typename T>
-struct DevConsts {
-    T b4;                                  // Carnahan-Starling, 2/G folded in: see eos_psi
-    T rtc, a2, c3;
-    T psi0, rho0;
-    T th_v, th_m, th_l, rho1, rho2, p_rho1, p_rho2;
-    T two_over_G;
-    T G, mG12, qk3;                        // G, -G/12, kappa G / 6
+// The update's constants as values of type C: the arithmetic type itself in kernel parameters
+// (DevConsts), pairs (v, v) where a kernel keeps them in shared memory (lb_tile.cuh): a packed
+// operation then takes its constant as loaded.
+template <typename C>
+struct ConstFields {
+    C b4;                                  // Carnahan-Starling, 2/G folded in: see eos_psi
+    C rtc, a2, c3;
+    C psi0, rho0;
+    C th_v, th_m, th_l, rho1, rho2, p_rho1, p_rho2;
+    C two_over_G;
+    C G, mG12, qk3;                        // G, -G/12, kappa G / 6
     // Eq. 17 coefficients of the moments as M^-1 uses them (collide): (e + 2 rho)/36,
     // (zeta - rho)/36, q/12, p/4. *_m multiplies the moment itself (1 - s); the others, in the
     // order of the terms of collide, the equilibrium, the forcing (1 - s/2) and the source.
     // Rounded once from FP64.
-    T e_m, e_w, e_fs, e_ss, e_tr;
-    T z_m, z_w, z_fs, z_ss, z_tr;
-    T q_m, q_j, q_f;
-    T v_m, v_u, v_f2, v_f4, v_q4, v_q16;
+    C e_m, e_w, e_fs, e_ss, e_tr;
+    C z_m, z_w, z_fs, z_ss, z_tr;
+    C q_m, q_j, q_f;
+    C v_m, v_u, v_f2, v_f4, v_q4, v_q16;
     // storage shift w_a rho_s: LB_BF16 stores f_a - w_a rho_s (zero for FP32 / FP64)
-    T wshift[9];
-    T rho_s;
+    C wshift[9];
+    C rho_s;
     // nu(rho) (open-boundary kernels only): sites with rho < rho_sw relax p_xx, p_xy at
     // s_vV; the v_* coefficients for that rate
-    T rho_sw, v_m_V, v_u_V, v_f2_V, v_f4_V, v_q4_V, v_q16_V;
+    C rho_sw, v_m_V, v_u_V, v_f2_V, v_f4_V, v_q4_V, v_q16_V;
+};
+template <typename T>
+struct DevConsts : ConstFields<T> {
     int stall_row;
     // LB_BF16 stochastic rounding: the step of the launch (the counter)
     unsigned sr_step;
@@ -192,33 +198,41 @@ __device__ __forceinline__ T pop_enc(Arith<T> v, int a, const DevConsts<Arith<T>
     }
 }
 
+// a constant as a scalar, however the kernel keeps it (ConstFields)
+template <typename T>
+struct V2;
+template <typename T>
+__device__ __forceinline__ T scalar(T v) { return v; }
+template <typename T>
+__device__ __forceinline__ T scalar(const V2<T> &v) { return v.lo(); }
+
 // Interaction potential psi(rho) (Sec. II): psi0 exp(-rho0/rho), or
 // sqrt(2 (p_EOS - rho c_s^2) / G) with p_EOS the Carnahan-Starling EOS or Eq. 23.
 // Sets `bad` when rho <= 0 or psi^2 <= 0 (the value is then not usable).
-template <typename T, int EOS>
-__device__ __forceinline__ T eos_psi(T rho, const DevConsts<T> &P, bool &bad) {
+template <typename T, int EOS, typename PT>
+__device__ __forceinline__ T eos_psi(T rho, const PT &P, bool &bad) {
     if constexpr (EOS == LB_EOS_EXP) {
         bad |= !(rho > T(0));
-        return rmul(P.psi0, lb_exp(-lb_div(P.rho0, rho)));
+        return rmul(scalar<T>(P.psi0), lb_exp(-lb_div(scalar<T>(P.rho0), rho)));
     } else {
         T arg;   // 2 (p_EOS - rho/3) / G
         if constexpr (EOS == LB_EOS_CS) {
             // p = rho RT (1 + eta + eta^2 - eta^3) / (1 - eta)^3 - a rho^2; with 2/G folded
             // into the constants, arg = rho RT' poly / den - a' rho^2 - 2 rho/(3G)
-            const T eta = rmul(P.b4, rho);
+            const T eta = rmul(scalar<T>(P.b4), rho);
             const T om = rsub(T(1), eta);
             const T poly = rfma(eta, rfma(eta, om, T(1)), T(1));
-            const T num = rmul(rmul(rho, P.rtc), poly);
+            const T num = rmul(rmul(rho, scalar<T>(P.rtc)), poly);
             const T q = rmul(num, lb_rcp(rmul(rmul(om, om), om)));
             if constexpr (std::is_same<T, float>::value)   // the three terms rounded apart: see eos_psi2
-                arg = rsub(rsub(q, rmul(P.a2, rmul(rho, rho))), rmul(rho, P.c3));
+                arg = rsub(rsub(q, rmul(scalar<T>(P.a2), rmul(rho, rho))), rmul(rho, scalar<T>(P.c3)));
             else
-                arg = rfma(rho, -rfma(P.a2, rho, P.c3), q);
+                arg = rfma(rho, -rfma(scalar<T>(P.a2), rho, scalar<T>(P.c3)), q);
         } else {
-            const T p = (rho <= P.rho1) ? rmul(rho, P.th_v)
-                      : (rho < P.rho2) ? rfma(rsub(rho, P.rho1), P.th_m, P.p_rho1)
-                                       : rfma(rsub(rho, P.rho2), P.th_l, P.p_rho2);
-            arg = rmul(rsub(p, rmul(rho, T(1.0 / 3.0))), P.two_over_G);
+            const T p = (rho <= scalar<T>(P.rho1)) ? rmul(rho, scalar<T>(P.th_v))
+                      : (rho < scalar<T>(P.rho2)) ? rfma(rsub(rho, scalar<T>(P.rho1)), scalar<T>(P.th_m), scalar<T>(P.p_rho1))
+                                       : rfma(rsub(rho, scalar<T>(P.rho2)), scalar<T>(P.th_l), scalar<T>(P.p_rho2));
+            arg = rmul(rsub(p, rmul(rho, T(1.0 / 3.0))), scalar<T>(P.two_over_G));
         }
         bad |= !(arg > T(0)) || !(rho > T(0));
         return lb_sqrt_pos(arg);
@@ -236,6 +250,7 @@ struct V2<float> {
     __device__ __forceinline__ V2(float2 a) : v(a) {}
     __device__ __forceinline__ V2(float a, float b) : v(make_float2(a, b)) {}
     __device__ __forceinline__ static V2 all(float a) { return V2(a, a); }
+    __device__ __forceinline__ static V2 all(V2 a) { return a; }   // a constant kept as a pair
     __device__ __forceinline__ float lo() const { return v.x; }
     __device__ __forceinline__ float hi() const { return v.y; }
 };
@@ -315,9 +330,8 @@ __device__ __forceinline__ V1<T> pick_ge(V1<T> a, T limit, T x, T y) {
 // psi of two densities; lane by lane the same operations, in the same order and with
 // the same rounding, as eos_psi (so a site's psi does not depend on which lane or which
 // kernel computes it). `hi_valid` = false: the second lane is padding and is not checked.
-template <typename T, int EOS>
-__device__ __forceinline__ V2<T> eos_psi2(V2<T> rho, const DevConsts<T> &P, bool hi_valid,
-                                          bool &bad) {
+template <typename T, int EOS, typename PT>
+__device__ __forceinline__ V2<T> eos_psi2(V2<T> rho, const PT &P, bool hi_valid, bool &bad) {
     if constexpr (EOS == LB_EOS_CS) {
         using V = V2<T>;
         const V one = V::all(T(1));
@@ -371,8 +385,8 @@ __device__ __forceinline__ V2<T> eos_psi2(V2<T> rho, const DevConsts<T> &P, bool
 //   SH (LB_BF16): f holds the stored shifted populations f_a - w_a rho_s. Of the quantities
 //   above the shift only moves rho (to which rho_s is added) and the rest state w_a rho, in
 //   which the shifted sum then gives the shifted f* that is stored.
-template <typename T, bool VSW = false, bool SH = false, typename V>
-__device__ __forceinline__ void collide(V (&f)[9], const V (&pn)[9], const DevConsts<T> &P) {
+template <typename T, bool VSW = false, bool SH = false, typename V, typename PT>
+__device__ __forceinline__ void collide(V (&f)[9], const V (&pn)[9], const PT &P) {
     const V four = V::all(T(4)), half = V::all(T(0.5)), mtwo = V::all(T(-2)), mfour = V::all(T(-4));
     const V pc = pn[0];
 

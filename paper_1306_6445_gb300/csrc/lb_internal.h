@@ -79,6 +79,18 @@ struct BatchItem {
     int yb, n, dir;     // first row, row count, march direction (+1 / -1)
 };
 
+// Lattices that the direct batched step takes in one launch (a kernel parameter: what a CTA needs
+// to start its loads comes from the constant bank).
+constexpr int GROUP_LATTICES = 64;
+struct BatchGroup {
+    struct Lattice {
+        void *g[2];         // the lattice's two population buffers
+        int nx, ny, pitch;
+        unsigned plane;
+        int tiles_x, lat;
+    } l[GROUP_LATTICES];
+};
+
 // One CTA's share of a batched measurement: rows row0 .. row0 + rows - 1 of a lattice.
 struct MeasureChunk {
     int lat, row0, rows;
@@ -95,9 +107,13 @@ struct StepLaunch {
 int step_variant_count();
 int ring_variant_count();               // variants 0 .. ring_variant_count() - 1 use a TMA ring
 int direct_variant();                   // the variant of the direct kernels (lb_tile.cuh)
+int staged_variant();                   // their TMA-staged tiles (LB_FP32 and LB_BF16)
 bool direct_fits(const Geom &g);        // the direct kernels' grid holds the lattice
 int default_variant(int prec, const Geom &g);   // what a context starts with
 constexpr int DIRECT_COLS = 64, DIRECT_ROWS = 4;   // tile of the direct FP32 and BF16 kernels
+// its TMA box: columns x0 - 4 .. x0 + 67 (a 16-byte aligned start in both types), the rows of the
+// tile and one on either side, three planes
+constexpr int TILE_BOX_LEFT = 4, TILE_BOX_W = DIRECT_COLS + 8, TILE_BOX_ROWS = DIRECT_ROWS + 2;
 int step_variant_tx(int variant);
 int step_variant_planes(int variant);   // population planes per TMA box (9 or 3)
 int default_ring_variant();
@@ -132,22 +148,27 @@ LB_DECLARE_BATCH_UNIT(f64, 0)
 LB_DECLARE_BATCH_UNIT(f64, 1)
 #undef LB_DECLARE_BATCH_UNIT
 
-// direct step units (lb_tile_f32.cu, lb_tile_bf16.cu, lb_split_f64.cu); psi: ny * pitch elements
-cudaError_t tile_f32(const Consts &c, const Geom &g, int order, const void *gin,
-                     void *gout, int *err, cudaStream_t st);
-cudaError_t tile_bf16(const Consts &c, const Geom &g, int order, const void *gin,
-                      void *gout, int *err, cudaStream_t st);
+// direct step units (lb_split_f64.cu, lb_batch_tile.cu; lb_tile_f32.cu and lb_tile_bf16.cu below);
+// psi: ny * pitch elements
 cudaError_t split_f64(const Consts &c, const Geom &g, const void *gin, void *psi, void *gout,
                       int *err, cudaStream_t st);
 
-// What a step reads and writes: the input buffer (the ring variants reach it through its
-// tensor map), the output buffer, and psi scratch (FP64 direct kernels only).
+// n lattices of a group, at most max_tiles tiles each
+cudaError_t batch_tile_f32(int eos, const BatchGroup &group, int n, int max_tiles, const void *maps,
+                           const void *lats, int phase, int *errs, cudaStream_t st);
+
+// What a step reads and writes: the input buffer and its tensor map (none for the direct FP64
+// kernels), the output buffer, and psi scratch (direct FP64 kernels only).
 struct StepBuffers {
     const void *gin;
     const void *tensor_map_in;
     void *gout;
     void *psi;
 };
+cudaError_t tile_f32(const Consts &c, const Geom &g, int variant, int order,
+                     const StepBuffers &b, int *err, cudaStream_t st);
+cudaError_t tile_bf16(const Consts &c, const Geom &g, int variant, int order,
+                      const StepBuffers &b, int *err, cudaStream_t st);
 // order 0 / 1: visit the row blocks (and the rows inside them) forward / in reverse
 cudaError_t launch_step(int prec, const Consts &c, const Geom &g, const StepLaunch &l, int order,
                         const StepBuffers &b, int *err, cudaStream_t stream);

@@ -383,28 +383,38 @@ k_reduce_final(const double *__restrict__ partials, int nblocks, double *__restr
 
 // the variants of LB_STEP_VARIANTS (lb_step.cuh): strip width and planes per TMA box (9:
 // whole stored rows, 3: one plane group of the stage ring)
-int step_variant_count() { return 8; }
+int step_variant_count() { return 9; }
 int ring_variant_count() { return 7; }
 int direct_variant() { return 7; }
+int staged_variant() { return 8; }
 
 int step_variant_tx(int variant) {
-    static const int tx[] = {128, 128, 240, 64, 128, 128, 240, 64};
-    return (variant >= 0 && variant < 8) ? tx[variant] : 0;
+    static const int tx[] = {128, 128, 240, 64, 128, 128, 240, 64, 64};
+    return (variant >= 0 && variant < 9) ? tx[variant] : 0;
 }
 
 int step_variant_kind(int variant) { return variant >= 4 ? 1 : 0; }
 
 bool direct_fits(const Geom &g) { return g.ny <= 65535; }   // one grid row per lattice row (FP64)
 
-// The direct kernels, except where the state of an FP32 or BF16 lattice does not stay in L2:
-// there the step is bound by memory, which the ring's TMA loads keep busier. FP32 periodic
-// droplets on GB300, direct against autotuned ring: 64^2 2.3 / 9.4 us, 512^2 4.6 / 8.5,
-// 1024^2 12.1 / 15.1, 1448^2 26.5 / 26.4 (75.5 MB a buffer), 2048^2 51.6 / 48.7. FP64 is
-// bound by its pipe at every size: 128^2 9.1 / 118 us, 1000 x 700 225 / 341.
+// Which kernel a context starts with, from steps measured on GB300 (direct / staged / ring with
+// the autotuner's launch, us):
+//   FP64: bound by its pipe at every size, direct: 128^2 8.9 / - / 118, 1000 x 700 219 / - / 280.
+//   BF16 (stochastic rounding): staged at every size: 64^2 2.7 / 2.6 / -, 1024^2 16.0 / 14.4 / 21,
+//   2048^2 58.2 / 49.6 / 63, 4096 x 2048 114 / 96 / more.
+//   FP32, open boundaries (nu(rho) takes registers from the direct kernel): staged: 600 x 225
+//   4.5 / 4.0 / 12.8, 1800 x 675 16.5 / 14.9 / -.
+//   FP32 otherwise: direct while latency counts, up to 1.1 M sites: 64^2 2.2 / 2.3 / 9.4, 512^2
+//   4.5 / 5.2 / 8.5, 1024^2 11.8 / 12.2 / 15.1; staged to 72 MiB a buffer: 1448^2 25.9 / 25.3 /
+//   26.4; beyond, memory is the bound and the ring's longer loads are ahead: 2048^2 50.5 / 49.0 /
+//   48.7, 4096 x 2048 98.6 / 94.0 / 91.7 (walls 123 / 95.9 / 94.4).
 int default_variant(int prec, const Geom &g) {
     if (!direct_fits(g)) return default_ring_variant();
-    const long long bytes = 9 * g.plane * (prec == LB_FP32 ? 4 : 2);
-    return prec == LB_FP64 || bytes <= (72ll << 20) ? direct_variant() : default_ring_variant();
+    if (prec == LB_FP64) return direct_variant();
+    if (prec == LB_BF16) return staged_variant();
+    const long long bytes = 9 * g.plane * 4;
+    if (bytes > (72ll << 20)) return default_ring_variant();
+    return g.walls == 2 || bytes > (40ll << 20) ? staged_variant() : direct_variant();
 }
 
 int step_variant_planes(int variant) { return step_variant_kind(variant) ? 3 : 9; }
@@ -418,7 +428,7 @@ StepLaunch make_step_launch(int prec, int eos_kind, const Geom &g, int num_sms, 
     StepLaunch l;
     l.variant = variant;
     l.tx = step_variant_tx(variant);
-    if (variant == direct_variant()) {
+    if (variant >= direct_variant()) {
         // its grid is fixed by the lattice: rows_override does not apply
         l.rows = prec == LB_FP64 ? 1 : std::min(DIRECT_ROWS, g.ny);
         l.ctas_per_sm = prec == LB_FP64 ? 2048 / DIRECT_COLS : 65536 / (32 * DIRECT_ROWS * 80);
@@ -458,16 +468,16 @@ static cudaError_t launch_step_unit(int prec, const Consts &c, const Geom &g, co
 }
 
 cudaError_t configure_step(int prec, const Consts &c, const Geom &g, const StepLaunch &l) {
-    if (l.variant == direct_variant()) return cudaSuccess;
+    if (l.variant >= direct_variant()) return cudaSuccess;
     static const CUtensorMap dummy{};
     return launch_step_unit(prec, c, g, l, 0, &dummy, nullptr, nullptr, nullptr, true);
 }
 
 cudaError_t launch_step(int prec, const Consts &c, const Geom &g, const StepLaunch &l, int order,
                         const StepBuffers &b, int *err, cudaStream_t st) {
-    if (l.variant == direct_variant()) {
+    if (l.variant >= direct_variant()) {
         if (prec == LB_FP64) return split_f64(c, g, b.gin, b.psi, b.gout, err, st);
-        return (prec == LB_FP32 ? tile_f32 : tile_bf16)(c, g, order, b.gin, b.gout, err, st);
+        return (prec == LB_FP32 ? tile_f32 : tile_bf16)(c, g, l.variant, order, b, err, st);
     }
     return launch_step_unit(prec, c, g, l, order, b.tensor_map_in, b.gout, err, st, false);
 }

@@ -267,9 +267,8 @@ __device__ __forceinline__ V2<Arith<T>> ring_pair(const T *p) {
 }
 
 // the density of two sites from their stored values (plus rho_s for LB_BF16)
-template <typename T>
-__device__ __forceinline__ V2<Arith<T>> site_rho(const V2<Arith<T>> (&f)[9],
-                                                 const DevConsts<Arith<T>> &P) {
+template <typename T, typename PT>
+__device__ __forceinline__ V2<Arith<T>> site_rho(const V2<Arith<T>> (&f)[9], const PT &P) {
     if constexpr (std::is_same<T, __nv_bfloat16>::value)
         return rho_pair(f) + V2<float>::all(P.rho_s);
     else
@@ -349,9 +348,7 @@ __device__ __forceinline__ void store_pair<double>(double *p, V2<double> v, bool
 // rounding, r32 its random bits for the pair (low half for the first site, high half for
 // the second)
 template <typename T, bool SR = false>
-__device__ __forceinline__ void store_pop_pair(T *p, V2<Arith<T>> v, bool both, int a,
-                                               const DevConsts<Arith<T>> &P, unsigned r32 = 0) {
-    (void)a; (void)P;
+__device__ __forceinline__ void store_pop_pair(T *p, V2<Arith<T>> v, bool both, unsigned r32 = 0) {
     if constexpr (std::is_same<T, __nv_bfloat16>::value) {
         const V2<float> d = v;
         if constexpr (SR) {
@@ -368,15 +365,15 @@ __device__ __forceinline__ void store_pop_pair(T *p, V2<Arith<T>> v, bool both, 
 }
 
 // the stochastic-rounding key of a site pair (SR: LB_BF16 with stochastic rounding), else 0
-template <typename T, bool SR>
-__device__ __forceinline__ unsigned store_key(int x, int y, const DevConsts<Arith<T>> &P) {
+template <typename T, bool SR, typename PT>
+__device__ __forceinline__ unsigned store_key(int x, int y, const PT &P) {
     if constexpr (SR && std::is_same<T, __nv_bfloat16>::value)
         return sr_pair_key(x, y, P.sr_step);
     else
         return 0u;
 }
 template <typename T, bool SR>
-__device__ __forceinline__ unsigned store_bits(unsigned key, int a, const DevConsts<Arith<T>> &) {
+__device__ __forceinline__ unsigned store_bits(unsigned key, int a) {
     if constexpr (SR && std::is_same<T, __nv_bfloat16>::value)
         return sr_bits(key, a);
     else
@@ -389,11 +386,11 @@ __device__ __forceinline__ unsigned store_bits(unsigned key, int a, const DevCon
 template <typename T, int BC, bool SR>
 __device__ __forceinline__ void store_ghosts(T *__restrict__ gout, const V2<Arith<T>> (&f)[9], int x,
                                              unsigned rowi, int nx, unsigned plane, bool both,
-                                             unsigned key, const DevConsts<Arith<T>> &P) {
+                                             unsigned key) {
     if (BC == 2 ? !(x == 0 || x + 1 >= nx - 1) : !(x < 2 || x + 1 >= nx - 2)) return;
 #pragma unroll
     for (int a = 0; a < 9; ++a) {
-        const unsigned r = store_bits<T, SR>(key, a, P);
+        const unsigned r = store_bits<T, SR>(key, a);
         const T v0 = stored_enc<T, SR>(f[a].lo(), r), v1 = stored_enc<T, SR>(f[a].hi(), r >> 16);
         T *rb = gout + (rowi + plane_of(a) * plane);
         if (BC == 2) {
@@ -588,9 +585,9 @@ __device__ __forceinline__ int march(const CUtensorMap *tmap, T *__restrict__ go
             const unsigned key = store_key<T, SR>(x, yr, P);
 #pragma unroll
             for (int a = 0; a < 9; ++a)
-                store_pop_pair<T, SR>(gout + (idx + plane_of(a) * plane), fc[a], both, a, P,
-                                  store_bits<T, SR>(key, a, P));
-            store_ghosts<T, BC, SR>(gout, fc, x, (unsigned)yr * (unsigned)pitch, nx, plane, both, key, P);
+                store_pop_pair<T, SR>(gout + (idx + plane_of(a) * plane), fc[a], both,
+                                  store_bits<T, SR>(key, a));
+            store_ghosts<T, BC, SR>(gout, fc, x, (unsigned)yr * (unsigned)pitch, nx, plane, both, key);
         }
         return true;
     };
@@ -841,15 +838,15 @@ __device__ __forceinline__ int march_stage(const CUtensorMap *tmap, T *__restric
             if (w == TX) {   // a whole strip (CTA-uniform): every thread stores two sites
 #pragma unroll
                 for (int a = 0; a < 9; ++a)
-                    store_pop_pair<T, SR>(gout + (idx + plane_of(a) * plane), fc[a], true, a, P,
-                                      store_bits<T, SR>(key, a, P));
+                    store_pop_pair<T, SR>(gout + (idx + plane_of(a) * plane), fc[a], true,
+                                      store_bits<T, SR>(key, a));
             } else {
 #pragma unroll
                 for (int a = 0; a < 9; ++a)
-                    store_pop_pair<T, SR>(gout + (idx + plane_of(a) * plane), fc[a], both, a, P,
-                                      store_bits<T, SR>(key, a, P));
+                    store_pop_pair<T, SR>(gout + (idx + plane_of(a) * plane), fc[a], both,
+                                      store_bits<T, SR>(key, a));
             }
-            store_ghosts<T, BC, SR>(gout, fc, x, (unsigned)y * (unsigned)pitch, nx, plane, both, key, P);
+            store_ghosts<T, BC, SR>(gout, fc, x, (unsigned)y * (unsigned)pitch, nx, plane, both, key);
         }
         return true;
     };

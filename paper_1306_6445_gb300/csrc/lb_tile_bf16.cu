@@ -3,9 +3,9 @@
 
 namespace lbm {
 
-cudaError_t tile_bf16(const Consts &c, const Geom &g, int order, const void *gin,
-                      void *gout, int *err, cudaStream_t st) {
-    return tile_dispatch<__nv_bfloat16>(c, g, order, gin, gout, err, st);
+cudaError_t tile_bf16(const Consts &c, const Geom &g, int variant, int order,
+                     const StepBuffers &b, int *err, cudaStream_t st) {
+    return tile_dispatch<__nv_bfloat16>(c, g, variant, order, b, err, st);
 }
 
 }  // namespace lbm

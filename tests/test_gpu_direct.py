@@ -1,6 +1,6 @@
 """The direct step kernels (launch variant 7: one CTA per 64-column tile in FP32 and BF16, a psi
-and a collision pass in FP64) give the bits of the ring kernels (variant 4) at the edges of
-their tiles: lattices narrower than a tile, one column short of, exactly and one or two beyond
+and a collision pass in FP64; variant 8: pipelined tiles) give the bits of the ring kernels
+(variant 4) at the edges of their tiles: lattices narrower than a tile, one column short of, exactly and one or two beyond
 it, and rows around the tile height, for every boundary, EOS and storage type."""
 import numpy as np
 import pytest
@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 torch = pytest.importorskip("torch")
 
-SIZES = [(3, 3), (5, 4), (63, 5), (64, 8), (65, 7), (66, 3), (127, 12), (128, 9), (130, 17), (257, 4)]
+SIZES = [(3, 3), (5, 4), (63, 5), (64, 8), (65, 7), (66, 3), (127, 12), (128, 9), (130, 17), (257, 4), (66, 21), (70, 22), (192, 19), (700, 401)]
 
 
 @pytest.mark.parametrize("prec", ["fp32", "fp64", "bf16", "bf16-stochastic"])
@@ -32,7 +32,7 @@ def test_direct_kernels_give_the_ring_kernels_bits(lbm, prec, bc, kind):  # noqa
         rho = I.smooth_random_density(rng, nx, ny, lo, hi)
         ux, uy = I.random_velocity(rng, rho.shape, 1e-3)
         outs = []
-        for variant in (4, 7):
+        for variant in (4, 7) if prec == "fp64" else (4, 7, 8):
             lat = lbm.Lattice(nx, ny, eos, G, kappa=0.4, sigma_force=0.05,
                               rates=lbm.RateParams.from_viscosity(0.1), prec=prec.split("-")[0], **kw)
             lbm.lb_set_launch(lat.ctx, variant, 0)
@@ -41,4 +41,5 @@ def test_direct_kernels_give_the_ring_kernels_bits(lbm, prec, bc, kind):  # noqa
             lat.step(3)
             outs.append(lat.populations())
             lat.close()
-        assert np.array_equal(outs[0], outs[1]), (nx, ny)
+        for o in outs[1:]:
+            assert np.array_equal(o, outs[0]), (nx, ny)
