@@ -60,6 +60,8 @@ struct BatchCommon {
     int *d_first = nullptr;                  // first chunk of lattice i, n + 1 entries
     double *d_partials = nullptr;            // 8 doubles per chunk
     int n_chunks = 0;
+    int *h_errs = nullptr;                   // page-locked: error words, radii, measured sums
+    double *h_radius = nullptr, *h_meas = nullptr;
     int variant = 0, rows = 16, grid = 0, ctas_per_sm = 1, num_sms = 0;
     int phase = 0;                       // which buffer holds the active lattices' state
     std::vector<unsigned char> active;   // lattices stepped by lb_batch_step
@@ -147,15 +149,19 @@ bool make_items(const lb_batch *b, int tx, int rows, std::vector<lbm::BatchItem>
     return true;
 }
 
-// The chunks of a measurement: whole rows, about 8192 sites each (32 per thread), at most 256
-// per lattice (one pass of k_batch_measure_sum's lanes over eight).
+// The chunks of a measurement: whole rows, 8192 sites each (32 per thread) or, in a small batch,
+// as few as 1024, so that the SMs have four CTAs each; at most 256 per lattice (one pass of
+// k_batch_measure_sum's lanes over eight).
 lb_status make_chunks(lb_batch *b) {
+    long long all = 0;
+    for (const auto &g : b->geom) all += (long long)g.nx * g.ny;
+    const int sites = (int)std::max<long long>(1024, std::min<long long>(8192, all / (4 * b->num_sms)));
     std::vector<lbm::MeasureChunk> chunks;
     std::vector<int> first(b->n + 1);
     for (int i = 0; i < b->n; ++i) {
         first[i] = (int)chunks.size();
         const int nx = b->geom[i].nx, ny = b->geom[i].ny;
-        const int rows = std::max(std::max(1, 8192 / nx), (ny + 255) / 256);
+        const int rows = std::max(std::max(1, sites / nx), (ny + 255) / 256);
         for (int y = 0; y < ny; y += rows) chunks.push_back({i, y, std::min(rows, ny - y)});
     }
     first[b->n] = b->n_chunks = (int)chunks.size();
@@ -199,7 +205,7 @@ int make_groups(lb_batch *b) {
         }
         auto &gr = b->groups.back();
         const int tx = (g.nx + lbm::DIRECT_COLS - 1) / lbm::DIRECT_COLS;
-        const int tiles = tx * ((g.ny + lbm::DIRECT_ROWS - 1) / lbm::DIRECT_ROWS);
+        const int tiles = tx * ((g.ny + lbm::STAGED_ROWS - 1) / lbm::STAGED_ROWS);
         gr.lattices.l[gr.n++] = {{buf(b, i, 0), buf(b, i, 1)}, g.nx, g.ny, g.pitch, (unsigned)g.plane, tx, i};
         gr.max_tiles = std::max(gr.max_tiles, tiles);
         in_group += sites(i);
@@ -252,7 +258,7 @@ lb_status apply_batch_launch(lb_batch *b, int variant, int rows) {
         const lb_status st = make_maps(b, lbm::TILE_BOX_W, lbm::TILE_BOX_ROWS, 3);
         if (st != LB_OK) return st;
         b->variant = variant;
-        b->rows = lbm::DIRECT_ROWS;
+        b->rows = lbm::STAGED_ROWS;
         b->ctas_per_sm = 1;
         b->grid = b->groups.empty() ? 0 : b->groups[0].n * b->groups[0].max_tiles;
         drop_graphs(b);
@@ -385,12 +391,13 @@ lb_status ensure_graph(lb_batch *b, int phase) {
     return LB_OK;
 }
 
+// waits for the stream; h_errs then holds the lattices' error words
 lb_status batch_sync(lb_batch *b) {
+    LB_BCUDA(b, cudaMemcpyAsync(b->h_errs, b->d_errs, b->n * sizeof(int), cudaMemcpyDeviceToHost,
+                                b->stream));
     LB_BCUDA(b, cudaStreamSynchronize(b->stream));
-    std::vector<int> errs(b->n);
-    LB_BCUDA(b, cudaMemcpy(errs.data(), b->d_errs, b->n * sizeof(int), cudaMemcpyDeviceToHost));
     int any = 0;
-    for (int v : errs) any |= v;
+    for (int i = 0; i < b->n; ++i) any |= b->h_errs[i];
     if (any & lbm::ERR_TIMEOUT)
         return bfail(b, LB_ETIMEOUT, "a bounded device-side wait gave up", true);
     return LB_OK;   // per-lattice domain errors are reported by lb_batch_errors
@@ -503,6 +510,9 @@ lb_status lb_batch_create(lb_batch **out, int n, const lb_lattice_desc *descs, i
         cudaMalloc(&b->d_stage, 3 * b->stage_sites * sizeof(double)) != cudaSuccess ||
         cudaMalloc(&b->d_radius, n * sizeof(double)) != cudaSuccess ||
         cudaMalloc(&b->d_meas, 8 * (size_t)n * sizeof(double)) != cudaSuccess ||
+        cudaMallocHost(&b->h_errs, n * sizeof(int)) != cudaSuccess ||
+        cudaMallocHost(&b->h_radius, n * sizeof(double)) != cudaSuccess ||
+        cudaMallocHost(&b->h_meas, 8 * (size_t)n * sizeof(double)) != cudaSuccess ||
         cudaMemset(b->pool, 0, total) != cudaSuccess ||
         cudaMemset(b->d_errs, 0, n * sizeof(int)) != cudaSuccess) {
         lb_batch_free(b);
@@ -670,7 +680,7 @@ lb_status lb_batch_errors(lb_batch *b, int *flags) {
     if (!b || !flags) return LB_EINVAL;
     lb_status s = batch_sync(b);
     if (s != LB_OK && s != LB_ETIMEOUT) return s;
-    LB_BCUDA(b, cudaMemcpy(flags, b->d_errs, b->n * sizeof(int), cudaMemcpyDeviceToHost));
+    std::memcpy(flags, b->h_errs, b->n * sizeof(int));
     return s;
 }
 
@@ -703,21 +713,20 @@ lb_status lb_batch_measure(lb_batch *b, const double *radius, double *out) {
     const lbm::NvtxRange nvtx_range("lb_batch_measure");
     if (!b || !radius || !out) return LB_EINVAL;
     if (b->sticky != LB_OK) return b->sticky;
-    LB_BCUDA(b, cudaMemcpyAsync(b->d_radius, radius, b->n * sizeof(double), cudaMemcpyHostToDevice,
-                                b->stream));
+    // every call that uses h_radius waits for its stream before it returns
+    std::memcpy(b->h_radius, radius, b->n * sizeof(double));
+    LB_BCUDA(b, cudaMemcpyAsync(b->d_radius, b->h_radius, b->n * sizeof(double),
+                                cudaMemcpyHostToDevice, b->stream));
     LB_BCUDA(b, lbm::launch_batch_measure(b->prec, b->eos_kind, b->d_lats, b->n, b->d_chunks,
                                           b->d_first, b->n_chunks, b->phase, b->d_radius,
                                           b->d_partials, b->d_meas, b->stream));
-    std::vector<double> raw(8 * (size_t)b->n);
-    LB_BCUDA(b, cudaMemcpyAsync(raw.data(), b->d_meas, raw.size() * sizeof(double),
+    LB_BCUDA(b, cudaMemcpyAsync(b->h_meas, b->d_meas, 8 * (size_t)b->n * sizeof(double),
                                 cudaMemcpyDeviceToHost, b->stream));
     lb_status s = batch_sync(b);
     if (s != LB_OK) return s;
-    std::vector<int> errs(b->n);
-    LB_BCUDA(b, cudaMemcpy(errs.data(), b->d_errs, b->n * sizeof(int), cudaMemcpyDeviceToHost));
     for (int i = 0; i < b->n; ++i)
-        lbm::droplet_results(&raw[8 * (size_t)i], (double)b->geom[i].nx * b->geom[i].ny,
-                             errs[i] != 0, out + 8 * (size_t)i);
+        lbm::droplet_results(b->h_meas + 8 * (size_t)i, (double)b->geom[i].nx * b->geom[i].ny,
+                             b->h_errs[i] != 0, out + 8 * (size_t)i);
     return LB_OK;
 }
 
@@ -762,6 +771,9 @@ void lb_batch_free(lb_batch *b) {
     cudaFree(b->d_radius);
     cudaFree(b->d_meas);
     cudaFree(b->d_chunks);
+    cudaFreeHost(b->h_errs);
+    cudaFreeHost(b->h_radius);
+    cudaFreeHost(b->h_meas);
     cudaFree(b->d_first);
     cudaFree(b->d_partials);
     delete b;

@@ -1,33 +1,11 @@
 // Batched-lattice kernels: the persistent step over work items with the whole-row ring
 // (FP32, FP64; the stage ring is in lb_batch_stage.cu) and the per-lattice Laplace
 // measurement.
-#include <climits>
-
 #include "lb_step.cuh"
 
 namespace lbm {
 
 namespace {
-
-// Squared distances from the lattice centre ((nx-1)/2, (ny-1)/2) are quarters of integers
-// D = (2x - nx + 1)^2 + (2y - ny + 1)^2, so r < r_in is D < below(r_in) and r > r_out is
-// D >= above(r_out) exactly as with r = sqrt(D / 4), without a root per site.
-__device__ long long below(double r) {      // smallest D with sqrt(D / 4) >= r
-    if (!(r > 0)) return 0;
-    if (r > 1e9) return LLONG_MAX;
-    long long d = (long long)(4.0 * r * r);
-    while (d > 0 && sqrt(0.25 * (double)(d - 1)) >= r) --d;
-    while (sqrt(0.25 * (double)d) < r) ++d;
-    return d;
-}
-__device__ long long above(double r) {      // smallest D with sqrt(D / 4) > r
-    if (r < 0) return 0;
-    if (!(r <= 1e9)) return LLONG_MAX;
-    long long d = (long long)(4.0 * r * r);
-    while (d > 0 && sqrt(0.25 * (double)(d - 1)) > r) --d;
-    while (!(sqrt(0.25 * (double)d) > r)) ++d;
-    return d;
-}
 
 // Laplace sums of a chunk of rows of one lattice (fixed per-thread order and fixed tree, so
 // deterministic). Inside: r < R/2; outside: r > R + 0.3 min(nx,ny)/2; p = rho/3 + (G/2) psi^2,
@@ -40,7 +18,6 @@ template <typename T, int EOS>
 __global__ void __launch_bounds__(RED_THREADS)
 k_batch_measure(const BatchLattice<T> *__restrict__ lats, const MeasureChunk *__restrict__ chunks,
                 int phase, const double *__restrict__ radius, double *__restrict__ partials) {
-    __shared__ double s[8][RED_THREADS / 32];
     __shared__ long long limit[2];
     const MeasureChunk ch = chunks[blockIdx.x];
     const BatchLattice<T> &L = lats[ch.lat];
@@ -49,7 +26,7 @@ k_batch_measure(const BatchLattice<T> *__restrict__ lats, const MeasureChunk *__
     const T *__restrict__ g = L.g[L.frozen ? 0 : phase];
     if (threadIdx.x < 2) {
         const double R = radius[ch.lat];
-        limit[threadIdx.x] = threadIdx.x == 0 ? below(0.5 * R) : above(R + 0.3 * 0.5 * min(nx, ny));
+        limit[threadIdx.x] = threadIdx.x == 0 ? quarters_below(0.5 * R) : quarters_above(R + 0.3 * 0.5 * min(nx, ny));
     }
     __syncthreads();
     const long long d_in = limit[0], d_out = limit[1];
@@ -61,7 +38,7 @@ k_batch_measure(const BatchLattice<T> *__restrict__ lats, const MeasureChunk *__
         const int x = (int)(i - row * (unsigned)nx), y = ch.row0 + (int)row;
         T v[9];
 #pragma unroll
-        for (int a = 0; a < 9; ++a) v[a] = pull_padded<T>(g, a, x, y, ny, pitch, L.plane);
+        for (int a = 0; a < 9; ++a) v[a] = pull_padded<T, 0>(g, a, x, y, ny, pitch, L.plane);
         const T rho = sum9(v);
         bool bad = false;
         const T psi = eos_psi<T, EOS>(rho, P, bad);
@@ -81,22 +58,8 @@ k_batch_measure(const BatchLattice<T> *__restrict__ lats, const MeasureChunk *__
         }
         if (bad || !(rho == rho) || !(psi == psi)) ++n_bad;
     }
-    const double hg = 0.5 * double(P.G);
-    double acc[8] = {m_in + m_out + m_rest, m_in, (double)n_in, m_out, (double)n_out,
-                     m_in / 3.0 + hg * q_in, m_out / 3.0 + hg * q_out, (double)n_bad};
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-#pragma unroll
-        for (int w = 16; w > 0; w >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], w);
-        if ((threadIdx.x & 31) == 0) s[k][threadIdx.x >> 5] = acc[k];
-    }
-    __syncthreads();
-    if (threadIdx.x < 8) {
-        double t = 0;
-#pragma unroll
-        for (int w = 0; w < RED_THREADS / 32; ++w) t += s[threadIdx.x][w];
-        partials[(size_t)blockIdx.x * 8 + threadIdx.x] = t;
-    }
+    droplet_combine(m_in, m_out, m_rest, q_in, q_out, n_in, n_out, n_bad, double(P.G),
+                    partials + (size_t)blockIdx.x * 8);
 }
 
 // Sum of the chunks of each lattice in a fixed order: warp k of CTA i adds quantity k.

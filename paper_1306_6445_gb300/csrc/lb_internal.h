@@ -110,10 +110,11 @@ int direct_variant();                   // the variant of the direct kernels (lb
 int staged_variant();                   // their TMA-staged tiles (LB_FP32 and LB_BF16)
 bool direct_fits(const Geom &g);        // the direct kernels' grid holds the lattice
 int default_variant(int prec, const Geom &g);   // what a context starts with
-constexpr int DIRECT_COLS = 64, DIRECT_ROWS = 4;   // tile of the direct FP32 and BF16 kernels
-// its TMA box: columns x0 - 4 .. x0 + 67 (a 16-byte aligned start in both types), the rows of the
-// tile and one on either side, three planes
-constexpr int TILE_BOX_LEFT = 4, TILE_BOX_W = DIRECT_COLS + 8, TILE_BOX_ROWS = DIRECT_ROWS + 2;
+// tiles of the direct and of the staged FP32 and BF16 kernels
+constexpr int DIRECT_COLS = 64, DIRECT_ROWS = 4, STAGED_ROWS = 4;
+// the staged tile's TMA box: columns x0 - 4 .. x0 + 67 (a 16-byte aligned start in both types), the
+// rows of the tile and one on either side, three planes
+constexpr int TILE_BOX_LEFT = 4, TILE_BOX_W = DIRECT_COLS + 8, TILE_BOX_ROWS = STAGED_ROWS + 2;
 int step_variant_tx(int variant);
 int step_variant_planes(int variant);   // population planes per TMA box (9 or 3)
 int default_ring_variant();
@@ -186,20 +187,46 @@ cudaError_t launch_psi_field(int prec, const Consts &c, const Geom &g, const voi
 cudaError_t launch_macro_fields(int prec, const Consts &c, const Geom &g, const void *gbuf,
                                 const void *psi, double *rho, double *ux, double *uy,
                                 cudaStream_t stream);
-// Deterministic FP64 reduction: partials must hold 4 * reduce_blocks(n) doubles.
+// Words of a context that its kernels write into page-locked host memory: after a wait for the
+// stream the host reads them, without a copy. Error bits are written only when there is an error.
+struct HostWords {
+    int err;
+    double out8[8];
+};
+
+// Deterministic FP64 reductions; partials must hold 8 * reduce_blocks(n) doubles, ticket is a device
+// word that is zero between launches. Results in out (host or device memory): mass, momentum, max
+// |v|^2 (4 doubles), and the Laplace sums of a droplet (8 doubles, layout of k_droplet_sums).
 int reduce_blocks(long long n_sites);
 cudaError_t launch_macro_reduce(int prec, const Consts &c, const Geom &g, const void *gbuf,
-                                const void *psi, double *partials, double *out4,
-                                cudaStream_t stream);
-
-// Laplace sums of a droplet (8 doubles into out8, layout of k_droplet_sums); partials must
-// hold 8 * reduce_blocks(n) doubles
+                                const void *psi, double *partials, unsigned *ticket,
+                                double *out, cudaStream_t stream);
 cudaError_t launch_droplet_sums(int prec, const Consts &c, const Geom &g, const void *gbuf,
-                                double cx, double cy, double r_in, double r_out,
-                                double *partials, double *out8, cudaStream_t stream);
+                                double r_in, double r_out, double *partials, unsigned *ticket,
+                                double *out, cudaStream_t stream);
 // interface height of every column into h (nx doubles); first: nx ints of scratch
 cudaError_t launch_interface_height(int prec, const Consts &c, const Geom &g, const void *gbuf,
                                     double rho_mid, int *first, double *h, cudaStream_t stream);
+
+// Squared distances from the lattice centre ((nx-1)/2, (ny-1)/2) are quarters of integers
+// D = (2x - nx + 1)^2 + (2y - ny + 1)^2, so r < r_in is D < quarters_below(r_in) and r > r_out is
+// D >= quarters_above(r_out) exactly as with r = sqrt(D / 4), without a root per site.
+__host__ __device__ inline long long quarters_below(double r) {   // smallest D with sqrt(D / 4) >= r
+    if (!(r > 0)) return 0;
+    if (r > 1e9) return 0x7fffffffffffffffll;
+    long long d = (long long)(4.0 * r * r);
+    while (d > 0 && sqrt(0.25 * (double)(d - 1)) >= r) --d;
+    while (sqrt(0.25 * (double)d) < r) ++d;
+    return d;
+}
+__host__ __device__ inline long long quarters_above(double r) {   // smallest D with sqrt(D / 4) > r
+    if (r < 0) return 0;
+    if (!(r <= 1e9)) return 0x7fffffffffffffffll;
+    long long d = (long long)(4.0 * r * r);
+    while (d > 0 && sqrt(0.25 * (double)(d - 1)) > r) --d;
+    while (!(sqrt(0.25 * (double)d) > r)) ++d;
+    return d;
+}
 
 // Laplace-law results from the 8 sums of a droplet measurement (the layout of
 // lb_batch_measure / lb_measure_droplet's out): theta, rho_in, rho_out, R (from the mass),

@@ -120,13 +120,12 @@ __global__ void k_init_feq(const double *__restrict__ rho, const double *__restr
 template <typename T, int EOS, int BC>
 __global__ void k_psi_field(const T *__restrict__ g, Arith<T> *__restrict__ psi,
                             const DevConsts<Arith<T>> P, int nx, int ny, int pitch,
-                            long long plane, int *__restrict__ err) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (long long)nx * ny) return;
-    const int y = (int)(i / nx), x = (int)(i % nx);
+                            unsigned plane, int *__restrict__ err) {
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (unsigned)nx * (unsigned)ny) return;
+    const unsigned y = i / (unsigned)nx, x = i - y * (unsigned)nx;
     Arith<T> v[9];
-#pragma unroll
-    for (int a = 0; a < 9; ++a) v[a] = pull_val<T, BC>(g, a, x, y, nx, ny, pitch, plane, P);
+    pull_site_vals<T, BC>(v, g, (int)x, (int)y, ny, pitch, plane, P);
     bool bad = false;
     psi[i] = eos_psi<Arith<T>, EOS>(sum9(v), P, bad);
     if (bad) atomicOr(err, ERR_DOMAIN);
@@ -136,11 +135,10 @@ __global__ void k_psi_field(const T *__restrict__ g, Arith<T> *__restrict__ psi,
 template <typename T, int BC, typename A = Arith<T>>
 __device__ __forceinline__ void site_macro(const T *__restrict__ g, const A *__restrict__ psi,
                                            const DevConsts<A> &P, int nx, int ny, int pitch,
-                                           long long plane, int x, int y, A &rho, A &vx, A &vy) {
+                                           unsigned plane, int x, int y, A &rho, A &vx, A &vy) {
     const A G = P.G;
     A v[9];
-#pragma unroll
-    for (int a = 0; a < 9; ++a) v[a] = pull_val<T, BC>(g, a, x, y, nx, ny, pitch, plane, P);
+    pull_site_vals<T, BC>(v, g, x, y, ny, pitch, plane, P);
     rho = sum9(v);
     const A jx = (v[1] - v[3]) + (v[5] - v[7]) - (v[6] - v[8]);
     const A jy = (v[2] - v[4]) + (v[5] - v[7]) + (v[6] - v[8]);
@@ -157,7 +155,7 @@ __device__ __forceinline__ void site_macro(const T *__restrict__ g, const A *__r
         yp = (y + 1 == ny) ? 0 : y + 1;
         ym = (y == 0) ? ny - 1 : y - 1;
     }
-    auto ps = [&](int xx, int yy) { return psi[(long long)yy * nx + xx]; };
+    auto ps = [&](int xx, int yy) { return psi[(unsigned)yy * (unsigned)nx + (unsigned)xx]; };
     const A third = A(1.0 / 3.0), twelfth = A(1.0 / 12.0);
     const A pc = ps(x, y);
     const A sx = (ps(xp, y) - ps(xm, y)) * third +
@@ -173,16 +171,15 @@ __device__ __forceinline__ void site_macro(const T *__restrict__ g, const A *__r
 template <typename T, int BC>
 __global__ void k_macro_fields(const T *__restrict__ g, const Arith<T> *__restrict__ psi,
                                const DevConsts<Arith<T>> P, int nx, int ny, int pitch,
-                               long long plane, double *__restrict__ rho,
+                               unsigned plane, double *__restrict__ rho,
                                double *__restrict__ ux, double *__restrict__ uy) {
     using A = Arith<T>;
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (long long)nx * ny) return;
-    const int y = (int)(i / nx), x = (int)(i % nx);
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (unsigned)nx * (unsigned)ny) return;
+    const int y = (int)(i / (unsigned)nx), x = (int)(i - (unsigned)y * (unsigned)nx);
     if (!ux && !uy) {  // density only: psi is not needed
         A v[9];
-#pragma unroll
-        for (int a = 0; a < 9; ++a) v[a] = pull_val<T, BC>(g, a, x, y, nx, ny, pitch, plane, P);
+        pull_site_vals<T, BC>(v, g, x, y, ny, pitch, plane, P);
         rho[i] = double(sum9(v));
         return;
     }
@@ -193,114 +190,105 @@ __global__ void k_macro_fields(const T *__restrict__ g, const Arith<T> *__restri
     if (uy) uy[i] = double(vy);
 }
 
+// The last CTA of a reduction to write its N partials (a ticket, which returns to zero) combines
+// all of them in a fixed order into out: no second launch.
+template <int N, int MAX>
+__device__ __forceinline__ void combine_last(const double *__restrict__ partials,
+                                             unsigned *__restrict__ ticket,
+                                             double *__restrict__ out) {
+    __shared__ bool last;
+    __threadfence();                   // this CTA's partials before its ticket
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double q[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) q[k] = 0;
+    for (unsigned b = threadIdx.x; b < gridDim.x; b += RED_THREADS) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            const double p = __ldcg(partials + (size_t)b * N + k);
+            q[k] = k < MAX ? q[k] + p : ((p > q[k] || p != p) ? p : q[k]);
+        }
+    }
+    __syncthreads();                   // block_combine's shared memory has been read
+    block_combine<N, MAX>(q, out);
+}
 
-// Block b reduces the contiguous site range [b*chunk, (b+1)*chunk) in FP64 with a fixed
-// per-thread order and a fixed shared-memory tree: the result does not depend on timing.
+// Mass, momentum and max |v|^2 in FP64 with a fixed order: thread t of CTA b takes sites
+// 256 b + t, + 256 gridDim, ...; |v| is compared squared (the root is taken of the maximum) and
+// only where FP32 does not rule it out. What bounds it: memory next to the FP64 pipe (2 operations
+// per clock and SM); with a root per site and 64-bit divisions it took 158 us at 2048^2 in FP32
+// (lb_reduce as a whole 124 against 235 us; of 501 x 383 39 against 64).
 template <typename T, int BC>
 __global__ void __launch_bounds__(RED_THREADS)
 k_macro_reduce(const T *__restrict__ g, const Arith<T> *__restrict__ psi,
-               const DevConsts<Arith<T>> P, int nx, int ny, int pitch, long long plane,
-               long long chunk, double *__restrict__ partials) {
-    __shared__ double s[4][RED_THREADS];
-    const long long n = (long long)nx * ny;
-    const long long beg = (long long)blockIdx.x * chunk;
-    const long long end = min(n, beg + chunk);
-    double m = 0, px = 0, py = 0, vmax = 0;
-    for (long long i = beg + threadIdx.x; i < end; i += RED_THREADS) {
-        const int y = (int)(i / nx), x = (int)(i % nx);
+               const DevConsts<Arith<T>> P, int nx, int ny, int pitch, unsigned plane,
+               double *__restrict__ partials, unsigned *__restrict__ ticket,
+               double *__restrict__ out) {
+    const unsigned n = (unsigned)nx * (unsigned)ny;
+    double q[4] = {0, 0, 0, 0};
+    float least = -1.f;                // |v|^2 below this cannot be the maximum
+    for (unsigned i = blockIdx.x * RED_THREADS + threadIdx.x; i < n; i += gridDim.x * RED_THREADS) {
+        const int y = (int)(i / (unsigned)nx), x = (int)(i - (unsigned)y * (unsigned)nx);
         Arith<T> r, vx, vy;
         site_macro<T, BC>(g, psi, P, nx, ny, pitch, plane, x, y, r, vx, vy);
         const double dr = r, dvx = vx, dvy = vy;
-        m += dr;
-        px += dr * dvx;
-        py += dr * dvy;
-        const double sp = sqrt(dvx * dvx + dvy * dvy);
-        vmax = (sp > vmax || sp != sp) ? sp : vmax;  // NaN propagates
-    }
-    s[0][threadIdx.x] = m;
-    s[1][threadIdx.x] = px;
-    s[2][threadIdx.x] = py;
-    s[3][threadIdx.x] = vmax;
-    __syncthreads();
-    for (int wdt = RED_THREADS / 2; wdt > 0; wdt >>= 1) {
-        if (threadIdx.x < wdt) {
-            s[0][threadIdx.x] += s[0][threadIdx.x + wdt];
-            s[1][threadIdx.x] += s[1][threadIdx.x + wdt];
-            s[2][threadIdx.x] += s[2][threadIdx.x + wdt];
-            const double o = s[3][threadIdx.x + wdt];
-            const double c = s[3][threadIdx.x];
-            s[3][threadIdx.x] = (o > c || o != o) ? o : c;
+        q[0] += dr;
+        q[1] = fma(dr, dvx, q[1]);
+        q[2] = fma(dr, dvy, q[2]);
+        const float fx = (float)vx, fy = (float)vy, f2 = fmaf(fx, fx, fy * fy);
+        if (!(f2 < least)) {           // also NaN
+            const double v2 = dvx * dvx + dvy * dvy;
+            q[3] = (v2 > q[3] || v2 != v2) ? v2 : q[3];
+            least = (float)q[3] * 0.99999f;
         }
-        __syncthreads();
     }
-    if (threadIdx.x < 4) partials[blockIdx.x * 4 + threadIdx.x] = s[threadIdx.x][0];
+    block_combine<4, 3>(q, partials + (size_t)blockIdx.x * 4);
+    combine_last<4, 3>(partials, ticket, out);
 }
 
-// Laplace-law sums of a droplet (Sec. V.A): block b sums the site range [b*chunk,
-// (b+1)*chunk) with a fixed per-thread order and a fixed tree. q[0] mass, q[1] / q[2] sum
-// of rho / count over r < r_in, q[3] / q[4] over r > r_out, q[5] / q[6] sum of the bulk
-// pressure p = rho/3 + (G/2) psi^2 inside / outside, q[7] sites with a non-finite rho or p
-// or psi off its real branch; r is the distance from (cx, cy).
+// Laplace-law sums of a droplet (Sec. V.A), sites taken as in k_macro_reduce. out[0] mass, [1] /
+// [2] sum of rho / count inside (D < d_in, see quarters_below), [3] / [4] outside (D >= d_out), [5]
+// / [6] sum of the bulk pressure p = rho/3 + (G/2) psi^2 inside / outside, [7] sites with a
+// non-finite rho or psi or psi off its real branch. FP64 operations as in k_batch_measure.
 template <typename T, int EOS, int BC>
 __global__ void __launch_bounds__(RED_THREADS)
 k_droplet_sums(const T *__restrict__ g, const DevConsts<Arith<T>> P, int nx, int ny, int pitch,
-               long long plane, long long chunk, double cx, double cy, double r_in,
-               double r_out, double *__restrict__ partials) {
+               unsigned plane, long long d_in, long long d_out, double *__restrict__ partials,
+               unsigned *__restrict__ ticket, double *__restrict__ out) {
     using A = Arith<T>;
-    __shared__ double s[8][RED_THREADS];
-    const long long n = (long long)nx * ny;
-    const long long beg = (long long)blockIdx.x * chunk;
-    const long long end = min(n, beg + chunk);
-    double q[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (long long i = beg + threadIdx.x; i < end; i += RED_THREADS) {
-        const int y = (int)(i / nx), x = (int)(i % nx);
+    const unsigned n = (unsigned)nx * (unsigned)ny;
+    double m_in = 0, m_out = 0, m_rest = 0, q_in = 0, q_out = 0;
+    int n_in = 0, n_out = 0, n_bad = 0;
+    for (unsigned i = blockIdx.x * RED_THREADS + threadIdx.x; i < n; i += gridDim.x * RED_THREADS) {
+        const int y = (int)(i / (unsigned)nx), x = (int)(i - (unsigned)y * (unsigned)nx);
         A v[9];
-#pragma unroll
-        for (int a = 0; a < 9; ++a) v[a] = pull_val<T, BC>(g, a, x, y, nx, ny, pitch, plane, P);
+        pull_site_vals<T, BC>(v, g, x, y, ny, pitch, plane, P);
         const A rho = sum9(v);
         bool bad = false;
         const A psi = eos_psi<A, EOS>(rho, P, bad);
-        const double dr = double(rho);
-        const double pr = dr / 3.0 + 0.5 * double(P.G) * double(psi) * double(psi);
-        q[0] += dr;
-        const double r = sqrt((x - cx) * (x - cx) + (y - cy) * (y - cy));
-        if (r < r_in) { q[1] += dr; q[2] += 1; q[5] += pr; }
-        if (r > r_out) { q[3] += dr; q[4] += 1; q[6] += pr; }
-        if (bad || !(dr == dr) || !(pr == pr)) q[7] += 1;
-    }
-#pragma unroll
-    for (int k = 0; k < 8; ++k) s[k][threadIdx.x] = q[k];
-    __syncthreads();
-    for (int wdt = RED_THREADS / 2; wdt > 0; wdt >>= 1) {
-        if (threadIdx.x < wdt) {
-#pragma unroll
-            for (int k = 0; k < 8; ++k) s[k][threadIdx.x] += s[k][threadIdx.x + wdt];
+        const double dr = double(rho), ds = double(psi);
+        const int a = 2 * x - (nx - 1), b = 2 * y - (ny - 1);
+        const long long d = (long long)a * a + (long long)b * b;
+        if (d < d_in) {
+            m_in += dr;
+            q_in = fma(ds, ds, q_in);
+            ++n_in;
+        } else if (d >= d_out) {
+            m_out += dr;
+            q_out = fma(ds, ds, q_out);
+            ++n_out;
+        } else {
+            m_rest += dr;
         }
-        __syncthreads();
+        if (bad || !(rho == rho) || !(psi == psi)) ++n_bad;
     }
-    if (threadIdx.x < 8) partials[blockIdx.x * 8 + threadIdx.x] = s[threadIdx.x][0];
-}
-
-// Sum of nblocks partial 8-vectors in a fixed order.
-__global__ void __launch_bounds__(RED_THREADS)
-k_sum8_final(const double *__restrict__ partials, int nblocks, double *__restrict__ out) {
-    __shared__ double s[8][RED_THREADS];
-    double q[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int b = threadIdx.x; b < nblocks; b += RED_THREADS) {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) q[k] += partials[b * 8 + k];
-    }
-#pragma unroll
-    for (int k = 0; k < 8; ++k) s[k][threadIdx.x] = q[k];
-    __syncthreads();
-    for (int wdt = RED_THREADS / 2; wdt > 0; wdt >>= 1) {
-        if (threadIdx.x < wdt) {
-#pragma unroll
-            for (int k = 0; k < 8; ++k) s[k][threadIdx.x] += s[k][threadIdx.x + wdt];
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x < 8) out[threadIdx.x] = s[threadIdx.x][0];
+    droplet_combine(m_in, m_out, m_rest, q_in, q_out, n_in, n_out, n_bad, double(P.G),
+                    partials + (size_t)blockIdx.x * 8);
+    combine_last<8, 8>(partials, ticket, out);
 }
 
 // Interface height per column (Sec. V.B), pass 1: thread (x, segment) scans the rows of
@@ -308,15 +296,14 @@ k_sum8_final(const double *__restrict__ partials, int nblocks, double *__restric
 // first[x] (atomicMin: the minimum does not depend on the order of the updates).
 template <typename T, int BC>
 __global__ void k_interface_first(const T *__restrict__ g, const DevConsts<Arith<T>> P, int nx,
-                                  int ny, int pitch, long long plane, double rho_mid, int seg,
+                                  int ny, int pitch, unsigned plane, double rho_mid, int seg,
                                   int *__restrict__ first) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= nx) return;
     const int y0 = blockIdx.y * seg, y1 = min(ny, y0 + seg);
     for (int y = y0; y < y1; ++y) {
         Arith<T> v[9];
-#pragma unroll
-        for (int a = 0; a < 9; ++a) v[a] = pull_val<T, BC>(g, a, x, y, nx, ny, pitch, plane, P);
+        pull_site_vals<T, BC>(v, g, x, y, ny, pitch, plane, P);
         if (double(sum9(v)) < rho_mid) {
             atomicMin(&first[x], y);
             return;
@@ -329,7 +316,7 @@ __global__ void k_interface_first(const T *__restrict__ g, const DevConsts<Arith
 // rho_mid or no row is
 template <typename T, int BC>
 __global__ void k_interface_height(const T *__restrict__ g, const DevConsts<Arith<T>> P, int nx,
-                                   int ny, int pitch, long long plane, double rho_mid,
+                                   int ny, int pitch, unsigned plane, double rho_mid,
                                    const int *__restrict__ first, double *__restrict__ h) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= nx) return;
@@ -340,42 +327,11 @@ __global__ void k_interface_height(const T *__restrict__ g, const DevConsts<Arit
     }
     auto rho_at = [&](int yy) {
         Arith<T> v[9];
-#pragma unroll
-        for (int a = 0; a < 9; ++a) v[a] = pull_val<T, BC>(g, a, x, yy, nx, ny, pitch, plane, P);
+        pull_site_vals<T, BC>(v, g, x, yy, ny, pitch, plane, P);
         return double(sum9(v));
     };
     const double r0 = rho_at(y - 1), r1 = rho_at(y);
     h[x] = double(y - 1) + (r0 - rho_mid) / (r0 - r1);
-}
-
-__global__ void __launch_bounds__(RED_THREADS)
-k_reduce_final(const double *__restrict__ partials, int nblocks, double *__restrict__ out) {
-    __shared__ double s[4][RED_THREADS];
-    double m = 0, px = 0, py = 0, vmax = 0;
-    for (int b = threadIdx.x; b < nblocks; b += RED_THREADS) {
-        m += partials[b * 4 + 0];
-        px += partials[b * 4 + 1];
-        py += partials[b * 4 + 2];
-        const double o = partials[b * 4 + 3];
-        vmax = (o > vmax || o != o) ? o : vmax;
-    }
-    s[0][threadIdx.x] = m;
-    s[1][threadIdx.x] = px;
-    s[2][threadIdx.x] = py;
-    s[3][threadIdx.x] = vmax;
-    __syncthreads();
-    for (int wdt = RED_THREADS / 2; wdt > 0; wdt >>= 1) {
-        if (threadIdx.x < wdt) {
-            s[0][threadIdx.x] += s[0][threadIdx.x + wdt];
-            s[1][threadIdx.x] += s[1][threadIdx.x + wdt];
-            s[2][threadIdx.x] += s[2][threadIdx.x + wdt];
-            const double o = s[3][threadIdx.x + wdt];
-            const double c = s[3][threadIdx.x];
-            s[3][threadIdx.x] = (o > c || o != o) ? o : c;
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x < 4) out[threadIdx.x] = s[threadIdx.x][0];
 }
 
 }  // namespace
@@ -430,7 +386,8 @@ StepLaunch make_step_launch(int prec, int eos_kind, const Geom &g, int num_sms, 
     l.tx = step_variant_tx(variant);
     if (variant >= direct_variant()) {
         // its grid is fixed by the lattice: rows_override does not apply
-        l.rows = prec == LB_FP64 ? 1 : std::min(DIRECT_ROWS, g.ny);
+        l.rows = prec == LB_FP64 ? 1
+               : std::min(variant == staged_variant() ? STAGED_ROWS : DIRECT_ROWS, g.ny);
         l.ctas_per_sm = prec == LB_FP64 ? 2048 / DIRECT_COLS : 65536 / (32 * DIRECT_ROWS * 80);
         return l;
     }
@@ -566,7 +523,7 @@ cudaError_t launch_psi_field(int prec, const Consts &c, const Geom &g, const voi
     k_psi_field<T, EOSK, W><<<nb, 256, 0, st>>>(static_cast<const T *>(gbuf),                \
                                                 static_cast<Arith<T> *>(psi),                \
                                                 to_dev<Arith<T>>(c), g.nx, g.ny, g.pitch,    \
-                                                g.plane, err)
+                                                (unsigned)g.plane, err)
 #define LB_PSI_W(T, EOSK)                                              \
     do {                                                               \
         if (g.walls == 2) LB_PSI(T, EOSK, 2);                          \
@@ -599,7 +556,7 @@ cudaError_t launch_macro_fields(int prec, const Consts &c, const Geom &g, const 
     k_macro_fields<T, W><<<nb, 256, 0, st>>>(static_cast<const T *>(gbuf),                    \
                                              static_cast<const Arith<T> *>(psi),              \
                                              to_dev<Arith<T>>(c), g.nx, g.ny, g.pitch,        \
-                                             g.plane, rho, ux, uy)
+                                             (unsigned)g.plane, rho, ux, uy)
     if (prec == LB_FP32) {
         BC3(LB_MAC, float);
     } else if (prec == LB_BF16) {
@@ -611,22 +568,22 @@ cudaError_t launch_macro_fields(int prec, const Consts &c, const Geom &g, const 
     return cudaGetLastError();
 }
 
+// a site per thread while that gives two CTAs per SM (the combination costs FP64 operations per
+// CTA), then more sites, and from 2^20 on four CTAs per SM (loads in flight count)
 int reduce_blocks(long long n_sites) {
-    long long nb = (n_sites + RED_THREADS * 4 - 1) / (RED_THREADS * 4);
-    return (int)std::max<long long>(1, std::min<long long>(nb, RED_MAX_BLOCKS));
+    const long long nb = (n_sites + RED_THREADS - 1) / RED_THREADS;
+    return (int)std::max<long long>(1, std::min<long long>(nb, n_sites < (1 << 20) ? 304 : 608));
 }
 
 cudaError_t launch_macro_reduce(int prec, const Consts &c, const Geom &g, const void *gbuf,
-                                const void *psi, double *partials, double *out4,
-                                cudaStream_t st) {
-    const long long n = (long long)g.nx * g.ny;
-    const int nb = reduce_blocks(n);
-    const long long chunk = (n + nb - 1) / nb;
+                                const void *psi, double *partials, unsigned *ticket,
+                                double *out, cudaStream_t st) {
+    const int nb = reduce_blocks((long long)g.nx * g.ny);
 #define LB_RED(T, W)                                                                           \
     k_macro_reduce<T, W><<<nb, RED_THREADS, 0, st>>>(static_cast<const T *>(gbuf),              \
                                                      static_cast<const Arith<T> *>(psi),       \
                                                      to_dev<Arith<T>>(c), g.nx, g.ny, g.pitch, \
-                                                     g.plane, chunk, partials)
+                                                     (unsigned)g.plane, partials, ticket, out)
     if (prec == LB_FP32) {
         BC3(LB_RED, float);
     } else if (prec == LB_BF16) {
@@ -635,23 +592,19 @@ cudaError_t launch_macro_reduce(int prec, const Consts &c, const Geom &g, const 
         BC3(LB_RED, double);
     }
 #undef LB_RED
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_reduce_final<<<1, RED_THREADS, 0, st>>>(partials, nb, out4);
     return cudaGetLastError();
 }
 
 cudaError_t launch_droplet_sums(int prec, const Consts &c, const Geom &g, const void *gbuf,
-                                double cx, double cy, double r_in, double r_out,
-                                double *partials, double *out8, cudaStream_t st) {
-    const long long n = (long long)g.nx * g.ny;
-    const int nb = reduce_blocks(n);
-    const long long chunk = (n + nb - 1) / nb;
+                                double r_in, double r_out, double *partials, unsigned *ticket,
+                                double *out, cudaStream_t st) {
+    const int nb = reduce_blocks((long long)g.nx * g.ny);
+    const long long d_in = quarters_below(r_in), d_out = quarters_above(r_out);
 #define LB_DS(T, EOSK, W)                                                                     \
     k_droplet_sums<T, EOSK, W><<<nb, RED_THREADS, 0, st>>>(static_cast<const T *>(gbuf),       \
                                                            to_dev<Arith<T>>(c), g.nx, g.ny,    \
-                                                           g.pitch, g.plane, chunk, cx, cy,    \
-                                                           r_in, r_out, partials)
+                                                           g.pitch, (unsigned)g.plane, d_in,   \
+                                                           d_out, partials, ticket, out)
 #define LB_DS_W(T, EOSK)                                              \
     do {                                                              \
         if (g.walls == 2) LB_DS(T, EOSK, 2);                          \
@@ -670,9 +623,6 @@ cudaError_t launch_droplet_sums(int prec, const Consts &c, const Geom &g, const 
 #undef LB_DS_E
 #undef LB_DS_W
 #undef LB_DS
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_sum8_final<<<1, RED_THREADS, 0, st>>>(partials, nb, out8);
     return cudaGetLastError();
 }
 
@@ -688,10 +638,12 @@ cudaError_t launch_interface_height(int prec, const Consts &c, const Geom &g, co
     do {                                                                                      \
         k_interface_first<T, W><<<grid1, TPB, 0, st>>>(static_cast<const T *>(gbuf),          \
                                                        to_dev<Arith<T>>(c), g.nx, g.ny,       \
-                                                       g.pitch, g.plane, rho_mid, SEG, first); \
+                                                       g.pitch, (unsigned)g.plane, rho_mid,   \
+                                                       SEG, first);                            \
         k_interface_height<T, W><<<grid2, TPB, 0, st>>>(static_cast<const T *>(gbuf),         \
                                                         to_dev<Arith<T>>(c), g.nx, g.ny,      \
-                                                        g.pitch, g.plane, rho_mid, first, h); \
+                                                        g.pitch, (unsigned)g.plane, rho_mid,  \
+                                                        first, h);                            \
     } while (0)
     if (prec == LB_FP32) {
         BC3(LB_IH, float);

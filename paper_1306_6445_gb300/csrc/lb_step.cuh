@@ -62,7 +62,6 @@ constexpr int AL = GH<T>;
 template <typename T, int TX>
 constexpr int ring_width() { return TX + AL<T> + 4; }
 constexpr int RED_THREADS = 256;      // reduction blocks (diagnostics, batch measurement)
-constexpr int RED_MAX_BLOCKS = 1024;
 
 // ---------------------------------------------------------------- PTX helpers
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
@@ -176,14 +175,16 @@ __device__ __forceinline__ T pull_global(const T *__restrict__ g, int a, int x, 
     return g[plane_of(a) * plane + (long long)sy * pitch + sx + GH<T>];
 }
 
-// f_a(x, y) of a periodic lattice pulled from g through its ghost columns (no wrap in x)
-template <typename T>
+// f_a(x, y) pulled from g through its ghost columns (no wrap in x)
+template <typename T, int BC>
 __device__ __forceinline__ T pull_padded(const T *__restrict__ g, int a, int x, int y, int ny,
                                          int pitch, unsigned plane) {
     int sy = y - EYv(a);
-    sy = sy < 0 ? sy + ny : (sy >= ny ? sy - ny : sy);
-    const T *pl = g + (size_t)plane_of(a) * plane;
-    return pl[(unsigned)sy * (unsigned)pitch + (unsigned)(x - EXv(a) + GH<T>)];
+    if ((BC != 0 && sy < 0) || (BC == 1 && sy >= ny))
+        return g[(size_t)plane_of(opp(a)) * plane + (unsigned)y * (unsigned)pitch + (unsigned)(x + GH<T>)];
+    if (BC == 0) sy = sy < 0 ? sy + ny : (sy >= ny ? sy - ny : sy);
+    if (BC == 2) sy = sy >= ny ? ny - 1 : sy;
+    return g[(size_t)plane_of(a) * plane + (unsigned)sy * (unsigned)pitch + (unsigned)(x - EXv(a) + GH<T>)];
 }
 
 // the value of f_a(x, y) (decoded from the storage type)
@@ -195,6 +196,76 @@ __device__ __forceinline__ Arith<T> pull_val(const T *__restrict__ g, int a, int
     return pop_dec<T>(pull_global<T, BC>(g, a, x, y, nx, ny, pitch, plane), a, P);
 }
 
+// the nine populations of (x, y) through the ghost columns, decoded
+template <typename T, int BC>
+__device__ __forceinline__ void pull_site_vals(Arith<T> (&v)[9], const T *__restrict__ g, int x, int y,
+                                               int ny, int pitch, unsigned plane,
+                                               const DevConsts<Arith<T>> &P) {
+#pragma unroll
+    for (int a = 0; a < 9; ++a) v[a] = pop_dec<T>(pull_padded<T, BC>(g, a, x, y, ny, pitch, plane), a, P);
+}
+
+// Sum over the CTA (RED_THREADS threads) of each thread's q[0 .. N-1] in a fixed order, into
+// out[0 .. N-1]; the quantities from MAX on are maxima instead (a NaN wins). Warp k combines
+// quantity k: 12 FP64 operations per quantity, where a shuffle tree in every warp takes 40 (at two
+// FP64 operations per clock and SM the combination was most of a reduction over a small lattice).
+template <int N, int MAX>
+__device__ __forceinline__ void block_combine(const double (&q)[N], double *__restrict__ out) {
+    constexpr int W = RED_THREADS / 32;
+    static_assert(N <= W, "one warp per quantity");
+    __shared__ double s[N][RED_THREADS];
+    auto both = [](int k, double a, double b) {
+        return k < MAX ? a + b : ((b > a || b != b) ? b : a);
+    };
+#pragma unroll
+    for (int k = 0; k < N; ++k) s[k][threadIdx.x] = q[k];
+    __syncthreads();
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (k < N) {
+        double t = s[k][lane];
+#pragma unroll
+        for (int w = 1; w < W; ++w) t = both(k, t, s[k][lane + 32 * w]);
+#pragma unroll
+        for (int w = 16; w > 0; w >>= 1) t = both(k, t, __shfl_xor_sync(0xffffffffu, t, w));
+        if (lane == 0) out[k] = t;
+    }
+}
+
+// Sum over the CTA of a count, in every thread.
+__device__ __forceinline__ int block_count(int n) {
+    __shared__ int s[RED_THREADS / 32];
+    n = __reduce_add_sync(0xffffffffu, n);
+    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = n;
+    __syncthreads();
+    int t = 0;
+#pragma unroll
+    for (int w = 0; w < RED_THREADS / 32; ++w) t += s[w];
+    __syncthreads();
+    return t;
+}
+
+// The partial sums of a droplet measurement by a CTA from its threads' sums: out[0] mass, [1] / [2]
+// rho / count inside, [3] / [4] outside, [5] / [6] p = rho/3 + (G/2) psi^2 inside / outside, [7]
+// failed sites (see k_droplet_sums).
+__device__ __forceinline__ void droplet_combine(double m_in, double m_out, double m_rest, double q_in,
+                                                double q_out, int n_in, int n_out, int n_bad,
+                                                double G, double *__restrict__ out) {
+    __shared__ double t[5];
+    const double q[5] = {m_in, m_out, m_rest, q_in, q_out};
+    block_combine<5, 5>(q, t);
+    const int c_in = block_count(n_in), c_out = block_count(n_out), c_bad = block_count(n_bad);
+    if (threadIdx.x == 0) {            // block_count's barriers come after t was written
+        const double hg = 0.5 * G;
+        out[0] = t[0] + t[1] + t[2];
+        out[1] = t[0];
+        out[2] = (double)c_in;
+        out[3] = t[1];
+        out[4] = (double)c_out;
+        out[5] = t[0] / 3.0 + hg * t[3];
+        out[6] = t[1] / 3.0 + hg * t[4];
+        out[7] = (double)c_bad;
+    }
+}
 // ---------------------------------------------------------------- the hot kernel
 
 template <typename T>

@@ -550,23 +550,24 @@ template <typename T, int EOS, int BC>
 cudaError_t tile_launch(const Consts &c, const Geom &g, int variant, int order,
                         const StepBuffers &b, int *err, cudaStream_t st) {
     constexpr bool BF = std::is_same<T, __nv_bfloat16>::value;
-    constexpr int R = DIRECT_ROWS;
-    const int tx = (g.nx + TILE_W - 1) / TILE_W, ty = (g.ny + R - 1) / R;
+    const int tx = (g.nx + TILE_W - 1) / TILE_W;
     const T *gin = static_cast<const T *>(b.gin);
     T *gout = static_cast<T *>(b.gout);
     if (variant == direct_variant()) {
+        constexpr int R = DIRECT_ROWS;
         auto kern = k_tile_step<T, EOS, BC, R, false>;
         if constexpr (BF) {
             if (c.stochastic) kern = k_tile_step<T, EOS, BC, R, true>;
         }
-        return launch_dependent(kern, dim3(tx, ty), dim3(32 * R), st, gin, gout, to_dev<Arith<T>>(c),
+        return launch_dependent(kern, dim3(tx, (g.ny + R - 1) / R), dim3(32 * R), st, gin, gout, to_dev<Arith<T>>(c),
                                 g.nx, g.ny, g.pitch, (unsigned)g.plane, order, err);
     }
+    constexpr int R = STAGED_ROWS;
     auto kern = k_staged_tile_step<T, EOS, BC, R, false>;
     if constexpr (BF) {
         if (c.stochastic) kern = k_staged_tile_step<T, EOS, BC, R, true>;
     }
-    return launch_dependent(kern, dim3(tx, ty), dim3(32 * R), st,
+    return launch_dependent(kern, dim3(tx, (g.ny + R - 1) / R), dim3(32 * R), st,
                             *static_cast<const CUtensorMap *>(b.tensor_map_in), gin, gout,
                             to_dev<Arith<T>>(c), g.nx, g.ny, g.pitch, (unsigned)g.plane, order, err);
 }
@@ -598,7 +599,7 @@ template <typename T>
 cudaError_t batch_tile_dispatch(int eos, const BatchGroup &group, int n, int max_tiles,
                                 const void *maps, const void *lats, int phase, int *errs,
                                 cudaStream_t st) {
-    constexpr int R = DIRECT_ROWS;
+    constexpr int R = STAGED_ROWS;
     auto kern = eos == LB_EOS_CS    ? k_batch_tile<T, LB_EOS_CS, R>
                 : eos == LB_EOS_EXP ? k_batch_tile<T, LB_EOS_EXP, R>
                                     : k_batch_tile<T, LB_EOS_PIECEWISE, R>;
