@@ -443,7 +443,8 @@ __global__ void k_mlp_refresh_bf16(const float *__restrict__ master, __nv_bfloat
 // 64-long sum), times 42 evaluations for the inversion. One thread per sample (weights re-read
 // from shared memory) took 2346 us for 4097 inversions and as long for 24, 33 CTAs busy; a
 // warp per sample shortens the chain by 30 and fills the chip: lb_mlp_forward and
-// lb_mlp_invert_kappa of 4097 samples, copies included, 181 us against 2449 us.
+// lb_mlp_invert_kappa of 4097 samples, copies included, 181 us against 2449 us (153 us without
+// the halvings that change nothing).
 // ---------------------------------------------------------------------------------
 constexpr int kInferThreads = 128, kInferWarps = kInferThreads / 32;
 constexpr int kInferCtas = 2;      // resident CTAs per SM (the weights take 128 registers a thread)
@@ -590,7 +591,7 @@ k_mlp_invert(const __nv_bfloat16 *__restrict__ wbf, const MlpNorm *__restrict__ 
         for (int it = -2; it < kBisect; ++it) {
             float k[Q];
             float2 g[Q];
-            bool any = false;
+            bool any = false;          // a query that is still being bisected
 #pragma unroll
             for (int q = 0; q < Q; ++q) {
                 k[q] = it == -2 ? lo[q] : (it == -1 ? hi[q] : 0.5f * (lo[q] + hi[q]));
@@ -600,11 +601,16 @@ k_mlp_invert(const __nv_bfloat16 *__restrict__ wbf, const MlpNorm *__restrict__ 
 #pragma unroll
             for (int q = 0; q < Q; ++q) {
                 const float s = sigma_of(nm, output_unit(w3, b3, g[q]));
-                if (it == -2) ok[q] = s >= target[q];
-                else if (it == -1) ok[q] = ok[q] && s <= target[q];
-                else if (s > target[q]) lo[q] = k[q];
-                else hi[q] = k[q];
-                any |= ok[q];
+                if (it < 0) {
+                    ok[q] = it == -2 ? s >= target[q] : ok[q] && s <= target[q];
+                    any |= ok[q];
+                } else {
+                    // a halving that moves neither end (the ends are adjacent floats after 24 to
+                    // 30 of them) would be followed by the same one: the rest is left out
+                    float &end = s > target[q] ? lo[q] : hi[q];
+                    any |= ok[q] && end != k[q];
+                    end = k[q];
+                }
             }
             if (!any) break;                   // the same in every lane
         }
