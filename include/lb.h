@@ -135,7 +135,10 @@ lb_status lb_init_ex(lb_ctx **out, int nx, int ny, const lb_eos *eos, double G, 
  * LB_FP64 lattices whose scratch cannot be allocated, take variant 4 in their place. Every
  * variant gives identical results. Contexts start with the variant that suits their type and
  * size: 7 for LB_FP64 and for LB_FP32 up to 40 MiB a buffer, 8 for LB_BF16, for LB_BC_OPEN
- * and up to 72 MiB, 4 beyond. LB_FP32 batches have variants 0-6 and 8 (7 is taken as 8) and
+ * and up to 72 MiB, 4 beyond. With variant 7 an lb_step of several steps of an LB_FP32 lattice of
+ * at most 16384 sites (LB_BC_PERIODIC or LB_BC_WALLS_Y, even nx >= 4, ny >= 16, at most 512 site
+ * pairs per 1/16 of the rows) is one launch of a 16-CTA cluster that holds the lattice in shared
+ * memory; lb_autotune chooses variant 7 for these. LB_FP32 batches have variants 0-6 and 8 (7 is taken as 8) and
  * start with 8, LB_FP64 batches 0-6 (7 and 8 are taken as 4) and start with 4. */
 int lb_launch_variants(void);
 
@@ -199,7 +202,8 @@ lb_status lb_debug_stall_row(lb_ctx *ctx, int row);
  * and positive at some site (rho <= 0, or (p_EOS - rho/3)/G <= 0), LB_ECUDA. */
 lb_status lb_set_rho_u(lb_ctx *ctx, const double *rho, const double *ux, const double *uy);
 
-/* Advance n >= 0 time steps (Eqs. 4-8, 17-19), lb_kernels_per_step launches each. Queued on the
+/* Advance n >= 0 time steps (Eqs. 4-8, 17-19), lb_kernels_per_step launches each (small
+ * LB_FP32 lattices with variant 7: up to 1024 steps in one launch). Queued on the
  * stream; returns without waiting. A psi-domain violation found on the device is reported
  * by the next call that synchronises (lb_sync, lb_get_*, lb_reduce) as LB_EDOMAIN; a
  * device-side wait that gave up (about one second) as LB_ETIMEOUT. */

@@ -37,6 +37,7 @@ struct lb_ctx {
     double *d_host_in = nullptr; // 3*nx*ny staging for lb_set_rho_u
     void *d_psi = nullptr;       // FP64 direct kernels: psi of the step, ny * pitch elements
     lbm::StepLaunch launch{};
+    bool cluster = false;        // several steps at once go to the cluster kernel (variant 7)
     long long steps = 0;
     lb_status sticky = LB_OK;
     std::string msg;
@@ -45,6 +46,7 @@ struct lb_ctx {
 namespace {
 
 const char *kNoCtx = "no context";
+constexpr int kClusterSteps = 1024;   // of one cluster launch
 
 lb_status fail(lb_ctx *c, lb_status s, const std::string &m) {
     if (c) c->msg = m;
@@ -233,6 +235,7 @@ lb_status apply_launch(lb_ctx *c, int variant, int rows) {
         if (c->prec == LB_FP64) variant = lbm::direct_variant();     // no staged FP64 kernel
         if (!direct_usable(c)) variant = lbm::default_ring_variant();
     }
+    c->cluster = variant == lbm::direct_variant() && lbm::cluster_fits(c->prec, c->consts, c->geom);
     c->launch = lbm::make_step_launch(c->prec, c->consts.eos_kind, c->geom, c->num_sms, variant, rows);
     LB_CUDA(c, lbm::configure_step(c->prec, c->consts, c->geom, c->launch));
     return variant >= lbm::direct_variant() && c->prec == LB_FP64 ? LB_OK : make_maps(c);
@@ -410,6 +413,7 @@ lb_status lb_autotune(lb_ctx *c, int trial_steps, int *variant, int *rows) {
     if (trial_steps < 1) return fail(c, LB_EINVAL, "lb_autotune: trial_steps < 1");
     // device errors of earlier steps are the state's: report them before any trial
     if ((s = sync_and_check(c)) != LB_OK) return s;
+    const bool cluster = direct_usable(c) && lbm::cluster_fits(c->prec, c->consts, c->geom);
     static const int cand[] = {0, 6, 8, 9, 10, 11, 12, 13, 14, 15, 16, 20, 24};
     // Trial launches take real steps on a scratch copy of the state, ping-ponging with the
     // spare buffer as lb_step does (each launch reads what the previous one wrote, in the
@@ -501,6 +505,9 @@ lb_status lb_autotune(lb_ctx *c, int trial_steps, int *variant, int *rows) {
     if (c->words->err & lbm::ERR_TIMEOUT)       // (the stream has been waited for)
         return poison(c, LB_ETIMEOUT, "a bounded device-side wait gave up");
     c->words->err = 0;
+    // the trials are launches of one step: a lattice that the cluster kernel takes is faster with it
+    // than with any of them
+    if (cluster) best_v = lbm::direct_variant(), best_r = lbm::DIRECT_ROWS;
     if ((s = apply_launch(c, best_v, best_r)) != LB_OK) return s;
     if (variant) *variant = best_v;
     if (rows) *rows = best_r;
@@ -581,6 +588,15 @@ lb_status lb_step(lb_ctx *c, int n) {
     lb_status s = check_usable(c);
     if (s != LB_OK) return s;
     if (n < 0) return fail(c, LB_EINVAL, "lb_step: n < 0");
+    // a small lattice takes several steps in one launch (at most kClusterSteps: about a millisecond)
+    while (c->cluster && n > 1) {
+        const int m = std::min(n, kClusterSteps);
+        LB_CUDA(c, lbm::launch_cluster_steps(c->consts, c->geom, c->f[c->cur], c->f[c->cur ^ 1], m,
+                                             c->d_err, c->stream));
+        c->cur ^= 1;
+        c->steps += m;
+        n -= m;
+    }
     for (int i = 0; i < n; ++i) {
         // alternate the visiting order: each step first reads the rows the previous one
         // wrote last (still in L2 when the state is not much larger than L2)

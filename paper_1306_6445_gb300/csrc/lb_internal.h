@@ -158,6 +158,11 @@ cudaError_t split_f64(const Consts &c, const Geom &g, const void *gin, void *psi
 cudaError_t batch_tile_f32(int eos, const BatchGroup &group, int n, int max_tiles, const void *maps,
                            const void *lats, int phase, int *errs, cudaStream_t st);
 
+// n_steps steps of a small lattice in one launch (lb_cluster.cu); cluster_fits: whether it can
+bool cluster_fits(int prec, const Consts &c, const Geom &g);
+cudaError_t launch_cluster_steps(const Consts &c, const Geom &g, const void *gin, void *gout,
+                                 int n_steps, int *err, cudaStream_t st);
+
 // What a step reads and writes: the input buffer and its tensor map (none for the direct FP64
 // kernels), the output buffer, and psi scratch (direct FP64 kernels only).
 struct StepBuffers {
