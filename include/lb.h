@@ -135,11 +135,15 @@ lb_status lb_init_ex(lb_ctx **out, int nx, int ny, const lb_eos *eos, double G, 
  * LB_FP64 lattices whose scratch cannot be allocated, take variant 4 in their place. Every
  * variant gives identical results. Contexts start with the variant that suits their type and
  * size: 7 for LB_FP64 and for LB_FP32 up to 40 MiB a buffer, 8 for LB_BF16, for LB_BC_OPEN
- * and up to 72 MiB, 4 beyond. With variant 7 an lb_step of several steps of an LB_FP32 lattice of
- * at most 16384 sites (LB_BC_PERIODIC or LB_BC_WALLS_Y, even nx >= 4, ny >= 16, at most 512 site
- * pairs per 1/16 of the rows) is one launch of a 16-CTA cluster that holds the lattice in shared
- * memory; lb_autotune chooses variant 7 for these. LB_FP32 batches have variants 0-6 and 8 (7 is taken as 8) and
- * start with 8, LB_FP64 batches 0-6 (7 and 8 are taken as 4) and start with 4. */
+ * and up to 72 MiB, 4 beyond. An lb_step of several steps of an LB_FP32 context with the variant
+ * it started with is one launch for lattices that fit the SMs' shared memory: of a 16-CTA cluster
+ * up to 16384 sites (LB_BC_PERIODIC or LB_BC_WALLS_Y, even nx >= 4, ny >= 16, at most 512 site
+ * pairs per 1/16 of the rows), of one CTA per SM from 32768 sites on as long as tiles of 64
+ * columns and at most 35 rows suffice (a cooperative launch, between 96 tiles and one per SM, the last of
+ * a row at least two columns wide; an exchange buffer is allocated by the library, without it the
+ * steps are single launches). lb_autotune keeps the variant of these. LB_FP32 batches have
+ * variants 0-6 and 8 (7 is taken as 8) and start with 8, LB_FP64 batches 0-6 (7 and 8 are taken
+ * as 4) and start with 4. */
 int lb_launch_variants(void);
 
 /* Density-dependent viscosity of Sec. V.C (LB_BC_OPEN contexts): sites with rho < rho_1

@@ -23,7 +23,7 @@ LIB = os.path.join(LIBDIR, "liblb_gb300.so")
 SOURCES = ["lb_step_f32.cu", "lb_step_f32_stage.cu", "lb_step_f64.cu", "lb_step_f64_stage.cu",
            "lb_step_bf16.cu", "lb_step_bf16_stage.cu", "lb_batch_kernels.cu", "lb_batch_stage.cu",
            "lb_tile_f32.cu", "lb_tile_bf16.cu",
-           "lb_split_f64.cu", "lb_batch_tile.cu", "lb_cluster.cu", "lb_kernels.cu", "lb_api.cu", "lb_thermo.cpp", "lb_noalloc.cu", "lb_batch.cu",
+           "lb_split_f64.cu", "lb_batch_tile.cu", "lb_cluster.cu", "lb_resident.cu", "lb_kernels.cu", "lb_api.cu", "lb_thermo.cpp", "lb_noalloc.cu", "lb_batch.cu",
            "lb_mlp.cu", "lb_probe.cu"]
 HEADERS = ["lb_internal.h", "lb_device.cuh", "lb_step.cuh", "lb_tile.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

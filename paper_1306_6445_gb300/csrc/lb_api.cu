@@ -37,7 +37,8 @@ struct lb_ctx {
     double *d_host_in = nullptr; // 3*nx*ny staging for lb_set_rho_u
     void *d_psi = nullptr;       // FP64 direct kernels: psi of the step, ny * pitch elements
     lbm::StepLaunch launch{};
-    bool cluster = false;        // several steps at once go to the cluster kernel (variant 7)
+    int many = 0;                // several steps at once: 1 the cluster kernel, 2 the resident one
+    void *d_words = nullptr;     // exchange words of the resident kernel
     long long steps = 0;
     lb_status sticky = LB_OK;
     std::string msg;
@@ -46,7 +47,7 @@ struct lb_ctx {
 namespace {
 
 const char *kNoCtx = "no context";
-constexpr int kClusterSteps = 1024;   // of one cluster launch
+constexpr int kManySteps = 1024;      // of one launch of the cluster or the resident kernel
 
 lb_status fail(lb_ctx *c, lb_status s, const std::string &m) {
     if (c) c->msg = m;
@@ -227,6 +228,21 @@ bool direct_usable(lb_ctx *c) {
     return false;
 }
 
+// which kernel takes several steps of this lattice in one launch, see lb_ctx::many
+int many_usable(lb_ctx *c) {
+    if (lbm::cluster_fits(c->prec, c->consts, c->geom)) return 1;
+    const size_t bytes = lbm::resident_bytes(c->prec, c->consts, c->geom, c->num_sms);
+    if (bytes == 0) return 0;
+    if (c->d_words) return 2;
+    if (cudaMalloc(&c->d_words, bytes) == cudaSuccess &&
+        cudaMemsetAsync(c->d_words, 0, bytes, c->stream) == cudaSuccess)
+        return 2;
+    (void)cudaGetLastError();
+    cudaFree(c->d_words);
+    c->d_words = nullptr;
+    return 0;
+}
+
 lb_status apply_launch(lb_ctx *c, int variant, int rows) {
     if (variant < 0 || variant >= lbm::step_variant_count())
         return fail(c, LB_EINVAL, "unknown launch variant");
@@ -235,7 +251,7 @@ lb_status apply_launch(lb_ctx *c, int variant, int rows) {
         if (c->prec == LB_FP64) variant = lbm::direct_variant();     // no staged FP64 kernel
         if (!direct_usable(c)) variant = lbm::default_ring_variant();
     }
-    c->cluster = variant == lbm::direct_variant() && lbm::cluster_fits(c->prec, c->consts, c->geom);
+    c->many = variant == lbm::default_variant(c->prec, c->geom) ? many_usable(c) : 0;
     c->launch = lbm::make_step_launch(c->prec, c->consts.eos_kind, c->geom, c->num_sms, variant, rows);
     LB_CUDA(c, lbm::configure_step(c->prec, c->consts, c->geom, c->launch));
     return variant >= lbm::direct_variant() && c->prec == LB_FP64 ? LB_OK : make_maps(c);
@@ -413,7 +429,13 @@ lb_status lb_autotune(lb_ctx *c, int trial_steps, int *variant, int *rows) {
     if (trial_steps < 1) return fail(c, LB_EINVAL, "lb_autotune: trial_steps < 1");
     // device errors of earlier steps are the state's: report them before any trial
     if ((s = sync_and_check(c)) != LB_OK) return s;
-    const bool cluster = direct_usable(c) && lbm::cluster_fits(c->prec, c->consts, c->geom);
+    if (many_usable(c)) {
+        // launches of many steps beat all that could be tried here
+        if ((s = apply_launch(c, lbm::default_variant(c->prec, c->geom), 0)) != LB_OK) return s;
+        if (variant) *variant = c->launch.variant;
+        if (rows) *rows = c->launch.rows;
+        return LB_OK;
+    }
     static const int cand[] = {0, 6, 8, 9, 10, 11, 12, 13, 14, 15, 16, 20, 24};
     // Trial launches take real steps on a scratch copy of the state, ping-ponging with the
     // spare buffer as lb_step does (each launch reads what the previous one wrote, in the
@@ -505,9 +527,6 @@ lb_status lb_autotune(lb_ctx *c, int trial_steps, int *variant, int *rows) {
     if (c->words->err & lbm::ERR_TIMEOUT)       // (the stream has been waited for)
         return poison(c, LB_ETIMEOUT, "a bounded device-side wait gave up");
     c->words->err = 0;
-    // the trials are launches of one step: a lattice that the cluster kernel takes is faster with it
-    // than with any of them
-    if (cluster) best_v = lbm::direct_variant(), best_r = lbm::DIRECT_ROWS;
     if ((s = apply_launch(c, best_v, best_r)) != LB_OK) return s;
     if (variant) *variant = best_v;
     if (rows) *rows = best_r;
@@ -588,12 +607,22 @@ lb_status lb_step(lb_ctx *c, int n) {
     lb_status s = check_usable(c);
     if (s != LB_OK) return s;
     if (n < 0) return fail(c, LB_EINVAL, "lb_step: n < 0");
-    // a small lattice takes several steps in one launch (at most kClusterSteps: about a millisecond)
-    while (c->cluster && n > 1) {
-        const int m = std::min(n, kClusterSteps);
-        LB_CUDA(c, lbm::launch_cluster_steps(c->consts, c->geom, c->f[c->cur], c->f[c->cur ^ 1], m,
-                                             c->d_err, c->stream));
-        c->cur ^= 1;
+    // a lattice that fits the SMs takes several steps in one launch (at most kManySteps: a few
+    // milliseconds)
+    while (c->many && n > 1) {
+        const int m = std::min(n, kManySteps);
+        const void *gin = c->f[c->cur];
+        void *gout = c->f[c->cur ^ (m & 1)];     // the buffer that m launches would end in
+        const cudaError_t e =
+            c->many == 1 ? lbm::launch_cluster_steps(c->consts, c->geom, gin, gout, m, c->d_err, c->stream)
+                         : lbm::launch_resident_steps(c->consts, c->geom, c->num_sms, gin, gout, m, c->d_words,
+                                                      c->d_err, c->stream);
+        if (e != cudaSuccess) {       // not every SM can be had (a limited context): single launches
+            (void)cudaGetLastError();
+            c->many = 0;
+            break;
+        }
+        c->cur ^= m & 1;
         c->steps += m;
         n -= m;
     }
@@ -745,6 +774,7 @@ void lb_free(lb_ctx *c) {
     cudaFree(c->d_first);
     cudaFree(c->d_host_in);
     cudaFree(c->d_psi);
+    cudaFree(c->d_words);
     delete c;
 }
 

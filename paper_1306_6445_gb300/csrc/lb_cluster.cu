@@ -41,7 +41,7 @@ __device__ __forceinline__ void store_remote(uint32_t addr, V2<float> v) {
 // in all): with two pairs per thread 140^2 took 2.3, 160^2 2.6 us, no less than the launches.
 template <int EOS, int BC>
 __global__ void __launch_bounds__(CL_MAX_THREADS, 1)
-k_cluster_steps(const float *__restrict__ gin, float *__restrict__ gout,
+k_cluster_steps(const float *gin, float *gout,          // (may be the same)
                 const __grid_constant__ DevConsts<float> P, const int nx, const int ny,
                 const int pitch, const unsigned plane, const int n_steps, int *__restrict__ err) {
     extern __shared__ __align__(16) float cl_smem[];

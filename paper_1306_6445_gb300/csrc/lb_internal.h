@@ -158,6 +158,12 @@ cudaError_t split_f64(const Consts &c, const Geom &g, const void *gin, void *psi
 cudaError_t batch_tile_f32(int eos, const BatchGroup &group, int n, int max_tiles, const void *maps,
                            const void *lats, int phase, int *errs, cudaStream_t st);
 
+// n_steps steps of a mid-size lattice in one launch (lb_resident.cu), with `words` of resident_bytes
+// bytes, zero before the first launch (resident_bytes 0: the lattice does not fit)
+size_t resident_bytes(int prec, const Consts &c, const Geom &g, int num_sms);
+cudaError_t launch_resident_steps(const Consts &c, const Geom &g, int num_sms, const void *gin, void *gout,
+                                  int n_steps, void *words, int *err, cudaStream_t st);
+
 // n_steps steps of a small lattice in one launch (lb_cluster.cu); cluster_fits: whether it can
 bool cluster_fits(int prec, const Consts &c, const Geom &g);
 cudaError_t launch_cluster_steps(const Consts &c, const Geom &g, const void *gin, void *gout,
