@@ -3,15 +3,14 @@
 //   k_mlp_prepare  one CTA: FP64 means / scales of the input features
 //                  (ln(1 - T/T_c), ln(1 - kappa), tau_v) and of the transformed targets,
 //                  standardised copies (float)
-//   k_mlp_grad     forward + backward over tiles of 4 or 16 samples; each CTA accumulates
-//                  its tiles' gradient in registers and writes one partial vector
+//   k_mlp_grad     forward + backward over tiles of 16 samples, one CTA or a cluster of four
+//                  each, which sums the tile's gradient and writes one partial vector
 //   k_mlp_adam     sums the partials in a fixed order, Adam update of the FP32 master
 //                  copy, refreshes the BF16 image used by the next forward pass
 //   k_mlp_forward  inference, one warp per sample or pair of samples
 //   k_mlp_invert   bisection on kappa for a target sigma, one warp per query or pair
-// The weights are read as BF16 and every product is accumulated in FP32 (fmaf; the hidden
-// layers in the order of the sums' indices, the output layer of inference over a fixed
-// butterfly of the lanes).
+// The weights are read as BF16 and every product is accumulated in FP32 (fmaf; in the order of
+// the sums' indices, the output layer of inference over a fixed butterfly of the lanes).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -21,6 +20,7 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "lb_internal.h"
@@ -33,7 +33,8 @@ constexpr int OW1 = 0, OB1 = OW1 + H * IN, OW2 = OB1 + H, OB2 = OW2 + H * H, OW3
               OB3 = OW3 + OUT * H;
 static_assert(OB3 + OUT == NP, "parameter layout");
 
-constexpr int kSmallTile = 4, kLargeTile = 16;   // samples per tile of k_mlp_grad
+constexpr int kTile = 16;          // samples per tile of k_mlp_grad
+constexpr int kSplit = 4;          // CTAs that share a tile while the grid leaves room (a cluster)
 constexpr int kThreads = 256;      // k_mlp_grad block
 constexpr int kMaxGradCtas = 304;  // 2 x 152 SMs: bounds the partial-gradient buffer
 constexpr int kW2Pitch = H + 4;    // padded rows of W2 in shared memory (16-byte rows, no bank conflicts)
@@ -187,19 +188,23 @@ k_mlp_prepare(float *__restrict__ x, float *__restrict__ y, int n, MlpNorm *__re
 }
 
 // ---------------------------------------------------------------------------------
-// Forward + backward. Block of 256 threads, tiles of TILE samples; the CTA walks tiles
-// blockIdx.x, blockIdx.x + gridDim.x, ... and keeps the gradient entries it owns in
-// registers:
-//   gW2: 16 per thread (k = t & 63, j = 16 (t >> 6) + q)   gb2: threads 0..63
-//   gW3 / gb3: threads 0..191 / 192..194                   gW1 / gb1: 0..191 / 192..255
+// Forward + backward. Tiles of 16 samples, in blocks of 256 threads:
+//   SPLIT = 1: CTA b takes tiles b, b + gridDim.x, ... and keeps the gradient entries it owns in
+//     registers: gW2: 16 per thread (k = t & 63, j = 16 (t >> 6) + q), gb2: threads 0..63,
+//     gW3 / gb3: threads 0..191 / 192..194, gW1 / gb1: 0..191 / 192..255.
+//   SPLIT = 4: cluster b takes tile b. Each of its CTAs carries four samples forward and back and
+//     sends the others what they need of it through distributed shared memory; then CTA r sums
+//     the gradient entries of hidden units 16 r .. 16 r + 15 over the tile's 16 samples.
 // Activations of a tile live in shared memory; dz overwrites z in place.
 // What bounds it: the chain load weights -> layer -> layer -> back, once per tile, not the
-// arithmetic (14 MFLOP at 512 samples). So the tile is 4 samples (one per thread in the
-// hidden layers) while that gives at most kMaxGradCtas tiles, and 16 beyond, where a CTA's
-// weight load and partial vector are shared by more samples. Rows of W2 are padded to 68
-// floats: 16-byte row reads (forward) and column reads (backward) are both free of bank
-// conflicts. 50 Adam steps at 512 samples (both kernels, the call included): 439 us, against
-// 1469 us with 16-sample tiles (32 CTAs), a serial partial sum and no launch overlap.
+// arithmetic (14 MFLOP at 512 samples): so four CTAs share a tile while they all are resident,
+// kMaxGradCtas in all. Every sum runs in the order of the samples and of the tiles, however
+// they are split: weights are used rounded to BF16, so a gradient off by one rounding sends
+// some weight to the other neighbour at some step, and with tiles of 4 samples two of three runs
+// of 50 steps ended 3e-5 away from the others. Rows of W2 are padded to 68 floats: 16-byte row
+// reads (forward) and column reads (backward) are both free of bank conflicts. 50 Adam steps at
+// 512 samples (both kernels, the call included): 520 us, against 1465 us with one CTA per
+// tile, a serial partial sum and no launch overlap.
 // ---------------------------------------------------------------------------------
 __device__ __forceinline__ void grid_dependency_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -208,16 +213,49 @@ __device__ __forceinline__ void grid_dependents_launch() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-template <int TILE>
+__device__ __forceinline__ unsigned cluster_rank() {
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// address of the same shared-memory variable in CTA `rank` of the cluster
+__device__ __forceinline__ uint32_t in_cta(const void *p, unsigned rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                 : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void store_cta(uint32_t addr, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
+// what a CTA of a cluster sums over the tile's samples: a_1 and, of its own 16 hidden units, a_2,
+// dz_2 and dz_1; inputs, residuals and their scaled form
+struct TileShare {
+    __align__(16) float a1[kTile * H];
+    float a2[kTile * 16], dz2[kTile * 16], dz1[kTile * 16];
+    float x[kTile * IN], dout[kTile * OUT], res[kTile * OUT];
+};
+
+template <int SPLIT>
 __global__ void __launch_bounds__(kThreads, 2)
 k_mlp_grad(const __nv_bfloat16 *__restrict__ wbf, const float *__restrict__ xn,
            const float *__restrict__ tn, MlpState *__restrict__ st, int bump_step,
            float *__restrict__ part, float *__restrict__ lpart) {
+    constexpr int TILE = kTile / SPLIT;   // samples of the CTA
     constexpr int NQ = TILE / 4;          // samples per thread in the hidden layers
+    constexpr bool CL = SPLIT > 1;
+    struct None {};
     __shared__ SmemW w;
     __shared__ float sx[TILE * IN], dout[TILE * OUT], res[TILE * OUT];
     __shared__ __align__(16) float z1[TILE * H], a1[TILE * H], z2[TILE * H], a2[TILE * H];
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    __shared__ std::conditional_t<CL, TileShare, None> sh;
+    const int t = threadIdx.x;
+    const unsigned rank = CL ? cluster_rank() : 0;
+    const int tile0 = blockIdx.x / SPLIT, tiles = gridDim.x / SPLIT;
+    if constexpr (CL) cluster_arrive();   // (waited for before the first store to another CTA)
     // the weights are the previous kernel's: wait for it (programmatic dependent launch)
     grid_dependency_wait();
     grid_dependents_launch();
@@ -236,7 +274,7 @@ k_mlp_grad(const __nv_bfloat16 *__restrict__ wbf, const float *__restrict__ xn,
     float gb2 = 0.f, g3 = 0.f, g1 = 0.f, lsum = 0.f;
 
     const int jj = t & 63, sg = t >> 6;   // unit and sample group (uniform in a warp)
-    for (int base = blockIdx.x * TILE; base < n; base += gridDim.x * TILE) {
+    for (int base = tile0 * kTile + (int)rank * TILE; base < n || CL; base += tiles * kTile) {
         __syncthreads();   // weights loaded / previous tile consumed
         if (t < TILE * IN) sx[t] = base + t / IN < n ? xn[(size_t)base * IN + t] : 0.f;
         __syncthreads();
@@ -251,6 +289,16 @@ k_mlp_grad(const __nv_bfloat16 *__restrict__ wbf, const float *__restrict__ xn,
             a1[s * H + jj] = gelu(z);
         }
         __syncthreads();
+        if constexpr (CL) {
+            cluster_wait();               // the others have started
+            const int s = (int)rank * TILE + sg;
+            const float v = a1[sg * H + jj];
+#pragma unroll
+            for (int c = 0; c < SPLIT; ++c) store_cta(in_cta(&sh.a1[s * H + jj], c), v);
+            if (t < TILE * IN)
+#pragma unroll
+                for (int c = 0; c < SPLIT; ++c) store_cta(in_cta(&sh.x[(int)rank * TILE * IN + t], c), sx[t]);
+        }
         // layer 2
         {
             float acc[NQ];
@@ -271,38 +319,49 @@ k_mlp_grad(const __nv_bfloat16 *__restrict__ wbf, const float *__restrict__ xn,
 #pragma unroll
             for (int q = 0; q < NQ; ++q) {
                 z2[(sg + 4 * q) * H + jj] = acc[q];
-                a2[(sg + 4 * q) * H + jj] = gelu(acc[q]);
+                const float g = gelu(acc[q]);
+                a2[(sg + 4 * q) * H + jj] = g;
+                if constexpr (CL)
+                    store_cta(in_cta(&sh.a2[((int)rank * TILE + sg) * 16 + (jj & 15)], jj >> 4), g);
             }
         }
         __syncthreads();
-        // output layer (summed as in inference) and loss residual: one warp per output
-        for (int p = warp; p < TILE * OUT; p += kThreads / 32) {
-            const int s = p / OUT, c = p % OUT;
-            const float2 g = *reinterpret_cast<const float2 *>(&a2[s * H + 2 * lane]);
-            const float o = output_unit(make_float2(w.w3[c * H + 2 * lane], w.w3[c * H + 2 * lane + 1]),
-                                        w.b3[c], g);
-            if (lane == 0) {
-                const float r = base + s < n ? o - tn[(size_t)base * OUT + p] : 0.f;
-                dout[p] = r * dscale;
-                res[p] = r;
+        // output layer and loss residual
+        if (t < TILE * OUT) {
+            const int s = t / OUT, c = t % OUT;
+            const float target = base + s < n ? tn[(size_t)base * OUT + t] : 0.f;
+            float o = w.b3[c];
+#pragma unroll
+            for (int k = 0; k < H; k += 4) {
+                const float4 wv = *reinterpret_cast<const float4 *>(&w.w3[c * H + k]);
+                const float4 av = *reinterpret_cast<const float4 *>(&a2[s * H + k]);
+                o = fmaf(wv.x, av.x, o);
+                o = fmaf(wv.y, av.y, o);
+                o = fmaf(wv.z, av.z, o);
+                o = fmaf(wv.w, av.w, o);
+            }
+            const float r = base + s < n ? o - target : 0.f;
+            dout[t] = r * dscale;
+            res[t] = r;
+            if constexpr (CL) {
+#pragma unroll
+                for (int d = 0; d < SPLIT; ++d) store_cta(in_cta(&sh.dout[(int)rank * TILE * OUT + t], d), r * dscale);
+                store_cta(in_cta(&sh.res[(int)rank * TILE * OUT + t], 0), r);
             }
         }
         __syncthreads();
-        if (warp == kThreads / 32 - 1) {
-            float l = lane < TILE * OUT ? res[lane] * res[lane] : 0.f;
-            if (TILE * OUT > 32 && lane + 32 < TILE * OUT) l = fmaf(res[lane + 32], res[lane + 32], l);
+        // gW3, gb3, loss; dz2 = (dout W3) * gelu'(z2) in place
+        if constexpr (!CL) {
+            if (t < OUT * H) {
+                const int c = t >> 6, k = t & 63;
 #pragma unroll
-            for (int m = 16; m > 0; m >>= 1) l += __shfl_xor_sync(0xffffffffu, l, m);
-            lsum += l;
-        }
-        // gW3, gb3; dz2 = (dout W3) * gelu'(z2) in place
-        if (t < OUT * H) {
-            const int c = t >> 6, k = t & 63;
-#pragma unroll
-            for (int s = 0; s < TILE; ++s) g3 = fmaf(dout[s * OUT + c], a2[s * H + k], g3);
-        } else if (t < OUT * H + OUT) {
-            const int c = t - OUT * H;
-            for (int s = 0; s < TILE; ++s) g3 += dout[s * OUT + c];
+                for (int s = 0; s < TILE; ++s) g3 = fmaf(dout[s * OUT + c], a2[s * H + k], g3);
+            } else if (t < OUT * H + OUT) {
+                const int c = t - OUT * H;
+                for (int s = 0; s < TILE; ++s) g3 += dout[s * OUT + c];
+            } else if (t == kThreads - 1) {
+                for (int k = 0; k < TILE * OUT; ++k) lsum = fmaf(res[k], res[k], lsum);
+            }
         }
 #pragma unroll
         for (int q = 0; q < NQ; ++q) {
@@ -310,24 +369,29 @@ k_mlp_grad(const __nv_bfloat16 *__restrict__ wbf, const float *__restrict__ xn,
             float d = 0.f;
 #pragma unroll
             for (int c = 0; c < OUT; ++c) d = fmaf(dout[s * OUT + c], w.w3[c * H + jj], d);
-            z2[s * H + jj] = d * gelu_grad(z2[s * H + jj]);
+            d = d * gelu_grad(z2[s * H + jj]);
+            z2[s * H + jj] = d;
+            if constexpr (CL)
+                store_cta(in_cta(&sh.dz2[((int)rank * TILE + sg) * 16 + (jj & 15)], jj >> 4), d);
         }
         __syncthreads();
         // gW2, gb2; dz1 = (dz2 W2) * gelu'(z1) in place
+        if constexpr (!CL) {
 #pragma unroll 4
-        for (int s = 0; s < TILE; ++s) {
-            const float av = a1[s * H + jj];
+            for (int s = 0; s < TILE; ++s) {
+                const float av = a1[s * H + jj];
 #pragma unroll
-            for (int q = 0; q < 16; q += 4) {
-                const float4 d = *reinterpret_cast<const float4 *>(&z2[s * H + 16 * sg + q]);
-                gw2[q] = fmaf(d.x, av, gw2[q]);
-                gw2[q + 1] = fmaf(d.y, av, gw2[q + 1]);
-                gw2[q + 2] = fmaf(d.z, av, gw2[q + 2]);
-                gw2[q + 3] = fmaf(d.w, av, gw2[q + 3]);
+                for (int q = 0; q < 16; q += 4) {
+                    const float4 d = *reinterpret_cast<const float4 *>(&z2[s * H + 16 * sg + q]);
+                    gw2[q] = fmaf(d.x, av, gw2[q]);
+                    gw2[q + 1] = fmaf(d.y, av, gw2[q + 1]);
+                    gw2[q + 2] = fmaf(d.z, av, gw2[q + 2]);
+                    gw2[q + 3] = fmaf(d.w, av, gw2[q + 3]);
+                }
             }
+            if (t < H)
+                for (int s = 0; s < TILE; ++s) gb2 += z2[s * H + t];
         }
-        if (t < H)
-            for (int s = 0; s < TILE; ++s) gb2 += z2[s * H + t];
         {
             float acc[NQ];
 #pragma unroll
@@ -349,9 +413,14 @@ k_mlp_grad(const __nv_bfloat16 *__restrict__ wbf, const float *__restrict__ xn,
 #pragma unroll
             for (int q = 0; q < NQ; ++q) {
                 const int s = sg + 4 * q;
-                z1[s * H + jj] = acc[q] * gelu_grad(z1[s * H + jj]);
+                const float d = acc[q] * gelu_grad(z1[s * H + jj]);
+                if constexpr (CL)
+                    store_cta(in_cta(&sh.dz1[((int)rank * TILE + sg) * 16 + (jj & 15)], jj >> 4), d);
+                else
+                    z1[s * H + jj] = d;
             }
         }
+        if constexpr (CL) break;
         __syncthreads();
         // gW1, gb1
         if (t < H * IN) {
@@ -364,22 +433,63 @@ k_mlp_grad(const __nv_bfloat16 *__restrict__ wbf, const float *__restrict__ xn,
             for (int s = 0; s < TILE; ++s) g1 += z1[s * H + j];
         }
     }
-    float *out = part + (size_t)blockIdx.x * NP;
+    float *out = part + (size_t)tile0 * NP;
+    if constexpr (CL) {
+        cluster_arrive();
+        cluster_wait();                   // the tile's samples are here; nothing is sent any more
+        const int j = t >> 4, k = t & 15, u = 16 * (int)rank;
+        // first the entries that a warp or two own, while the others go on to W2
+        if (t >= 208) {
+            if (t < 256) {                // gW3 of units u ..
+                const int c = (t - 208) >> 4;
 #pragma unroll
-    for (int q = 0; q < 16; ++q) out[OW2 + (16 * sg + q) * H + jj] = gw2[q];
-    if (t < H) out[OB2 + t] = gb2;
-    if (t < OUT * H) out[OW3 + t] = g3;
-    else if (t < OUT * H + OUT) out[OB3 + t - OUT * H] = g3;
-    if (t < H * IN) out[OW1 + t] = g1;
-    else out[OB1 + t - H * IN] = g1;
-    if (t == kThreads - 1) lpart[blockIdx.x] = lsum;
+                for (int s = 0; s < kTile; ++s) g3 = fmaf(sh.dout[s * OUT + c], sh.a2[s * 16 + k], g3);
+                out[OW3 + c * H + u + k] = g3;
+            }
+        } else if (t >= 160) {            // gW1 of units u ..
+            const int e = t - 160;
+#pragma unroll
+            for (int s = 0; s < kTile; ++s) g1 = fmaf(sh.dz1[s * 16 + e / IN], sh.x[s * IN + e % IN], g1);
+            out[OW1 + u * IN + e] = g1;
+        } else if (t >= 128) {            // gb1, gb2
+            const float *d = t < 144 ? sh.dz1 : sh.dz2;
+#pragma unroll
+            for (int s = 0; s < kTile; ++s) gb2 += d[s * 16 + k];
+            out[(t < 144 ? OB1 : OB2) + u + k] = gb2;
+        } else if (t >= 96 && t < 96 + OUT && rank == 0) {
+#pragma unroll
+            for (int s = 0; s < kTile; ++s) g3 += sh.dout[s * OUT + t - 96];
+            out[OB3 + t - 96] = g3;
+        } else if (t == 64 && rank == 0) {
+#pragma unroll
+            for (int e = 0; e < kTile * OUT; ++e) lsum = fmaf(sh.res[e], sh.res[e], lsum);
+            lpart[tile0] = lsum;
+        }
+#pragma unroll
+        for (int s = 0; s < kTile; ++s) {
+            const float d = sh.dz2[s * 16 + j];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) gw2[q] = fmaf(d, sh.a1[s * H + 16 * q + k], gw2[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) out[OW2 + (u + j) * H + 16 * q + k] = gw2[q];
+    } else {
+#pragma unroll
+        for (int q = 0; q < 16; ++q) out[OW2 + (16 * sg + q) * H + jj] = gw2[q];
+        if (t < H) out[OB2 + t] = gb2;
+        if (t < OUT * H) out[OW3 + t] = g3;
+        else if (t < OUT * H + OUT) out[OB3 + t - OUT * H] = g3;
+        if (t < H * IN) out[OW1 + t] = g1;
+        else out[OB1 + t - H * IN] = g1;
+        if (t == kThreads - 1) lpart[tile0] = lsum;
+    }
 }
 
-// Sum of the partial gradients in a fixed order, then Adam on the FP32 master copy. A CTA
-// owns 32 parameters: warp w sums partials w, w + 8, ... (128-byte reads, several in
-// flight), then the eight sums are added in warp order; the bias corrections come from the
-// running powers of beta1 and beta2 that k_mlp_grad advances in FP64. One thread per
-// parameter with a serial sum of 32 partials and two FP64 pow took 17.6 us at 512 samples.
+// Sum of the partial gradients in the order of the tiles, then Adam on the FP32 master copy. A
+// CTA owns 32 parameters: its warps fetch the partials into shared memory (128-byte reads,
+// several in flight), then one warp adds them; the bias corrections come from the running powers
+// of beta1 and beta2 that k_mlp_grad advances in FP64. One thread per parameter with a serial
+// sum of 32 partials and two FP64 pow took 17.6 us at 512 samples.
 constexpr int kAdamThreads = 256, kAdamParams = 32;
 
 __global__ void __launch_bounds__(kAdamThreads)
@@ -387,17 +497,15 @@ k_mlp_adam(const float *__restrict__ part, const float *__restrict__ lpart, int 
            MlpState *__restrict__ st, float *__restrict__ master, float *__restrict__ m1,
            float *__restrict__ m2, __nv_bfloat16 *__restrict__ wbf, float *__restrict__ grad_out) {
     constexpr int NW = kAdamThreads / 32;
-    __shared__ float sums[NW][kAdamParams];
+    __shared__ float parts[kMaxGradCtas][kAdamParams];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int p = blockIdx.x * kAdamParams + lane;
     grid_dependency_wait();
     grid_dependents_launch();
-    float g = 0.f;
     if (p < NP) {
 #pragma unroll 8
-        for (int c = warp; c < nparts; c += NW) g += part[(size_t)c * NP + p];
+        for (int c = warp; c < nparts; c += NW) parts[c][lane] = part[(size_t)c * NP + p];
     }
-    sums[warp][lane] = g;
     __syncthreads();
     if (blockIdx.x == 0 && warp == 1) {   // the loss: lanes take every 32nd partial, then a butterfly
         double l = 0.0;
@@ -407,9 +515,9 @@ k_mlp_adam(const float *__restrict__ part, const float *__restrict__ lpart, int 
         if (lane == 0) st->loss = (float)(l / (3.0 * st->n));
     }
     if (warp != 0 || p >= NP) return;
-    g = 0.f;
-#pragma unroll
-    for (int w = 0; w < NW; ++w) g += sums[w][lane];
+    float g = 0.f;
+#pragma unroll 16
+    for (int c = 0; c < nparts; ++c) g += parts[c][lane];
     if (grad_out) {   // gradient only (no update)
         grad_out[p] = g;
         return;
@@ -640,8 +748,8 @@ InferLaunch infer_launch(int sms, int n) {
 
 struct lb_mlp {
     cudaStream_t stream = nullptr;
-    int max_samples = 0, n = 0, grad_ctas = 0;
-    int tile = 0;
+    int max_samples = 0, n = 0;
+    int parts = 0, split = 1;     // partial gradients, CTAs that share one (k_mlp_grad)
     int sms = 1;
     float *master = nullptr, *m1 = nullptr, *m2 = nullptr, *xn = nullptr, *tn = nullptr;
     float *part = nullptr, *lpart = nullptr, *grad = nullptr;
@@ -677,32 +785,34 @@ bool finite3(const float *v) {
 // launch with programmatic dependent launch: the kernel's set-up overlaps the previous
 // kernel's end, it waits (griddepcontrol.wait) before its first access to global memory
 template <typename K, typename... A>
-cudaError_t launch_dependent(K kern, int grid, int block, cudaStream_t s, A... args) {
+cudaError_t launch_dependent(K kern, int grid, int block, int cluster, cudaStream_t s, A... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-// samples per tile for n samples (see k_mlp_grad)
-int tile_for(int n) { return n <= kSmallTile * kMaxGradCtas ? kSmallTile : kLargeTile; }
+// CTAs per tile for n samples (see k_mlp_grad)
+int split_for(int n) { return n <= kTile * (kMaxGradCtas / kSplit) ? kSplit : 1; }
 
 cudaError_t launch_grad(lb_mlp *m, int bump, cudaStream_t s) {
-    return launch_dependent(tile_for(m->n) == kSmallTile ? k_mlp_grad<kSmallTile> : k_mlp_grad<kLargeTile>,
-                            m->grad_ctas, kThreads, s, (const __nv_bfloat16 *)m->wbf,
-                            (const float *)m->xn, (const float *)m->tn, m->st, bump, m->part,
-                            m->lpart);
+    return launch_dependent(m->split == kSplit ? k_mlp_grad<kSplit> : k_mlp_grad<1>, m->parts * m->split, kThreads,
+                            m->split, s, (const __nv_bfloat16 *)m->wbf, (const float *)m->xn,
+                            (const float *)m->tn, m->st, bump, m->part, m->lpart);
 }
 
 cudaError_t launch_adam(lb_mlp *m, float *grad_out, cudaStream_t s) {
-    return launch_dependent(k_mlp_adam, (NP + kAdamParams - 1) / kAdamParams, kAdamThreads, s,
-                            (const float *)m->part, (const float *)m->lpart, m->grad_ctas, m->st,
+    return launch_dependent(k_mlp_adam, (NP + kAdamParams - 1) / kAdamParams, kAdamThreads, 1, s,
+                            (const float *)m->part, (const float *)m->lpart, m->parts, m->st,
                             m->master, m->m1, m->m2, m->wbf, grad_out);
 }
 
@@ -842,12 +952,11 @@ lb_status lb_mlp_set_data(lb_mlp *m, const float *x, const float *y, int n) {
     LB_MCUDA(m, cudaMemcpyAsync(&m->st->n, &n, sizeof(int), cudaMemcpyHostToDevice, m->stream));
     LB_MCUDA(m, cudaStreamSynchronize(m->stream));
     m->n = n;
-    const int tile = tile_for(n), tiles = (n + tile - 1) / tile;
-    const int ctas = tiles < kMaxGradCtas ? tiles : kMaxGradCtas;
-    // the captured graph carries the grid and the tile kernel
-    if (ctas != m->grad_ctas || tile != m->tile) drop_graph(m);
-    m->tile = tile;
-    m->grad_ctas = ctas;
+    const int split = split_for(n), parts = std::min((n + kTile - 1) / kTile, kMaxGradCtas);
+    // the captured graph carries the grid and the kernel
+    if (parts != m->parts || split != m->split) drop_graph(m);
+    m->split = split;
+    m->parts = parts;
     m->have_norm = true;
     return LB_OK;
 }

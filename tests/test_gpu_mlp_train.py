@@ -1,6 +1,6 @@
-"""The training kernels at the edges of the tile rule (4 samples per tile while that gives at
-most 304 tiles, 16 beyond): ragged tiles, the last count of small tiles, the first of large
-ones, more tiles than CTAs; and the running powers of beta1, beta2 behind the bias correction
+"""The training kernels at the edges of how a tile of 16 samples is split (over four CTAs while
+there are at most 76 tiles, beyond not): ragged tiles, the last count that is split, the first
+that is not, more tiles than CTAs; and the running powers of beta1, beta2 behind the bias correction
 over calls with other betas. Gradients within 1e-4 of the largest entry and losses within 1e-4
 (FP32 sums of up to 5000 samples, about 1e-6, and FP32 erf / exp)."""
 import numpy as np
