@@ -95,7 +95,9 @@ def measured_peaks():
 def kernel_source_sha(prec: str = "fp32") -> str:
     h = hashlib.sha256()
     unit = {"fp32": "f32", "fp64": "f64", "bf16": "bf16"}[prec]
-    for name in ("lb_device.cuh", "lb_step.cuh", f"lb_step_{unit}.cu", f"lb_step_{unit}_stage.cu"):
+    tile = "lb_split_f64.cu" if prec == "fp64" else f"lb_tile_{unit}.cu"
+    for name in ("lb_device.cuh", "lb_step.cuh", "lb_tile.cuh", f"lb_step_{unit}.cu",
+                 f"lb_step_{unit}_stage.cu", tile):
         with open(os.path.join(ROOT, "paper_1306_6445_gb300", "csrc", name), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -239,7 +241,11 @@ def time_precision(lbm, torch, inputs, prec, nx, ny, inner, steps, warmup, dist,
         dist.barrier()
     total_ms = t0.elapsed_time(t1)
     step_kernel_ms = sum(a.elapsed_time(b) for a, b in ev)
-    launches = steps * (inner * lbm.lb_kernels_per_step(lat.ctx) + 3)
+    # lb_reduce launches two kernels; an FP32 lattice that fits the SMs' shared memory (at most 152
+    # tiles of 64 x 35 sites) may take all its steps in one launch: counted as one
+    per_step = 1 if prec == "fp32" and nx * ny <= 152 * 64 * 35 else \
+        inner * lbm.lb_kernels_per_step(lat.ctx)
+    launches = steps * (per_step + 2)
     lat.close()
     return total_ms, step_kernel_ms / (steps * inner), launches, shape
 
@@ -710,7 +716,9 @@ def native(args):
     hbm, peak_src = measured_peaks()
     alg = ALG_BYTES_PER_SITE["fp32"] * sites
     achieved = alg / (kern_ms * 1e-3) / 1e9
-    kname = "k_pull_collide_stage<float>" if shape["variant"] >= 4 else "k_pull_collide<float>"
+    kname = ("k_pull_collide", "k_pull_collide_stage", "k_tile_step",
+             "k_staged_tile_step")[(shape["variant"] >= 4) + (shape["variant"] >= 7)
+                                   + (shape["variant"] >= 8)] + "<float>"
     # the committed capture counts only for the kernel it was taken on
     traffic = profiled_traffic("fp32") if profiled_kernel("fp32") == kname else None
     roof = {"bound": "hbm", "achieved": round(achieved, 1), "peak": hbm, "unit": "GB/s",

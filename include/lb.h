@@ -206,8 +206,9 @@ lb_status lb_debug_stall_row(lb_ctx *ctx, int row);
  * and positive at some site (rho <= 0, or (p_EOS - rho/3)/G <= 0), LB_ECUDA. */
 lb_status lb_set_rho_u(lb_ctx *ctx, const double *rho, const double *ux, const double *uy);
 
-/* Advance n >= 0 time steps (Eqs. 4-8, 17-19), lb_kernels_per_step launches each (small
- * LB_FP32 lattices with variant 7: up to 1024 steps in one launch). Queued on the
+/* Advance n >= 0 time steps (Eqs. 4-8, 17-19), lb_kernels_per_step launches each
+ * (LB_FP32 lattices that fit the SMs, see lb_launch_variants: up to 1024 steps in one launch,
+ * which ends in the same one of the two buffers). Queued on the
  * stream; returns without waiting. A psi-domain violation found on the device is reported
  * by the next call that synchronises (lb_sync, lb_get_*, lb_reduce) as LB_EDOMAIN; a
  * device-side wait that gave up (about one second) as LB_ETIMEOUT. */

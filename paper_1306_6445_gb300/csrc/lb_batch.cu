@@ -1,6 +1,8 @@
 // Batched lattices (lb_batch_*): many independent periodic droplet lattices of uneven size
-// and parameters advanced together by one persistent kernel per time step (k_batch_step),
-// replayed from a captured CUDA graph, plus per-lattice Laplace measurements on the GPU.
+// and parameters advanced together, plus per-lattice Laplace measurements on the GPU. FP32 batches
+// take their steps by groups of lattices whose state stays in L2 (k_batch_tile, queue_groups); FP64
+// and the ring variants by one persistent kernel per time step over all lattices (k_batch_step),
+// replayed from a captured CUDA graph, as is a batch of a single small group.
 #include <cuda.h>
 #include <cuda_runtime.h>
 

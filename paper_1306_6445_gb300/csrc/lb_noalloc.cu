@@ -8,8 +8,8 @@
 // Differences from lb_reduce (which stores a psi field and allocates its partial sums on
 // first use): psi at a site's eight neighbours is recomputed from their populations, so
 // the only scratch is the per-block partial sums, the final four values and an error
-// word. The block split and per-thread order are those of lb_reduce, and the per-site
-// arithmetic is the same, so the two usually agree to the last bit.
+// word. The per-site arithmetic is that of lb_reduce; the blocks are its own, so the sums
+// agree to the rounding of FP64 sums taken in another (fixed) order.
 #include <cuda_runtime.h>
 
 #include <climits>
@@ -84,8 +84,8 @@ __device__ __forceinline__ T na_psi(const T *__restrict__ g, const DevConsts<T> 
     return lbm::eos_psi<T, EOS>(na_sum9(v), P, bad);
 }
 
-// Block b sums sites [b*chunk, (b+1)*chunk) in the same order as lb_reduce and writes its
-// four partials to scratch[4b .. 4b+3]; a psi-domain violation sets scratch[NA_ERR].
+// Block b sums sites [b*chunk, (b+1)*chunk) in a fixed order and writes its four partials to
+// scratch[4b .. 4b+3]; a psi-domain violation sets scratch[NA_ERR].
 template <typename T, int EOS, bool WALLS>
 __global__ void __launch_bounds__(NA_THREADS)
 k_na_partials(const T *__restrict__ g, const DevConsts<T> P, int nx, int ny, int pitch,
@@ -251,7 +251,7 @@ extern "C" lb_status lb_reduce_noalloc(lb_ctx *ctx, double out[4]) {
     cudaError_t e = scratch_address(&scratch);
     if (e != cudaSuccess)
         return lbm::ctx_fail(ctx, LB_ECUDA, cudaGetErrorString(e), false);
-    // same block split as lb_reduce
+    // four sites per thread, up to the blocks that the scratch has room for
     long long nbl = (n + NA_THREADS * 4 - 1) / (NA_THREADS * 4);
     const int nb = (int)(nbl < 1 ? 1 : (nbl > NA_MAX_BLOCKS ? NA_MAX_BLOCKS : nbl));
     const long long chunk = (n + nb - 1) / nb;

@@ -21,10 +21,12 @@
 // GH-1 and nx+GH, nx+GH+1 are ghost copies of columns nx-2, nx-1 and 0, 1 (periodic
 // images), rewritten by every kernel that writes g.
 //
-// Hot kernels: a CTA owns a strip of TX columns (two per thread) and marches over `rows`
+// Kernels of this file, the ring kernels (launch variants 0-6; the default for FP32 states beyond
+// L2, where their long loads keep memory busiest; the others are in lb_tile.cuh, lb_cluster.cu and
+// lb_resident.cu): a CTA owns a strip of TX columns (two per thread) and marches over `rows`
 // rows. The populations arrive in shared memory through 3-D TMA loads
-// (cp.async.bulk.tensor) completing on per-stage mbarriers: k_pull_collide_stage (the
-// default) stages, per psi row, exactly the three plane groups that row is pulled from,
+// (cp.async.bulk.tensor) completing on per-stage mbarriers: k_pull_collide_stage
+// stages, per psi row, exactly the three plane groups that row is pulled from,
 // one stage in use at a time; k_pull_collide stages whole rows of the strip (9 planes x
 // (TX + AL + 4) columns: the strip, an apron of AL columns on the left, 8 for float
 // storage and 4 otherwise, and 4 on the right), three rows in use at a time. From the
@@ -32,9 +34,6 @@
 // HBM; a four-row psi ring with one halo column on each side lives in shared memory), then
 // collides (Eqs. 3-8, 17-19) in packed two-lane arithmetic and stores f* as one 8-byte
 // (FP32) or 16-byte (FP64) store per population. Both give identical results.
-
-
-
 #pragma once
 
 #include <cuda.h>
@@ -185,15 +184,6 @@ __device__ __forceinline__ T pull_padded(const T *__restrict__ g, int a, int x, 
     if (BC == 0) sy = sy < 0 ? sy + ny : (sy >= ny ? sy - ny : sy);
     if (BC == 2) sy = sy >= ny ? ny - 1 : sy;
     return g[(size_t)plane_of(a) * plane + (unsigned)sy * (unsigned)pitch + (unsigned)(x - EXv(a) + GH<T>)];
-}
-
-// the value of f_a(x, y) (decoded from the storage type)
-template <typename T, int BC>
-__device__ __forceinline__ Arith<T> pull_val(const T *__restrict__ g, int a, int x, int y,
-                                             int nx, int ny, int pitch, long long plane,
-                                             const DevConsts<Arith<T>> &P) {
-    // a bounced-back link reads the opposite population, whose storage shift is the same
-    return pop_dec<T>(pull_global<T, BC>(g, a, x, y, nx, ny, pitch, plane), a, P);
 }
 
 // the nine populations of (x, y) through the ghost columns, decoded

@@ -425,7 +425,7 @@ k_batch_tile(const __grid_constant__ BatchGroup G, const CUtensorMap *__restrict
 // columns beside it) and a collision pass reads it; the 16 extra bytes per site cost nothing
 // beside the pipe. One site per thread: any lattice spreads over all SMs. Per step: 128^2 8.9
 // against 118 us in the ring kernel (16 CTAs), 1000 x 700 219 against 280 us (which forms psi
-// of the strip's rim in a pass of its own); 0.89 of the measured FP64 rate.
+// of the strip's rim in a pass of its own); 0.85 of the measured FP64 rate at 2048^2.
 constexpr int SPLIT_THREADS = 64;
 
 template <typename T, int BC>
