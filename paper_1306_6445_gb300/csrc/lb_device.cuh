@@ -25,6 +25,8 @@ template <>
 struct ArithOf<__nv_bfloat16> { using type = float; };
 template <typename T>
 using Arith = typename ArithOf<T>::type;
+template <typename T>
+constexpr bool PLAIN_OF = std::is_same<T, __nv_bfloat16>::value;   // see collide_plain
 
 // The update's constants as values of type C: the arithmetic type itself in kernel parameters
 // (DevConsts), pairs (v, v) where a kernel keeps them in shared memory (lb_tile.cuh): a packed
@@ -52,17 +54,17 @@ struct ConstFields {
     // s_vV; the v_* coefficients for that rate
     C rho_sw, v_m_V, v_u_V, v_f2_V, v_f4_V, v_q4_V, v_q16_V;
 };
-// The coefficients of collide_switched: Eq. 17's (1 - s), s, (1 - s/2) and source weights of the
-// unscaled moments, rounded once from FP64; *_V: of the vapour's rate.
+// The constants of collide_plain and of its psi: Eq. 17's (1 - s), s, (1 - s/2) and source weights
+// of the unscaled moments, rounded once from FP64; *_V: of the vapour's rate.
 template <typename T>
-struct SwitchedConsts {
-    T mG, kG2, sig_coef, rho_sw;
+struct PlainConsts {
+    T a, RT, mG, kG2, sig_coef, rho_sw, rho_s;
     T e_keep, s_e, e_half, e_src, z_keep, s_z, z_half, z_src, q_keep, s_q, q_half;
     T v_keep, s_v, v_half, v_src, v_keep_V, s_v_V, v_half_V, v_src_V;
 };
 template <typename T>
 struct DevConsts : ConstFields<T> {
-    SwitchedConsts<T> sw;
+    PlainConsts<T> sw;
     int stall_row;
     // LB_BF16 stochastic rounding: the step of the launch (the counter)
     unsigned sr_step;
@@ -109,7 +111,8 @@ inline DevConsts<T> to_dev(const Consts &c) {
         d.wshift[a] = T((a == 0 ? 4.0 / 9.0 : (a <= 4 ? 1.0 / 9.0 : 1.0 / 36.0)) * c.shift_rho);
     d.rho_s = T(c.shift_rho);
     d.rho_sw = T(c.rho_sw);
-    SwitchedConsts<T> &w = d.sw;
+    PlainConsts<T> &w = d.sw;
+    w.a = T(c.a); w.RT = T(c.RT); w.rho_s = T(c.shift_rho);
     w.mG = T(-c.G); w.kG2 = T(c.kG2); w.sig_coef = T(c.sig_coef); w.rho_sw = T(c.rho_sw);
     w.e_keep = T(1.0 - c.s_e); w.s_e = T(c.s_e); w.e_half = T(1.0 - 0.5 * c.s_e); w.e_src = T(1.5 * c.s_e);
     w.z_keep = T(1.0 - c.s_z); w.s_z = T(c.s_z); w.z_half = T(1.0 - 0.5 * c.s_z); w.z_src = T(1.5 * c.s_z);
@@ -226,7 +229,8 @@ __device__ __forceinline__ T scalar(const V2<T> &v) { return v.lo(); }
 // Interaction potential psi(rho) (Sec. II): psi0 exp(-rho0/rho), or
 // sqrt(2 (p_EOS - rho c_s^2) / G) with p_EOS the Carnahan-Starling EOS or Eq. 23.
 // Sets `bad` when rho <= 0 or psi^2 <= 0 (the value is then not usable).
-template <typename T, int EOS, typename PT>
+// PLAIN: psi of the BF16 steps, whose arithmetic stays as it is (see collide_plain).
+template <typename T, int EOS, bool PLAIN = false, typename PT>
 __device__ __forceinline__ T eos_psi(T rho, const PT &P, bool &bad) {
     if constexpr (EOS == LB_EOS_EXP) {
         bad |= !(rho > T(0));
@@ -239,9 +243,14 @@ __device__ __forceinline__ T eos_psi(T rho, const PT &P, bool &bad) {
             const T eta = rmul(scalar<T>(P.b4), rho);
             const T om = rsub(T(1), eta);
             const T poly = rfma(eta, rfma(eta, om, T(1)), T(1));
-            const T num = rmul(rmul(rho, scalar<T>(P.rtc)), poly);
+            T rt;
+            if constexpr (PLAIN) rt = P.sw.RT;
+            else rt = scalar<T>(P.rtc);
+            const T num = rmul(rmul(rho, rt), poly);
             const T q = rmul(num, lb_rcp(rmul(rmul(om, om), om)));
-            if constexpr (std::is_same<T, float>::value)   // the three terms rounded apart: see eos_psi2
+            if constexpr (PLAIN)
+                arg = rmul(rsub(rsub(q, rmul(P.sw.a, rmul(rho, rho))), rmul(rho, T(1.0 / 3.0))), P.two_over_G);
+            else if constexpr (std::is_same<T, float>::value)   // the three terms rounded apart: see eos_psi2
                 arg = rsub(rsub(q, rmul(scalar<T>(P.a2), rmul(rho, rho))), rmul(rho, scalar<T>(P.c3)));
             else
                 arg = rfma(rho, -rfma(scalar<T>(P.a2), rho, scalar<T>(P.c3)), q);
@@ -347,7 +356,7 @@ __device__ __forceinline__ V1<T> pick_ge(V1<T> a, T limit, T x, T y) {
 // psi of two densities; lane by lane the same operations, in the same order and with
 // the same rounding, as eos_psi (so a site's psi does not depend on which lane or which
 // kernel computes it). `hi_valid` = false: the second lane is padding and is not checked.
-template <typename T, int EOS, typename PT>
+template <typename T, int EOS, bool PLAIN = false, typename PT>
 __device__ __forceinline__ V2<T> eos_psi2(V2<T> rho, const PT &P, bool hi_valid, bool &bad) {
     if constexpr (EOS == LB_EOS_CS) {
         using V = V2<T>;
@@ -355,14 +364,21 @@ __device__ __forceinline__ V2<T> eos_psi2(V2<T> rho, const PT &P, bool hi_valid,
         const V eta = V::all(P.b4) * rho;
         const V om = one - eta;
         const V poly = vfma(eta, vfma(eta, om, one), one);
-        const V num = (rho * V::all(P.rtc)) * poly;
-        const V q = num * vrcp((om * om) * om);
+        V rt;
+        if constexpr (PLAIN) rt = V::all(P.sw.RT);
+        else rt = V::all(P.rtc);
+        const V num = (rho * rt) * poly, den = (om * om) * om;
+        V q;
+        if constexpr (PLAIN) q = V(lb_div(num.lo(), den.lo()), lb_div(num.hi(), den.hi()));
+        else q = num * vrcp(den);
         // In FP32 the three terms are rounded one by one: arg is a small difference of terms of
         // the order of rho, and the fused form (two operations fewer) rounds 2 a rho + 2/3, twice
         // their size; the pressure it left in a liquid at 0.8 T_c doubled the error of a droplet
         // after 200 steps against FP64 (1.3e-6 against 6e-7).
         V arg;
-        if constexpr (std::is_same<T, float>::value)
+        if constexpr (PLAIN)
+            arg = ((q - V::all(P.sw.a) * (rho * rho)) - rho * V::all(T(1.0 / 3.0))) * V::all(P.two_over_G);
+        else if constexpr (std::is_same<T, float>::value)
             arg = (q - V::all(P.a2) * (rho * rho)) - rho * V::all(P.c3);
         else
             arg = vfma(rho, -vfma(V::all(P.a2), rho, V::all(P.c3)), q);
@@ -371,21 +387,25 @@ __device__ __forceinline__ V2<T> eos_psi2(V2<T> rho, const PT &P, bool hi_valid,
         return V(lb_sqrt_pos(arg.lo()), lb_sqrt_pos(arg.hi()));
     } else {
         bool b2 = false;
-        const T lo = eos_psi<T, EOS>(rho.lo(), P, bad);
-        const T hi = eos_psi<T, EOS>(rho.hi(), P, b2);
+        const T lo = eos_psi<T, EOS, PLAIN>(rho.lo(), P, bad);
+        const T hi = eos_psi<T, EOS, PLAIN>(rho.hi(), P, b2);
         if (hi_valid) bad |= b2;
         return V2<T>(lo, hi);
     }
 }
 
-// The collision of FP32 sites whose viscosity switches at rho_sw (open boundaries), with the
-// moments as they are: m* = (1 - s) m + s m_eq + (1 - s/2) S + C of Eq. 17, then M^-1 m*. The switch
-// is a discontinuity: a site whose rho lies within the rounding errors of rho_sw takes one
+// The collision of the steps in which a rounding decides, with the moments as they are: m* = (1 - s)
+// m + s m_eq + (1 - s/2) S + C of Eq. 17, then M^-1 m*. VSW: the viscosity switch of FP32 lattices
+// with open boundaries: a site whose rho lies within the rounding errors of rho_sw takes one
 // viscosity or the other, which moves populations by up to 1e-3 of the largest and is carried on.
-// So its arithmetic stays as it is, operation by operation (collide, below, has 30 operations fewer
-// and a smaller error where no site switches, but sends other sites across).
-template <typename V, typename T>
-__device__ __forceinline__ void collide_switched(V (&f)[9], const V (&pn)[9], const SwitchedConsts<T> &P) {
+// SH: BF16 storage, where one rounding of the FP32 value sends the stored one to its other
+// neighbour, and with it a reproducible run (with stochastic rounding, one of its random walks) to
+// another. So the arithmetic of these stays as it is, operation by operation (collide, below, has
+// 30 operations fewer and a smaller error, but another one). SH: f holds f_a - w_a rho_s; the shift
+// only moves the moments rho, e and zeta (M w = (1, -2, 1, 0, ..., 0)), so those are corrected by
+// rho_s, and the same is taken off m* before M^-1 gives the shifted f* that is stored.
+template <typename T, bool VSW, bool SH, typename V>
+__device__ __forceinline__ void collide_plain(V (&f)[9], const V (&pn)[9], const PlainConsts<T> &P) {
     const V third = V::all(T(1.0 / 3.0)), twelfth = V::all(T(1.0 / 12.0));
     const V two = V::all(T(2)), four = V::all(T(4)), half = V::all(T(0.5)), mtwo = V::all(T(-2));
     const V pc = pn[0];
@@ -408,10 +428,17 @@ __device__ __forceinline__ void collide_switched(V (&f)[9], const V (&pn)[9], co
     const V s57 = f[5] + f[7], s68 = f[6] + f[8];
     const V d57 = f[5] - f[7], d68 = f[6] - f[8];
     const V axis = ax + ay, diag = s57 + s68;
-    const V rho = f[0] + (axis + diag);
+    const V rsum = f[0] + (axis + diag);       // sum of f (of the shifted f when SH)
+    const V rs = V::all(P.rho_s);
+    V rho = rsum;
+    if constexpr (SH) rho = rsum + rs;
     const V jx = d13 + (d57 - d68), jy = d24 + (d57 + d68);
-    const V m1 = vfma(two, diag, vfma(V::all(T(-4)), f[0], -axis));
-    const V m2 = vfma(four, f[0], vfma(mtwo, axis, diag));
+    V m1 = vfma(two, diag, vfma(V::all(T(-4)), f[0], -axis));
+    V m2 = vfma(four, f[0], vfma(mtwo, axis, diag));
+    if constexpr (SH) {
+        m1 = vfma(mtwo, rs, m1);
+        m2 = m2 + rs;
+    }
     const V m4 = vfma(mtwo, d13, d57 - d68), m6 = vfma(mtwo, d24, d57 + d68);
 
     // Eq. 6 velocity, Eq. 3 equilibria, Eqs. 5 and 8 forcing, Eq. 18 source
@@ -427,20 +454,29 @@ __device__ __forceinline__ void collide_switched(V (&f)[9], const V (&pn)[9], co
     const V tr = Qxx + Qyy;
 
     // Eq. 17
-    const V ms1 = vfma(V::all(P.e_keep), m1, vfma(V::all(P.s_e), meq1, vfma(V::all(P.e_half), S1, V::all(P.e_src) * tr)));
-    const V ms2 = vfma(V::all(P.z_keep), m2, vfma(V::all(P.s_z), meq2, -vfma(V::all(P.z_half), S1, V::all(P.z_src) * tr)));
+    V ms1 = vfma(V::all(P.e_keep), m1, vfma(V::all(P.s_e), meq1, vfma(V::all(P.e_half), S1, V::all(P.e_src) * tr)));
+    V ms2 = vfma(V::all(P.z_keep), m2, vfma(V::all(P.s_z), meq2, -vfma(V::all(P.z_half), S1, V::all(P.z_src) * tr)));
     const V ms3 = jx + Fx, ms5 = jy + Fy;
     const V ms4 = vfma(V::all(P.q_keep), m4, -vfma(V::all(P.s_q), rvx, V::all(P.q_half) * Fx));
     const V ms6 = vfma(V::all(P.q_keep), m6, -vfma(V::all(P.s_q), rvy, V::all(P.q_half) * Fy));
-    const V vkeep = pick_ge(rho, P.rho_sw, P.v_keep, P.v_keep_V), vs = pick_ge(rho, P.rho_sw, P.s_v, P.s_v_V);
-    const V vhalf = pick_ge(rho, P.rho_sw, P.v_half, P.v_half_V), vsrc = pick_ge(rho, P.rho_sw, P.v_src, P.v_src_V);
+    V vkeep = V::all(P.v_keep), vs = V::all(P.s_v), vhalf = V::all(P.v_half), vsrc = V::all(P.v_src);
+    if constexpr (VSW) {
+        vkeep = pick_ge(rho, P.rho_sw, P.v_keep, P.v_keep_V);
+        vs = pick_ge(rho, P.rho_sw, P.s_v, P.s_v_V);
+        vhalf = pick_ge(rho, P.rho_sw, P.v_half, P.v_half_V);
+        vsrc = pick_ge(rho, P.rho_sw, P.v_src, P.v_src_V);
+    }
     const V ms7 = vfma(vkeep, ax - ay, vfma(vs, rho * (vxx - vyy), vfma(vhalf, S7, vsrc * (Qxx - Qyy))));
     const V ms8 = vfma(vkeep, s57 - s68, vfma(vs, rvx * vy, vfma(vhalf, S8, vsrc * Qxy)));
 
     // f* = M^-1 m*; f*_0 from mass conservation, so that rounded constants add no mass
+    if constexpr (SH) {                        // back to the moments of the shifted f*
+        ms1 = vfma(two, rs, ms1);
+        ms2 = ms2 - rs;
+    }
     const V c18 = V::all(T(1.0 / 18.0)), c36 = V::all(T(1.0 / 36.0));
     const V c6 = V::all(T(1.0 / 6.0)), c4 = V::all(T(0.25));
-    const V a0 = V::all(T(1.0 / 9.0)) * rho;
+    const V a0 = V::all(T(1.0 / 9.0)) * rsum;
     const V base_axis = a0 - vfma(c36, ms1, c18 * ms2);
     const V base_diag = vfma(c18, ms1, vfma(c36, ms2, a0));
     const V jx6 = c6 * ms3, qx6 = c6 * ms4, jy6 = c6 * ms5, qy6 = c6 * ms6;
@@ -456,7 +492,7 @@ __device__ __forceinline__ void collide_switched(V (&f)[9], const V (&pn)[9], co
     f[6] = base_diag - (xy_m + pxy4);
     f[7] = base_diag - (xy_p - pxy4);
     f[8] = base_diag + (xy_m - pxy4);
-    f[0] = rho - (((f[1] + f[3]) + (f[2] + f[4])) + ((f[5] + f[7]) + (f[6] + f[8])));
+    f[0] = rsum - (((f[1] + f[3]) + (f[2] + f[4])) + ((f[5] + f[7]) + (f[6] + f[8])));
 }
 
 // One collision for the sites of a vector V (V2: two sites, V1: one): f[9] (populations
@@ -477,16 +513,14 @@ __device__ __forceinline__ void collide_switched(V (&f)[9], const V (&pn)[9], co
 //   too. The products with rho v are taken before the division by rho is multiplied back.
 //   That is 120 operations and one reciprocal per site (FP64, whose pipe is the bound of
 //   the FP64 step; the form with unscaled moments took 150: 1000 x 700 FP64 steps in 280
-//   against 333 us, BF16 2048^2 steps in 63 against 65 us, FP32 2048^2 1 % faster).
+//   against 333 us, FP32 2048^2 1 % faster).
 //   VSW: nu(rho) of Sec. V.C, the rate of p_xx, p_xy (and the weight of their source
 //   terms) taken per site as s_v where rho >= rho_sw, else s_vV.
-//   SH (LB_BF16): f holds the stored shifted populations f_a - w_a rho_s. Of the quantities
-//   above the shift only moves rho (to which rho_s is added) and the rest state w_a rho, in
-//   which the shifted sum then gives the shifted f* that is stored.
+//   SH: LB_BF16, see collide_plain.
 template <typename T, bool VSW = false, bool SH = false, typename V, typename PT>
 __device__ __forceinline__ void collide(V (&f)[9], const V (&pn)[9], const PT &P) {
-    if constexpr (VSW && std::is_same<T, float>::value) {
-        collide_switched<V, T>(f, pn, P.sw);
+    if constexpr (SH || (VSW && std::is_same<T, float>::value)) {
+        collide_plain<T, VSW, SH>(f, pn, P.sw);
         return;
     }
     const V four = V::all(T(4)), half = V::all(T(0.5)), mtwo = V::all(T(-2)), mfour = V::all(T(-4));
@@ -515,9 +549,7 @@ __device__ __forceinline__ void collide(V (&f)[9], const V (&pn)[9], const PT &P
     const V d57 = f[5] - f[7], d68 = f[6] - f[8];
     const V axis = ax + ay, diag = s57 + s68;
     const V moving = axis + diag;
-    const V rsum = f[0] + moving;              // sum of f (of the shifted f when SH)
-    V rho = rsum;
-    if constexpr (SH) rho = rsum + V::all(P.rho_s);
+    const V rho = f[0] + moving;
     const V dm = d57 - d68, dp = d57 + d68;
     const V jx = d13 + dm;
     const V jy = d24 + dp;
@@ -562,8 +594,8 @@ __device__ __forceinline__ void collide(V (&f)[9], const V (&pn)[9], const PT &P
 
     // f* = M^-1 m*, M^-1 = M^T diag(1/9, 1/36, 1/36, 1/6, 1/12, 1/6, 1/12, 1/4, 1/4)
     const V c6 = V::all(T(1.0 / 6.0));
-    const V base_axis = vfma(V::all(T(1.0 / 9.0)), rsum, -vfma(V::all(T(2)), dz, de));
-    const V base_diag = vfma(V::all(T(1.0 / 36.0)), rsum, vfma(V::all(T(2)), de, dz));
+    const V base_axis = vfma(V::all(T(1.0 / 9.0)), rho, -vfma(V::all(T(2)), dz, de));
+    const V base_diag = vfma(V::all(T(1.0 / 36.0)), rho, vfma(V::all(T(2)), de, dz));
     // j* = j + F as 4 (j*/6 + q/12) along the diagonals and the rest along the axes, so that a
     // rounded 1/6 (which in FP32 adds 3e-8 of the momentum at every step) does not enter it (160
     // steps of a 600 x 225 splash with this collision, error against FP64: 2.6e-7 against 1.5e-6)
@@ -587,7 +619,7 @@ __device__ __forceinline__ void collide(V (&f)[9], const V (&pn)[9], const PT &P
     // FP64: 7e-7 against 1.1e-6). In FP64 the eight f*_a sum to 4 (base_axis + base_diag) up
     // to their own unbiased roundings, two operations instead of nine.
     if constexpr (std::is_same<T, double>::value)
-        f[0] = vfma(mfour, base_axis + base_diag, rsum);
+        f[0] = vfma(mfour, base_axis + base_diag, rho);
     else
         f[0] = f[0] + (moving - (((f[1] + f[3]) + (f[2] + f[4])) + ((f[5] + f[7]) + (f[6] + f[8]))));
 }

@@ -89,7 +89,7 @@ __global__ void k_init_feq(const double *__restrict__ rho, const double *__restr
     const int y = (int)(i / nx), x = (int)(i % nx);
     const double r = rho[i], vx = ux[i], vy = uy[i];
     bool bad = false;
-    (void)eos_psi<Arith<T>, EOS>(Arith<T>(r), P, bad);
+    (void)eos_psi<Arith<T>, EOS, PLAIN_OF<T>>(Arith<T>(r), P, bad);
     if (bad) atomicOr(err, ERR_DOMAIN);
     const double v2 = vx * vx + vy * vy;
     const double m[9] = {r, r * (-2.0 + 3.0 * v2), r * (1.0 - 3.0 * v2), r * vx, -r * vx,
@@ -127,7 +127,7 @@ __global__ void k_psi_field(const T *__restrict__ g, Arith<T> *__restrict__ psi,
     Arith<T> v[9];
     pull_site_vals<T, BC>(v, g, (int)x, (int)y, ny, pitch, plane, P);
     bool bad = false;
-    psi[i] = eos_psi<Arith<T>, EOS>(sum9(v), P, bad);
+    psi[i] = eos_psi<Arith<T>, EOS, PLAIN_OF<T>>(sum9(v), P, bad);
     if (bad) atomicOr(err, ERR_DOMAIN);
 }
 
@@ -269,7 +269,7 @@ k_droplet_sums(const T *__restrict__ g, const DevConsts<Arith<T>> P, int nx, int
         pull_site_vals<T, BC>(v, g, x, y, ny, pitch, plane, P);
         const A rho = sum9(v);
         bool bad = false;
-        const A psi = eos_psi<A, EOS>(rho, P, bad);
+        const A psi = eos_psi<A, EOS, PLAIN_OF<T>>(rho, P, bad);
         const double dr = double(rho), ds = double(psi);
         const int a = 2 * x - (nx - 1), b = 2 * y - (ny - 1);
         const long long d = (long long)a * a + (long long)b * b;

@@ -563,7 +563,7 @@ __device__ __forceinline__ int march(const CUtensorMap *tmap, T *__restrict__ go
         const bool bottom = WALLS && Y == 0, top = WALLS && Y == ny - 1;
         if (act) {
             pull2<T, BC, BW, true>(keep, r, c0 + L, c0 + L + 1, bottom, top, P);
-            const V2<A> psi = eos_psi2<A, EOS>(site_rho<T>(keep, P), P, both, bad);
+            const V2<A> psi = eos_psi2<A, EOS, PLAIN_OF<T>>(site_rho<T>(keep, P), P, both, bad);
             if (both) {
                 store_pair<A>(ps + c0 + 2, psi, true);
             } else {
@@ -578,7 +578,7 @@ __device__ __forceinline__ int march(const CUtensorMap *tmap, T *__restrict__ go
                 if (x0 + w == nx) hb = w + L - 1;
             }
             pull2<T, BC, BW, false>(h, r, ha, hb, bottom, top, P);
-            const V2<A> psi = eos_psi2<A, EOS>(site_rho<T>(h, P), P, true, bad);
+            const V2<A> psi = eos_psi2<A, EOS, PLAIN_OF<T>>(site_rho<T>(h, P), P, true, bad);
             ps[1] = psi.lo();
             ps[w + 2] = psi.hi();
         }
@@ -822,7 +822,7 @@ __device__ __forceinline__ int march_stage(const CUtensorMap *tmap, T *__restric
         const bool bottom = WALLS && Y == 0, top = WALLS && Y == ny - 1;
         if (act) {
             pull_stage<T, BC, BW, GS, true>(keep, stg, c0 + L, c0 + L + 1, bottom, top, P);
-            const V2<A> psi = eos_psi2<A, EOS>(site_rho<T>(keep, P), P, both, bad);
+            const V2<A> psi = eos_psi2<A, EOS, PLAIN_OF<T>>(site_rho<T>(keep, P), P, both, bad);
             if (both) {
                 store_pair<A>(ps + c0 + 2, psi, true);
             } else {
@@ -837,7 +837,7 @@ __device__ __forceinline__ int march_stage(const CUtensorMap *tmap, T *__restric
                 if (x0 + w == nx) hb = w + L - 1;
             }
             pull_stage<T, BC, BW, GS, false>(h, stg, ha, hb, bottom, top, P);
-            const V2<A> psi = eos_psi2<A, EOS>(site_rho<T>(h, P), P, true, bad);
+            const V2<A> psi = eos_psi2<A, EOS, PLAIN_OF<T>>(site_rho<T>(h, P), P, true, bad);
             ps[1] = psi.lo();
             ps[w + 2] = psi.hi();
         }

@@ -198,7 +198,7 @@ __device__ __forceinline__ void tile_step(const T *__restrict__ gin, T *__restri
                     return two_at<T>(plane_bytes(gin, plane, a), o[r] + oa, o[r] + ob, dx);
                 });
             }
-            const V2<A> psi = eos_psi2<A, EOS>(site_rho<T>(h, P), P, warp == 2 || both, bad);
+            const V2<A> psi = eos_psi2<A, EOS, PLAIN_OF<T>>(site_rho<T>(h, P), P, warp == 2 || both, bad);
             A *ps = psis[yr - y0 + 1];
             if (warp == 2) {
                 ps[1] = psi.lo();
@@ -211,7 +211,7 @@ __device__ __forceinline__ void tile_step(const T *__restrict__ gin, T *__restri
         }
     }
     if (act) {
-        const V2<A> psi = eos_psi2<A, EOS>(site_rho<T>(f, P), P, both, bad);
+        const V2<A> psi = eos_psi2<A, EOS, PLAIN_OF<T>>(site_rho<T>(f, P), P, both, bad);
         A *ps = psis[warp + 1];
         if (both) store_pair<A>(ps + c0 + 2, psi, true);
         else ps[c0 + 2] = psi.lo();
@@ -356,7 +356,7 @@ __device__ __forceinline__ void staged_tile_step(const CUtensorMap *tmap,
 
     bool bad = false;
     if (rim) {
-        const V2<A> psi = eos_psi2<A, EOS>(site_rho<T>(h, P), P, warp == 2 || both, bad);
+        const V2<A> psi = eos_psi2<A, EOS, PLAIN_OF<T>>(site_rho<T>(h, P), P, warp == 2 || both, bad);
         A *ps = sm.psis[yr - y0 + 1];
         if (warp == 2) {
             ps[1] = psi.lo();
@@ -368,7 +368,7 @@ __device__ __forceinline__ void staged_tile_step(const CUtensorMap *tmap,
         }
     }
     if (act) {
-        const V2<A> psi = eos_psi2<A, EOS>(site_rho<T>(f, P), P, both, bad);
+        const V2<A> psi = eos_psi2<A, EOS, PLAIN_OF<T>>(site_rho<T>(f, P), P, both, bad);
         A *ps = sm.psis[warp + 1];
         if (both) store_pair<A>(ps + c0 + 2, psi, true);
         else ps[c0 + 2] = psi.lo();
