@@ -356,8 +356,8 @@ bool direct_fits(const Geom &g) { return g.ny <= 65535; }   // one grid row per 
 // Which kernel a context starts with, from steps measured on GB300 (direct / staged / ring with
 // the autotuner's launch, us):
 //   FP64: bound by its pipe at every size, direct: 128^2 8.9 / - / 118, 1000 x 700 219 / - / 280.
-//   BF16 (stochastic rounding): staged at every size: 64^2 2.7 / 2.6 / -, 1024^2 16.0 / 14.4 / 21,
-//   2048^2 58.2 / 49.6 / 63, 4096 x 2048 114 / 96 / more.
+//   BF16 (stochastic rounding): staged at every size: 64^2 2.8 / 2.8 / -, 1024^2 16.6 / 15.1 / 21,
+//   2048^2 60.6 / 51.9 / 65, 4096 x 2048 with walls 155 / 109 / 137.
 //   FP32, open boundaries (nu(rho) takes registers from the direct kernel): staged: 600 x 225
 //   4.5 / 4.0 / 12.8, 1800 x 675 16.5 / 14.9 / -.
 //   FP32 otherwise: direct while latency counts, up to 1.1 M sites: 64^2 2.2 / 2.3 / 9.4, 512^2

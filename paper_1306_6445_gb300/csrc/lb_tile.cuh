@@ -137,7 +137,7 @@ __host__ __device__ constexpr int tile_ctas(int R, bool sr) {
 // row) and their per-row bookkeeping for 3 extra psi passes per 4 rows. Per step, against the
 // ring kernel with the autotuner's launch: 64^2 2.3 / 9.4 us, 501 x 383 4.6 / 9.8, 600 x 225
 // splash 4.1 / 12.8, 1024^2 12.0 / 15.1, 2048^2 51 / 49 (memory), BF16 stochastic 2048^2
-// 56-58 / 65. Tiles of 3, 5, 6 and 8 rows were within 3 % of 4 or slower, as were 64 and 96
+// 61 / 65. Tiles of 3, 5, 6 and 8 rows were within 3 % of 4 or slower, as were 64 and 96
 // registers.
 template <typename T, int EOS, int BC, int R, bool SR, typename PT>
 __device__ __forceinline__ void tile_step(const T *__restrict__ gin, T *__restrict__ gout,
