@@ -284,6 +284,12 @@ long long lb_steps_done(const lb_ctx *ctx);
 /* Number of kernel launches one lb_step(ctx, 1) queues (for launch accounting). */
 int lb_kernels_per_step(const lb_ctx *ctx);
 
+/* Kernel launches that the context's lb_step calls have queued so far: lb_kernels_per_step for
+ * each step taken singly, one for several steps taken together (see lb_launch_variants), which
+ * shows whether they were. A launch recorded into a graph counts once, however often it is
+ * replayed. */
+long long lb_step_launches(const lb_ctx *ctx);
+
 /* Last error message of the context (static string "no context" for NULL). */
 const char *lb_last_error(const lb_ctx *ctx);
 

@@ -40,6 +40,7 @@ struct lb_ctx {
     int many = 0;                // several steps at once: 1 the cluster kernel, 2 the resident one
     void *d_words = nullptr;     // exchange words of the resident kernel
     long long steps = 0;
+    long long launches = 0;      // kernel launches that lb_step has queued
     lb_status sticky = LB_OK;
     std::string msg;
 };
@@ -255,6 +256,13 @@ lb_status apply_launch(lb_ctx *c, int variant, int rows) {
     c->launch = lbm::make_step_launch(c->prec, c->consts.eos_kind, c->geom, c->num_sms, variant, rows);
     LB_CUDA(c, lbm::configure_step(c->prec, c->consts, c->geom, c->launch));
     return variant >= lbm::direct_variant() && c->prec == LB_FP64 ? LB_OK : make_maps(c);
+}
+
+// a launch of many steps that the GPU (or this process's share of it) has no room for: the steps can
+// still be taken one by one. Any other error is the caller's to know.
+bool no_room(cudaError_t e) {
+    return e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorInvalidClusterSize ||
+           e == cudaErrorLaunchOutOfResources || e == cudaErrorInvalidConfiguration;
 }
 
 lb_status check_usable(lb_ctx *c) {
@@ -617,13 +625,15 @@ lb_status lb_step(lb_ctx *c, int n) {
             c->many == 1 ? lbm::launch_cluster_steps(c->consts, c->geom, gin, gout, m, c->d_err, c->stream)
                          : lbm::launch_resident_steps(c->consts, c->geom, c->num_sms, gin, gout, m, c->d_words,
                                                       c->d_err, c->stream);
-        if (e != cudaSuccess) {       // not every SM can be had (a limited context): single launches
+        if (no_room(e)) {             // not every SM can be had (a limited context): single launches
             (void)cudaGetLastError();
             c->many = 0;
             break;
         }
+        LB_CUDA(c, e);
         c->cur ^= m & 1;
         c->steps += m;
+        ++c->launches;
         n -= m;
     }
     for (int i = 0; i < n; ++i) {
@@ -635,6 +645,7 @@ lb_status lb_step(lb_ctx *c, int n) {
                                     b, c->d_err, c->stream));
         c->cur ^= 1;
         ++c->steps;
+        c->launches += lb_kernels_per_step(c);
     }
     return LB_OK;
 }
@@ -749,6 +760,8 @@ lb_status lb_interface_height(lb_ctx *c, double rho_mid, double *heights) {
 }
 
 long long lb_steps_done(const lb_ctx *c) { return c ? c->steps : 0; }
+
+long long lb_step_launches(const lb_ctx *c) { return c ? c->launches : 0; }
 
 int lb_kernels_per_step(const lb_ctx *c) {
     if (!c) return 0;

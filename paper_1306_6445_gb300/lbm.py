@@ -29,7 +29,8 @@ LB_BC_PERIODIC, LB_BC_WALLS_Y, LB_BC_OPEN = 0, 1, 2
 # every exported symbol of include/lb.h
 EXPORTED = ["lb_pitch", "lb_buffer_bytes", "lb_init", "lb_init_ex", "lb_set_rho_u", "lb_step",
             "lb_sync", "lb_get_rho", "lb_get_u", "lb_get_populations", "lb_set_populations",
-            "lb_reduce", "lb_steps_done", "lb_kernels_per_step", "lb_last_error",
+            "lb_reduce", "lb_steps_done", "lb_kernels_per_step", "lb_step_launches",
+            "lb_last_error",
             "lb_status_of", "lb_free", "lb_cs_critical", "lb_maxwell", "lb_launch_variants",
             "lb_probe_fp64_fma_rate", "lb_measure_droplet", "lb_interface_height",
             "lb_set_launch", "lb_get_launch", "lb_debug_stall_row", "lb_reduce_noalloc",
@@ -109,6 +110,7 @@ def load_library():
         "lb_reduce": (I, [P, DP]),
         "lb_steps_done": (C.c_longlong, [P]),
         "lb_kernels_per_step": (I, [P]),
+        "lb_step_launches": (C.c_longlong, [P]),
         "lb_last_error": (C.c_char_p, [P]),
         "lb_status_of": (I, [P]),
         "lb_free": (None, [P]),
@@ -356,6 +358,10 @@ def lb_steps_done(ctx) -> int:
 
 def lb_kernels_per_step(ctx) -> int:
     return int(load_library().lb_kernels_per_step(ctx))
+
+
+def lb_step_launches(ctx) -> int:
+    return int(load_library().lb_step_launches(ctx))
 
 
 def lb_launch_variants() -> int:
