@@ -222,6 +222,7 @@ def time_precision(lbm, torch, inputs, prec, nx, ny, inner, steps, warmup, dist,
     ev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True))
           for _ in range(steps)]
     t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    launched = lbm.lb_step_launches(lat.ctx)
     if dist is not None:
         dist.barrier()
     torch.cuda.synchronize()
@@ -241,11 +242,8 @@ def time_precision(lbm, torch, inputs, prec, nx, ny, inner, steps, warmup, dist,
         dist.barrier()
     total_ms = t0.elapsed_time(t1)
     step_kernel_ms = sum(a.elapsed_time(b) for a, b in ev)
-    # lb_reduce launches two kernels; an FP32 lattice that fits the SMs' shared memory (at most 152
-    # tiles of 64 x 35 sites) may take all its steps in one launch: counted as one
-    per_step = 1 if prec == "fp32" and nx * ny <= 152 * 64 * 35 else \
-        inner * lbm.lb_kernels_per_step(lat.ctx)
-    launches = steps * (per_step + 2)
+    # the library counts the launches of its steps; lb_reduce launches two kernels
+    launches = lbm.lb_step_launches(lat.ctx) - launched + 2 * steps
     lat.close()
     return total_ms, step_kernel_ms / (steps * inner), launches, shape
 
