@@ -9,6 +9,7 @@ namespace {
 
 constexpr int CL_SIZE = 16;           // CTAs of the cluster
 constexpr int CL_MAX_THREADS = 512;   // of a CTA: as many as it has site pairs, in warps
+constexpr int CL_SMEM_MOST = 200 * 1024;
 
 __device__ __forceinline__ unsigned cluster_rank() {
     unsigned r;
@@ -165,7 +166,8 @@ cudaError_t cluster_launch(const Consts &c, const Geom &g, const void *gin, void
                            int *err, cudaStream_t st, bool probe) {
     auto kern = k_cluster_steps<EOS, BC>;
     const int smem = cluster_smem(g);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    // the kernel's limit, not this lattice's size: contexts of several threads share the attribute
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, CL_SMEM_MOST);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -211,7 +213,7 @@ cudaError_t cluster_dispatch(const Consts &c, const Geom &g, const void *gin, vo
 bool cluster_fits(int prec, const Consts &c, const Geom &g) {
     if (prec != LB_FP32 || g.walls == 2 || (g.nx & 1) || g.nx < 4 || g.ny < CL_SIZE) return false;
     if ((long long)g.nx * g.ny > CL_SIZE * 2ll * CL_MAX_THREADS) return false;
-    if (cluster_pairs(g) > CL_MAX_THREADS || cluster_smem(g) > 200 * 1024) return false;
+    if (cluster_pairs(g) > CL_MAX_THREADS || cluster_smem(g) > CL_SMEM_MOST) return false;
     if (cluster_dispatch(c, g, nullptr, nullptr, 0, nullptr, nullptr, true) == cudaSuccess) return true;
     (void)cudaGetLastError();
     return false;

@@ -400,10 +400,12 @@ k_resident_steps(const float *gin, float *gout,
     }
 }
 
-int resident_smem(const ResidentShape &s) {
-    return (18 * (s.max_rows + 4) + s.max_rows + 2) * RS_STRIDE * (int)sizeof(float) +
-           max_items(s.max_rows) * (int)sizeof(int2);
+constexpr int smem_of_rows(int rows) {
+    return (18 * (rows + 4) + rows + 2) * RS_STRIDE * (int)sizeof(float) + max_items(rows) * (int)sizeof(int2);
 }
+int resident_smem(const ResidentShape &s) { return smem_of_rows(s.max_rows); }
+constexpr int RS_SMEM_MOST = smem_of_rows(RS_MAX_ROWS);
+static_assert(RS_SMEM_MOST + 1024 <= 228 * 1024, "a tile fits an SM (1 KB per CTA is the system's)");
 
 // Tiles of at least 6 rows (with fewer there are more CTAs to exchange with and no less to wait for:
 // 160^2 in tiles of 2, 4, 6, 12 rows 2.61, 2.30, 2.28, 2.62 us a step). false: the lattice does not fit,
@@ -427,7 +429,8 @@ cudaError_t resident_launch(const Consts &c, const Geom &g, const ResidentShape 
                             void *gout, int n_steps, uint64_t *words, int *err, cudaStream_t st, bool probe) {
     auto kern = k_resident_steps<EOS, BC>;
     const int smem = resident_smem(s);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    // the kernel's limit, not this lattice's size: contexts of several threads share the attribute
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, RS_SMEM_MOST);
     if (e != cudaSuccess) return e;
     if (probe) {
         int n = 0;

@@ -1,5 +1,7 @@
 """Which lattices take several steps in one launch (the cluster kernel and the resident one), as counted
 by lb_step_launches, and what a launch that cannot be made does to the context."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -81,3 +83,31 @@ def test_a_launch_that_fails_is_reported_and_changes_nothing(lbm, nx, ny):  # no
     lat.sync()
     assert lat.steps_done == STEPS
     lat.close()
+
+
+@pytest.mark.parametrize("sizes", [((4, 16), (128, 128)), ((195, 200), (560, 560))])
+def test_lattices_of_different_size_step_side_by_side(lbm, sizes):  # noqa: F811
+    """Two host threads step a small and a large lattice, which one kernel takes with different amounts
+    of shared memory: neither loses its launches of many steps."""
+    lats = []
+    for size in sizes:
+        with torch.cuda.stream(torch.cuda.Stream()):
+            lats.append(lattice(lbm, *size))
+    calls = 2000
+    before = [lbm.lb_step_launches(lat.ctx) for lat in lats]
+
+    def work(lat):
+        for i in range(calls):
+            lat.step(STEPS)
+            if i % 50 == 0:
+                lat.sync()
+        lat.sync()
+
+    threads = [threading.Thread(target=work, args=(lat,)) for lat in lats]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert [lbm.lb_step_launches(lat.ctx) - b for lat, b in zip(lats, before)] == [calls, calls]
+    for lat in lats:
+        lat.close()
