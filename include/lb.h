@@ -194,10 +194,14 @@ lb_status lb_autotune(lb_ctx *ctx, int trial_steps, int *variant, int *rows);
 lb_status lb_get_launch(const lb_ctx *ctx, int *variant, int *tx, int *rows, int *ctas_per_sm);
 
 /* Test hook for the failure path of the bounded device-side waits: from the next lb_step
- * on, the step kernel never requests lattice row `row` (as staged in its shared-memory
- * ring; a context with variant 7 or 8 changes to variant 4), so the CTAs that need it give up after about one second and the next
- * synchronising call returns LB_ETIMEOUT. Nothing faults and no copy is left in flight.
- * INT_MIN (the default) switches it off. Not part of the method; for tests only. */
+ * on, the step kernels wait for lattice row `row` in vain: it is never requested (as staged in
+ * the shared-memory ring, or in a staged tile), or taken from an exchange word that nobody
+ * publishes (many steps in one launch, from 32768 sites on). The CTAs that need it give up after
+ * about a second per wait and the next synchronising call returns LB_ETIMEOUT. Nothing faults and no
+ * copy is left in flight. While it is on, kernels that wait for nothing, or not for this row (variant
+ * 7, the tiles of variant 8 beside a periodic seam, many steps of up to 16384 sites), are replaced by
+ * variant 4. INT_MIN (the default) switches it off and the launch is what it was. Not part of the
+ * method; for tests only. */
 lb_status lb_debug_stall_row(lb_ctx *ctx, int row);
 
 /* f = f_eq(rho, u) = M^-1 m_eq(rho, u) of Eq. 3 at every site (the initial state).

@@ -37,6 +37,7 @@ struct lb_ctx {
     double *d_host_in = nullptr; // 3*nx*ny staging for lb_set_rho_u
     void *d_psi = nullptr;       // FP64 direct kernels: psi of the step, ny * pitch elements
     lbm::StepLaunch launch{};
+    int asked_variant = 0, asked_rows = 0;   // what apply_launch was last asked for
     int many = 0;                // several steps at once: 1 the cluster kernel, 2 the resident one
     void *d_words = nullptr;     // exchange words of the resident kernel
     long long steps = 0;
@@ -248,11 +249,20 @@ lb_status apply_launch(lb_ctx *c, int variant, int rows) {
     if (variant < 0 || variant >= lbm::step_variant_count())
         return fail(c, LB_EINVAL, "unknown launch variant");
     if (rows < 0) return fail(c, LB_EINVAL, "rows must be >= 0");
+    c->asked_variant = variant;
+    c->asked_rows = rows;
     if (variant >= lbm::direct_variant()) {
         if (c->prec == LB_FP64) variant = lbm::direct_variant();     // no staged FP64 kernel
         if (!direct_usable(c)) variant = lbm::default_ring_variant();
     }
     c->many = variant == lbm::default_variant(c->prec, c->geom) ? many_usable(c) : 0;
+    const int stall = c->consts.stall_row;
+    if (stall != INT_MIN) {      // test hook: kernels that wait for the row
+        if (c->many == 1 || !lbm::resident_waits_for_row(c->geom, stall)) c->many = 0;
+        if (variant == lbm::direct_variant() ||
+            (variant == lbm::staged_variant() && !lbm::staged_loads_row(c->geom, stall)))
+            variant = lbm::default_ring_variant();
+    }
     c->launch = lbm::make_step_launch(c->prec, c->consts.eos_kind, c->geom, c->num_sms, variant, rows);
     LB_CUDA(c, lbm::configure_step(c->prec, c->consts, c->geom, c->launch));
     return variant >= lbm::direct_variant() && c->prec == LB_FP64 ? LB_OK : make_maps(c);
@@ -579,10 +589,7 @@ lb_status lb_debug_stall_row(lb_ctx *c, int row) {
     lb_status s = check_usable(c);
     if (s != LB_OK) return s;
     c->consts.stall_row = row;
-    // the direct kernels stage no rows: a stalled row needs a ring
-    if (row != INT_MIN && c->launch.variant >= lbm::direct_variant())
-        return apply_launch(c, lbm::default_ring_variant(), 0);
-    return LB_OK;
+    return apply_launch(c, c->asked_variant, c->asked_rows);
 }
 
 lb_status lb_get_launch(const lb_ctx *c, int *variant, int *tx, int *rows, int *ctas_per_sm) {

@@ -56,7 +56,7 @@ struct Consts {
     double kG2;     // kappa G / 2 of Eq. 19
     double sig_coef;  // 12 sigma G^2 / (tau_e - 1/2): Eq. 8 with |F|^2/psi^2 = G^2 |sum w psi e|^2
     double s_e, s_z, s_q, s_v;  // non-conserved relaxation rates (s_rho, s_j drop out, see kernels)
-    int stall_row;  // test hook: the step kernel never requests this ring row (INT_MIN = off)
+    int stall_row;  // test hook: the kernels wait for this row in vain (INT_MIN = off)
     double shift_rho;  // rho_s of the LB_BF16 storage shift f_a - w_a rho_s (0 otherwise)
     int stochastic;    // LB_BF16: 1 = stochastic rounding of the stored values (0 = nearest)
     unsigned step_key; // the step a launch takes (the stochastic-rounding counter)
@@ -115,6 +115,14 @@ constexpr int DIRECT_COLS = 64, DIRECT_ROWS = 4, STAGED_ROWS = 4;
 // the staged tile's TMA box: columns x0 - 4 .. x0 + 67 (a 16-byte aligned start in both types), the
 // rows of the tile and one on either side, three planes
 constexpr int TILE_BOX_LEFT = 4, TILE_BOX_W = DIRECT_COLS + 8, TILE_BOX_ROWS = STAGED_ROWS + 2;
+// whether the staged kernel brings the tile of rows y0 .. y0 + r - 1 into shared memory: not where rows
+// wrap, nor where the row above the tile is the last below a wall (it bounces populations of its own
+// row, which its plane group's box does not reach)
+__host__ __device__ constexpr bool tile_staged(int bc, int y0, int r, int ny) {
+    return bc == 0 ? y0 >= 2 && y0 + r + 2 <= ny : !(bc == 1 && y0 + r == ny - 1);
+}
+bool staged_loads_row(const Geom &g, int row);      // some staged tile's boxes hold this lattice row
+bool resident_waits_for_row(const Geom &g, int row);   // some tile has it beside it (lb_resident.cu)
 int step_variant_tx(int variant);
 int step_variant_planes(int variant);   // population planes per TMA box (9 or 3)
 int default_ring_variant();

@@ -353,6 +353,12 @@ int step_variant_kind(int variant) { return variant >= 4 ? 1 : 0; }
 
 bool direct_fits(const Geom &g) { return g.ny <= 65535; }   // one grid row per lattice row (FP64)
 
+bool staged_loads_row(const Geom &g, int row) {
+    for (int y0 = 0; y0 < g.ny; y0 += STAGED_ROWS)
+        if (tile_staged(g.walls, y0, STAGED_ROWS, g.ny) && row >= y0 - 2 && row < y0 + STAGED_ROWS + 2) return true;
+    return false;
+}
+
 // Which kernel a context starts with, from steps measured on GB300 (direct / staged / ring with
 // the autotuner's launch, us):
 //   FP64: bound by its pipe at every size, direct: 128^2 8.9 / - / 118, 1000 x 700 219 / - / 280.

@@ -43,9 +43,13 @@ __host__ __device__ constexpr int max_items(int rows) { return RS_ROW_SLOTS * (R
 //   rows:    [ty][18][64 tx]  of a tile's row 0 planes 3..8, row 1 planes 6..8, last row planes 0..5,
 //                             last but one planes 0..2
 //   columns: [tx][4][9][ny]   of its column 0, column 1, last, last but one
+//   one that nobody publishes (the test hook, see lb_debug_stall_row, waits for it)
 // A word is a value and the time (epoch + step) it belongs to.
 __host__ __device__ constexpr unsigned row_words(int tx, int ty) { return (unsigned)ty * RS_ROW_SLOTS * RS_W * (unsigned)tx; }
 __host__ __device__ constexpr unsigned col_words(int tx, int ny) { return (unsigned)tx * RS_COL_SLOTS * (unsigned)ny; }
+__host__ __device__ constexpr unsigned exchange_words(int tx, int ty, int ny) {
+    return row_words(tx, ty) + col_words(tx, ny) + 1;
+}
 
 __device__ __forceinline__ uint64_t load_word(const uint64_t *p) {
     uint64_t v;
@@ -99,7 +103,7 @@ k_resident_steps(const float *gin, float *gout,
     const int PS = (max_rows + 4) * RS_STRIDE;
     float *const psis = rs_smem + 18 * PS;                    // rows -1 .. n
     int2 *const items = reinterpret_cast<int2 *>(psis + (max_rows + 2) * RS_STRIDE);
-    const unsigned n_words = row_words(tx, ty) + col_words(tx, ny);
+    const unsigned n_words = exchange_words(tx, ty, ny);
     uint64_t *const exch = words + 2;
     const unsigned epoch = (unsigned)load_word(words);
     const int c0 = 2 * lane, cr = (w - 1) & ~1;               // the lane's pair, the last pair
@@ -111,6 +115,7 @@ k_resident_steps(const float *gin, float *gout,
     for (int base = 32 * warp; base < row_items + RS_COL_SLOTS * n; base += (int)blockDim.x) {
         const int i = base + lane;
         int2 it = make_int2(-1, 0);
+        int from = 0;                             // the lattice row it comes from
         if (i < row_items) {
             // slots as published: the row above the tile is row 0 or 1 of the next tile
             const int slot = i / wide, col = i - slot * wide - 2;
@@ -119,6 +124,7 @@ k_resident_steps(const float *gin, float *gout,
             int nb = slot < 9 ? by + 1 : by - 1, gx = x0 + col;
             const bool in = BC == 0 || (nb >= 0 && nb < ty);
             nb = nb < 0 ? ty - 1 : nb >= ty ? 0 : nb;
+            from = y0 + row < 0 ? y0 + row + ny : y0 + row >= ny ? y0 + row - ny : y0 + row;
             if (BC == 2) gx = gx < 0 ? 0 : gx >= nx ? nx - 1 : gx;
             else gx = gx < 0 ? gx + nx : gx >= nx ? gx - nx : gx;
             if (in)
@@ -135,10 +141,12 @@ k_resident_steps(const float *gin, float *gout,
             const int ex = plane_ex(p), into = s < 2 ? -1 : 1;
             if (BC == 0) in = in && ((s & 1) ? ex == into : ex != -into);
             nb = nb < 0 ? tx - 1 : nb >= tx ? 0 : nb;
+            from = y0 + r;
             if (in)
                 it = make_int2((int)row_words(tx, ty) + (nb * RS_COL_SLOTS + slot) * ny + y0 + r,
                                p * PS + (r + 2) * RS_STRIDE + col + 2);
         }
+        if (it.x >= 0 && from == P.stall_row) it.x = (int)n_words - 1;   // test hook
         const unsigned have = __ballot_sync(0xffffffffu, it.x >= 0);
         int at = 0;
         if (lane == 0) at = atomicAdd(&n_items, __popc(have));
@@ -480,9 +488,15 @@ size_t resident_bytes(int prec, const Consts &c, const Geom &g, int num_sms) {
     if (cudaGetDevice(&dev) == cudaSuccess &&
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
         resident_dispatch(c, g, s, nullptr, nullptr, 0, nullptr, nullptr, nullptr, true) == cudaSuccess)
-        return (2 + 2 * ((size_t)row_words(s.tx, s.ty) + col_words(s.tx, g.ny))) * sizeof(uint64_t);
+        return (2 + 2 * (size_t)exchange_words(s.tx, s.ty, g.ny)) * sizeof(uint64_t);
     (void)cudaGetLastError();
     return 0;
+}
+
+// every row is beside a tile of the next column of tiles, if there is one (around the lattice unless
+// its sides are open)
+bool resident_waits_for_row(const Geom &g, int row) {
+    return row >= 0 && row < g.ny && (g.walls != 2 || g.nx > RS_W);
 }
 
 cudaError_t launch_resident_steps(const Consts &c, const Geom &g, int num_sms, const void *gin, void *gout,

@@ -4,6 +4,8 @@
 // layout, arithmetic and results, bit for bit, as the ring kernels of lb_step.cuh.
 #pragma once
 
+#include <climits>
+
 #include "lb_step.cuh"
 
 namespace lbm {
@@ -254,6 +256,12 @@ __host__ __device__ constexpr int staged_ctas(int R, bool sr) {
     return 65536 / (32 * R * (sr ? 128 : 64));
 }
 
+// the test hook's row (see lb_debug_stall_row); batches have no such hook
+template <typename T>
+__device__ __forceinline__ int stall_row_of(const DevConsts<T> &P) { return P.stall_row; }
+template <typename C>
+__device__ __forceinline__ constexpr int stall_row_of(const ConstFields<C> &) { return INT_MIN; }
+
 // As tile_step, with the populations brought into shared memory by three TMA loads, so that a
 // pull is a load at a constant offset: no address arithmetic, no wrap (414 instead of 471 warp
 // instructions per 64 sites). The loads take longer to arrive than a warp's own, so the direct
@@ -277,9 +285,7 @@ __device__ __forceinline__ void staged_tile_step(const CUtensorMap *tmap,
     const int w = min(TILE_W, nx - x0), n = min(R, ny - y0);
     const int y = y0 + warp, c0 = 2 * lane, x = x0 + c0;
     const bool act = warp < n && c0 < w, both = c0 + 1 < w;
-    // CTA-uniform: not where rows wrap, nor where the row above the tile is the last below a wall
-    // (it bounces populations of its own row, which its plane group's box does not reach)
-    const bool staged = BC == 0 ? y0 >= 2 && y0 + R + 2 <= ny : !(BC == 1 && y0 + R == ny - 1);
+    const bool staged = tile_staged(BC, y0, R, ny);   // CTA-uniform
 
     if (staged && threadIdx.x == 0) {
         mbar_init(&sm.bar, 1);
@@ -290,8 +296,11 @@ __device__ __forceinline__ void staged_tile_step(const CUtensorMap *tmap,
     if (staged && threadIdx.x == 0) {
         mbar_arrive_expect_tx(&sm.bar, 9u * SM::ROWS * TILE_BOX_W * (unsigned)sizeof(T));
 #pragma unroll
-        for (int q = 0; q < 3; ++q)   // rows outside the lattice (walls, open top) are zero-filled, not used
+        for (int q = 0; q < 3; ++q) { // rows outside the lattice (walls, open top) are zero-filled, not used
+            // test hook: the bytes of a box that holds this row stay expected and never come
+            if ((unsigned)stall_row_of(P) - (unsigned)(y0 - 2 + q) < (unsigned)SM::ROWS) continue;
             tma_load_3d(sm.pop + q * SM::GROUP, tmap, x0 + GH<T> - TILE_BOX_LEFT, y0 - 2 + q, 3 * q, &sm.bar);
+        }
     }
     if (staged || CONSTS) __syncthreads();   // the barrier is initialised, the constants are written
 
