@@ -311,7 +311,8 @@ void lb_free(lb_ctx *ctx);
  * captured once in a CUDA graph and replayed. With variant 8 (LB_FP32) the lattices form groups
  * that stay in the L2 cache: a group takes all the steps of a call before the next one, three
  * groups side by side on the batch's stream and two streams of its own that it forks and joins
- * (work queued on the stream before and after a call is ordered as ever). The update of each lattice is the one of lb_step (Eqs. 4-8,
+ * (work queued on the stream before and after a call is ordered as ever), or as graphs (see
+ * lb_batch_step). The update of each lattice is the one of lb_step (Eqs. 4-8,
  * 17-19), bit for bit. All lattices share the precision and the EOS kind.
  * --------------------------------------------------------------------------------- */
 typedef struct {
@@ -340,7 +341,12 @@ lb_status lb_batch_create(lb_batch **out, int n, const lb_lattice_desc *descs, i
 lb_status lb_batch_set_rho_u(lb_batch *b, int i, const double *rho, const double *ux,
                              const double *uy);
 
-/* Advance every lattice n >= 0 time steps (queued; returns without waiting). */
+/* Advance every lattice n >= 0 time steps (queued; returns without waiting for them). Few operations
+ * are queued: runs of 64 steps are one graph launch, with variant 8 and several groups of lattices
+ * runs of 16 steps one per 48 groups. What is left of n, and with several groups the first 128 steps of
+ * a batch and those after its launch or its active lattices have changed, is launched step by step
+ * and group by group, which takes as long as the GPU takes once its queue (about 1000 launches) is
+ * full. Inside a capture of the caller's all steps are launched one by one. */
 lb_status lb_batch_step(lb_batch *b, int n);
 
 /* Wait for queued work. LB_ETIMEOUT (and poisoning) if a bounded device wait gave up;

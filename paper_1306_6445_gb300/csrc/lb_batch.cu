@@ -20,8 +20,20 @@
 
 namespace {
 
-constexpr int kGraphSteps = 64;   // steps per captured graph (even: the phase returns)
-// Most sites of a group of the direct launch (or one lattice): both buffers of the kChains groups
+constexpr int kGraphSteps = 64;   // steps per captured graph of a batch of one group (even: the phase returns)
+// Several groups: graphs of 16 steps (even) of blocks of 48 groups each. lb_batch_step can return without
+// waiting only if it queues few operations: launched one by one, 64 steps of 512 lattices of 64^2 to
+// 512^2 (12 600 launches) hold the calling thread for 30.1 of their 39.2 ms and 64 of 24 x 128^2 for 0.38
+// of 0.40 ms; as graphs 0.1 of 39.25 ms and 0.01 of 0.36 ms. Blocks of 24, 12 or 6 groups took 39.6,
+// 40.7 and 45.2 ms (each starts and drains the three chains), graphs of 32 steps 38.7 ms, but twice as
+// long to make. Making them costs 4 us per launch and step, 13 ms for the 512 lattices, during which
+// the GPU takes the steps of the blocks before; so the first 128 steps of a batch, and after its
+// launch or active lattices have changed, are launched one by one (with graphs at once the first 64
+// steps took 44.5 against 39.2 ms).
+constexpr int kGroupSteps = 16;
+constexpr size_t kBlockGroups = 48;
+constexpr int kDirectSteps = 128;
+// Most sites of a group of the staged tiles (or one lattice): both buffers of the kChains groups
 // that run side by side (57 MB in FP32) stay in L2 over their steps. 64 steps of 512 lattices of
 // 64^2 to 512^2, sites / groups side by side: 2^18 / 3 39.4 ms, 2^18 / 2 45.8, 2^18 / 4 41.4, 0.7 2^18
 // / 3 40.4, 1.4 2^18 / 3 41.0, 2^19 / 2 40.4, 2^20 / 1 51.7; of 512 lattices of 128^2: 6.7, 6.8, 8.6,
@@ -44,10 +56,10 @@ struct BatchCommon {
     void *d_lats = nullptr;              // BatchLattice<T> table
     lbm::BatchItem *d_items = nullptr;
     int n_items = 0;
-    // Lattices that take their steps together (lb_batch_step): the direct launch (variant 7) has
+    // Lattices that take their steps together (lb_batch_step): the staged tiles (variant 8) have
     // groups that stay in L2, the ring variants one group of all items.
     struct Group {
-        lbm::BatchGroup lattices{};      // direct launch: the lattices, how many, most tiles of one
+        lbm::BatchGroup lattices{};      // staged tiles: the lattices, how many, most tiles of one
         int n = 0, max_tiles = 0;
     };
     std::vector<Group> groups;
@@ -69,7 +81,10 @@ struct BatchCommon {
     std::vector<unsigned char> active;   // lattices stepped by lb_batch_step
     std::vector<long long> lat_steps;    // steps taken by each lattice
     long long steps = 0;
-    cudaGraphExec_t graph[2] = {nullptr, nullptr};   // kGraphSteps steps from phase 0 / 1
+    // kGraphSteps steps of the one group, or kGroupSteps steps of each block of kBlockGroups groups,
+    // from phase 0 / 1
+    std::vector<cudaGraphExec_t> graphs[2];
+    int direct_steps = 0;                // launched one by one since the groups were formed
     lb_status sticky = LB_OK;
     std::string msg;
 };
@@ -181,7 +196,7 @@ lb_status make_chunks(lb_batch *b) {
     return LB_OK;
 }
 
-// The groups of the direct launch: active lattices by size (so that the lattices of a group have
+// The groups of the staged tiles: active lattices by size (so that the lattices of a group have
 // about as many tiles), each group of at most kGroupSites sites (or one lattice) and of at most
 // GROUP_LATTICES lattices. Returns the number of tiles.
 int make_groups(lb_batch *b) {
@@ -217,10 +232,32 @@ int make_groups(lb_batch *b) {
 }
 
 void drop_graphs(lb_batch *b) {
-    for (auto &g : b->graph) {
-        if (g) cudaGraphExecDestroy(g);
-        g = nullptr;
+    for (auto &v : b->graphs) {
+        for (cudaGraphExec_t g : v)
+            if (g) cudaGraphExecDestroy(g);
+        v.clear();
     }
+}
+
+// room for the graphs of the groups as they are now
+void renew_graphs(lb_batch *b) {
+    drop_graphs(b);
+    b->direct_steps = 0;
+    for (auto &v : b->graphs) v.assign((b->groups.size() + kBlockGroups - 1) / kBlockGroups, nullptr);
+}
+
+int graph_steps(const lb_batch *b) { return b->groups.size() > 1 ? kGroupSteps : kGraphSteps; }
+
+// The side streams of several groups.
+cudaError_t ensure_side(lb_batch *b) {
+    cudaError_t e = cudaSuccess;
+    if (!b->fork) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
+    for (int c = 0; c < kChains - 1 && e == cudaSuccess; ++c) {
+        if (!b->side[c]) e = cudaStreamCreateWithFlags(&b->side[c], cudaStreamNonBlocking);
+        if (e == cudaSuccess && !b->join[c])
+            e = cudaEventCreateWithFlags(&b->join[c], cudaEventDisableTiming);
+    }
+    return e;
 }
 
 // the tensor maps of every lattice's two buffers, for boxes of cols x rows x planes
@@ -263,7 +300,8 @@ lb_status apply_batch_launch(lb_batch *b, int variant, int rows) {
         b->rows = lbm::STAGED_ROWS;
         b->ctas_per_sm = 1;
         b->grid = b->groups.empty() ? 0 : b->groups[0].n * b->groups[0].max_tiles;
-        drop_graphs(b);
+        if (b->groups.size() > 1) LB_BCUDA(b, ensure_side(b));
+        renew_graphs(b);
         return LB_OK;
     }
     const int tx = lbm::step_variant_tx(variant);
@@ -285,7 +323,7 @@ lb_status apply_batch_launch(lb_batch *b, int variant, int rows) {
     const lb_status st = make_maps(b, tx + lbm::ghost_of_prec(b->prec) + 4, 1,
                                    lbm::step_variant_planes(variant));
     if (st != LB_OK) return st;
-    drop_graphs(b);
+    renew_graphs(b);
     return LB_OK;
 }
 
@@ -325,72 +363,76 @@ cudaError_t launch_group(const lb_batch *b, const BatchCommon::Group &g, int pha
                                   b->d_items, b->n_items, phase, b->d_errs, st);
 }
 
-// n steps of a batch of one group from phase `phase`, queued on st
-cudaError_t queue_steps(const lb_batch *b, int n, int phase, cudaStream_t st) {
+// n steps from phase `phase` of groups first .. last - 1, queued on `main`. Several groups: a group
+// takes all its steps before the next one (lattices are independent), so that its state stays in L2,
+// and kChains groups run side by side: one computes while another starts a launch or drains one.
+cudaError_t queue_groups(lb_batch *b, size_t first, size_t last, int n, int phase, cudaStream_t main) {
     cudaError_t e = cudaSuccess;
-    for (const auto &g : b->groups)
-        for (int i = 0; i < n && e == cudaSuccess; ++i) e = launch_group(b, g, phase ^ (i & 1), st);
-    return e;
-}
-
-// The side streams of several groups, made on first use.
-cudaError_t ensure_side(lb_batch *b) {
-    cudaError_t e = cudaSuccess;
-    if (!b->fork) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
-    for (int c = 0; c < kChains - 1 && e == cudaSuccess; ++c) {
-        if (!b->side[c]) e = cudaStreamCreateWithFlags(&b->side[c], cudaStreamNonBlocking);
-        if (e == cudaSuccess && !b->join[c])
-            e = cudaEventCreateWithFlags(&b->join[c], cudaEventDisableTiming);
+    if (last - first <= 1) {
+        for (int i = 0; i < n && first < last && e == cudaSuccess; ++i)
+            e = launch_group(b, b->groups[first], phase ^ (i & 1), main);
+        return e;
     }
-    return e;
-}
-
-// n steps of a batch of several groups: a group takes all its steps before the next one (lattices
-// are independent), so that its state stays in L2, and kChains groups run side by side: one
-// computes while another starts a launch or drains one.
-cudaError_t queue_groups(lb_batch *b, int n) {
-    cudaError_t e = ensure_side(b);
-    if (e == cudaSuccess) e = cudaEventRecord(b->fork, b->stream);
+    e = cudaEventRecord(b->fork, main);
     for (int c = 0; c < kChains - 1 && e == cudaSuccess; ++c)
         e = cudaStreamWaitEvent(b->side[c], b->fork, 0);
-    for (size_t k = 0; k < b->groups.size() && e == cudaSuccess; k += kChains)
+    for (size_t k = first; k < last && e == cudaSuccess; k += kChains)
         for (int i = 0; i < n && e == cudaSuccess; ++i)
-            for (size_t c = 0; c < kChains && k + c < b->groups.size() && e == cudaSuccess; ++c)
-                e = launch_group(b, b->groups[k + c], b->phase ^ (i & 1),
-                                 c == 0 ? b->stream : b->side[c - 1]);
+            for (size_t c = 0; c < kChains && k + c < last && e == cudaSuccess; ++c)
+                e = launch_group(b, b->groups[k + c], phase ^ (i & 1), c == 0 ? main : b->side[c - 1]);
     for (int c = 0; c < kChains - 1; ++c) {       // also after an error: nothing is left unjoined
         cudaError_t j = cudaEventRecord(b->join[c], b->side[c]);
-        if (j == cudaSuccess) j = cudaStreamWaitEvent(b->stream, b->join[c], 0);
+        if (j == cudaSuccess) j = cudaStreamWaitEvent(main, b->join[c], 0);
         if (e == cudaSuccess) e = j;
     }
     return e;
 }
 
 lb_status launch_steps(lb_batch *b, int n) {
-    LB_BCUDA(b, b->groups.size() > 1 ? queue_groups(b, n)
-                                     : queue_steps(b, n, b->phase, b->stream));
+    if (n > 0) LB_BCUDA(b, queue_groups(b, 0, b->groups.size(), n, b->phase, b->stream));
+    b->direct_steps = std::min(b->direct_steps + std::min(n, kDirectSteps), kDirectSteps);
     b->phase ^= n & 1;
     count_steps(b, n);
     return LB_OK;
 }
 
-lb_status ensure_graph(lb_batch *b, int phase) {
-    if (b->graph[phase]) return LB_OK;
+cudaError_t capture_graph(lb_batch *b, size_t first, size_t last, cudaGraphExec_t *exec) {
     cudaStream_t cap = nullptr;
-    LB_BCUDA(b, cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
     cudaGraph_t g = nullptr;
-    cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
+    cudaError_t e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
+    if (e != cudaSuccess) return e;
+    e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        e = queue_steps(b, kGraphSteps, phase, cap);
-        cudaError_t e2 = cudaStreamEndCapture(cap, &g);
+        e = queue_groups(b, first, last, graph_steps(b), b->phase, cap);
+        const cudaError_t e2 = cudaStreamEndCapture(cap, &g);
         if (e == cudaSuccess) e = e2;
     }
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&b->graph[phase], g, 0);
+    if (e == cudaSuccess) e = cudaGraphInstantiate(exec, g, 0);
     if (g) cudaGraphDestroy(g);
     cudaStreamDestroy(cap);
-    if (e != cudaSuccess)
-        return bfail(b, LB_ECUDA, std::string("graph capture: ") + cudaGetErrorString(e));
+    return e;
+}
+
+// graph_steps steps as graphs, captured when they are first launched: those of a block of groups
+// while the GPU takes the steps of the block before.
+lb_status launch_graphs(lb_batch *b) {
+    auto &graphs = b->graphs[b->phase];
+    for (size_t k = 0; k < graphs.size(); ++k) {
+        const size_t first = k * kBlockGroups;
+        if (!graphs[k])
+            LB_BCUDA(b, capture_graph(b, first, std::min(first + kBlockGroups, b->groups.size()), &graphs[k]));
+        LB_BCUDA(b, cudaGraphLaunch(graphs[k], b->stream));
+    }
+    count_steps(b, graph_steps(b));   // even: the phase is unchanged
     return LB_OK;
+}
+
+// a capture of the caller's takes the steps launch by launch (a graph launch cannot be captured)
+bool capturing(const lb_batch *b) {
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(b->stream, &s) == cudaSuccess) return s != cudaStreamCaptureStatusNone;
+    (void)cudaGetLastError();
+    return false;
 }
 
 // waits for the stream; h_errs then holds the lattices' error words
@@ -659,16 +701,17 @@ lb_status lb_batch_step(lb_batch *b, int n) {
     const lbm::NvtxRange nvtx_range("lb_batch_step");
     if (!b || n < 0) return LB_EINVAL;
     if (b->sticky != LB_OK) return b->sticky;
-    // several groups are launched one by one: a graph of all their steps would cost more to build
-    // (2 us a node) than the launches, which run ahead of the GPU
-    while (n >= kGraphSteps && b->groups.size() <= 1) {
-        if (b->n_items > 0) {
-            lb_status s = ensure_graph(b, b->phase);
+    if (n >= graph_steps(b) && !capturing(b)) {
+        if (b->groups.size() > 1 && b->direct_steps < kDirectSteps) {
+            const int m = std::min(n, kDirectSteps - b->direct_steps);
+            const lb_status s = launch_steps(b, m);
             if (s != LB_OK) return s;
-            LB_BCUDA(b, cudaGraphLaunch(b->graph[b->phase], b->stream));
+            n -= m;
         }
-        count_steps(b, kGraphSteps);   // even: the phase is unchanged
-        n -= kGraphSteps;
+        for (; n >= graph_steps(b); n -= graph_steps(b)) {
+            const lb_status s = launch_graphs(b);
+            if (s != LB_OK) return s;
+        }
     }
     return launch_steps(b, n);
 }

@@ -1,0 +1,96 @@
+"""Batches of several groups of lattices: their steps are queued as graphs once the first 128 have been
+launched one by one, and give the bits of the ring kernel's single launch per step over blocks of
+groups, from either buffer, after a change of the active lattices and inside a capture. The calling
+thread is not held while the GPU works."""
+import time
+
+import numpy as np
+import pytest
+
+from paper_1306_6445_gb300 import inputs as I
+from test_gpu_parity import lbm  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+def batch(lbm, sides, stream=None):  # noqa: F811
+    eos = lbm.cs_eos(0.8)
+    rv, rl, _ = lbm.lb_maxwell(eos, -1.0)
+    b = lbm.Batch([lbm.LatticeDesc(s, s + 1, eos, -1.0, kappa=0.3, sigma_force=0.05,
+                                   rates=lbm.RateParams.from_viscosity(0.1)) for s in sides], stream=stream)
+    for i, s in enumerate(sides):
+        b.set_rho_u(i, I.droplet_density(s, s + 1, 0.2 * s + 0.01 * i, rl, rv))
+    return b
+
+
+# 2 groups, 3, 4 (15 lattices each), 50 (the second block has two), 49 (the second block has one)
+@pytest.mark.parametrize("sides", [[256] * 2, [512, 511, 301], [128] * 60, [511] * 50, [512] * 49])
+def test_bits_of_single_launches(lbm, sides):  # noqa: F811
+    a, b = batch(lbm, sides), batch(lbm, sides)
+    b.set_launch(4, 16)
+    active = np.ones(len(sides), np.uint8)
+    pick = sorted({0, 1, len(sides) // 2, len(sides) - 1})
+
+    def same():
+        for i in pick:
+            assert np.array_equal(a.populations(i), b.populations(i)), i
+        assert a.steps_done == b.steps_done
+
+    for x in (a, b):
+        x.step(100)                # one by one
+        x.step(60)                 # the last of these, then graphs
+        x.step(16)
+    same()
+    for x in (a, b):
+        x.step(1)                  # from the other buffer
+        x.step(35)
+    same()
+    active[0] = 0
+    for x in (a, b):
+        x.set_active(active)
+        x.step(129 + 33)
+    same()
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("warm", [False, True])
+def test_captured_steps(lbm, warm):  # noqa: F811
+    """recorded by the caller, before and after the batch has graphs of its own"""
+    st = torch.cuda.Stream()
+    sides = [512, 511, 301]
+    a, b = batch(lbm, sides, st.cuda_stream), batch(lbm, sides)
+    if warm:
+        a.step(192)
+        b.step(192)
+    a.sync()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=st):
+        a.step(34)
+    with torch.cuda.stream(st):
+        for _ in range(2):
+            graph.replay()
+    a.sync()
+    b.step(68)
+    for i in range(3):
+        assert np.array_equal(a.populations(i), b.populations(i))
+    a.close()
+    b.close()
+
+
+def test_the_calling_thread_is_not_held(lbm):  # noqa: F811
+    b = batch(lbm, [128] * 60)
+    b.step(128)
+    b.step(16)                     # the graphs are made
+    held, whole = [], []
+    for _ in range(5):
+        b.sync()
+        t = time.perf_counter()
+        b.step(640)
+        held.append(time.perf_counter() - t)
+        b.sync()
+        whole.append(time.perf_counter() - t)
+    assert sorted(held)[2] < 0.5 * sorted(whole)[2], (held, whole)
+    b.close()
