@@ -248,12 +248,19 @@ void renew_graphs(lb_batch *b) {
 
 int graph_steps(const lb_batch *b) { return b->groups.size() > 1 ? kGroupSteps : kGraphSteps; }
 
+// A stream beside the batch's, with its priority (launches recorded into a graph keep it).
+cudaError_t side_stream(const lb_batch *b, cudaStream_t *st) {
+    int priority = 0;
+    const cudaError_t e = cudaStreamGetPriority(b->stream, &priority);
+    return e != cudaSuccess ? e : cudaStreamCreateWithPriority(st, cudaStreamNonBlocking, priority);
+}
+
 // The side streams of several groups.
 cudaError_t ensure_side(lb_batch *b) {
     cudaError_t e = cudaSuccess;
     if (!b->fork) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
     for (int c = 0; c < kChains - 1 && e == cudaSuccess; ++c) {
-        if (!b->side[c]) e = cudaStreamCreateWithFlags(&b->side[c], cudaStreamNonBlocking);
+        if (!b->side[c]) e = side_stream(b, &b->side[c]);
         if (e == cudaSuccess && !b->join[c])
             e = cudaEventCreateWithFlags(&b->join[c], cudaEventDisableTiming);
     }
@@ -399,7 +406,7 @@ lb_status launch_steps(lb_batch *b, int n) {
 cudaError_t capture_graph(lb_batch *b, size_t first, size_t last, cudaGraphExec_t *exec) {
     cudaStream_t cap = nullptr;
     cudaGraph_t g = nullptr;
-    cudaError_t e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
+    cudaError_t e = side_stream(b, &cap);
     if (e != cudaSuccess) return e;
     e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {

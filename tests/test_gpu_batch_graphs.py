@@ -7,6 +7,7 @@ import time
 import numpy as np
 import pytest
 
+import _capture
 from paper_1306_6445_gb300 import inputs as I
 from test_gpu_parity import lbm  # noqa: F401
 
@@ -93,4 +94,17 @@ def test_the_calling_thread_is_not_held(lbm):  # noqa: F811
         b.sync()
         whole.append(time.perf_counter() - t)
     assert sorted(held)[2] < 0.5 * sorted(whole)[2], (held, whole)
+    b.close()
+
+
+def test_every_group_has_the_priority_of_the_stream(lbm):  # noqa: F811
+    st = torch.cuda.Stream(priority=-1)
+    assert st.priority < 0
+    b = batch(lbm, [512, 511, 301], st.cuda_stream)
+    b.sync()
+    _capture.begin(st.cuda_stream)
+    b.step(2)
+    graph = _capture.end(st.cuda_stream)
+    assert _capture.kernel_priorities(graph) == [st.priority] * 6
+    _capture.destroy(graph)
     b.close()
