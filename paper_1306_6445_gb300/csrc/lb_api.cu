@@ -53,7 +53,7 @@ constexpr int kManySteps = 1024;      // of one launch of the cluster or the res
 
 lb_status fail(lb_ctx *c, lb_status s, const std::string &m) {
     if (c) c->msg = m;
-    return s;
+    return lbm::reported(s);
 }
 
 lb_status poison(lb_ctx *c, lb_status s, const std::string &m) {
@@ -64,8 +64,7 @@ lb_status poison(lb_ctx *c, lb_status s, const std::string &m) {
 
 lb_status cuda_fail(lb_ctx *c, cudaError_t e, const char *where) {
     std::string m = std::string(where) + ": " + cudaGetErrorString(e);
-    if (c) c->msg = m;
-    return LB_ECUDA;
+    return fail(c, LB_ECUDA, m);
 }
 
 #define LB_CUDA(ctx, call)                                        \
@@ -336,7 +335,7 @@ lb_status create(lb_ctx **out, int nx, int ny, const lb_eos *eos, double G, doub
     if (e != cudaSuccess) {
         std::fprintf(stderr, "lb_init: %s\n", cudaGetErrorString(e));
         delete c;
-        return LB_ECUDA;
+        return lbm::reported(LB_ECUDA);
     }
     const size_t bytes = lb_buffer_bytes(nx, ny, prec);
     if (external) {
@@ -347,7 +346,7 @@ lb_status create(lb_ctx **out, int nx, int ny, const lb_eos *eos, double G, doub
         c->own_f = true;
         if (cudaMalloc(&c->f[0], bytes) != cudaSuccess || cudaMalloc(&c->f[1], bytes) != cudaSuccess) {
             lb_free(c);
-            return LB_ENOMEM;
+            return lbm::reported(LB_ENOMEM);
         }
     }
     lbm::HostWords *dev_words = nullptr;
@@ -355,7 +354,7 @@ lb_status create(lb_ctx **out, int nx, int ny, const lb_eos *eos, double G, doub
         cudaHostAlloc(&c->words, sizeof(lbm::HostWords), cudaHostAllocMapped) != cudaSuccess ||
         cudaHostGetDevicePointer(&dev_words, c->words, 0) != cudaSuccess) {
         lb_free(c);
-        return LB_ENOMEM;
+        return lbm::reported(LB_ENOMEM);
     }
     std::memset(c->words, 0, sizeof(lbm::HostWords));
     c->d_err = &dev_words->err;
@@ -365,12 +364,12 @@ lb_status create(lb_ctx **out, int nx, int ny, const lb_eos *eos, double G, doub
         cudaMemsetAsync(c->f[1], 0, bytes, c->stream) != cudaSuccess ||
         cudaStreamSynchronize(c->stream) != cudaSuccess) {
         lb_free(c);
-        return LB_ECUDA;
+        return lbm::reported(LB_ECUDA);
     }
     if ((s = apply_launch(c, lbm::default_variant(prec, c->geom), 0)) != LB_OK) {
         std::fprintf(stderr, "lb_init: %s\n", c->msg.c_str());
         lb_free(c);
-        return s;
+        return lbm::reported(s);
     }
     *out = c;
     return LB_OK;
@@ -395,7 +394,7 @@ lb_status ctx_fail(lb_ctx *c, lb_status s, const char *msg, bool poison_ctx) {
     if (!c) return s;
     c->msg = msg ? msg : "";
     if (poison_ctx) c->sticky = s;
-    return s;
+    return reported(s);
 }
 
 lb_status ctx_sync_check(lb_ctx *c) {

@@ -100,7 +100,7 @@ lb_status bfail(lb_batch *b, lb_status s, const std::string &m, bool poison = fa
         b->msg = m;
         if (poison) b->sticky = s;
     }
-    return s;
+    return lbm::reported(s);
 }
 
 #define LB_BCUDA(b, call)                                                            \
@@ -565,7 +565,7 @@ lb_status lb_batch_create(lb_batch **out, int n, const lb_lattice_desc *descs, i
         cudaMemset(b->pool, 0, total) != cudaSuccess ||
         cudaMemset(b->d_errs, 0, n * sizeof(int)) != cudaSuccess) {
         lb_batch_free(b);
-        return LB_ENOMEM;
+        return lbm::reported(LB_ENOMEM);
     }
     // one page-locked block: each allocation of one costs about 0.15 ms
     b->h_radius = b->h_meas + 8 * (size_t)n;
@@ -574,14 +574,14 @@ lb_status lb_batch_create(lb_batch **out, int n, const lb_lattice_desc *descs, i
     b->lat_steps.assign(n, 0);
     if ((s = make_chunks(b)) != LB_OK) {
         lb_batch_free(b);
-        return s;
+        return lbm::reported(s);
     }
     s = prec == LB_FP32 ? upload_lattices<float>(b) : upload_lattices<double>(b);
     if (s == LB_OK) s = apply_batch_launch(b, lbm::staged_variant(), 16);
     if (s != LB_OK) {
         std::fprintf(stderr, "lb_batch_create: %s\n", b->msg.c_str());
         lb_batch_free(b);
-        return s;
+        return lbm::reported(s);
     }
     *out = b;
     return LB_OK;

@@ -22,6 +22,13 @@ struct NvtxRange {
     NvtxRange &operator=(const NvtxRange &) = delete;
 };
 
+// An error that a call returns is reported: it does not stay behind as the runtime's last error, which
+// the next launch of this host thread, of any context, would take for its own.
+inline lb_status reported(lb_status s) {
+    if (s == LB_ECUDA || s == LB_ENOMEM) (void)cudaGetLastError();
+    return s;
+}
+
 // Error bits written by kernels into the context's device flag word.
 enum : int { ERR_DOMAIN = 1, ERR_TIMEOUT = 2 };
 

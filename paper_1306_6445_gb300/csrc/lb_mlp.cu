@@ -768,7 +768,7 @@ namespace {
 
 lb_status mfail(lb_mlp *m, lb_status s, const std::string &msg) {
     if (m) m->msg = msg;
-    return s;
+    return lbm::reported(s);
 }
 
 #define LB_MCUDA(m, call)                                                              \

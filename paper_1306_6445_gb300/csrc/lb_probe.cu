@@ -3,7 +3,7 @@
 // its 144 bytes of population traffic on a GPU with a reduced FP64 rate.
 #include <cuda_runtime.h>
 
-#include "lb.h"
+#include "lb_internal.h"
 
 namespace {
 
@@ -38,10 +38,10 @@ extern "C" lb_status lb_probe_fp64_fma_rate(void *cuda_stream, int iters, double
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return LB_ECUDA;
+        return lbm::reported(LB_ECUDA);
     const int blocks = sms * PROBE_BLOCKS_PER_SM;
     double *out = nullptr;
-    if (cudaMalloc(&out, sizeof(double) * blocks) != cudaSuccess) return LB_ENOMEM;
+    if (cudaMalloc(&out, sizeof(double) * blocks) != cudaSuccess) return lbm::reported(LB_ENOMEM);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaError_t e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
@@ -63,7 +63,7 @@ extern "C" lb_status lb_probe_fp64_fma_rate(void *cuda_stream, int iters, double
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     cudaFree(out);
-    if (e != cudaSuccess || !(ms > 0.f)) return LB_ECUDA;
+    if (e != cudaSuccess || !(ms > 0.f)) return lbm::reported(LB_ECUDA);
     *fma_per_s = (double)blocks * PROBE_THREADS * PROBE_CHAINS * (double)iters / (ms * 1e-3);
     return LB_OK;
 }
