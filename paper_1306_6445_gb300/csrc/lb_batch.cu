@@ -85,6 +85,7 @@ struct BatchCommon {
     // from phase 0 / 1
     std::vector<cudaGraphExec_t> graphs[2];
     int direct_steps = 0;                // launched one by one since the groups were formed
+    long long queued = 0;                // launches of steps, also of graphs of them
     lb_status sticky = LB_OK;
     std::string msg;
 };
@@ -362,12 +363,15 @@ void count_steps(lb_batch *b, int n) {
         if (b->active[i]) b->lat_steps[i] += n;
 }
 
-cudaError_t launch_group(const lb_batch *b, const BatchCommon::Group &g, int phase, cudaStream_t st) {
-    if (b->variant == lbm::staged_variant())
-        return lbm::batch_tile_f32(b->eos_kind, g.lattices, g.n, g.max_tiles, b->d_maps, b->d_lats,
-                                   phase, b->d_errs, st);
-    return lbm::launch_batch_step(b->prec, b->eos_kind, b->variant, b->grid, b->d_maps, b->d_lats,
-                                  b->d_items, b->n_items, phase, b->d_errs, st);
+cudaError_t launch_group(lb_batch *b, const BatchCommon::Group &g, int phase, cudaStream_t st) {
+    const cudaError_t e =
+        b->variant == lbm::staged_variant()
+            ? lbm::batch_tile_f32(b->eos_kind, g.lattices, g.n, g.max_tiles, b->d_maps, b->d_lats, phase,
+                                  b->d_errs, st)
+            : lbm::launch_batch_step(b->prec, b->eos_kind, b->variant, b->grid, b->d_maps, b->d_lats,
+                                     b->d_items, b->n_items, phase, b->d_errs, st);
+    if (e == cudaSuccess) ++b->queued;
+    return e;
 }
 
 // n steps from phase `phase` of groups first .. last - 1, queued on `main`. Several groups: a group
@@ -410,7 +414,9 @@ cudaError_t capture_graph(lb_batch *b, size_t first, size_t last, cudaGraphExec_
     if (e != cudaSuccess) return e;
     e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
+        const long long queued = b->queued;
         e = queue_groups(b, first, last, graph_steps(b), b->phase, cap);
+        b->queued = queued;              // recorded only
         const cudaError_t e2 = cudaStreamEndCapture(cap, &g);
         if (e == cudaSuccess) e = e2;
     }
@@ -429,6 +435,7 @@ lb_status launch_graphs(lb_batch *b) {
         if (!graphs[k])
             LB_BCUDA(b, capture_graph(b, first, std::min(first + kBlockGroups, b->groups.size()), &graphs[k]));
         LB_BCUDA(b, cudaGraphLaunch(graphs[k], b->stream));
+        ++b->queued;
     }
     count_steps(b, graph_steps(b));   // even: the phase is unchanged
     return LB_OK;
@@ -440,6 +447,22 @@ bool capturing(const lb_batch *b) {
     if (cudaStreamIsCapturing(b->stream, &s) == cudaSuccess) return s != cudaStreamCaptureStatusNone;
     (void)cudaGetLastError();
     return false;
+}
+
+lb_status take_steps(lb_batch *b, int n) {
+    if (n >= graph_steps(b) && !capturing(b)) {
+        if (b->groups.size() > 1 && b->direct_steps < kDirectSteps) {
+            const int m = std::min(n, kDirectSteps - b->direct_steps);
+            const lb_status s = launch_steps(b, m);
+            if (s != LB_OK) return s;
+            n -= m;
+        }
+        for (; n >= graph_steps(b); n -= graph_steps(b)) {
+            const lb_status s = launch_graphs(b);
+            if (s != LB_OK) return s;
+        }
+    }
+    return launch_steps(b, n);
 }
 
 // waits for the stream; h_errs then holds the lattices' error words
@@ -708,19 +731,11 @@ lb_status lb_batch_step(lb_batch *b, int n) {
     const lbm::NvtxRange nvtx_range("lb_batch_step");
     if (!b || n < 0) return LB_EINVAL;
     if (b->sticky != LB_OK) return b->sticky;
-    if (n >= graph_steps(b) && !capturing(b)) {
-        if (b->groups.size() > 1 && b->direct_steps < kDirectSteps) {
-            const int m = std::min(n, kDirectSteps - b->direct_steps);
-            const lb_status s = launch_steps(b, m);
-            if (s != LB_OK) return s;
-            n -= m;
-        }
-        for (; n >= graph_steps(b); n -= graph_steps(b)) {
-            const lb_status s = launch_graphs(b);
-            if (s != LB_OK) return s;
-        }
-    }
-    return launch_steps(b, n);
+    const long long queued = b->queued;
+    const lb_status s = take_steps(b, n);
+    // some lattices have gone on and others not: nothing can be made of the batch any more
+    if (s != LB_OK && b->queued != queued) b->sticky = s;
+    return s;
 }
 
 lb_status lb_batch_sync(lb_batch *b) {

@@ -2,6 +2,7 @@
 launched one by one, and give the bits of the ring kernel's single launch per step over blocks of
 groups, from either buffer, after a change of the active lattices and inside a capture. The calling
 thread is not held while the GPU works."""
+import threading
 import time
 
 import numpy as np
@@ -107,4 +108,40 @@ def test_every_group_has_the_priority_of_the_stream(lbm):  # noqa: F811
     graph = _capture.end(st.cuda_stream)
     assert _capture.kernel_priorities(graph) == [st.priority] * 6
     _capture.destroy(graph)
+    b.close()
+
+
+@pytest.mark.parametrize("variant,partly", [(8, False), (8, True), (4, True)])
+def test_steps_that_fail(lbm, variant, partly):  # noqa: F811
+    """A capture that is spoilt while the steps are being recorded: some lattices have moved on and
+    others not, so the batch refuses everything afterwards. Spoilt before, nothing has happened."""
+    st = torch.cuda.Stream()
+    b = batch(lbm, [512, 511, 301], st.cuda_stream)
+    b.set_launch(variant, 16)
+    b.sync()
+    _capture.begin(st.cuda_stream)
+
+    def spoil():                   # waiting for a stream that is being captured
+        if partly:
+            time.sleep(0.01)
+        st.synchronize()
+
+    t = threading.Thread(target=lambda: pytest.raises(RuntimeError, spoil))
+    t.start()
+    if not partly:
+        t.join()
+    with pytest.raises(lbm.LBError) as e:
+        b.step(100000)             # far longer than the wait
+    assert e.value.status == lbm.LB_ECUDA
+    t.join()
+    assert _capture.end(st.cuda_stream) is None
+    if partly:
+        for call in (lambda: b.step(1), b.sync, lambda: b.measure([50.0] * 3), lambda: b.populations(0)):
+            with pytest.raises(lbm.LBError) as e:
+                call()
+            assert e.value.status == lbm.LB_ECUDA
+    else:
+        b.step(2)
+        b.sync()
+        assert b.steps_done == 2
     b.close()
