@@ -141,7 +141,7 @@ lb_status lb_init_ex(lb_ctx **out, int nx, int ny, const lb_eos *eos, double G, 
  * pairs per 1/16 of the rows), of one CTA per SM from 32768 sites on as long as tiles of 64
  * columns and at most 35 rows suffice (a cooperative launch, between 96 tiles and one per SM, the last of
  * a row at least two columns wide; an exchange buffer is allocated by the library, without it the
- * steps are single launches). lb_autotune keeps the variant of these. LB_FP32 batches have
+ * steps are single launches); also after lb_autotune, whatever variant it chose for single steps. LB_FP32 batches have
  * variants 0-6 and 8 (7 is taken as 8) and start with 8, LB_FP64 batches 0-6 (7 and 8 are taken
  * as 4) and start with 4. */
 int lb_launch_variants(void);
@@ -178,7 +178,8 @@ lb_status lb_set_launch(lb_ctx *ctx, int variant, int rows);
 
 /* Autotuner: time every compiled variant with rows per CTA from {default, 6, 8, 9, 10,
  * 11, 12, 13, 14, 15, 16, 20, 24} (at most ny; variants 7 and 8 once) on this lattice and keep the
- * fastest. Each
+ * fastest; lattices that take several steps in one launch (see lb_launch_variants) have their
+ * single steps timed with variants 7 and 8. Each
  * candidate runs one untimed launch and then three timed runs of `trial_steps` >= 1
  * launches (its time is the fastest run). The trial launches take real steps on a scratch
  * copy of the state (a temporary device buffer of lb_buffer_bytes, freed before return),

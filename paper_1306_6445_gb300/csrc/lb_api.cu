@@ -38,6 +38,7 @@ struct lb_ctx {
     void *d_psi = nullptr;       // FP64 direct kernels: psi of the step, ny * pitch elements
     lbm::StepLaunch launch{};
     int asked_variant = 0, asked_rows = 0;   // what apply_launch was last asked for
+    bool asked_many = false;
     int many = 0;                // several steps at once: 1 the cluster kernel, 2 the resident one
     void *d_words = nullptr;     // exchange words of the resident kernel
     long long steps = 0;
@@ -244,17 +245,19 @@ int many_usable(lb_ctx *c) {
     return 0;
 }
 
-lb_status apply_launch(lb_ctx *c, int variant, int rows) {
+// any_many: several steps go together with any variant, not only with the one that contexts start with
+lb_status apply_launch(lb_ctx *c, int variant, int rows, bool any_many = false) {
     if (variant < 0 || variant >= lbm::step_variant_count())
         return fail(c, LB_EINVAL, "unknown launch variant");
     if (rows < 0) return fail(c, LB_EINVAL, "rows must be >= 0");
     c->asked_variant = variant;
     c->asked_rows = rows;
+    c->asked_many = any_many;
     if (variant >= lbm::direct_variant()) {
         if (c->prec == LB_FP64) variant = lbm::direct_variant();     // no staged FP64 kernel
         if (!direct_usable(c)) variant = lbm::default_ring_variant();
     }
-    c->many = variant == lbm::default_variant(c->prec, c->geom) ? many_usable(c) : 0;
+    c->many = any_many || variant == lbm::default_variant(c->prec, c->geom) ? many_usable(c) : 0;
     const int stall = c->consts.stall_row;
     if (stall != INT_MIN) {      // test hook: kernels that wait for the row
         if (c->many == 1 || !lbm::resident_waits_for_row(c->geom, stall)) c->many = 0;
@@ -446,13 +449,9 @@ lb_status lb_autotune(lb_ctx *c, int trial_steps, int *variant, int *rows) {
     if (trial_steps < 1) return fail(c, LB_EINVAL, "lb_autotune: trial_steps < 1");
     // device errors of earlier steps are the state's: report them before any trial
     if ((s = sync_and_check(c)) != LB_OK) return s;
-    if (many_usable(c)) {
-        // launches of many steps beat all that could be tried here
-        if ((s = apply_launch(c, lbm::default_variant(c->prec, c->geom), 0)) != LB_OK) return s;
-        if (variant) *variant = c->launch.variant;
-        if (rows) *rows = c->launch.rows;
-        return LB_OK;
-    }
+    // Launches of many steps beat all that could be tried here: what is chosen is the launch of single
+    // steps, between the two tile kernels (the ring kernels take twice their time and more at these sizes).
+    const bool many = many_usable(c) != 0;
     static const int cand[] = {0, 6, 8, 9, 10, 11, 12, 13, 14, 15, 16, 20, 24};
     // Trial launches take real steps on a scratch copy of the state, ping-ponging with the
     // spare buffer as lb_step does (each launch reads what the previous one wrote, in the
@@ -482,6 +481,7 @@ lb_status lb_autotune(lb_ctx *c, int trial_steps, int *variant, int *rows) {
     for (int v = 0; v < lbm::step_variant_count() && e == cudaSuccess; ++v) {
         int tried_rows[16], n_tried = 0;
         const bool direct = v >= lbm::direct_variant();
+        if (many && !direct) continue;
         if (direct && !direct_usable(c)) continue;
         if (v == lbm::staged_variant() && c->prec == LB_FP64) continue;
         for (int r : cand) {
@@ -544,7 +544,7 @@ lb_status lb_autotune(lb_ctx *c, int trial_steps, int *variant, int *rows) {
     if (c->words->err & lbm::ERR_TIMEOUT)       // (the stream has been waited for)
         return poison(c, LB_ETIMEOUT, "a bounded device-side wait gave up");
     c->words->err = 0;
-    if ((s = apply_launch(c, best_v, best_r)) != LB_OK) return s;
+    if ((s = apply_launch(c, best_v, best_r, many)) != LB_OK) return s;
     if (variant) *variant = best_v;
     if (rows) *rows = best_r;
     return sync_and_check(c);
@@ -588,7 +588,7 @@ lb_status lb_debug_stall_row(lb_ctx *c, int row) {
     lb_status s = check_usable(c);
     if (s != LB_OK) return s;
     c->consts.stall_row = row;
-    return apply_launch(c, c->asked_variant, c->asked_rows);
+    return apply_launch(c, c->asked_variant, c->asked_rows, c->asked_many);
 }
 
 lb_status lb_get_launch(const lb_ctx *c, int *variant, int *tx, int *rows, int *ctas_per_sm) {

@@ -1,6 +1,7 @@
 """Which lattices take several steps in one launch (the cluster kernel and the resident one), as counted
 by lb_step_launches, and what a launch that cannot be made does to the context."""
 import threading
+import time
 
 import numpy as np
 import pytest
@@ -111,3 +112,24 @@ def test_lattices_of_different_size_step_side_by_side(lbm, sizes):  # noqa: F811
     assert [lbm.lb_step_launches(lat.ctx) - b for lat, b in zip(lats, before)] == [calls, calls]
     for lat in lats:
         lat.close()
+
+
+@pytest.mark.parametrize("nx,ny,bc", [(64, 64, "walls"), (200, 200, "periodic"), (600, 225, "open")])
+def test_autotuning(lbm, nx, ny, bc):  # noqa: F811
+    """The launch of single steps is chosen by trials (each takes a microsecond a step at the very
+    least), also where many steps go together, which they do afterwards whatever was chosen."""
+    lat = lattice(lbm, nx, ny, bc)
+    lbm.lb_set_launch(lat.ctx, 4, 0)
+    lat.step(2)
+    before = lat.populations()
+    t = time.perf_counter()
+    variant, _ = lat.autotune(3000)
+    assert time.perf_counter() - t > 2 * 3 * 3000 * 1e-6
+    assert variant in (7, 8) and lbm.lb_get_launch(lat.ctx)["variant"] == variant
+    assert np.array_equal(lat.populations(), before) and lat.steps_done == 2
+    assert launches(lbm, lat, 1) == 1 and launches(lbm, lat, STEPS) == 1
+    lbm.lb_debug_stall_row(lat.ctx, 3)      # (a test hook that renews the launch)
+    lbm.lb_debug_stall_row(lat.ctx, -2**31)
+    assert launches(lbm, lat, STEPS) == 1
+    lat.sync()
+    lat.close()
