@@ -596,7 +596,10 @@ lb_status lb_get_launch(const lb_ctx *c, int *variant, int *tx, int *rows, int *
     if (variant) *variant = c->launch.variant;
     if (tx) *tx = c->launch.tx;
     if (rows) *rows = c->launch.rows;
-    if (ctas_per_sm) *ctas_per_sm = c->launch.ctas_per_sm;
+    if (ctas_per_sm)
+        *ctas_per_sm = c->launch.variant >= lbm::direct_variant()
+                           ? lbm::tile_occupancy(c->prec, c->consts, c->geom, c->launch.variant)
+                           : c->launch.ctas_per_sm;
     return LB_OK;
 }
 

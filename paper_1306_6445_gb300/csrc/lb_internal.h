@@ -107,7 +107,8 @@ struct StepLaunch {
     int variant;        // compiled (strip width, ring depth) choice, see step_variant_tx
     int tx;             // lattice columns per CTA (two per thread)
     int rows;           // rows each CTA marches over
-    int ctas_per_sm;    // resident CTAs per SM reported by the occupancy calculator
+    int ctas_per_sm;    // resident CTAs per SM reported by the occupancy calculator (ring variants; the
+                        // others' rows do not depend on it, see tile_occupancy)
 };
 
 // ---- kernels (lb_kernels.cu) -------------------------------------------------------
@@ -165,9 +166,9 @@ LB_DECLARE_BATCH_UNIT(f64, 1)
 #undef LB_DECLARE_BATCH_UNIT
 
 // direct step units (lb_split_f64.cu, lb_batch_tile.cu; lb_tile_f32.cu and lb_tile_bf16.cu below);
-// psi: ny * pitch elements
-cudaError_t split_f64(const Consts &c, const Geom &g, const void *gin, void *psi, void *gout,
-                      int *err, cudaStream_t st);
+// StepBuffers::psi: ny * pitch elements
+struct StepBuffers;
+cudaError_t split_f64(const Consts &c, const Geom &g, const StepBuffers &b, int *err, cudaStream_t st);
 
 // n lattices of a group, at most max_tiles tiles each
 cudaError_t batch_tile_f32(int eos, const BatchGroup &group, int n, int max_tiles, const void *maps,
@@ -185,13 +186,16 @@ cudaError_t launch_cluster_steps(const Consts &c, const Geom &g, const void *gin
                                  int n_steps, int *err, cudaStream_t st);
 
 // What a step reads and writes: the input buffer and its tensor map (none for the direct FP64
-// kernels), the output buffer, and psi scratch (direct FP64 kernels only).
+// kernels), the output buffer, and psi scratch (direct FP64 kernels only). occ (variants 7 and 8): not
+// launched, the smallest of *occ and the kernels' resident CTAs per SM goes there.
 struct StepBuffers {
     const void *gin;
     const void *tensor_map_in;
     void *gout;
     void *psi;
+    int *occ = nullptr;
 };
+int tile_occupancy(int prec, const Consts &c, const Geom &g, int variant);   // of variants 7 and 8
 cudaError_t tile_f32(const Consts &c, const Geom &g, int variant, int order,
                      const StepBuffers &b, int *err, cudaStream_t st);
 cudaError_t tile_bf16(const Consts &c, const Geom &g, int variant, int order,

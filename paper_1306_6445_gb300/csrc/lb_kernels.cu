@@ -394,7 +394,7 @@ StepLaunch make_step_launch(int prec, int eos_kind, const Geom &g, int num_sms, 
         // its grid is fixed by the lattice: rows_override does not apply
         l.rows = prec == LB_FP64 ? 1
                : std::min(variant == staged_variant() ? STAGED_ROWS : DIRECT_ROWS, g.ny);
-        l.ctas_per_sm = prec == LB_FP64 ? 2048 / DIRECT_COLS : 65536 / (32 * DIRECT_ROWS * 80);
+        l.ctas_per_sm = 0;
         return l;
     }
     const bool st = step_variant_kind(variant) == 1;
@@ -439,10 +439,21 @@ cudaError_t configure_step(int prec, const Consts &c, const Geom &g, const StepL
 cudaError_t launch_step(int prec, const Consts &c, const Geom &g, const StepLaunch &l, int order,
                         const StepBuffers &b, int *err, cudaStream_t st) {
     if (l.variant >= direct_variant()) {
-        if (prec == LB_FP64) return split_f64(c, g, b.gin, b.psi, b.gout, err, st);
+        if (prec == LB_FP64) return split_f64(c, g, b, err, st);
         return (prec == LB_FP32 ? tile_f32 : tile_bf16)(c, g, l.variant, order, b, err, st);
     }
     return launch_step_unit(prec, c, g, l, order, b.tensor_map_in, b.gout, err, st, false);
+}
+
+int tile_occupancy(int prec, const Consts &c, const Geom &g, int variant) {
+    static const CUtensorMap dummy{};
+    StepLaunch l{};
+    l.variant = variant;
+    int occ = INT_MAX;
+    const StepBuffers b{nullptr, &dummy, nullptr, nullptr, &occ};
+    if (launch_step(prec, c, g, l, 0, b, nullptr, nullptr) == cudaSuccess) return occ;
+    (void)cudaGetLastError();
+    return 0;
 }
 
 cudaError_t launch_unstream(int prec, const Geom &g, const void *f, void *gbuf, bool packed,

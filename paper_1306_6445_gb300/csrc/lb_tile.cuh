@@ -4,6 +4,7 @@
 // layout, arithmetic and results, bit for bit, as the ring kernels of lb_step.cuh.
 #pragma once
 
+#include <algorithm>
 #include <climits>
 
 #include "lb_step.cuh"
@@ -555,6 +556,16 @@ cudaError_t launch_dependent(K kern, dim3 grid, dim3 block, cudaStream_t st, Arg
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
+// a step's launch, or the kernel's resident CTAs per SM (StepBuffers::occ)
+template <typename K, typename... Args>
+cudaError_t launch_or_count(const StepBuffers &b, K kern, dim3 grid, dim3 block, cudaStream_t st, Args... args) {
+    if (!b.occ) return launch_dependent(kern, grid, block, st, args...);
+    int n = 0;
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, (int)block.x, 0);
+    *b.occ = std::min(*b.occ, n);
+    return e;
+}
+
 template <typename T, int EOS, int BC>
 cudaError_t tile_launch(const Consts &c, const Geom &g, int variant, int order,
                         const StepBuffers &b, int *err, cudaStream_t st) {
@@ -568,17 +579,17 @@ cudaError_t tile_launch(const Consts &c, const Geom &g, int variant, int order,
         if constexpr (BF) {
             if (c.stochastic) kern = k_tile_step<T, EOS, BC, R, true>;
         }
-        return launch_dependent(kern, dim3(tx, (g.ny + R - 1) / R), dim3(32 * R), st, gin, gout, to_dev<Arith<T>>(c),
-                                g.nx, g.ny, g.pitch, (unsigned)g.plane, order, err);
+        return launch_or_count(b, kern, dim3(tx, (g.ny + R - 1) / R), dim3(32 * R), st, gin, gout, to_dev<Arith<T>>(c),
+                               g.nx, g.ny, g.pitch, (unsigned)g.plane, order, err);
     }
     constexpr int R = STAGED_ROWS;
     auto kern = k_staged_tile_step<T, EOS, BC, R, false>;
     if constexpr (BF) {
         if (c.stochastic) kern = k_staged_tile_step<T, EOS, BC, R, true>;
     }
-    return launch_dependent(kern, dim3(tx, (g.ny + R - 1) / R), dim3(32 * R), st,
-                            *static_cast<const CUtensorMap *>(b.tensor_map_in), gin, gout,
-                            to_dev<Arith<T>>(c), g.nx, g.ny, g.pitch, (unsigned)g.plane, order, err);
+    return launch_or_count(b, kern, dim3(tx, (g.ny + R - 1) / R), dim3(32 * R), st,
+                           *static_cast<const CUtensorMap *>(b.tensor_map_in), gin, gout,
+                           to_dev<Arith<T>>(c), g.nx, g.ny, g.pitch, (unsigned)g.plane, order, err);
 }
 
 template <typename T, int EOS>
@@ -618,26 +629,24 @@ cudaError_t batch_tile_dispatch(int eos, const BatchGroup &group, int n, int max
 }
 
 template <typename T, int EOS, int BC>
-cudaError_t split_launch(const Consts &c, const Geom &g, const void *gin, void *psi, void *gout,
-                         int *err, cudaStream_t st) {
+cudaError_t split_launch(const Consts &c, const Geom &g, const StepBuffers &b, int *err, cudaStream_t st) {
     const dim3 grid((g.nx + SPLIT_THREADS - 1) / SPLIT_THREADS, g.ny);
     const DevConsts<T> P = to_dev<T>(c);
-    cudaError_t e = launch_dependent(k_psi_site<T, EOS, BC>, grid, dim3(SPLIT_THREADS), st,
-                                     static_cast<const T *>(gin), static_cast<T *>(psi), P, g.nx,
-                                     g.ny, g.pitch, (unsigned)g.plane, err);
+    const T *gin = static_cast<const T *>(b.gin);
+    T *psi = static_cast<T *>(b.psi), *gout = static_cast<T *>(b.gout);
+    cudaError_t e = launch_or_count(b, k_psi_site<T, EOS, BC>, grid, dim3(SPLIT_THREADS), st, gin, psi, P, g.nx,
+                                    g.ny, g.pitch, (unsigned)g.plane, err);
     if (e != cudaSuccess) return e;
-    return launch_dependent(k_collide_site<T, BC>, grid, dim3(SPLIT_THREADS), st,
-                            static_cast<const T *>(gin), static_cast<const T *>(psi),
-                            static_cast<T *>(gout), P, g.nx, g.ny, g.pitch, (unsigned)g.plane);
+    return launch_or_count(b, k_collide_site<T, BC>, grid, dim3(SPLIT_THREADS), st, gin, (const T *)psi, gout, P,
+                           g.nx, g.ny, g.pitch, (unsigned)g.plane);
 }
 
 template <typename T, int EOS>
-cudaError_t split_bc(const Consts &c, const Geom &g, const void *gin, void *psi, void *gout,
-                     int *err, cudaStream_t st) {
+cudaError_t split_bc(const Consts &c, const Geom &g, const StepBuffers &b, int *err, cudaStream_t st) {
     switch (g.walls) {
-        case 0: return split_launch<T, EOS, 0>(c, g, gin, psi, gout, err, st);
-        case 1: return split_launch<T, EOS, 1>(c, g, gin, psi, gout, err, st);
-        default: return split_launch<T, EOS, 2>(c, g, gin, psi, gout, err, st);
+        case 0: return split_launch<T, EOS, 0>(c, g, b, err, st);
+        case 1: return split_launch<T, EOS, 1>(c, g, b, err, st);
+        default: return split_launch<T, EOS, 2>(c, g, b, err, st);
     }
 }
 
