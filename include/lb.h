@@ -136,9 +136,9 @@ lb_status lb_init_ex(lb_ctx **out, int nx, int ny, const lb_eos *eos, double G, 
  * variant gives identical results. Contexts start with the variant that suits their type and
  * size: 7 for LB_FP64 and for LB_FP32 up to 40 MiB a buffer, 8 for LB_BF16, for LB_BC_OPEN
  * and up to 72 MiB, 4 beyond. An lb_step of several steps of an LB_FP32 context with the variant
- * it started with is one launch for lattices that fit the SMs' shared memory: of a 16-CTA cluster
- * up to 16384 sites (LB_BC_PERIODIC or LB_BC_WALLS_Y, even nx >= 4, ny >= 16, at most 512 site
- * pairs per 1/16 of the rows), of one CTA per SM from 32768 sites on as long as tiles of 64
+ * it started with is one launch for lattices that fit the SMs' shared memory: from 7 steps on, of a
+ * 16-CTA cluster, up to 16384 sites (LB_BC_PERIODIC or LB_BC_WALLS_Y, even nx >= 4, ny >= 16, at most 512 site
+ * pairs per 1/16 of the rows), from 10 steps on, of one CTA per SM, from 32768 sites on as long as tiles of 64
  * columns and at most 35 rows suffice (a cooperative launch, between 96 tiles and one per SM, the last of
  * a row at least two columns wide; an exchange buffer is allocated by the library, without it the
  * steps are single launches); also after lb_autotune, whatever variant it chose for single steps. LB_FP32 batches have

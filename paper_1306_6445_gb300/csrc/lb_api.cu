@@ -50,7 +50,14 @@ struct lb_ctx {
 namespace {
 
 const char *kNoCtx = "no context";
-constexpr int kManySteps = 1024;      // of one launch of the cluster or the resident kernel
+// Most steps of one launch of the cluster or the resident kernel, and the fewest (lb_ctx::many). Such
+// a launch loads the lattice, and the resident kernel sets up its exchange, for the time of several
+// single steps: together / singly, us, cluster kernel: 64^2 2 steps 11.6 / 5.7, 6 15.4 / 13.7, 7 15.5 /
+// 15.8, 24 30 / 51; resident kernel: 501 x 383 2 steps 21.9 / 10.1, 8 40.3 / 36.9, 10 46.4 / 45.9, 12 52.5
+// / 55.1, 24 89 / 108; 600 x 225 splash 10 43.8 / 43.3, 24 87 / 102. The lines lie where the first
+// lattice gains; others gain later (128^2 from 20 steps on, 512^2 from 35).
+constexpr int kManySteps = 1024;
+constexpr int kManyLeast[3] = {0, 7, 10};
 
 lb_status fail(lb_ctx *c, lb_status s, const std::string &m) {
     if (c) c->msg = m;
@@ -626,7 +633,7 @@ lb_status lb_step(lb_ctx *c, int n) {
     if (n < 0) return fail(c, LB_EINVAL, "lb_step: n < 0");
     // a lattice that fits the SMs takes several steps in one launch (at most kManySteps: a few
     // milliseconds)
-    while (c->many && n > 1) {
+    while (c->many && n >= kManyLeast[c->many]) {
         const int m = std::min(n, kManySteps);
         const void *gin = c->f[c->cur];
         void *gout = c->f[c->cur ^ (m & 1)];     // the buffer that m launches would end in
