@@ -243,7 +243,8 @@ k_macro_reduce(const T *__restrict__ g, const Arith<T> *__restrict__ psi,
         if (!(f2 < least)) {           // also NaN
             const double v2 = dvx * dvx + dvy * dvy;
             q[3] = (v2 > q[3] || v2 != v2) ? v2 : q[3];
-            least = (float)q[3] * 0.99999f;
+            const float most = (float)q[3];
+            least = most > 1e-30f ? most * 0.99999f : -1.f;   // (f2 of less is subnormal: too coarse)
         }
     }
     block_combine<4, 3>(q, partials + (size_t)blockIdx.x * 4);
