@@ -294,7 +294,13 @@ k_droplet_sums(const T *__restrict__ g, const DevConsts<Arith<T>> P, int nx, int
 
 // Interface height per column (Sec. V.B), pass 1: thread (x, segment) scans the rows of
 // its segment upward and records the first row whose density is below rho_mid in
-// first[x] (atomicMin: the minimum does not depend on the order of the updates).
+// first[x] (atomicMin: the minimum does not depend on the order of the updates). What bounds it: the
+// latency of one row's loads after another, so two rows are loaded at a time, and with open sides,
+// whose conditions keep a row's loads apart, without conditions away from the top and bottom.
+// lb_interface_height, whole columns scanned, one row at a time / as here: 4096 x 2048 with walls FP32
+// 122 / 106 us, 1000 x 700 with walls FP64 69 / 68, 600 x 225 open FP64 101 / 69, 2048^2 open FP32 111 / 88,
+// 16 x 60000 periodic FP64 160 / 130. Four rows took 118, 74, 80, 117, 154; without conditions with walls
+// 136 and 70.
 template <typename T, int BC>
 __global__ void k_interface_first(const T *__restrict__ g, const DevConsts<Arith<T>> P, int nx,
                                   int ny, int pitch, unsigned plane, double rho_mid, int seg,
@@ -302,13 +308,29 @@ __global__ void k_interface_first(const T *__restrict__ g, const DevConsts<Arith
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= nx) return;
     const int y0 = blockIdx.y * seg, y1 = min(ny, y0 + seg);
-    for (int y = y0; y < y1; ++y) {
-        Arith<T> v[9];
-        pull_site_vals<T, BC>(v, g, x, y, ny, pitch, plane, P);
-        if (double(sum9(v)) < rho_mid) {
-            atomicMin(&first[x], y);
-            return;
+    constexpr int AHEAD = 2;
+    for (int y = y0; y < y1; y += AHEAD) {
+        Arith<T> rho[AHEAD];
+        const bool inner = BC == 2 && y > 0 && y + AHEAD < ny && y + AHEAD <= y1;
+#pragma unroll
+        for (int k = 0; k < AHEAD; ++k) {
+            Arith<T> v[9];
+            if (inner) {
+#pragma unroll
+                for (int a = 0; a < 9; ++a)
+                    v[a] = pop_dec<T>(g[(size_t)plane_of(a) * plane + (unsigned)(y + k - EYv(a)) * (unsigned)pitch +
+                                        (unsigned)(x - EXv(a) + GH<T>)], a, P);
+            } else {
+                pull_site_vals<T, BC>(v, g, x, min(y + k, y1 - 1), ny, pitch, plane, P);
+            }
+            rho[k] = sum9(v);
         }
+#pragma unroll
+        for (int k = 0; k < AHEAD; ++k)
+            if (double(rho[k]) < rho_mid) {
+                atomicMin(&first[x], min(y + k, y1 - 1));
+                return;
+            }
     }
 }
 
