@@ -7,6 +7,7 @@
 #include <climits>
 #include <cmath>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <new>
 #include <string>
@@ -27,10 +28,11 @@ struct lb_ctx {
     bool own_f = false;
     int cur = 0;                 // buffer holding the current state g (f = pull of g)
     int num_sms = 0;
-    lbm::HostWords *words = nullptr;   // page-locked: error bits and reduction results
+    lbm::HostWords *words = nullptr;   // host memory: error bits and reduction results (make_words)
+    bool words_locked = false;         // page-locked by the runtime
     int *d_err = nullptr;        // = &words->err, as the kernels address it
     double *d_out8 = nullptr;    // = words->out8, as the kernels address it
-    unsigned *d_ticket = nullptr;      // of the reductions
+    unsigned *d_ticket = nullptr;      // of the reductions (behind d_partials)
     double *d_field = nullptr;   // diagnostics: two nx*ny double fields
     double *d_partials = nullptr;  // 8 doubles per reduction block
     int *d_first = nullptr;        // interface height: nx ints
@@ -290,7 +292,7 @@ lb_status check_usable(lb_ctx *c) {
 }
 
 // Wait for the stream and fold device error bits into the sticky status. The kernels write them
-// (and a reduction's results) into page-locked host memory, so there is nothing to copy: a wait
+// (and a reduction's results) into host memory, so there is nothing to copy: a wait
 // and a blocking copy of the error word took 14 us, the wait alone takes 5.
 lb_status sync_and_check(lb_ctx *c) {
     LB_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -302,11 +304,45 @@ lb_status sync_and_check(lb_ctx *c) {
     return LB_OK;
 }
 
+// The words that the kernels write and the host reads. Where the GPU reads the host's page tables
+// (GB300) they are ordinary memory: a page-locked allocation and its release take 270 us, which made
+// lb_init and lb_free of a 64^2 lattice 560 us (55 now).
+cudaError_t make_words(lb_ctx *c, int dev) {
+    constexpr size_t line = 128;         // whole cache lines, nothing else in them
+    static_assert(sizeof(lbm::HostWords) <= line, "one line");
+    int host_tables = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&host_tables, cudaDevAttrPageableMemoryAccessUsesHostPageTables, dev);
+    if (e != cudaSuccess) return e;
+    void *host = nullptr, *device = nullptr;
+    if (host_tables) {
+        host = device = std::aligned_alloc(line, line);
+        if (!host) return cudaErrorMemoryAllocation;
+    } else {
+        e = cudaHostAlloc(&host, line, cudaHostAllocMapped);
+        c->words_locked = e == cudaSuccess;
+    }
+    c->words = static_cast<lbm::HostWords *>(host);
+    if (e == cudaSuccess && !host_tables) e = cudaHostGetDevicePointer(&device, host, 0);
+    if (e != cudaSuccess) return e;
+    std::memset(host, 0, line);
+    c->d_err = &static_cast<lbm::HostWords *>(device)->err;
+    c->d_out8 = static_cast<lbm::HostWords *>(device)->out8;
+    return cudaSuccess;
+}
+
 lb_status ensure_diag(lb_ctx *c) {
     const size_t n = (size_t)c->geom.nx * c->geom.ny;
     if (!c->d_field) LB_CUDA(c, cudaMalloc(&c->d_field, 2 * n * sizeof(double)));
-    if (!c->d_partials)
-        LB_CUDA(c, cudaMalloc(&c->d_partials, 8 * sizeof(double) * lbm::reduce_blocks((long long)n)));
+    if (!c->d_partials) {
+        const size_t k = 8 * (size_t)lbm::reduce_blocks((long long)n);
+        double *partials = nullptr;
+        LB_CUDA(c, cudaMalloc(&partials, (k + 1) * sizeof(double)));
+        const cudaError_t e = cudaMemsetAsync(partials + k, 0, sizeof(double), c->stream);
+        if (e != cudaSuccess) cudaFree(partials);
+        LB_CUDA(c, e);
+        c->d_partials = partials;
+        c->d_ticket = reinterpret_cast<unsigned *>(partials + k);
+    }
     if (!c->d_first) LB_CUDA(c, cudaMalloc(&c->d_first, sizeof(int) * (size_t)c->geom.nx));
     return LB_OK;
 }
@@ -359,18 +395,11 @@ lb_status create(lb_ctx **out, int nx, int ny, const lb_eos *eos, double G, doub
             return lbm::reported(LB_ENOMEM);
         }
     }
-    lbm::HostWords *dev_words = nullptr;
-    if (cudaMalloc(&c->d_ticket, sizeof(unsigned)) != cudaSuccess ||
-        cudaHostAlloc(&c->words, sizeof(lbm::HostWords), cudaHostAllocMapped) != cudaSuccess ||
-        cudaHostGetDevicePointer(&dev_words, c->words, 0) != cudaSuccess) {
+    if (make_words(c, dev) != cudaSuccess) {
         lb_free(c);
         return lbm::reported(LB_ENOMEM);
     }
-    std::memset(c->words, 0, sizeof(lbm::HostWords));
-    c->d_err = &dev_words->err;
-    c->d_out8 = dev_words->out8;
-    if (cudaMemsetAsync(c->d_ticket, 0, sizeof(unsigned), c->stream) != cudaSuccess ||
-        cudaMemsetAsync(c->f[0], 0, bytes, c->stream) != cudaSuccess ||
+    if (cudaMemsetAsync(c->f[0], 0, bytes, c->stream) != cudaSuccess ||
         cudaMemsetAsync(c->f[1], 0, bytes, c->stream) != cudaSuccess ||
         cudaStreamSynchronize(c->stream) != cudaSuccess) {
         lb_free(c);
@@ -796,14 +825,16 @@ void lb_free(lb_ctx *c) {
         cudaFree(c->f[0]);
         cudaFree(c->f[1]);
     }
-    cudaFree(c->d_ticket);
-    cudaFreeHost(c->words);
     cudaFree(c->d_field);
     cudaFree(c->d_partials);
     cudaFree(c->d_first);
     cudaFree(c->d_host_in);
     cudaFree(c->d_psi);
     cudaFree(c->d_words);
+    // as cudaFree does, for what other streams (replayed captures) may still write there
+    if (c->words) cudaDeviceSynchronize();
+    if (c->words_locked) cudaFreeHost(c->words);
+    else std::free(c->words);
     delete c;
 }
 

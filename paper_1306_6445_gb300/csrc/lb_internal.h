@@ -217,7 +217,7 @@ cudaError_t launch_psi_field(int prec, const Consts &c, const Geom &g, const voi
 cudaError_t launch_macro_fields(int prec, const Consts &c, const Geom &g, const void *gbuf,
                                 const void *psi, double *rho, double *ux, double *uy,
                                 cudaStream_t stream);
-// Words of a context that its kernels write into page-locked host memory: after a wait for the
+// Words of a context that its kernels write into host memory: after a wait for the
 // stream the host reads them, without a copy. Error bits are written only when there is an error.
 struct HostWords {
     int err;
