@@ -380,7 +380,9 @@ lb_status lb_batch_measure(lb_batch *b, const double *radius, double *out);
  * current states (set them first: the cost of a step depends on the state), after the
  * populations, per-lattice error flags, phase and step count have been saved to a
  * temporary device buffer the size of the batch's pool; they are restored afterwards, so
- * the batch is unchanged. Writes the choice if the pointers are not NULL. Synchronises.
+ * the batch is unchanged. A batch of several groups that then has variant 8 keeps the fastest ring
+ * variant beside it for calls of one step, or of up to 2 or 4, where that is faster. Writes the
+ * choice if the pointers are not NULL. Synchronises.
  * Errors: LB_EINVAL, LB_ENOMEM (no room for the copy; nothing changed), LB_ECUDA. */
 lb_status lb_batch_autotune(lb_batch *b, int trial_steps, int *variant, int *rows);
 

@@ -52,9 +52,16 @@ struct BatchCommon {
     std::vector<lbm::Consts> consts;
     std::vector<size_t> off[2];          // byte offsets of each lattice's two buffers
     void *pool = nullptr;                // all population buffers
-    void *d_maps = nullptr;              // 2 CUtensorMap per lattice
+    void *d_maps = nullptr;              // 2 CUtensorMap per lattice, of the staged tiles
     void *d_lats = nullptr;              // BatchLattice<T> table
-    lbm::BatchItem *d_items = nullptr;
+    // A ring variant's launch: all lattices, one step. `ring` is the batch's where its variant is one;
+    // `few` takes the calls of up to few_steps steps beside the staged tiles (lb_batch_autotune).
+    struct Ring {
+        int variant = 0, rows = 0, grid = 0, n_items = 0;
+        lbm::BatchItem *d_items = nullptr;
+        void *d_maps = nullptr;          // 2 CUtensorMap per lattice
+    } ring, few;
+    int few_steps = 0;
     int n_items = 0;
     // Lattices that take their steps together (lb_batch_step): the staged tiles (variant 8) have
     // groups that stay in L2, the ring variants one group of all items.
@@ -76,7 +83,7 @@ struct BatchCommon {
     int n_chunks = 0;
     int *h_errs = nullptr;                   // page-locked: error words, radii, measured sums
     double *h_radius = nullptr, *h_meas = nullptr;
-    int variant = 0, rows = 16, grid = 0, ctas_per_sm = 1, num_sms = 0;
+    int variant = 0, rows = 16, grid = 0, num_sms = 0;
     int phase = 0;                       // which buffer holds the active lattices' state
     std::vector<unsigned char> active;   // lattices stepped by lb_batch_step
     std::vector<long long> lat_steps;    // steps taken by each lattice
@@ -269,7 +276,7 @@ cudaError_t ensure_side(lb_batch *b) {
 }
 
 // the tensor maps of every lattice's two buffers, for boxes of cols x rows x planes
-lb_status make_maps(lb_batch *b, int cols, int rows, int planes) {
+lb_status make_maps(lb_batch *b, int cols, int rows, int planes, void **d_maps) {
     EncodeTiledFn enc = batch_encode_fn();
     if (!enc) return bfail(b, LB_ECUDA, "cuTensorMapEncodeTiled unavailable");
     std::vector<CUtensorMap> maps(2 * (size_t)b->n);
@@ -288,9 +295,34 @@ lb_status make_maps(lb_batch *b, int cols, int rows, int planes) {
             if (r != CUDA_SUCCESS) return bfail(b, LB_ECUDA, "cuTensorMapEncodeTiled failed");
         }
     }
-    LB_BCUDA(b, cudaMemcpy(b->d_maps, maps.data(), maps.size() * sizeof(CUtensorMap),
+    if (!*d_maps) LB_BCUDA(b, cudaMalloc(d_maps, maps.size() * sizeof(CUtensorMap)));
+    LB_BCUDA(b, cudaMemcpy(*d_maps, maps.data(), maps.size() * sizeof(CUtensorMap),
                            cudaMemcpyHostToDevice));
     return LB_OK;
+}
+
+void drop_ring(BatchCommon::Ring &r) {
+    cudaFree(r.d_items);
+    cudaFree(r.d_maps);
+    r = {};
+}
+
+lb_status make_ring(lb_batch *b, int variant, int rows, BatchCommon::Ring &r) {
+    const int tx = lbm::step_variant_tx(variant);
+    int occ = 0;
+    LB_BCUDA(b, lbm::configure_batch(b->prec, b->eos_kind, variant, &occ));
+    std::vector<lbm::BatchItem> items;
+    if (!make_items(b, tx, rows, items)) return bfail(b, LB_EINVAL, "bad strip decomposition");
+    cudaFree(r.d_items);
+    r.d_items = nullptr;
+    LB_BCUDA(b, cudaMalloc(&r.d_items, items.size() * sizeof(lbm::BatchItem)));
+    LB_BCUDA(b, cudaMemcpy(r.d_items, items.data(), items.size() * sizeof(lbm::BatchItem),
+                           cudaMemcpyHostToDevice));
+    r.n_items = (int)items.size();
+    r.variant = variant;
+    r.rows = rows;
+    r.grid = std::min(r.n_items, b->num_sms * std::max(occ, 1));
+    return make_maps(b, tx + lbm::ghost_of_prec(b->prec) + 4, 1, lbm::step_variant_planes(variant), &r.d_maps);
 }
 
 lb_status apply_batch_launch(lb_batch *b, int variant, int rows) {
@@ -300,37 +332,23 @@ lb_status apply_batch_launch(lb_batch *b, int variant, int rows) {
     // of the direct kernels batches have the staged tiles, compiled for LB_FP32
     if (variant >= lbm::direct_variant())
         variant = b->prec == LB_FP32 ? lbm::staged_variant() : lbm::default_ring_variant();
+    b->few_steps = 0;
     if (variant == lbm::staged_variant()) {
         b->n_items = make_groups(b);
-        const lb_status st = make_maps(b, lbm::TILE_BOX_W, lbm::TILE_BOX_ROWS, 3);
+        const lb_status st = make_maps(b, lbm::TILE_BOX_W, lbm::TILE_BOX_ROWS, 3, &b->d_maps);
         if (st != LB_OK) return st;
-        b->variant = variant;
         b->rows = lbm::STAGED_ROWS;
-        b->ctas_per_sm = 1;
         b->grid = b->groups.empty() ? 0 : b->groups[0].n * b->groups[0].max_tiles;
         if (b->groups.size() > 1) LB_BCUDA(b, ensure_side(b));
-        renew_graphs(b);
-        return LB_OK;
+    } else {
+        const lb_status st = make_ring(b, variant, rows, b->ring);
+        if (st != LB_OK) return st;
+        b->n_items = b->ring.n_items;
+        b->rows = rows;
+        b->grid = b->ring.grid;
+        b->groups.assign(b->n_items > 0 ? 1 : 0, {});
     }
-    const int tx = lbm::step_variant_tx(variant);
-    int occ = 0;
-    LB_BCUDA(b, lbm::configure_batch(b->prec, b->eos_kind, variant, &occ));
-    std::vector<lbm::BatchItem> items;
-    if (!make_items(b, tx, rows, items)) return bfail(b, LB_EINVAL, "bad strip decomposition");
-    if (b->d_items) cudaFree(b->d_items);
-    b->d_items = nullptr;
-    LB_BCUDA(b, cudaMalloc(&b->d_items, items.size() * sizeof(lbm::BatchItem)));
-    LB_BCUDA(b, cudaMemcpy(b->d_items, items.data(), items.size() * sizeof(lbm::BatchItem),
-                           cudaMemcpyHostToDevice));
-    b->n_items = (int)items.size();
     b->variant = variant;
-    b->rows = rows;
-    b->ctas_per_sm = std::max(occ, 1);
-    b->grid = std::min(b->n_items, b->num_sms * b->ctas_per_sm);
-    b->groups.assign(b->n_items > 0 ? 1 : 0, {});
-    const lb_status st = make_maps(b, tx + lbm::ghost_of_prec(b->prec) + 4, 1,
-                                   lbm::step_variant_planes(variant));
-    if (st != LB_OK) return st;
     renew_graphs(b);
     return LB_OK;
 }
@@ -363,13 +381,17 @@ void count_steps(lb_batch *b, int n) {
         if (b->active[i]) b->lat_steps[i] += n;
 }
 
+cudaError_t launch_ring(const lb_batch *b, const BatchCommon::Ring &r, int phase, cudaStream_t st) {
+    return lbm::launch_batch_step(b->prec, b->eos_kind, r.variant, r.grid, r.d_maps, b->d_lats, r.d_items,
+                                  r.n_items, phase, b->d_errs, st);
+}
+
 cudaError_t launch_group(lb_batch *b, const BatchCommon::Group &g, int phase, cudaStream_t st) {
     const cudaError_t e =
         b->variant == lbm::staged_variant()
             ? lbm::batch_tile_f32(b->eos_kind, g.lattices, g.n, g.max_tiles, b->d_maps, b->d_lats, phase,
                                   b->d_errs, st)
-            : lbm::launch_batch_step(b->prec, b->eos_kind, b->variant, b->grid, b->d_maps, b->d_lats,
-                                     b->d_items, b->n_items, phase, b->d_errs, st);
+            : launch_ring(b, b->ring, phase, st);
     if (e == cudaSuccess) ++b->queued;
     return e;
 }
@@ -399,8 +421,16 @@ cudaError_t queue_groups(lb_batch *b, size_t first, size_t last, int n, int phas
     return e;
 }
 
+// n steps, launched one by one
 lb_status launch_steps(lb_batch *b, int n) {
-    if (n > 0) LB_BCUDA(b, queue_groups(b, 0, b->groups.size(), n, b->phase, b->stream));
+    if (n <= b->few_steps) {
+        for (int i = 0; i < n && b->few.n_items > 0; ++i) {
+            LB_BCUDA(b, launch_ring(b, b->few, b->phase ^ (i & 1), b->stream));
+            ++b->queued;
+        }
+    } else if (n > 0) {
+        LB_BCUDA(b, queue_groups(b, 0, b->groups.size(), n, b->phase, b->stream));
+    }
     b->direct_steps = std::min(b->direct_steps + std::min(n, kDirectSteps), kDirectSteps);
     b->phase ^= n & 1;
     count_steps(b, n);
@@ -655,11 +685,23 @@ lb_status lb_batch_autotune(lb_batch *b, int trial_steps, int *variant, int *row
         e = cudaMemcpyAsync(saved_errs, b->d_errs, b->n * sizeof(int), cudaMemcpyDeviceToDevice,
                             b->stream);
     const int cand_rows[] = {8, 12, 16, 24, 32};
-    float best = 1e30f;
-    int bv = v0, br = r0;
+    float best = 1e30f, best_ring = 1e30f;   // ms a step
+    int bv = v0, br = r0, ring_v = 0, ring_r = 0, few = 0;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (e == cudaSuccess) e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
+    // ms a step of `calls` calls of `steps` steps, 0 if they cannot be launched
+    auto timed = [&](int calls, int steps) {
+        float ms = 0;
+        if (launch_steps(b, steps) != LB_OK) return 0.f;           // warm-up
+        cudaEventRecord(e0, b->stream);
+        for (int i = 0; i < calls; ++i)
+            if (launch_steps(b, steps) != LB_OK) return 0.f;
+        cudaEventRecord(e1, b->stream);
+        e = cudaEventSynchronize(e1);
+        if (e == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
+        return ms / (float)(calls * steps);
+    };
     for (int v = 0; v < lbm::step_variant_count() && e == cudaSuccess; ++v) {
         for (int r : cand_rows) {
             if (v == lbm::direct_variant()) break;   // batches take the staged tiles
@@ -667,22 +709,26 @@ lb_status lb_batch_autotune(lb_batch *b, int trial_steps, int *variant, int *row
             if (apply_batch_launch(b, v, r) != LB_OK) continue;
             // the groups of the staged tiles keep their state in L2 over the steps of a call: they
             // are timed over a call of some length
-            const int steps = v == lbm::staged_variant() ? std::max(trial_steps, 16) : trial_steps;
-            if (launch_steps(b, 1) != LB_OK) continue;                 // warm-up
-            cudaEventRecord(e0, b->stream);
-            if (launch_steps(b, steps) != LB_OK) continue;
-            cudaEventRecord(e1, b->stream);
-            e = cudaEventSynchronize(e1);
-            float ms = 0;
-            if (e == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
-            ms /= (float)steps;
+            const float ms = v == lbm::staged_variant() ? timed(1, std::max(trial_steps, 16)) : timed(trial_steps, 1);
             if (ms > 0 && ms < best) {
                 best = ms;
                 bv = v;
                 br = b->rows;
             }
+            if (ms > 0 && ms < best_ring && v < lbm::direct_variant()) {
+                best_ring = ms;
+                ring_v = v;
+                ring_r = r;
+            }
         }
     }
+    // In calls of one step or a few nothing stays in L2, and the groups' many launches take longer than
+    // the ring kernel's one where memory is the bound: staged / ring, us a step, 512 lattices of 64^2 to
+    // 512^2 812 / 741 (calls of four 658), 2 of 1024^2 36.2 / 29.3 (29.8), 60 of 64^2 to 512^2 97.9 / 78.7
+    // (73.5); 24 of 128^2 11.2 / 12.9.
+    if (bv == lbm::staged_variant() && best_ring < 1e30f && e == cudaSuccess &&
+        apply_batch_launch(b, bv, br) == LB_OK && b->groups.size() > 1)
+        for (int k = 1; k <= 4 && e == cudaSuccess && best_ring < timed(8 / k, k); k *= 2) few = k;
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     // put the states back (whatever the trials did)
@@ -699,7 +745,9 @@ lb_status lb_batch_autotune(lb_batch *b, int trial_steps, int *variant, int *row
     if (e != cudaSuccess) return bfail(b, LB_ECUDA, cudaGetErrorString(e));
     if (e2 != cudaSuccess) return bfail(b, LB_ECUDA, cudaGetErrorString(e2));
     lb_status s = apply_batch_launch(b, bv, br);
+    if (s == LB_OK && few > 0) s = make_ring(b, ring_v, ring_r, b->few);
     if (s != LB_OK) return s;
+    b->few_steps = few;
     if (variant) *variant = bv;
     if (rows) *rows = br;
     return LB_OK;
@@ -807,7 +855,10 @@ lb_status lb_batch_set_active(lb_batch *b, const unsigned char *active) {
     for (int i = 0; i < b->n; ++i) b->active[i] = active[i] ? 1 : 0;
     lb_status s = b->prec == LB_FP32 ? upload_lattices<float>(b) : upload_lattices<double>(b);
     if (s != LB_OK) return s;
-    return apply_batch_launch(b, b->variant, b->rows);
+    const int few = b->few_steps;
+    if ((s = apply_batch_launch(b, b->variant, b->rows)) != LB_OK || few == 0) return s;
+    if ((s = make_ring(b, b->few.variant, b->few.rows, b->few)) == LB_OK) b->few_steps = few;
+    return s;
 }
 
 long long lb_batch_lattice_steps(const lb_batch *b, int i) {
@@ -833,7 +884,8 @@ void lb_batch_free(lb_batch *b) {
     cudaFree(b->pool);
     cudaFree(b->d_maps);
     cudaFree(b->d_lats);
-    cudaFree(b->d_items);
+    drop_ring(b->ring);
+    drop_ring(b->few);
     cudaFree(b->d_errs);
     cudaFree(b->d_stage);
     cudaFree(b->d_radius);

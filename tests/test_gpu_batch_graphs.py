@@ -145,3 +145,49 @@ def test_steps_that_fail(lbm, variant, partly):  # noqa: F811
         b.sync()
         assert b.steps_done == 2
     b.close()
+
+
+def step_us(b, calls=40):
+    t = []
+    for _ in range(7):
+        b.sync()
+        a = time.perf_counter()
+        for _ in range(calls):
+            b.step(1)
+        b.sync()
+        t.append((time.perf_counter() - a) / calls * 1e6)
+    return sorted(t)[3]
+
+
+def test_single_steps_of_a_tuned_batch(lbm):  # noqa: F811
+    """A batch tuned for many steps takes single ones no slower than its fastest ring launch, with the
+    bits of any other launch, also after a change of the active lattices."""
+    sides = [1024, 1000]
+    a, b = batch(lbm, sides), batch(lbm, sides)
+    a.autotune(8)
+    assert a.launch()["variant"] == 8 and a.steps_done == 0
+    ring = 1e9
+    for variant in range(7):
+        for rows in (8, 16, 24):
+            b.set_launch(variant, rows)
+            ring = min(ring, step_us(b))
+    assert step_us(a) < 1.1 * ring
+    a.close()
+    a = batch(lbm, sides)
+    a.autotune(8)
+    b.close()
+    b = batch(lbm, sides)
+    b.set_launch(4, 16)
+    for x in (a, b):
+        for n in (1, 2, 64, 3, 4, 1, 1):
+            x.step(n)
+    for i in range(2):
+        assert np.array_equal(a.populations(i), b.populations(i))
+    for x in (a, b):
+        x.set_active(np.array([0, 1], np.uint8))
+        for n in (1, 17, 2, 4):
+            x.step(n)
+    for i in range(2):
+        assert np.array_equal(a.populations(i), b.populations(i)) and a.lattice_steps(i) == b.lattice_steps(i)
+    a.close()
+    b.close()
