@@ -99,8 +99,9 @@ lb_status lb_mlp_forward(lb_mlp *m, const float *x, float *y, int n);
 
 /* For each query q[i] = (T/T_c, tau_v, sigma_target), bisection on kappa in
  * [kappa_lo, kappa_hi] (kappa_lo < kappa_hi < 1, T/T_c < 1) for predicted sigma =
- * sigma_target, using that sigma decreases with kappa (Eq. 22): 40 halvings, each one
- * forward pass on the GPU (one warp per query or two). kappa[i] receives the midpoint of the final bracket, or
+ * sigma_target, using that sigma decreases with kappa (Eq. 22): up to 40 halvings,
+ * each one forward pass on the GPU (one warp per query or two), ended once a halving moves
+ * neither end (adjacent floats after 24 to 30). kappa[i] receives the midpoint of the final bracket, or
  * NaN when the target lies outside [sigma(kappa_hi), sigma(kappa_lo)] as predicted.
  * 0 <= n <= 1 << 20. Errors: LB_EINVAL, LB_ENOMEM, LB_ECUDA. */
 lb_status lb_mlp_invert_kappa(lb_mlp *m, const float *q, int n, float kappa_lo,

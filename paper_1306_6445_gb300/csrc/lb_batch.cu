@@ -2,7 +2,7 @@
 // and parameters advanced together, plus per-lattice Laplace measurements on the GPU. FP32 batches
 // take their steps by groups of lattices whose state stays in L2 (k_batch_tile, queue_groups); FP64
 // and the ring variants by one persistent kernel per time step over all lattices (k_batch_step),
-// replayed from a captured CUDA graph, as is a batch of a single small group.
+// replayed from a captured CUDA graph. Steps of the groups are graphs too (launch_graphs).
 #include <cuda.h>
 #include <cuda_runtime.h>
 

@@ -374,7 +374,8 @@ __device__ __forceinline__ V2<T> eos_psi2(V2<T> rho, const PT &P, bool hi_valid,
         // In FP32 the three terms are rounded one by one: arg is a small difference of terms of
         // the order of rho, and the fused form (two operations fewer) rounds 2 a rho + 2/3, twice
         // their size; the pressure it left in a liquid at 0.8 T_c doubled the error of a droplet
-        // after 200 steps against FP64 (1.3e-6 against 6e-7).
+        // after 200 steps against FP64 (1.3e-6 against 6e-7). In FP64 the error of a run is the same
+        // either way (1.1e-15 of the largest population), and two operations fewer count.
         V arg;
         if constexpr (PLAIN)
             arg = ((q - V::all(P.sw.a) * (rho * rho)) - rho * V::all(T(1.0 / 3.0))) * V::all(P.two_over_G);
@@ -616,7 +617,9 @@ __device__ __forceinline__ void collide(V (&f)[9], const V (&pn)[9], const PT &P
     // at about 7e-9 per step. In FP32 it is f_0 plus what the moving populations lost, the two
     // sums over them formed alike: in a uniform fluid their roundings cancel, where rho - sum
     // f*_a adds the same one at every step (a 501 x 383 droplet after 200 steps, error against
-    // FP64: 7e-7 against 1.1e-6). In FP64 the eight f*_a sum to 4 (base_axis + base_diag) up
+    // FP64: 7.3e-7 against 1.1e-6; the unscaled moments of collide_plain had 6.2e-7 there, and more
+    // than these elsewhere: a 4096 x 2048 wave 6.6e-7 / 3.0e-7, 24 droplets of 128^2 1.3e-6 / 3.7e-7).
+    // In FP64 the eight f*_a sum to 4 (base_axis + base_diag) up
     // to their own unbiased roundings, two operations instead of nine.
     if constexpr (std::is_same<T, double>::value)
         f[0] = vfma(mfour, base_axis + base_diag, rho);

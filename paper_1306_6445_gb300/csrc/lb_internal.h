@@ -113,7 +113,6 @@ struct StepLaunch {
 
 // ---- kernels (lb_kernels.cu) -------------------------------------------------------
 int step_variant_count();
-int ring_variant_count();               // variants 0 .. ring_variant_count() - 1 use a TMA ring
 int direct_variant();                   // the variant of the direct kernels (lb_tile.cuh)
 int staged_variant();                   // their TMA-staged tiles (LB_FP32 and LB_BF16)
 bool direct_fits(const Geom &g);        // the direct kernels' grid holds the lattice

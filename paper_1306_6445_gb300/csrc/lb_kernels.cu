@@ -363,7 +363,6 @@ __global__ void k_interface_height(const T *__restrict__ g, const DevConsts<Arit
 // the variants of LB_STEP_VARIANTS (lb_step.cuh): strip width and planes per TMA box (9:
 // whole stored rows, 3: one plane group of the stage ring)
 int step_variant_count() { return 9; }
-int ring_variant_count() { return 7; }
 int direct_variant() { return 7; }
 int staged_variant() { return 8; }
 
@@ -404,8 +403,8 @@ int default_variant(int prec, const Geom &g) {
 
 int step_variant_planes(int variant) { return step_variant_kind(variant) ? 3 : 9; }
 
-// the ring launch that batches, and contexts the direct kernels do not fit, start with: the
-// stage ring, 128-column strips, S = 3
+// the ring launch that FP64 batches, FP32 contexts beyond 72 MiB a buffer and contexts the direct
+// kernels do not fit start with: the stage ring, 128-column strips, S = 3
 int default_ring_variant() { return 4; }
 
 StepLaunch make_step_launch(int prec, int eos_kind, const Geom &g, int num_sms, int variant,

@@ -1,6 +1,8 @@
-// The direct step kernels (launch variant 7): no staging ring, one short dependent chain per
-// step. FP32 and BF16 storage use k_tile_step, one CTA per tile of 64 x R sites; FP64 uses a
-// psi pass and a collision pass (k_psi_site, k_collide_site), one site per thread. Same state
+// The tile kernels: no staging ring, one short dependent chain per step. FP32 and BF16 storage use
+// one CTA per tile of 64 x R sites, which reads memory (k_tile_step, launch variant 7) or brings the
+// tile into shared memory first (k_staged_tile_step, variant 8; k_batch_tile, the same for groups of
+// lattices); FP64 uses a psi pass and a collision pass (k_psi_site, k_collide_site, variant 7), one
+// site per thread. Same state
 // layout, arithmetic and results, bit for bit, as the ring kernels of lb_step.cuh.
 #pragma once
 
