@@ -344,8 +344,8 @@ lb_status lb_batch_set_rho_u(lb_batch *b, int i, const double *rho, const double
 
 /* Advance every lattice n >= 0 time steps (queued; returns without waiting for them). Few operations
  * are queued: runs of 64 steps are one graph launch, with variant 8 and several groups of lattices
- * runs of 16 steps one per 48 groups. What is left of n, and with several groups the first 128 steps of
- * a batch and those after its launch or its active lattices have changed, is launched step by step
+ * runs of 64 (up to 8 groups), 32 (16) or 16 steps one per 48 groups. What is left of n, and with several
+ * groups the first 512 steps of a batch and those after its launch or its active lattices have changed, is launched step by step
  * and group by group, which takes as long as the GPU takes once its queue (about 1000 launches) is
  * full. Inside a capture of the caller's all steps are launched one by one. An error after some of the
  * steps were queued leaves the lattices at different times: the batch is poisoned with it. */

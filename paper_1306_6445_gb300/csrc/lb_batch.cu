@@ -20,19 +20,18 @@
 
 namespace {
 
-constexpr int kGraphSteps = 64;   // steps per captured graph of a batch of one group (even: the phase returns)
-// Several groups: graphs of 16 steps (even) of blocks of 48 groups each. lb_batch_step can return without
-// waiting only if it queues few operations: launched one by one, 64 steps of 512 lattices of 64^2 to
-// 512^2 (12 600 launches) hold the calling thread for 30.1 of their 39.2 ms and 64 of 24 x 128^2 for 0.38
-// of 0.40 ms; as graphs 0.1 of 39.25 ms and 0.01 of 0.36 ms. Blocks of 24, 12 or 6 groups took 39.6,
-// 40.7 and 45.2 ms (each starts and drains the three chains), graphs of 32 steps 38.7 ms, but twice as
-// long to make. Making them costs 4 us per launch and step, 13 ms for the 512 lattices, during which
-// the GPU takes the steps of the blocks before; so the first 128 steps of a batch, and after its
-// launch or active lattices have changed, are launched one by one (with graphs at once the first 64
-// steps took 44.5 against 39.2 ms).
-constexpr int kGroupSteps = 16;
+constexpr int kGraphSteps = 64;   // steps per captured graph (even: the phase returns)
+// Several groups: graphs of 64 steps of up to 8 groups, 32 of up to 16, 16 of more, in blocks of 48
+// groups. lb_batch_step can return without waiting only if it queues few operations: launched one by
+// one, 64 steps of 512 lattices of 64^2 to 512^2 (229 groups) hold the calling thread for 30 of their
+// 39.1 ms, of 24 x 128^2 (3 groups) for 0.39 of 0.40 ms; as graphs 0.1 of 39.25 ms and 0.004 of 0.33. The
+// shorter the graphs, the more the groups' states are read again and the chains started and drained
+// (24 x 128^2: 16 steps 359 us; the 512 lattices: 32 steps 38.7 ms, blocks of 24 or 12 groups 39.6 and
+// 40.7), the longer, the longer they take to make: 4 us per group and step (15 ms for the 512
+// lattices, during which the GPU takes the steps of the blocks before). So the first 512 steps of a
+// batch, and after its launch or active lattices have changed, are launched one by one.
 constexpr size_t kBlockGroups = 48;
-constexpr int kDirectSteps = 128;
+constexpr int kDirectSteps = 512;
 // Most sites of a group of the staged tiles (or one lattice): both buffers of the kChains groups
 // that run side by side (57 MB in FP32) stay in L2 over their steps. 64 steps of 512 lattices of
 // 64^2 to 512^2, sites / groups side by side: 2^18 / 3 39.4 ms, 2^18 / 2 45.8, 2^18 / 4 41.4, 0.7 2^18
@@ -88,8 +87,7 @@ struct BatchCommon {
     std::vector<unsigned char> active;   // lattices stepped by lb_batch_step
     std::vector<long long> lat_steps;    // steps taken by each lattice
     long long steps = 0;
-    // kGraphSteps steps of the one group, or kGroupSteps steps of each block of kBlockGroups groups,
-    // from phase 0 / 1
+    // graph_steps steps of each block of kBlockGroups groups from phase 0 / 1
     std::vector<cudaGraphExec_t> graphs[2];
     int direct_steps = 0;                // launched one by one since the groups were formed
     long long queued = 0;                // launches of steps, also of graphs of them
@@ -254,7 +252,10 @@ void renew_graphs(lb_batch *b) {
     for (auto &v : b->graphs) v.assign((b->groups.size() + kBlockGroups - 1) / kBlockGroups, nullptr);
 }
 
-int graph_steps(const lb_batch *b) { return b->groups.size() > 1 ? kGroupSteps : kGraphSteps; }
+int graph_steps(const lb_batch *b) {
+    const size_t n = b->groups.size();
+    return n <= 8 ? kGraphSteps : n <= 16 ? kGraphSteps / 2 : kGraphSteps / 4;
+}
 
 // A stream beside the batch's, with its priority (launches recorded into a graph keep it).
 cudaError_t side_stream(const lb_batch *b, cudaStream_t *st) {

@@ -1,4 +1,4 @@
-"""Batches of several groups of lattices: their steps are queued as graphs once the first 128 have been
+"""Batches of several groups of lattices: their steps are queued as graphs once the first 512 have been
 launched one by one, and give the bits of the ring kernel's single launch per step over blocks of
 groups, from either buffer, after a change of the active lattices and inside a capture. The calling
 thread is not held while the GPU works."""
@@ -27,8 +27,9 @@ def batch(lbm, sides, stream=None):  # noqa: F811
     return b
 
 
-# 2 groups, 3, 4 (15 lattices each), 50 (the second block has two), 49 (the second block has one)
-@pytest.mark.parametrize("sides", [[256] * 2, [512, 511, 301], [128] * 60, [511] * 50, [512] * 49])
+# 2 groups, 3, 4 (15 lattices each), 12 (graphs of 32 steps), 50 (of 16, the second block has two), 49
+# (the second block has one)
+@pytest.mark.parametrize("sides", [[256] * 2, [512, 511, 301], [128] * 60, [512] * 12, [511] * 50, [512] * 49])
 def test_bits_of_single_launches(lbm, sides):  # noqa: F811
     a, b = batch(lbm, sides), batch(lbm, sides)
     b.set_launch(4, 16)
@@ -41,18 +42,18 @@ def test_bits_of_single_launches(lbm, sides):  # noqa: F811
         assert a.steps_done == b.steps_done
 
     for x in (a, b):
-        x.step(100)                # one by one
-        x.step(60)                 # the last of these, then graphs
+        x.step(500)                # one by one
+        x.step(150)                # the last of these, then graphs
         x.step(16)
     same()
     for x in (a, b):
         x.step(1)                  # from the other buffer
-        x.step(35)
+        x.step(135)
     same()
     active[0] = 0
     for x in (a, b):
         x.set_active(active)
-        x.step(129 + 33)
+        x.step(513 + 133)
     same()
     a.close()
     b.close()
@@ -65,17 +66,17 @@ def test_captured_steps(lbm, warm):  # noqa: F811
     sides = [512, 511, 301]
     a, b = batch(lbm, sides, st.cuda_stream), batch(lbm, sides)
     if warm:
-        a.step(192)
-        b.step(192)
+        a.step(640)
+        b.step(640)
     a.sync()
     graph = torch.cuda.CUDAGraph()
     with torch.cuda.graph(graph, stream=st):
-        a.step(34)
+        a.step(70)
     with torch.cuda.stream(st):
         for _ in range(2):
             graph.replay()
     a.sync()
-    b.step(68)
+    b.step(140)
     for i in range(3):
         assert np.array_equal(a.populations(i), b.populations(i))
     a.close()
@@ -84,8 +85,8 @@ def test_captured_steps(lbm, warm):  # noqa: F811
 
 def test_the_calling_thread_is_not_held(lbm):  # noqa: F811
     b = batch(lbm, [128] * 60)
-    b.step(128)
-    b.step(16)                     # the graphs are made
+    b.step(512)
+    b.step(64)                     # the graphs are made
     held, whole = [], []
     for _ in range(5):
         b.sync()
