@@ -196,10 +196,10 @@ lb_status lb_get_launch(const lb_ctx *ctx, int *variant, int *tx, int *rows, int
 
 /* Test hook for the failure path of the bounded device-side waits: from the next lb_step
  * on, the step kernels wait for lattice row `row` in vain: it is never requested (as staged in
- * the shared-memory ring, or in a staged tile), or taken from an exchange word that nobody
- * publishes (many steps in one launch, from 32768 sites on). The CTAs that need it give up after
- * about a second per wait and the next synchronising call returns LB_ETIMEOUT. Nothing faults and no
- * copy is left in flight. While it is on, kernels that wait for nothing, or not for this row (variant
+ * the shared-memory ring), expected by every staged tile with bytes that nobody sends (variant 8),
+ * or taken from an exchange word that nobody publishes (many steps in one launch, from 32768 sites
+ * on). The CTAs that need it give up after about a second per wait and the next synchronising call
+ * returns LB_ETIMEOUT. Nothing faults and no copy is left in flight. While it is on, kernels that wait for nothing, or not for this row (variant
  * 7, the tiles of variant 8 beside a periodic seam, many steps of up to 16384 sites), are replaced by
  * variant 4. INT_MIN (the default) switches it off and the launch is what it was. Not part of the
  * method; for tests only. */

@@ -11,6 +11,8 @@
 // are plain scalar doubles.
 #pragma once
 
+#include <climits>
+
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -65,7 +67,8 @@ struct PlainConsts {
 template <typename T>
 struct DevConsts : ConstFields<T> {
     PlainConsts<T> sw;
-    int stall_row;
+    int stall_row;                         // test hook (lb_debug_stall_row): kernels that wait for rows,
+    unsigned vain_bytes;                   // and staged tiles
     // LB_BF16 stochastic rounding: the step of the launch (the counter)
     unsigned sr_step;
 };
@@ -121,6 +124,7 @@ inline DevConsts<T> to_dev(const Consts &c) {
     w.v_keep_V = T(1.0 - c.s_v_vapour); w.s_v_V = T(c.s_v_vapour);
     w.v_half_V = T(1.0 - 0.5 * c.s_v_vapour); w.v_src_V = T(-c.s_v_vapour);
     d.stall_row = c.stall_row;
+    d.vain_bytes = c.stall_row != INT_MIN ? 16 : 0;
     d.sr_step = c.step_key;
     return d;
 }

@@ -7,7 +7,6 @@
 #pragma once
 
 #include <algorithm>
-#include <climits>
 
 #include "lb_step.cuh"
 
@@ -259,11 +258,12 @@ __host__ __device__ constexpr int staged_ctas(int R, bool sr) {
     return 65536 / (32 * R * (sr ? 128 : 64));
 }
 
-// the test hook's row (see lb_debug_stall_row); batches have no such hook
+// bytes that a staged tile expects and nobody sends: none but for the test hook (lb_debug_stall_row),
+// which batches do not have
 template <typename T>
-__device__ __forceinline__ int stall_row_of(const DevConsts<T> &P) { return P.stall_row; }
+__device__ __forceinline__ unsigned vain_bytes(const DevConsts<T> &P) { return P.vain_bytes; }
 template <typename C>
-__device__ __forceinline__ constexpr int stall_row_of(const ConstFields<C> &) { return INT_MIN; }
+__device__ __forceinline__ constexpr unsigned vain_bytes(const ConstFields<C> &) { return 0; }
 
 // As tile_step, with the populations brought into shared memory by three TMA loads, so that a
 // pull is a load at a constant offset: no address arithmetic, no wrap (414 instead of 471 warp
@@ -297,13 +297,10 @@ __device__ __forceinline__ void staged_tile_step(const CUtensorMap *tmap,
     grid_dependency_wait();           // the previous step's state (programmatic dependent launch)
     grid_dependents_launch();
     if (staged && threadIdx.x == 0) {
-        mbar_arrive_expect_tx(&sm.bar, 9u * SM::ROWS * TILE_BOX_W * (unsigned)sizeof(T));
+        mbar_arrive_expect_tx(&sm.bar, 9u * SM::ROWS * TILE_BOX_W * (unsigned)sizeof(T) + vain_bytes(P));
 #pragma unroll
-        for (int q = 0; q < 3; ++q) { // rows outside the lattice (walls, open top) are zero-filled, not used
-            // test hook: the bytes of a box that holds this row stay expected and never come
-            if ((unsigned)stall_row_of(P) - (unsigned)(y0 - 2 + q) < (unsigned)SM::ROWS) continue;
+        for (int q = 0; q < 3; ++q)   // rows outside the lattice (walls, open top) are zero-filled, not used
             tma_load_3d(sm.pop + q * SM::GROUP, tmap, x0 + GH<T> - TILE_BOX_LEFT, y0 - 2 + q, 3 * q, &sm.bar);
-        }
     }
     if (staged || CONSTS) __syncthreads();   // the barrier is initialised, the constants are written
 
