@@ -90,6 +90,7 @@ struct BatchCommon {
     // graph_steps steps of each block of kBlockGroups groups from phase 0 / 1
     std::vector<cudaGraphExec_t> graphs[2];
     int direct_steps = 0;                // launched one by one since the groups were formed
+    bool no_graphs = false;              // one could not be made
     long long queued = 0;                // launches of steps, also of graphs of them
     lb_status sticky = LB_OK;
     std::string msg;
@@ -249,6 +250,7 @@ void drop_graphs(lb_batch *b) {
 void renew_graphs(lb_batch *b) {
     drop_graphs(b);
     b->direct_steps = 0;
+    b->no_graphs = false;
     for (auto &v : b->graphs) v.assign((b->groups.size() + kBlockGroups - 1) / kBlockGroups, nullptr);
 }
 
@@ -438,12 +440,17 @@ lb_status launch_steps(lb_batch *b, int n) {
     return LB_OK;
 }
 
+// The steps of a block of groups as a graph. The thread may be recording into another stream meanwhile,
+// in a mode that forbids it calls that this one makes (and ends the recording at the first): it is
+// relaxed for them.
 cudaError_t capture_graph(lb_batch *b, size_t first, size_t last, cudaGraphExec_t *exec) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) return e;
     cudaStream_t cap = nullptr;
     cudaGraph_t g = nullptr;
-    cudaError_t e = side_stream(b, &cap);
-    if (e != cudaSuccess) return e;
-    e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
+    e = side_stream(b, &cap);
+    if (e == cudaSuccess) e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
         const long long queued = b->queued;
         e = queue_groups(b, first, last, graph_steps(b), b->phase, cap);
@@ -453,20 +460,29 @@ cudaError_t capture_graph(lb_batch *b, size_t first, size_t last, cudaGraphExec_
     }
     if (e == cudaSuccess) e = cudaGraphInstantiate(exec, g, 0);
     if (g) cudaGraphDestroy(g);
-    cudaStreamDestroy(cap);
+    if (cap) cudaStreamDestroy(cap);
+    (void)cudaThreadExchangeStreamCaptureMode(&mode);
     return e;
 }
 
 // graph_steps steps as graphs, captured when they are first launched: those of a block of groups
-// while the GPU takes the steps of the block before.
+// while the GPU takes the steps of the block before. What cannot be captured (no memory for the
+// graph) is launched one by one.
 lb_status launch_graphs(lb_batch *b) {
     auto &graphs = b->graphs[b->phase];
     for (size_t k = 0; k < graphs.size(); ++k) {
-        const size_t first = k * kBlockGroups;
-        if (!graphs[k])
-            LB_BCUDA(b, capture_graph(b, first, std::min(first + kBlockGroups, b->groups.size()), &graphs[k]));
-        LB_BCUDA(b, cudaGraphLaunch(graphs[k], b->stream));
-        ++b->queued;
+        const size_t first = k * kBlockGroups, last = std::min(first + kBlockGroups, b->groups.size());
+        if (!graphs[k] && !b->no_graphs && capture_graph(b, first, last, &graphs[k]) != cudaSuccess) {
+            (void)cudaGetLastError();
+            graphs[k] = nullptr;
+            b->no_graphs = true;
+        }
+        if (graphs[k]) {
+            LB_BCUDA(b, cudaGraphLaunch(graphs[k], b->stream));
+            ++b->queued;
+        } else {
+            LB_BCUDA(b, queue_groups(b, first, last, graph_steps(b), b->phase, b->stream));
+        }
     }
     count_steps(b, graph_steps(b));   // even: the phase is unchanged
     return LB_OK;

@@ -192,3 +192,24 @@ def test_single_steps_of_a_tuned_batch(lbm):  # noqa: F811
         assert np.array_equal(a.populations(i), b.populations(i)) and a.lattice_steps(i) == b.lattice_steps(i)
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("sides,before", [([64] * 3, 2), ([512, 511, 301], 512)])   # 1 and 3 groups
+def test_steps_beside_a_capture_of_another_stream(lbm, sides, before):  # noqa: F811
+    """The thread records into a stream of its own while the batch, whose graphs are not made yet, steps
+    in another: the steps are taken, and the recording is not spoilt."""
+    st, other = torch.cuda.Stream(), torch.cuda.Stream()
+    a, b = batch(lbm, sides, st.cuda_stream), batch(lbm, sides)
+    a.step(before)
+    b.step(before)
+    a.sync()
+    _capture.begin(other.cuda_stream)
+    a.step(128)
+    graph = _capture.end(other.cuda_stream)
+    assert graph is not None
+    _capture.destroy(graph)
+    b.step(128)
+    for i in range(3):
+        assert np.array_equal(a.populations(i), b.populations(i))
+    a.close()
+    b.close()
