@@ -48,7 +48,7 @@ __host__ __device__ constexpr int max_items(int rows) { return RS_ROW_SLOTS * (R
 __host__ __device__ constexpr unsigned row_words(int tx, int ty) { return (unsigned)ty * RS_ROW_SLOTS * RS_W * (unsigned)tx; }
 __host__ __device__ constexpr unsigned col_words(int tx, int ny) { return (unsigned)tx * RS_COL_SLOTS * (unsigned)ny; }
 __host__ __device__ constexpr unsigned exchange_words(int tx, int ty, int ny) {
-    return row_words(tx, ty) + col_words(tx, ny) + 1;
+    return row_words(tx, ty) + col_words(tx, ny) + 4;   // (a sector: the copies stay aligned)
 }
 
 __device__ __forceinline__ uint64_t load_word(const uint64_t *p) {
@@ -83,7 +83,7 @@ __device__ __forceinline__ void bar_arrive(int id, int threads) {
 // What bounds it: the border's chain, in clocks of 501 x 383 (64 x 20 tiles): 2500 until the halo is
 // here, 1000 psi, 2100 collision and publishing, with the interior beside it; 2.3 us a step at
 // least. Per step, against a launch of the tile kernels per step: 256^2 2.3 / 2.7 us, 384^2 2.8 / 3.3,
-// 501 x 383 3.2 / 4.5, 512^2 3.7 / 4.4, 560^2 4.4 / 5.1, 600 x 225 splash 3.4 / 3.9. The same warps
+// 501 x 383 3.1 / 4.5, 512^2 3.7 / 4.4, 560^2 4.2 / 5.1, 600 x 225 splash 3.4 / 3.9. The same warps
 // for border and interior took 4.1 us at 501 x 383; polling one value after the other 3.7.
 template <int EOS, int BC>
 __global__ void __launch_bounds__(32 * (RS_BORDER + RS_INNER), 1)
