@@ -135,15 +135,17 @@ lb_status lb_init_ex(lb_ctx **out, int nx, int ny, const lb_eos *eos, double G, 
  * LB_FP64 lattices whose scratch cannot be allocated, take variant 4 in their place. Every
  * variant gives identical results. Contexts start with the variant that suits their type and
  * size: 7 for LB_FP64 and for LB_FP32 up to 40 MiB a buffer, 8 for LB_BF16, for LB_BC_OPEN
- * and up to 72 MiB, 4 beyond. An lb_step of several steps of an LB_FP32 context with the variant
- * it started with is one launch for lattices that fit the SMs' shared memory: from 7 steps on, of a
- * 16-CTA cluster, up to 16384 sites (LB_BC_PERIODIC or LB_BC_WALLS_Y, even nx >= 4, ny >= 16, at most 512 site
- * pairs per 1/16 of the rows), from 10 steps on, of one CTA per SM, from 32768 sites on as long as tiles of 64
- * columns and at most 35 rows suffice (a cooperative launch, between 96 tiles and one per SM, the last of
- * a row at least two columns wide; an exchange buffer is allocated by the library, without it the
- * steps are single launches); also after lb_autotune, whatever variant it chose for single steps. LB_FP32 batches have
- * variants 0-6 and 8 (7 is taken as 8) and start with 8, LB_FP64 batches 0-6 (7 and 8 are taken
- * as 4) and start with 4. */
+ * and up to 72 MiB, 4 beyond.
+ * An lb_step of several steps of an LB_FP32 context with the variant it started with, or the one that
+ * lb_autotune chose, is one launch for lattices that fit the SMs' shared memory: 7 steps or more of up
+ * to 16384 sites on a 16-CTA cluster (LB_BC_PERIODIC or LB_BC_WALLS_Y, even nx >= 4, ny >= 16, at most
+ * 512 site pairs per 1/16 of the rows), 10 steps or more of 32768 sites and up on one CTA per SM, as
+ * long as tiles of 64 columns and at most 35 rows suffice (a cooperative launch, between 96 tiles and
+ * one per SM, the last of a row at least two columns wide; an exchange buffer is allocated by the
+ * library). Without the buffer, or where the GPU has no room for such a launch, the steps are single
+ * launches.
+ * LB_FP32 batches have variants 0-6 and 8 (7 is taken as 8) and start with 8, LB_FP64 batches 0-6 (7
+ * and 8 are taken as 4) and start with 4. */
 int lb_launch_variants(void);
 
 /* Density-dependent viscosity of Sec. V.C (LB_BC_OPEN contexts): sites with rho < rho_1
@@ -344,10 +346,10 @@ lb_status lb_batch_set_rho_u(lb_batch *b, int i, const double *rho, const double
 
 /* Advance every lattice n >= 0 time steps (queued; returns without waiting for them). Few operations
  * are queued: runs of 64 steps are one graph launch, with variant 8 and several groups of lattices
- * runs of 64 (up to 8 groups), 32 (16) or 16 steps one per 48 groups. What is left of n, and with several
- * groups the first 512 steps of a batch and those after its launch or its active lattices have changed, is launched step by step
- * and group by group, which takes as long as the GPU takes once its queue (about 1000 launches) is
- * full. Inside a capture of the caller's all steps are launched one by one. An error after some of the
+ * runs of 64 (up to 8 groups), 32 (16) or 16 steps one per 48 groups. What is left of n, and with
+ * several groups the first 512 steps of a batch, and after its launch or its active lattices have
+ * changed, is launched step by step and group by group, which takes as long as the GPU takes once its
+ * queue (about 1000 launches) is full; so are steps whose graph cannot be made. Inside a capture of the caller's all steps are launched one by one. An error after some of the
  * steps were queued leaves the lattices at different times: the batch is poisoned with it. */
 lb_status lb_batch_step(lb_batch *b, int n);
 
